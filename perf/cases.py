@@ -185,13 +185,34 @@ def tolerance(case):
 # ---- a pass ---------------------------------------------------------------------------------
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """Per turn the calls that bring its prompts (sequences, kinds, tensors by name), and q, k, v of the decode steps."""
     n, hq, hkv, d, b = case["layers"], case["q_heads"], case["kv_heads"], case["head_dim"], case["batch"]
     gen = torch.Generator(device="cuda").manual_seed(int(seed))
 
     def normal(*shape):
         return torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
 
+    prompts = []
+    for turn in range(case["turns"]):
+        if not case["attend"]:
+            kinds = [_pieces(case, s, turn)[0] for s in range(b)]
+            total = sum(len(kind) for kind in kinds)
+            prompts.append([(list(range(b)), kinds, {"k": normal(n, total, hkv, d), "v": normal(n, total, hkv, d)})])
+            continue
+        calls = []
+        for s in range(b):
+            for kind in _pieces(case, s, turn):
+                t = len(kind)
+                calls.append(([s], [kind], {"q": normal(n, t, hq, d), "k": normal(n, t, hkv, d),
+                                            "v": normal(n, t, hkv, d)}))
+        prompts.append(calls)
+    q, k, v = (normal(case["turns"], case["steps"], n, b, h, d) for h in (hq, hkv, hkv))
+    return prompts, q, k, v
+
+
+def prepare(case, seed):
+    n, hq, hkv, d, b = case["layers"], case["q_heads"], case["kv_heads"], case["head_dim"], case["batch"]
     turns, steps = case["turns"], case["steps"]
     lens = _lengths(case)
     text = [before + after + (turns - 1) * case["later_text"] + turns * steps for before, _, after in lens]
@@ -203,23 +224,16 @@ def prepare(case, seed):
     if case["entry"] == "in_order":
         session.set_option("in_order_launches", 1)
 
-    prompts = []   # per turn: the calls that bring its prompts
-    for turn in range(turns):
-        if not case["attend"]:
-            kinds = [_pieces(case, s, turn)[0] for s in range(b)]
-            total = sum(len(k) for k in kinds)
-            prompts.append([(list(range(b)), [len(k) for k in kinds], np.concatenate(kinds), normal(n, total, hkv, d),
-                             normal(n, total, hkv, d))])
-            continue
-        calls = []
-        for s in range(b):
-            for kind in _pieces(case, s, turn):
-                t = len(kind)
-                calls.append((s, kind, normal(n, t, hq, d), normal(n, t, hkv, d), normal(n, t, hkv, d),
-                              torch.empty(n, t, hq, d, device="cuda", dtype=torch.bfloat16)))
-        prompts.append(calls)
+    drawn, q, k, v = _inputs(case, seed)
+    prompts = []   # per turn: the arguments of the calls that bring its prompts
+    for calls in drawn:
+        if case["attend"]:
+            prompts.append([(ids[0], kinds[0], t["q"], t["k"], t["v"], torch.empty_like(t["q"]))
+                            for ids, kinds, t in calls])
+        else:
+            prompts.append([(ids, [len(kind) for kind in kinds], np.concatenate(kinds), t["k"], t["v"])
+                            for ids, kinds, t in calls])
 
-    q, k, v = (normal(turns, steps, n, b, h, d) for h in (hq, hkv, hkv))
     out = torch.empty(turns, steps, n, b, hq, d, device="cuda", dtype=torch.bfloat16)
     if case["entry"] == "host":
         q, k, v, out = (t.cpu().pin_memory() for t in (q, k, v, out))
@@ -253,3 +267,75 @@ def run(state):
     if case["attend"]:
         outputs += [call[-1] for prompts in state["prompts"] for call in prompts]
     return outputs
+
+
+# ---- the same in 64 bits --------------------------------------------------------------------
+
+
+def _attention(q, q_visual, k, v, visual):
+    """Softmax attention of the last len(q) tokens of k and v, each over the tokens up to itself.
+
+    q: [new][hq][d]; k, v: [tokens][hkv][d]; where ``q_visual`` is given it scores the visual keys."""
+    new, hq, d = q.shape
+    tokens, hkv, _ = k.shape
+    group = hq // hkv
+    out = torch.empty_like(q)
+    at = torch.arange(tokens, device=q.device)
+    hidden = (at[None, :] > at[tokens - new:, None]).repeat(group, 1)          # [group * new][tokens]
+    step = max(1, int(2 ** 27 // (group * new * tokens)))
+    for h in range(0, hkv, step):
+        e = min(hkv, h + step)
+
+        def scores(x):
+            x = x[:, h * group:e * group].reshape(new, e - h, group, d).permute(1, 2, 0, 3).reshape(e - h, group * new, d)
+            return x @ k[:, h:e].permute(1, 2, 0)
+
+        s = scores(q)
+        if q_visual is not None:
+            s = torch.where(visual, scores(q_visual), s)
+        w = (s * d ** -0.5).masked_fill_(hidden, float("-inf")).softmax(-1)
+        o = (w @ v[:, h:e].permute(1, 0, 2)).reshape(e - h, group, new, d)
+        out[:, h * group:e * group] = o.permute(2, 0, 1, 3).reshape(new, (e - h) * group, d)
+    return out
+
+
+def exact(case, seed):
+    """Lazy attention written down directly: a lazy layer's queries and keys are its leader's, of all
+    tokens (gla) or of the visual ones; a generated token is text, and its query on visual keys is
+    the leader's in vla_qc, its own in vla_eq8."""
+    drawn, q, k, v = _inputs(case, seed)
+    n, steps, gla = case["layers"], case["steps"], case["mode"] == "gla"
+    kinds = _layer_kind(case)
+    leader = [max(x for x in range(l + 1) if not kinds[x]) for l in range(n)]
+    out = torch.empty(case["turns"], steps, n, case["batch"], case["q_heads"], case["head_dim"], device="cuda",
+                      dtype=torch.float64)
+    prompt_outs = [[torch.empty(t["q"].shape, device="cuda", dtype=torch.float64) for _, _, t in calls]
+                   if case["attend"] else [] for calls in drawn]
+    for s in range(case["batch"]):
+        for l in range(n):
+            c = leader[l]
+            keys, values, vis = [], [], []
+
+            def add(kind, key, key_lead, value):
+                visual = torch.from_numpy(kind != 0).cuda()
+                keys.append((key_lead if gla else torch.where(visual[:, None, None], key_lead, key)).double())
+                values.append(value.double())
+                vis.append(visual)
+                return torch.cat(keys), torch.cat(values), torch.cat(vis)
+
+            for turn, calls in enumerate(drawn):
+                for i, (ids, call_kinds, t) in enumerate(calls):
+                    if s not in ids:
+                        continue
+                    first = sum(len(x) for x in call_kinds[:ids.index(s)])
+                    kind = call_kinds[ids.index(s)]
+                    part = {name: x[:, first:first + len(kind)] for name, x in t.items()}
+                    kv = add(kind, part["k"][l], part["k"][c], part["v"][l])
+                    if case["attend"]:
+                        own = part["q"][c] if gla else torch.where(kv[2][-len(kind):, None, None], part["q"][c], part["q"][l])
+                        prompt_outs[turn][i][l] = _attention(own.double(), None, *kv)
+                kv = add(np.zeros(steps, np.uint8), k[turn, :, l, s], k[turn, :, c, s], v[turn, :, l, s])
+                lead_q = q[turn, :, c, s].double()
+                own_q = lead_q if gla else q[turn, :, l, s].double()
+                out[turn, :, l, s] = _attention(own_q, lead_q if case["mode"] == "vla_qc" else None, *kv)
+    return [out] + [x for outs in prompt_outs for x in outs]
