@@ -153,6 +153,7 @@ __device__ __forceinline__ void process_item_tc(WorkerState& st, const TcCtx* ct
                 P.qcache + ((static_cast<size_t>(it.k_layer) * P.max_seqs + it.seq_id) * P.hq + it.head) * D);
             for (int e = lane; e < n_heads * (D / 8); e += 32) dst[e] = src[e];
           }
+          fence_proxy_async();   // these generic-proxy writes precede the slot's next asynchronous refill
           __syncwarp();
         }
 #pragma unroll
@@ -193,8 +194,8 @@ __device__ __forceinline__ void process_item_tc(WorkerState& st, const TcCtx* ct
           t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, off));
         }
         const float m0 = fmaxf(m[x][0], t0), m1 = fmaxf(m[x][1], t1);   // finite: key 0 is always valid
-        const float c0 = exp2f(m[x][0] - m0), c1 = exp2f(m[x][1] - m1);
-        const float p0 = exp2f(s0 - m0), p1 = exp2f(s1 - m1), p2 = exp2f(s2 - m0), p3 = exp2f(s3 - m1);
+        const float c0 = ex2_approx(m[x][0] - m0), c1 = ex2_approx(m[x][1] - m1);
+        const float p0 = ex2_approx(s0 - m0), p1 = ex2_approx(s1 - m1), p2 = ex2_approx(s2 - m0), p3 = ex2_approx(s3 - m1);
         l[x][0] = fmaf(l[x][0], c0, p0 + p2);
         l[x][1] = fmaf(l[x][1], c1, p1 + p3);
         m[x][0] = m0;
@@ -318,16 +319,16 @@ __device__ __forceinline__ void process_item_tc(WorkerState& st, const TcCtx* ct
       }
     }
   }
-  finish_rows<D>(P, ctx[st.cons_k % kCtxSlots].ip, lane);
 }
 
 // A worker's life: take items (claimed from the list, or the pieces of its static ranges), keep
 // the tile ring full across item boundaries, process each item.  While item k is processed the
 // ring already fetches tiles of item k + 1 and the context of item k + 2 (descriptor, page ids)
 // arrives by asynchronous copies.
+// False if a wait ran out.
 template <int D, bool STATIC>
-__device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, uint32_t ring, uint64_t* full,
-                                                 RangeCursor* cursor, int32_t* stage, int wid, int lane) {
+__device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, uint32_t ring, uint64_t* full,
+                                                 RangeCursor* cursor, int32_t* stage, CtaDesc* cta, int wid, int lane) {
   auto ctx_of = [ctx](int k) -> const ItemPages& { return ctx[k % kCtxSlots].ip; };
   WorkerState st;
   worker_init(st, 0);
@@ -341,60 +342,77 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
     it = load_item(P, idx);
     return true;
   };
-  // ---- ahead of the wait for the previous kernel: the first items and their page ids (from the
+  // ---- ahead of the wait for the previous kernel: the first two items and their page ids (from the
   // launch plan, the step descriptors and the page tables, all written before that kernel
   // started), and the first tiles unless they could hold a new token that an earlier launch of the
-  // step stores (with the folded append the worker patches the new token's row itself)
+  // step stores (with the folded append the worker patches the new token's row itself).  After it,
+  // only the layer's inputs.
   Item first;
-  if (STATIC && P.wdesc != nullptr) {
-    // planned ahead: one read gives the first item, its first page ids and the cursor
-    if (wid >= P.part_workers) return;
-    if (!load_worker_desc(P, wid, ctx[0].ip, cursor, stage, lane)) return;
-    first = ctx[0].ip.item;
+  bool more;
+  if (STATIC) {
+    bool any = wid >= 0 && wid < P.part_workers;
+    if (P.wdesc != nullptr) {
+      // planned ahead: one read gives the first two items, the first page ids and the cursor
+      any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, cta, lane);
+      if (any) first = ctx[0].ip.item;
+    } else {
+      RangeCursor c;
+      any = any && cursor_init(c, part_view(P), wid);
+      if (lane == 0) *cursor = c;
+      __syncwarp();
+      any = any && take();
+      if (any) {
+        first = it;
+        begin_item_pages(ctx[0].ip, P, first, lane);
+        cp_async_wait_all();
+        __syncwarp();
+      }
+    }
+    if (!any) {
+      pdl_wait();   // (a warp without work may still merge)
+      return true;
+    }
     st.n_my = 1;
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRingTc);
     if (early_tiles) fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
-    begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
-  } else {
-    if (STATIC) {
-      if (wid >= P.part_workers) return;
-      RangeCursor c;
-      const bool any = cursor_init(c, part_view(P), wid, lane);
-      if (lane == 0) *cursor = c;
-      __syncwarp();
-      if (!any) return;
+    if (P.wdesc != nullptr) {
+      begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
+      it = ctx[1].ip.item;
+      more = it.n_pages > 0;
     } else {
-      pdl_wait();   // the item list and the work counter are the previous kernel's
-      pdl_launch_dependents();
-      issued = claim_issue(P, lane);
+      more = take();
     }
-    if (!take()) return;
-    begin_item_pages(ctx[0].ip, P, it, lane);
+    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    pdl_wait();
+    pdl_launch_dependents();
+  } else {
+    pdl_wait();   // the item list and the work counter are the previous kernel's
+    pdl_launch_dependents();
+    issued = claim_issue(P, lane);
+    if (!take()) return true;
     first = it;
+    begin_item_pages(ctx[0].ip, P, first, lane);
     cp_async_wait_all();
     __syncwarp();
     st.n_my = 1;
-    const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRingTc);
-    if (early_tiles) fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
+    fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
+    issued = claim_issue(P, lane);
   }
-  if (STATIC) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
-  // ---- this layer's inputs; the rest of the first tiles; the second item's context while they fly
   begin_new_rows(ctx[0].ip, P, first, lane, D);
-  fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
-  if (STATIC) record_row_slots(P, first, lane);
-  if (!STATIC) issued = claim_issue(P, lane);
-  bool more = take();
-  if (more) {
-    begin_item_pages(ctx[1].ip, P, it, lane);
-    begin_new_rows(ctx[1].ip, P, it, lane, D);
-    if (STATIC) record_row_slots(P, it, lane);
+  if (!STATIC) {
+    more = take();
+    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
   }
-  cp_async_wait_all();
+  cp_async_commit_group();
+  if (more) {
+    begin_new_rows(ctx[1].ip, P, it, lane, D);
+  }
+  cp_async_commit_group();   // the second item's inputs are waited for when the first item is done
+  if (STATIC) cp_async_wait_group<1>();
+  else cp_async_wait_all();
   __syncwarp();
   if (more) st.n_my = 2;
+  fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
   bool pending = false;   // a context is being filled for item st.n_my
   if (!STATIC && more) issued = claim_issue(P, lane);
 
@@ -408,7 +426,6 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
       if (more) {
         begin_item_pages(ctx[(k + 2) % kCtxSlots].ip, P, it, lane);
         begin_new_rows(ctx[(k + 2) % kCtxSlots].ip, P, it, lane, D);
-        if (STATIC) record_row_slots(P, it, lane);
         pending = true;
       }
     }
@@ -428,10 +445,11 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
     else if (shared) process_item_tc<D, 1, 4>(st, ctx, ring, full, P, lane);
     else process_item_tc<D, 2, 2>(st, ctx, ring, full, P, lane);   // own-query sweeps feed at most two layers here
     if (st.dead) break;
-    if (pending) {   // the context of item k + 2 has had this item's time to arrive
+    if (STATIC) record_row_slots(P, cur, lane);
+    if (k + 1 < st.n_my) {   // the contexts of items k + 1 and k + 2 have had this item's time to arrive
       cp_async_wait_all();
       __syncwarp();
-      st.n_my = k + 3;
+      if (pending) st.n_my = k + 3;
       pending = false;
     }
     st.cons_k = k + 1;
@@ -441,15 +459,18 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
     cp_async_wait_all();
     drain_ring<kRingTc>(st, full, P.debug_drop_tile ? kDebugSpinLimit : kSpinLimit);
   }
+  return !st.dead;
 }
 
 template <int D, bool STATIC>
-__global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_constant__ Params P) {
+__global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_tc_kernel(const __grid_constant__ Params P) {
   constexpr uint32_t kTile = kPage * D * 2;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_all[kWarps][kRingTc];
   __shared__ __align__(16) RangeCursor cursors[kWarps];
   __shared__ __align__(16) int32_t stages[kWarps][12];
+  __shared__ __align__(16) FinishSmem<D> finish;
+  __shared__ CtaDesc cta;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // swizzled tiles must sit on 1024-byte boundaries
@@ -463,9 +484,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     for (int s = 0; s < kRingTc; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
   }
+  if (threadIdx.x == 0) finish.dead = 0;
   __syncthreads();
 
-  attend_tc_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], worker_index(P, warp, kWarps), lane);
+  const bool ok = attend_tc_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], &cta, worker_index(P, warp), lane);
+  if (STATIC) finish_cta<D>(P, finish, cta, !ok, warp, lane);
 }
 
 template <int D>
@@ -475,18 +498,20 @@ constexpr int attend_tc_smem_bytes() {
 
 }  // namespace
 
+namespace {
+template <typename K>
+cudaError_t configure_attend(K kernel, int smem) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+}  // namespace
+
 cudaError_t configure_kernels_tc(int* attend_smem) {
-  cudaError_t e = cudaFuncSetAttribute(attend_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       attend_tc_smem_bytes<128>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           attend_tc_smem_bytes<128>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           attend_tc_smem_bytes<64>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_tc_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           attend_tc_smem_bytes<64>());
+  cudaError_t e = configure_attend(attend_tc_kernel<128, false>, attend_tc_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_tc_kernel<128, true>, attend_tc_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_tc_kernel<64, false>, attend_tc_smem_bytes<64>());
+  if (e == cudaSuccess) e = configure_attend(attend_tc_kernel<64, true>, attend_tc_smem_bytes<64>());
   if (attend_smem) *attend_smem = attend_tc_smem_bytes<128>();
   return e;
 }
@@ -494,7 +519,8 @@ cudaError_t configure_kernels_tc(int* attend_smem) {
 cudaError_t launch_attend_tc(const Params& p, int n_sms, cudaStream_t stream) {
   const int n_items = p.item_end - p.item_begin;
   if (!p.part_static && n_items <= 0) return cudaSuccess;
-  const int grid = min(n_sms, ((p.part_static ? p.part_workers : n_items) + kWarps - 1) / kWarps);
+  const int grid = p.part_static ? (p.part_workers + p.part_wpc - 1) / p.part_wpc
+                                 : min(n_sms * kAttendCtasPerSm, (n_items + kWarps - 1) / kWarps);
   if (p.d == 128) {
     if (p.part_static)
       return launch_pdl(attend_tc_kernel<128, true>, dim3(grid), dim3(kThreads), attend_tc_smem_bytes<128>(), stream, p);

@@ -98,6 +98,9 @@ __device__ __forceinline__ void cp_async_4(void* dst_smem, const void* src) {
 __device__ __forceinline__ void cp_async_16(void* dst_smem, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Programmatic dependent launch: the kernels of a decode step are launched back to back with
@@ -192,6 +195,44 @@ __device__ __forceinline__ size_t table_row(const Params& P, int layer, int stre
   return ((static_cast<size_t>(layer) * 4 + stream) * P.max_seqs + seq_id) * P.max_pages;
 }
 
+// 2^x, single MUFU instruction (2^-inf = 0; results below 2^-126 are 0)
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Two fp32 operations in one instruction: the pairs are adjacent elements.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint4& v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ float2 bf16x2_to_f32(uint32_t r) { return make_float2(__uint_as_float(r << 16), __uint_as_float(r & 0xffff0000u)); }
+__device__ __forceinline__ void bf16x8_to_f32x2(const uint4& r, float2* f) {
+  f[0] = bf16x2_to_f32(r.x), f[1] = bf16x2_to_f32(r.y), f[2] = bf16x2_to_f32(r.z), f[3] = bf16x2_to_f32(r.w);
+}
+
 // ------------------------------------------------------------------------------------------
 // per-warp tile ring
 // ------------------------------------------------------------------------------------------
@@ -206,7 +247,6 @@ __device__ __forceinline__ size_t table_row(const Params& P, int layer, int stre
 // Item descriptor and page ids of one item, as the ring needs them.
 struct ItemPages {
   Item item;
-  StepSeq sq;          // the item's sequence
   int32_t kv_head;     // item.head / group
   int32_t pad[3];
   uint4 new_k[16];     // folded append: the new token's k row of the item's K layer and the v row of its
@@ -218,67 +258,86 @@ struct WorkerState {
   int n_my;            // items this worker owns
   int cons_k;          // item being consumed
   int iss_k;           // item being fetched (cons_k or cons_k + 1)
-  int iss_page, iss_which;
+  int iss_pages;       // pages of it not yet requested (0: it has not been looked at, or is done)
+  int iss_which, iss_first, iss_last;   // stream of the next tile (0: K, 1 + x: V of consumer x), of a page's first and last tile
+  uint32_t iss_addr;   // where the next tile's page id is (shared memory)
+  int iss_kv_head;
   int iss_slot, cons_slot;
   uint32_t cons_phase;
   int in_flight;
   bool dead;           // a bounded wait ran out: stop fetching, drain, leave
   bool drop_next;      // test hook: the next tile's copy is left out
+  uint64_t policy;     // L2 policy of the tile copies
 };
 
 __device__ __forceinline__ void worker_init(WorkerState& st, int n_my) {
   st.n_my = n_my;
   st.cons_k = st.iss_k = 0;
-  st.iss_page = st.iss_which = 0;
+  st.iss_pages = st.iss_which = st.iss_first = st.iss_last = 0;
+  st.iss_addr = 0;
+  st.iss_kv_head = 0;
   st.iss_slot = st.cons_slot = 0;
   st.cons_phase = 0;
   st.in_flight = 0;
   st.dead = false;
   st.drop_next = false;
+  st.policy = l2_evict_first_policy();
 }
 
 // Issue the copy of the next tile.  D: head dim; RING: slots; TMAP: copy through the tensor
 // map (swizzled tile: two 64-element column halves per row when D == 128) instead of one
 // linear 16*D*2-byte bulk copy.  `ctx(k)` returns the ItemPages of the worker's k-th item.
+// What an item's tiles have in common is looked up once per item: a worker issues a copy for every
+// tile it consumes, between the arithmetic of two tiles, so each instruction here is on its path
+// (with the look-ups per tile, a proxy fence and a policy made for each copy, a copy cost 700
+// cycles and a page of a K and a V tile 3 100, in a CTA with every worker busy; now 550 and 2 500).  No proxy fence is needed for a slot that was only
+// read; where a worker writes into a tile (new rows, cleared rows) it fences itself.
 template <int D, int RING, bool TMAP, typename CtxFn>
 __device__ __forceinline__ bool issue_one(WorkerState& st, CtxFn ctx, uint32_t ring, uint64_t* full, const Params& P,
                                           int lane) {
   constexpr uint32_t kTile = kPage * D * 2;
-  if (st.dead || st.iss_k >= st.n_my || st.iss_k > st.cons_k + 1) return false;
-  const ItemPages& c = ctx(st.iss_k);
-  const int n_cons = c.item.n_cons;
-  if (st.iss_which == 0 && (c.item.flags & kFlagReadLogits)) st.iss_which = 1;   // scores come from the logit cache
-  int pid = c.pages[st.iss_which][st.iss_page];
+  if (st.iss_pages == 0) {   // the next item
+    if (st.dead || st.iss_k >= st.n_my || st.iss_k > st.cons_k + 1) return false;
+    const ItemPages& c = ctx(st.iss_k);
+    st.iss_pages = c.item.n_pages;
+    st.iss_first = (c.item.flags & kFlagReadLogits) ? 1 : 0;   // (scores from the logit cache: no K tile)
+    st.iss_last = c.item.n_cons;
+    st.iss_which = st.iss_first;
+    st.iss_kv_head = c.kv_head;
+    st.iss_addr = smem_u32(&c.pages[st.iss_first][0]);
+  }
+  int pid;
+  asm volatile("ld.shared.s32 %0, [%1];" : "=r"(pid) : "r"(st.iss_addr) : "memory");
   if (static_cast<uint32_t>(pid) >= static_cast<uint64_t>(P.n_pool_pages)) {   // never read outside the pool
     if (lane == 0) report_error(P.err, P.err_host, kErrBadPage);
     pid = 0;
   }
-  if (P.debug_drop_tile && st.drop_next) {
+  if (st.drop_next) {
     // test hook: count the tile as in flight without requesting it; its wait will run out
     st.drop_next = false;
   } else if (lane == 0) {
-    uint64_t* bar = &full[st.iss_slot];
+    uint64_t* bar = full + st.iss_slot;
     const uint32_t dst = ring + st.iss_slot * kTile;
-    fence_proxy_async();   // the slot's earlier generic-proxy accesses precede this async write
     mbar_expect_tx(bar, kTile);
-    const uint64_t policy = l2_evict_first_policy();
     if (TMAP) {
-      const int32_t row = (pid * P.hkv + c.kv_head) * kPage;
-      tensor_g2s_2d(dst, &P.tmap, 0, row, bar, policy);
-      if (D == 128) tensor_g2s_2d(dst + kTile / 2, &P.tmap, 64, row, bar, policy);
+      const int32_t row = (pid * P.hkv + st.iss_kv_head) * kPage;
+      tensor_g2s_2d(dst, &P.tmap, 0, row, bar, st.policy);
+      if (D == 128) tensor_g2s_2d(dst + kTile / 2, &P.tmap, 64, row, bar, st.policy);
     } else {
-      const uint16_t* src = P.pool + (static_cast<size_t>(pid) * P.hkv + c.kv_head) * (kPage * D);
-      bulk_g2s(dst, src, kTile, bar, policy);
+      const uint16_t* src = P.pool + (static_cast<size_t>(pid) * P.hkv + st.iss_kv_head) * (kPage * D);
+      bulk_g2s(dst, src, kTile, bar, st.policy);
     }
   }
   st.iss_slot = (st.iss_slot + 1 == RING) ? 0 : st.iss_slot + 1;
   st.in_flight++;
-  if (++st.iss_which > n_cons) {
-    st.iss_which = 0;
-    if (++st.iss_page == c.item.n_pages) {
-      st.iss_page = 0;
-      st.iss_k++;
-    }
+  constexpr uint32_t kStream = kMaxChunkPages * 4;   // bytes from one stream's page ids to the next one's
+  if (st.iss_which == st.iss_last) {   // next page
+    st.iss_addr -= (st.iss_last - st.iss_first) * kStream - 4;
+    st.iss_which = st.iss_first;
+    if (--st.iss_pages == 0) st.iss_k++;
+  } else {
+    st.iss_addr += kStream;
+    st.iss_which++;
   }
   return true;
 }
@@ -296,13 +355,15 @@ template <int D>
 __device__ __forceinline__ uint32_t wait_tile(WorkerState& st, uint32_t ring, uint64_t* full, const Params& P,
                                               int lane) {
   constexpr uint32_t kTile = kPage * D * 2;
-  uint64_t* bar = &full[st.cons_slot];
-  uint32_t done = mbar_try_wait(bar, st.cons_phase);
-  const uint32_t limit = P.debug_drop_tile ? kDebugSpinLimit : kSpinLimit;
-  for (uint32_t spin = 0; !done && spin < limit; ++spin) done = mbar_try_wait(bar, st.cons_phase);
-  if (!done) {
-    if (lane == 0) report_error(P.err, P.err_host, kErrTimeout);
-    st.dead = true;
+  uint64_t* bar = full + st.cons_slot;
+  if (!mbar_try_wait(bar, st.cons_phase)) {
+    uint32_t done = 0;
+    const uint32_t limit = P.debug_drop_tile ? kDebugSpinLimit : kSpinLimit;
+    for (uint32_t spin = 0; !done && spin < limit; ++spin) done = mbar_try_wait(bar, st.cons_phase);
+    if (!done) {
+      if (lane == 0) report_error(P.err, P.err_host, kErrTimeout);
+      st.dead = true;
+    }
   }
   return ring + st.cons_slot * kTile;
 }
@@ -345,7 +406,6 @@ __device__ __forceinline__ void begin_item_pages(ItemPages& c, const Params& P, 
     c.item = it;
     c.kv_head = it.head / P.group;
   }
-  if (lane >= 30) cp_async_16(reinterpret_cast<uint4*>(&c.sq) + (lane - 30), reinterpret_cast<const uint4*>(P.seqs + it.seq_idx) + (lane - 30));
   if (lane < it.n_pages) {
     cp_async_4(&c.pages[0][lane], P.table + table_row(P, it.k_layer, it.stream, it.seq_id) + it.first_page + lane);
     for (int x = 0; x < it.n_cons; ++x)
@@ -389,29 +449,31 @@ __device__ __forceinline__ int claim_take(const Params& P, int issued) {
 // static partition of a launch
 // ------------------------------------------------------------------------------------------
 //
-// The work of a launch is laid out in tiles: plan positions of the launch in order, inside a
-// position the listed sequences, inside a sequence the rows (one per query head, or per query
-// group with GQA), inside a row its pages, each page worth w tiles (one K tile unless the scores
-// come from the logit cache, one V tile per consumer) after a fixed part_row_cost per row (what
-// starting and finishing an item costs a worker).  The space of T tiles is cut into ranges of
-// part_q tiles; a page belongs to the range its first tile falls into.  Physical worker i takes
-// ranges i*part_k .. i*part_k + part_k - 1, which are adjacent, so it walks rows forward from one
-// starting point.  The pages of a row that one range owns are one piece: an Item whose partial
-// result goes to slot (range - range owning the row's first page) of the row's stream.  The host
-// plans part_q so that a range is at least as long as any page (every range between a row's
-// first and last owns a page of it: no slot is left unwritten), a piece has at most
-// kMaxChunkPages pages and a row at most slots_per_stream pieces; T < 2^31.
+// The work of a launch is laid out in tiles: listed sequences in order, inside a sequence the rows
+// (one per query head, or per query group with GQA), inside a row the launch's plan positions,
+// inside a position the row's pages, each page worth w tiles (one K tile unless the scores come
+// from the logit cache, one V tile per consumer) after a fixed part_row_cost (what starting and
+// finishing an item costs a worker).  The space of T tiles is cut into ranges of part_q tiles; a
+// page belongs to the range its first tile falls into.  Physical worker i takes ranges i*part_k ..
+// i*part_k + part_k - 1, which are adjacent, so it walks forward from one starting point; the
+// workers of a CTA are adjacent too, so a CTA owns one stretch of tiles and with it, apart from the
+// rows at the two ends of the stretch, everything that the output rows in it need (finish_cta).
+// The pages of a row and position that one range owns are one piece: an Item whose partial result
+// goes to slot (range - range owning the first of those pages) of the row's stream.  The host plans
+// part_q so that a range is at least as long as any page (every range between a row's first and
+// last owns a page of it: no slot is left unwritten), a piece has at most kMaxChunkPages pages and
+// a row at most slots_per_stream pieces per stream; T < 2^31.
 
 struct __align__(16) RangeCursor {
-  int32_t r0;        // tile offset of the current row's first page
+  int32_t r0;        // tile offset of the first page of the current row and position
   int32_t vw_end;    // first tile beyond the current range
   int32_t vw, vw_stop;
   int32_t pos, si, u;
-  int32_t row_pages, w;     // pages of the current row; tiles per page of its job
-  int32_t page;             // next page of the current row to hand out
-  int32_t owner0;           // range that owns the row's first page
-  int32_t len, seq_id;      // tokens of the row's stream; its sequence
-  int32_t pad[3];
+  int32_t row_pages, w;     // pages of the current row and position; tiles per page of its job
+  int32_t page;             // next page to hand out
+  int32_t owner0;           // range that owns the first page
+  int32_t len_text, len_vis, seq_id;   // of the current sequence
+  int32_t pad[2];
   Job job;
 };
 static_assert(sizeof(RangeCursor) == 80, "RangeCursor layout");
@@ -424,9 +486,9 @@ struct PartView {
   int32_t* err;
   int32_t* err_host;
   int32_t pos_begin, pos_end, n_seqs;
-  int32_t q, k, vw, row_cost;          // tiles per range, ranges per worker, ranges, fixed tiles per row
-  int32_t tp_v, tp_t;                  // pages of the visual / text streams over the listed sequences
-  int32_t rows, heads_per_item, group, slots_per_stream;   // rows per (position, sequence); query heads per row
+  int32_t q, k, vw, row_cost;          // tiles per range, ranges per worker, ranges, fixed tiles per row and position
+  int32_t wv, wt;                      // tiles per page summed over the launch's visual / text positions
+  int32_t rows, heads_per_item, group, slots_per_stream;   // rows per sequence; query heads per row
 };
 
 __device__ __forceinline__ PartView part_view(const Params& P) {
@@ -434,156 +496,78 @@ __device__ __forceinline__ PartView part_view(const Params& P) {
   V.plan = P.plan, V.seqs = P.seqs, V.err = P.err, V.err_host = P.err_host;
   V.pos_begin = P.pos_begin, V.pos_end = P.pos_end, V.n_seqs = P.n_seqs;
   V.q = P.part_q, V.k = P.part_k, V.vw = P.part_vw, V.row_cost = P.part_row_cost;
-  V.tp_v = P.tp_v, V.tp_t = P.tp_t;
+  V.wv = P.part_wv, V.wt = P.part_wt;
   V.rows = P.heads_per_item_dim, V.heads_per_item = P.heads_per_item, V.group = P.group;
   V.slots_per_stream = P.slots_per_stream;
+  return V;
+}
+__device__ __forceinline__ PartView part_view(const Params& P, const LaunchDesc& L) {
+  PartView V = part_view(P);
+  V.pos_begin = L.pos_begin, V.pos_end = L.pos_end;
+  V.q = L.part_q, V.k = L.part_k, V.vw = L.part_vw, V.row_cost = L.part_row_cost;
+  V.wv = L.part_wv, V.wt = L.part_wt;
   return V;
 }
 
 __device__ __forceinline__ int job_tiles_per_page(const Job& j) {
   return ((j.flags & kFlagReadLogits) ? 0 : 1) + j.n_cons;
 }
+__device__ __forceinline__ int pages_of(int tokens) { return (tokens + kPage - 1) / kPage; }
 
-// Load the job of plan position c.pos (if it changed) and the sequence c.si into the cursor.
-__device__ __forceinline__ void cursor_load_segment(RangeCursor& c, const PartView& V, bool new_pos) {
-  if (new_pos) {
-    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(V.plan + c.pos));
-    *reinterpret_cast<uint4*>(&c.job) = raw;
-    c.w = job_tiles_per_page(c.job);
-  }
-  const StepSeq sq = V.seqs[c.si];
-  c.len = c.job.stream ? sq.len_vis : sq.len_text;
-  c.seq_id = sq.seq_id;
-  c.row_pages = (c.len + kPage - 1) / kPage;
+// Tile offset at which the rows of listed sequence si start; tiles of one of its rows.
+__device__ __forceinline__ int32_t seq_base(const PartView& V, int32_t pre_v, int32_t pre_t, int si) {
+  return V.rows * (V.wv * pre_v + V.wt * pre_t + V.row_cost * (V.pos_end - V.pos_begin) * si);
+}
+__device__ __forceinline__ int32_t row_tiles(const PartView& V, int32_t len_vis, int32_t len_text) {
+  return V.wv * pages_of(len_vis) + V.wt * pages_of(len_text) + V.row_cost * (V.pos_end - V.pos_begin);
 }
 
-// Tile offset at which the rows of a plan position start (index: its place in the launch).
-__device__ __forceinline__ int32_t pos_base_of(const PartView& V, int wv_before, int wt_before, int index) {
-  return V.rows * (wv_before * V.tp_v + wt_before * V.tp_t + V.row_cost * V.n_seqs * index);
-}
-
-// With position, job, sequence and its length in place: the row and page at which tile t0 falls.
-__device__ __forceinline__ void cursor_place(RangeCursor& c, const PartView& V, int32_t t0, int32_t pos_base,
-                                             int32_t my_pre) {
-  c.w = job_tiles_per_page(c.job);
-  c.row_pages = (c.len + kPage - 1) / kPage;
-  const int32_t seg_base = pos_base + V.rows * (c.w * my_pre + V.row_cost * c.si);
-  // a row costs its fixed part and then its pages; r0 is where its first page starts
-  const int32_t row_cost = V.row_cost + c.w * c.row_pages;
-  c.u = row_cost > 0 ? min(V.rows - 1, (t0 - seg_base) / row_cost) : 0;
-  c.r0 = seg_base + c.u * row_cost + V.row_cost;
-  c.page = t0 > c.r0 ? (t0 - c.r0 + c.w - 1) / c.w : 0;   // first page that starts at or after t0
-  c.owner0 = c.r0 / V.q;
-  c.pad[0] = c.pad[1] = c.pad[2] = 0;
-}
-
-// Place the cursor of worker `wid` at its first range; false if the worker has no work.  All
-// lanes of a warp compute the same values.  Reads the launch plan and the step's sequence
-// descriptors only, the first 32 of each in one round of loads.
-__device__ __forceinline__ bool cursor_init(RangeCursor& c, const PartView& V, int wid, int lane) {
-  c.vw = wid * V.k;
-  c.vw_stop = min(c.vw + V.k, V.vw);
-  if (c.vw >= c.vw_stop) return false;
-  const int32_t t0 = c.vw * V.q;
-  c.vw_end = t0 + V.q;
-  const int n_pos = V.pos_end - V.pos_begin;
-  uint4 pj_lo = make_uint4(0, 0, 0, 0);
-  int4 pj_hi = make_int4(0, 0, 0, 0);
-  int4 sq_lo = make_int4(0, 0, 0, 0), sq_hi = make_int4(0, 0, 0, 0);
-  if (lane < n_pos) {
-    pj_lo = __ldg(reinterpret_cast<const uint4*>(V.plan + V.pos_begin + lane));
-    pj_hi = __ldg(reinterpret_cast<const int4*>(V.plan + V.pos_begin + lane) + 1);
-  }
-  if (lane < V.n_seqs) {
-    sq_lo = reinterpret_cast<const int4*>(V.seqs + lane)[0];   // seq_id, len_text, len_vis, n_slots
-    sq_hi = reinterpret_cast<const int4*>(V.seqs + lane)[1];   // pre_v, pre_t, ncv, pad
-  }
-  // plan position: the last one of the launch that starts at or before t0
-  int n_le = __popc(__ballot_sync(0xffffffffu, lane < n_pos && pos_base_of(V, pj_hi.z, pj_hi.w, lane) <= t0));
-  int32_t pos_base;
-  if (n_le == 32 && n_pos > 32) {   // beyond the first round
-    for (int base = V.pos_begin + 32; base < V.pos_end; base += 32) {
-      const int idx = base + lane;
-      bool le = false;
-      if (idx < V.pos_end) {
-        const int4 hi = __ldg(reinterpret_cast<const int4*>(V.plan + idx) + 1);
-        le = pos_base_of(V, hi.z, hi.w, idx - V.pos_begin) <= t0;
-      }
-      n_le += __popc(__ballot_sync(0xffffffffu, le));
-    }
-    c.pos = V.pos_begin + n_le - 1;
-    const PlanJob pj = V.plan[c.pos];
-    c.job = pj.job;
-    pos_base = pos_base_of(V, pj.wv_before, pj.wt_before, c.pos - V.pos_begin);
-  } else {
-    const int src = max(n_le, 1) - 1;
-    c.pos = V.pos_begin + src;
-    uint4 j;
-    j.x = __shfl_sync(0xffffffffu, pj_lo.x, src);
-    j.y = __shfl_sync(0xffffffffu, pj_lo.y, src);
-    j.z = __shfl_sync(0xffffffffu, pj_lo.z, src);
-    j.w = __shfl_sync(0xffffffffu, pj_lo.w, src);
-    *reinterpret_cast<uint4*>(&c.job) = j;
-    pos_base = pos_base_of(V, __shfl_sync(0xffffffffu, pj_hi.z, src), __shfl_sync(0xffffffffu, pj_hi.w, src), src);
-  }
-  const int w = job_tiles_per_page(c.job);
-  // listed sequence: the last one whose rows start at or before t0
-  const int32_t rc = V.row_cost;
-  n_le = __popc(__ballot_sync(0xffffffffu, lane < V.n_seqs && pos_base + V.rows * (w * (c.job.stream ? sq_hi.x : sq_hi.y) + rc * lane) <= t0));
-  int32_t my_pre;
-  if (n_le == 32 && V.n_seqs > 32) {
-    for (int base = 32; base < V.n_seqs; base += 32) {
-      const int idx = base + lane;
-      bool le = false;
-      if (idx < V.n_seqs) le = pos_base + V.rows * (w * (c.job.stream ? V.seqs[idx].pre_v : V.seqs[idx].pre_t) + rc * idx) <= t0;
-      n_le += __popc(__ballot_sync(0xffffffffu, le));
-    }
-    c.si = n_le - 1;
-    const StepSeq sq = V.seqs[c.si];
-    c.len = c.job.stream ? sq.len_vis : sq.len_text;
-    c.seq_id = sq.seq_id;
-    my_pre = c.job.stream ? sq.pre_v : sq.pre_t;
-  } else {
-    const int src = max(n_le, 1) - 1;
-    c.si = src;
-    c.len = __shfl_sync(0xffffffffu, c.job.stream ? sq_lo.z : sq_lo.y, src);
-    c.seq_id = __shfl_sync(0xffffffffu, sq_lo.x, src);
-    my_pre = __shfl_sync(0xffffffffu, c.job.stream ? sq_hi.x : sq_hi.y, src);
-  }
-  cursor_place(c, V, t0, pos_base, my_pre);
-  return true;
-}
-
-// The same by one thread alone (the kernel that plans a step's launches ahead).
-__device__ __forceinline__ bool cursor_init_scalar(RangeCursor& c, const PartView& V, int wid) {
-  c.vw = wid * V.k;
-  c.vw_stop = min(c.vw + V.k, V.vw);
-  if (c.vw >= c.vw_stop) return false;
-  const int32_t t0 = c.vw * V.q;
-  c.vw_end = t0 + V.q;
-  c.pos = V.pos_begin;
-  int32_t pos_base = 0;
-  for (int p = V.pos_begin + 1; p < V.pos_end; ++p) {
-    const int4 hi = __ldg(reinterpret_cast<const int4*>(V.plan + p) + 1);
-    const int32_t b = pos_base_of(V, hi.z, hi.w, p - V.pos_begin);
-    if (b > t0) break;
-    c.pos = p;
-    pos_base = b;
-  }
-  c.job = V.plan[c.pos].job;
-  const int w = job_tiles_per_page(c.job);
+// The listed sequence and the row that tile t falls into; returns the row's first tile.
+__device__ __forceinline__ int32_t find_row(const PartView& V, int32_t t, int& si, int& u, StepSeq& sq) {
   int lo = 0, hi = V.n_seqs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    const int32_t pre = c.job.stream ? V.seqs[mid].pre_v : V.seqs[mid].pre_t;
-    if (pos_base + V.rows * (w * pre + V.row_cost * mid) <= t0) lo = mid;
+    if (seq_base(V, V.seqs[mid].pre_v, V.seqs[mid].pre_t, mid) <= t) lo = mid;
     else hi = mid - 1;
   }
-  c.si = lo;
-  const StepSeq sq = V.seqs[c.si];
-  c.len = c.job.stream ? sq.len_vis : sq.len_text;
-  c.seq_id = sq.seq_id;
-  cursor_place(c, V, t0, pos_base, c.job.stream ? sq.pre_v : sq.pre_t);
+  si = lo;
+  sq = V.seqs[lo];
+  const int32_t base = seq_base(V, sq.pre_v, sq.pre_t, lo), per_row = row_tiles(V, sq.len_vis, sq.len_text);
+  u = per_row > 0 ? min(V.rows - 1, (t - base) / per_row) : 0;
+  return base + u * per_row;
+}
+
+// Load the job of plan position c.pos into the cursor.
+__device__ __forceinline__ void cursor_load_job(RangeCursor& c, const PartView& V) {
+  const uint4 raw = __ldg(reinterpret_cast<const uint4*>(V.plan + c.pos));
+  *reinterpret_cast<uint4*>(&c.job) = raw;
+  c.w = job_tiles_per_page(c.job);
+  c.row_pages = pages_of(c.job.stream ? c.len_vis : c.len_text);
+}
+
+// Place the cursor of worker `wid` at its first range; false if the worker has no work.  Reads the
+// launch plan and the step's sequence descriptors only.
+__device__ __forceinline__ bool cursor_init(RangeCursor& c, const PartView& V, int wid) {
+  c.vw = wid * V.k;
+  c.vw_stop = min(c.vw + V.k, V.vw);
+  if (c.vw >= c.vw_stop) return false;
+  const int32_t t0 = c.vw * V.q;
+  c.vw_end = t0 + V.q;
+  StepSeq sq;
+  const int32_t row0 = find_row(V, t0, c.si, c.u, sq);
+  c.len_text = sq.len_text, c.len_vis = sq.len_vis, c.seq_id = sq.seq_id;
+  // the first position of the row whose pages do not all start before t0, or the last one
+  c.r0 = row0 + V.row_cost;
+  c.pos = V.pos_begin;
+  cursor_load_job(c, V);
+  while (c.pos + 1 < V.pos_end && c.r0 + c.w * c.row_pages <= t0) {
+    c.r0 += c.w * c.row_pages + V.row_cost;
+    ++c.pos;
+    cursor_load_job(c, V);
+  }
+  c.page = t0 > c.r0 ? (t0 - c.r0 + c.w - 1) / c.w : 0;   // first page that starts at or after t0
+  c.owner0 = c.r0 / V.q;
+  c.pad[0] = c.pad[1] = 0;
   return true;
 }
 
@@ -591,22 +575,22 @@ __device__ __forceinline__ bool cursor_init_scalar(RangeCursor& c, const PartVie
 __device__ __forceinline__ bool cursor_next(RangeCursor& c, const PartView& V, Item& it) {
   for (;;) {
     if (c.vw >= c.vw_stop) return false;
-    if (c.page >= c.row_pages) {   // next row
+    if (c.page >= c.row_pages) {   // next position, row, sequence
       c.r0 += c.w * c.row_pages + V.row_cost;
       c.page = 0;
-      if (++c.u == V.rows) {
-        c.u = 0;
-        bool new_pos = false;
-        if (++c.si == V.n_seqs) {
-          c.si = 0;
-          new_pos = true;
-          if (++c.pos >= V.pos_end) {
+      if (++c.pos == V.pos_end) {
+        c.pos = V.pos_begin;
+        if (++c.u == V.rows) {
+          c.u = 0;
+          if (++c.si == V.n_seqs) {
             c.vw = c.vw_stop;
             return false;
           }
+          const StepSeq sq = V.seqs[c.si];
+          c.len_text = sq.len_text, c.len_vis = sq.len_vis, c.seq_id = sq.seq_id;
         }
-        cursor_load_segment(c, V, new_pos);
       }
+      cursor_load_job(c, V);
       c.owner0 = c.r0 / V.q;
       continue;
     }
@@ -634,12 +618,11 @@ __device__ __forceinline__ bool cursor_next(RangeCursor& c, const PartView& V, I
       it.n_pages = static_cast<uint16_t>(lim - c.page);
       const bool last = lim == c.row_pages;
       if (last) it.flags |= kFlagStreamEnd;
-      it.n_valid_last = static_cast<uint16_t>(last ? c.len - (c.row_pages - 1) * kPage : kPage);
+      it.n_valid_last = static_cast<uint16_t>(last ? (c.job.stream ? c.len_vis : c.len_text) - (c.row_pages - 1) * kPage : kPage);
       it.n_heads = static_cast<uint8_t>(min(hpi, V.group - sub * hpi));
       it.skip_new = c.job.skip_new;
-      it.finish = c.job.finish;
-      it.pad1 = 0;
-      // the piece that holds a row's first page tells the merge how many pieces the row has
+      it.pad0 = it.pad1 = 0;
+      // the piece that holds the first page tells the merge how many pieces there are
       it.n_pieces = c.page == 0 ? static_cast<uint16_t>((c.r0 + c.w * (c.row_pages - 1)) / V.q - c.owner0 + 1) : 0;
       if (lim - c.page > kMaxChunkPages || slot < 0 || slot >= V.slots_per_stream) {   // outside the plan's limits
         report_error(V.err, V.err_host, kErrPlan);
@@ -649,7 +632,7 @@ __device__ __forceinline__ bool cursor_next(RangeCursor& c, const PartView& V, I
       c.page = lim;
       return true;
     }
-    // the current range owns nothing (more) of this row
+    // the current range owns nothing (more) of this row and position
     ++c.vw;
     c.vw_end += V.q;
   }
@@ -692,14 +675,23 @@ __device__ __forceinline__ void begin_new_rows(ItemPages& c, const Params& P, co
 }
 
 // Start of a worker from the descriptor planned for it when the step began: the first item goes
-// into the context slot together with the page ids of its first two pages, the cursor into the
-// worker's cursor slot.  False if the worker has no work.  `stage`: 48 bytes of shared memory.
-__device__ __forceinline__ bool load_worker_desc(const Params& P, int wid, ItemPages& c0, RangeCursor* cursor,
-                                                 int32_t* stage, int lane) {
+// into the first context slot together with the page ids of its first two pages, the second item
+// into the second slot, the cursor into the worker's cursor slot.  False if the worker has no
+// work.  `stage`: 48 bytes of shared memory.  The first warp also fetches the CTA's descriptor,
+// where the launch merges its rows itself.
+__device__ __forceinline__ bool load_worker_desc(const Params& P, int wid, ItemPages& c0, ItemPages& c1, RangeCursor* cursor,
+                                                 int32_t* stage, CtaDesc* cta, int lane) {
   const uint4* d = reinterpret_cast<const uint4*>(P.wdesc + static_cast<size_t>(P.launch_index) * kPlanWorkers + wid);
-  if (lane < 2) cp_async_16(reinterpret_cast<uint4*>(&c0.item) + lane, d + lane);
-  else if (lane < 5) cp_async_16(reinterpret_cast<uint4*>(stage) + (lane - 2), d + lane);
-  else if (lane < 10) cp_async_16(reinterpret_cast<uint4*>(cursor) + (lane - 5), d + lane);
+  if (lane < 12) {
+    uint4* dst = lane < 2 ? reinterpret_cast<uint4*>(&c0.item) + lane
+                 : lane < 4 ? reinterpret_cast<uint4*>(&c1.item) + (lane - 2)
+                 : lane < 7 ? reinterpret_cast<uint4*>(stage) + (lane - 4)
+                            : reinterpret_cast<uint4*>(cursor) + (lane - 7);
+    cp_async_16(dst, d + lane);
+  } else if (lane < 17 && threadIdx.x < 32 && P.fused_merge) {
+    cp_async_16(reinterpret_cast<uint4*>(cta) + (lane - 12),
+                reinterpret_cast<const uint4*>(P.cdesc + static_cast<size_t>(P.launch_index) * kPlanCtas + blockIdx.x) + (lane - 12));
+  }
   cp_async_wait_all();
   __syncwarp();
   if (c0.item.n_pages == 0) return false;
@@ -709,20 +701,16 @@ __device__ __forceinline__ bool load_worker_desc(const Params& P, int wid, ItemP
   return true;
 }
 
-// Which worker of a launch a warp is.  Under the static partition the warps of a CTA are adjacent
-// workers (adjacent ranges: the same rows, page-table lines and queries), and a launch with fewer
-// workers than warps fills the first CTAs and leaves the other SMs to the next launch's early
-// part.  Measured against one worker of every CTA first (same call, in-order step): config 2
-// 1.117 -> 1.078 ms, configs 3 / 4 / 5 within 0.6 %; runs of adjacent workers spread over all CTAs: 1.092.
-__device__ __forceinline__ int worker_index(const Params& P, int warp, int warps_per_cta) {
-  if (!P.part_static) return warp * gridDim.x + blockIdx.x;
-  return static_cast<int>(blockIdx.x) * warps_per_cta + warp;
+// Which worker of a statically partitioned launch a warp is, or -1: the workers of a CTA are
+// adjacent (the same rows, page-table lines and queries, and the rows a CTA can merge by itself).
+__device__ __forceinline__ int worker_index(const Params& P, int warp) {
+  return warp < P.part_wpc ? static_cast<int>(blockIdx.x) * P.part_wpc + warp : -1;
 }
 
 // Under the static partition, the piece that holds a row's first page records how many pieces
 // the row has: one entry per consumer layer and query head, visual and text streams side by side.
 __device__ __forceinline__ void record_row_slots(const Params& P, const Item& it, int lane) {
-  if (it.n_pieces == 0) return;
+  if (it.n_pieces == 0 || P.planned_pieces) return;   // (planned: row_pieces has them)
   const int x = lane >> 3, h = lane & 7;
   if (x < it.n_cons && h < it.n_heads) {
     const size_t row = (static_cast<size_t>(it.v_layer[x]) * P.max_seqs + it.seq_idx) * P.hq + it.head + h;
@@ -731,166 +719,308 @@ __device__ __forceinline__ void record_row_slots(const Params& P, const Item& it
 }
 
 // ------------------------------------------------------------------------------------------
-// log-sum-exp merge of one output row's partials (one warp)
+// log-sum-exp merge of output rows
 // ------------------------------------------------------------------------------------------
 //
-// Used by the merge kernel and by the attention workers (the worker that delivers a row's last
-// partial merges it).  Partials may have been written by other SMs moments ago: they are read
-// past the L1 cache.  extra_leader >= 0 adds the step's new token as one more key (merge kernel,
-// rows of a GLA follower under the in-order schedule; Eq. 6).
+// An output row's partials are nv rows of the visual stream in slots 0 .. nv - 1 and nt rows of the
+// text stream in slots text0 .. text0 + nt - 1.  They may have been written by other SMs moments
+// ago: they are read past the L1 cache.
+
 template <int D>
-__device__ __forceinline__ void merge_row(const Params& P, int layer, int si, int head, const StepSeq& sq, int lane,
-                                          int extra_leader) {
+struct RowSum {   // one warp's sum over partials; lane i holds elements i * D/32 ...
+  float m, l, acc[D / 32];
+};
+
+template <int VPL>
+__device__ __forceinline__ void load_elems(float (&v)[VPL], const float* src) {
+  if constexpr (VPL == 4) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(src));
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+  } else {
+    const float2 a = __ldcg(reinterpret_cast<const float2*>(src));
+    v[0] = a.x, v[1] = a.y;
+  }
+}
+
+// Sum of partials first, first + step, ... of the n = nv + nt of one output row.  Lane s holds the
+// (max, sum) pair of the s-th of them; the accumulator rows do not depend on the pairs, so the
+// first of them are requested together with the pairs.
+template <int D>
+__device__ __forceinline__ void sum_partials(const Params& P, size_t base, int head, int nv, int nt, int text0, int first,
+                                             int step, int lane, RowSum<D>& r) {
+  constexpr int VPL = D / 32;
+  constexpr int kBatch = D == 128 ? 12 : 16;
+  const int n = nv + nt;
+  const float* acc0 = P.part_acc + (base * P.hq + head) * D + lane * VPL;
+  const float2* ml0 = P.part_ml + base * P.hq + head;
+  const uint32_t acc_stride = static_cast<uint32_t>(P.hq) * D;
+  auto slot_of = [&](int s) { return static_cast<uint32_t>(s < nv ? s : text0 + (s - nv)); };
+  r.m = -INFINITY, r.l = 0.f;
+#pragma unroll
+  for (int e = 0; e < VPL; ++e) r.acc[e] = 0.f;
+  for (int c0 = first; c0 < n; c0 += 32 * step) {
+    const int cnt = min(32, (n - c0 + step - 1) / step);
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (lane < cnt) ml = __ldcg(ml0 + static_cast<size_t>(slot_of(c0 + lane * step)) * P.hq);
+    float v[kBatch][VPL];
+    auto request = [&](int s0) {
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (s0 + u < cnt) load_elems<VPL>(v[u], acc0 + static_cast<size_t>(slot_of(c0 + (s0 + u) * step)) * acc_stride);
+    };
+    request(0);
+    float m_new = ml.y > 0.f ? ml.x : -INFINITY;   // (a sweep that left out its only key has an empty partial)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+    m_new = fmaxf(m_new, r.m);
+    if (m_new == -INFINITY) continue;
+    const float corr = exp2f(r.m - m_new);
+    const float w = ml.y > 0.f ? exp2f(ml.x - m_new) : 0.f;
+    float ls = ml.y > 0.f ? ml.y * w : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
+    r.m = m_new;
+    r.l = r.l * corr + ls;
+#pragma unroll
+    for (int e = 0; e < VPL; ++e) r.acc[e] *= corr;
+    for (int s0 = 0; s0 < cnt; s0 += kBatch) {
+      if (s0 > 0) request(s0);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const float wu = __shfl_sync(0xffffffffu, w, (s0 + u) & 31);
+        if (s0 + u < cnt && wu > 0.f) {
+#pragma unroll
+          for (int e = 0; e < VPL; ++e) r.acc[e] = fmaf(v[u][e], wu, r.acc[e]);
+        }
+      }
+    }
+  }
+}
+
+// The finished output row: normalised, bf16, with the optional log-sum-exp.
+template <int D>
+__device__ __forceinline__ void store_row(const Params& P, int layer, int si, int head, const RowSum<D>& r, int lane) {
+  constexpr int VPL = D / 32;
+  const float inv = 1.f / r.l;
+  const size_t orow = ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head);
+  uint16_t* dst = P.out + orow * D + lane * VPL;
+  uint32_t o[VPL / 2];
+#pragma unroll
+  for (int e = 0; e < VPL; e += 2)
+    o[e / 2] = f32_to_bf16_rne(r.acc[e] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(r.acc[e + 1] * inv)) << 16);
+  if constexpr (VPL == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(o[0], o[1]);
+  else *reinterpret_cast<uint32_t*>(dst) = o[0];
+  if (P.lse != nullptr && lane == 0) P.lse[orow] = (r.m + log2f(r.l)) * 0.6931471805599453f;
+}
+
+// Merge of one output row by a launch of its own (merge_kernel), including the wait for the launch
+// that leaves the last partials.  With claimed items the numbers of partials follow from the stream
+// lengths; launches of one layer under the static partition have them planned; otherwise the
+// sweeps recorded them.  P.extra_key_leader >= 0 adds the step's new token as one more key (rows of
+// a GLA follower under the in-order schedule; Eq. 6).
+template <int D>
+__device__ __forceinline__ void merge_row(const Params& P, int layer, int si, int head, int lane) {
   constexpr int VPL = D / 32;
   const size_t base = (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots;
-  // Partial rows of this output row: nv from the visual sweep in slots 0.., nt from the text
-  // sweep in slots text0...  With claimed items both counts follow from the stream lengths; under
-  // the static partition the sweeps recorded them.
+  const int kvh = head / P.group, extra_leader = P.extra_key_leader;
+  const StepSeq sq = P.seqs[si];
   int nv = sq.ncv, nt = sq.n_slots - sq.ncv, text0 = sq.ncv;
-  if (P.part_static) {
+  if (P.planned_pieces) {
+    const int hpi = P.heads_per_item, n_sub = (P.group + hpi - 1) / hpi, rows = P.heads_per_item_dim;
+    const int u = kvh * n_sub + (head - kvh * P.group) / hpi;
+    const uint32_t both = __ldcg(P.row_pieces + (static_cast<size_t>(P.launch_index) * P.max_seqs + si) * rows + u);
+    nv = both & 0xffffu, nt = both >> 16, text0 = P.slots_per_stream;
+  }
+  const int pos = sq.len_text - 1;
+  int pid = 0, pid_v = -1;
+  if (extra_leader >= 0) {
+    pid = P.table[table_row(P, extra_leader, 0, sq.seq_id) + pos / kPage];
+    if (P.fold_append && head % P.group == 0) pid_v = P.table[table_row(P, layer, 2, sq.seq_id) + pos / kPage];
+    if (static_cast<uint32_t>(pid) >= static_cast<uint64_t>(P.n_pool_pages)) {   // never read outside the pool
+      if (lane == 0) report_error(P.err, P.err_host, kErrBadPage);
+      pid = 0;
+    }
+  }
+  pdl_wait();
+  pdl_launch_dependents();
+  if (P.part_static && !P.planned_pieces) {
     const size_t row = (static_cast<size_t>(layer) * P.max_seqs + si) * P.hq + head;
     const uint32_t both = __ldcg(reinterpret_cast<const uint32_t*>(P.row_slots + 2 * row));
     nv = sq.len_vis > 0 ? static_cast<int>(both & 0xffffu) : 0;
     nt = static_cast<int>(both >> 16);
     text0 = P.slots_per_stream;
   }
-  const int n_slots = nv + nt;
-  auto phys = [&](int s) { return s < nv ? s : text0 + (s - nv); };
-
-  // Lane s holds the (max, sum) pair of slot s; the accumulator rows do not depend on them, so
-  // their loads are issued four at a time without waiting for the pairs.
-  float mmax = -INFINITY;
-  float2 my_ml = make_float2(-INFINITY, 0.f);
-  if (lane < n_slots) my_ml = __ldcg(P.part_ml + (base + phys(lane)) * P.hq + head);
-  mmax = my_ml.x;
-  for (int s = lane + 32; s < n_slots; s += 32) mmax = fmaxf(mmax, __ldcg(P.part_ml + (base + phys(s)) * P.hq + head).x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-
-  float s_new = -INFINITY;
-  const uint16_t* v_new = nullptr;
+  float s_new = -INFINITY, vn[VPL];
   if (extra_leader >= 0) {
-    const int kvh = head / P.group;
     const uint16_t* qrow = P.qcache + ((static_cast<size_t>(extra_leader) * P.max_seqs + sq.seq_id) * P.hq + head) * D;
     // the leader's new k: the last row of its text K stream (appended before this kernel ran)
-    const int pos = sq.len_text - 1;
-    int pid = P.table[table_row(P, extra_leader, 0, sq.seq_id) + pos / kPage];
-    if (static_cast<uint32_t>(pid) >= static_cast<uint64_t>(P.n_pool_pages)) {   // never read outside the pool
-      if (lane == 0) report_error(P.err, P.err_host, kErrBadPage);
-      pid = 0;
-    }
     const uint16_t* krow = P.pool + ((static_cast<size_t>(pid) * P.hkv + kvh) * kPage + pos % kPage) * D;
-    v_new = P.v + ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hkv + kvh) * D + lane * VPL;
+    const uint16_t* v_new = P.v + ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hkv + kvh) * D + lane * VPL;
+    uint32_t q2[VPL / 2], k2[VPL / 2], v2[VPL / 2];
+#pragma unroll
+    for (int e = 0; e < VPL / 2; ++e) {
+      q2[e] = __ldcg(reinterpret_cast<const uint32_t*>(qrow + lane * VPL) + e);
+      k2[e] = __ldcg(reinterpret_cast<const uint32_t*>(krow + lane * VPL) + e);
+      v2[e] = __ldcg(reinterpret_cast<const uint32_t*>(v_new) + e);
+    }
     float dot = 0.f;
 #pragma unroll
-    for (int e = 0; e < VPL; ++e)
-      dot = fmaf(__uint_as_float(static_cast<uint32_t>(qrow[lane * VPL + e]) << 16),
-                 __uint_as_float(static_cast<uint32_t>(krow[lane * VPL + e]) << 16), dot);
+    for (int e = 0; e < VPL / 2; ++e) {
+      dot = fmaf(__uint_as_float(q2[e] << 16), __uint_as_float(k2[e] << 16), dot);
+      dot = fmaf(__uint_as_float(q2[e] & 0xffff0000u), __uint_as_float(k2[e] & 0xffff0000u), dot);
+      vn[2 * e] = __uint_as_float(v2[e] << 16);
+      vn[2 * e + 1] = __uint_as_float(v2[e] & 0xffff0000u);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     s_new = dot * P.scale_log2;
-    mmax = fmaxf(mmax, s_new);
     if (P.fold_append && head % P.group == 0) {
       // this layer's new v row has no sweep to store it: the merge warp of the KV head's first query head does
-      int pid_v = P.table[table_row(P, layer, 2, sq.seq_id) + pos / kPage];
       if (static_cast<uint32_t>(pid_v) < static_cast<uint64_t>(P.n_pool_pages)) {
-        uint16_t* dst_v = P.pool + ((static_cast<size_t>(pid_v) * P.hkv + kvh) * kPage + pos % kPage) * D + lane * VPL;
+        uint32_t* dst_v = reinterpret_cast<uint32_t*>(
+            P.pool + ((static_cast<size_t>(pid_v) * P.hkv + kvh) * kPage + pos % kPage) * D + lane * VPL);
 #pragma unroll
-        for (int e = 0; e < VPL; ++e) dst_v[e] = v_new[e];
+        for (int e = 0; e < VPL / 2; ++e) dst_v[e] = v2[e];
       } else if (lane == 0) {
         report_error(P.err, P.err_host, kErrBadPage);
       }
     }
   }
-
-  float lsum = 0.f;
-  float acc[VPL];
+  RowSum<D> r;
+  sum_partials<D>(P, base, head, nv, nt, text0, 0, 1, lane, r);
+  if (extra_leader >= 0) {
+    const float m_new = fmaxf(r.m, s_new);
+    const float corr = exp2f(r.m - m_new), w = exp2f(s_new - m_new);
+    r.m = m_new;
+    r.l = r.l * corr + w;
 #pragma unroll
-  for (int e = 0; e < VPL; ++e) acc[e] = 0.f;
-  if (v_new != nullptr) {
-    const float w = exp2f(s_new - mmax);
-    lsum = w;
-#pragma unroll
-    for (int e = 0; e < VPL; ++e) acc[e] = w * __uint_as_float(static_cast<uint32_t>(v_new[e]) << 16);
+    for (int e = 0; e < VPL; ++e) r.acc[e] = fmaf(w, vn[e], r.acc[e] * corr);
   }
-  for (int s0 = 0; s0 < n_slots; s0 += 4) {
-    float v[4][VPL];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int s = phys(min(s0 + u, n_slots - 1));
-      const float* src = P.part_acc + ((base + s) * P.hq + head) * D + lane * VPL;
-      if (VPL == 4) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(src));
-        v[u][0] = a.x, v[u][1] = a.y, v[u][2 % VPL] = a.z, v[u][3 % VPL] = a.w;
-      } else {
-        const float2 a = __ldcg(reinterpret_cast<const float2*>(src));
-        v[u][0] = a.x, v[u][1] = a.y;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int s = s0 + u;
-      float2 ml;
-      if (s < 32) {
-        ml.x = __shfl_sync(0xffffffffu, my_ml.x, s & 31);
-        ml.y = __shfl_sync(0xffffffffu, my_ml.y, s & 31);
-      } else {
-        ml = __ldcg(P.part_ml + (base + phys(min(s, n_slots - 1))) * P.hq + head);
-      }
-      if (s < n_slots && ml.y > 0.f) {   // (a sweep that left out its only key has an empty partial)
-        const float w = exp2f(ml.x - mmax);
-        lsum = fmaf(ml.y, w, lsum);
-#pragma unroll
-        for (int e = 0; e < VPL; ++e) acc[e] = fmaf(v[u][e], w, acc[e]);
-      }
-    }
-  }
-  const float inv = 1.f / lsum;
-  const size_t orow = ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head);
-  uint16_t* dst = P.out + orow * D + lane * VPL;
-  if (VPL == 4) {
-    uint2 o;
-    o.x = f32_to_bf16_rne(acc[0] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[1] * inv)) << 16);
-    o.y = f32_to_bf16_rne(acc[2 % VPL] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[3 % VPL] * inv)) << 16);
-    *reinterpret_cast<uint2*>(dst) = o;
-  } else {
-    const uint32_t o = f32_to_bf16_rne(acc[0] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[1] * inv)) << 16);
-    *reinterpret_cast<uint32_t*>(dst) = o;
-  }
-  if (P.lse != nullptr && lane == 0) P.lse[orow] = (mmax + log2f(lsum)) * 0.6931471805599453f;
+  store_row<D>(P, layer, si, head, r, lane);
 }
 
-// After an item's partial rows have been stored: count the item's pages towards the output rows
-// that this launch completes (the job's finish bits), and merge a row whose count is full.  The
-// count of a row is the pages of its visual and text streams, or of the item's stream alone when
-// only that stream is swept for the row in this launch.  Release / acquire: every lane fences its
-// stores before lane 0's atomic, and the merging warp fences again before it reads.
+// ------------------------------------------------------------------------------------------
+// merge by the attention launch itself (static partition, launches of one layer)
+// ------------------------------------------------------------------------------------------
+//
+// A CTA's workers own one stretch of the launch's tiles, ordered by output row.  When they are done,
+// the rows that lie inside the stretch are complete: the CTA merges them.  The first and the
+// last row of the stretch may be shared with other CTAs: such a row has a page counter, and the CTA
+// whose pages complete the count merges it.  Everything but the partials themselves is known
+// from the plan (which rows, how many pages and pieces), so what is left when the last worker
+// stops is a barrier, one atomic per end (1 us), one round of reads and the store (2 us).  With the
+// rows, pages and pieces worked out here instead it took 4.6 us, longer than a merge launch.
+
 template <int D>
-__device__ __forceinline__ void finish_rows(const Params& P, const ItemPages& c, int lane) {
-  const Item& it = c.item;
-  if ((it.finish & 0xf) == 0) return;
-  __threadfence();
-  __syncwarp();
-  const StepSeq sq = c.sq;
-  const int own_pages = ((it.stream ? sq.len_vis : sq.len_text) + kPage - 1) / kPage;
-  const int total = (it.finish & kFinishOwnStream)
-                        ? own_pages
-                        : (sq.len_vis + kPage - 1) / kPage + (sq.len_text + kPage - 1) / kPage;
-  // one counter per (consumer layer, sequence, first head of the item)
-  int old = 0;
-  if (lane < it.n_cons && ((it.finish >> lane) & 1)) {
-    const size_t row = (static_cast<size_t>(it.v_layer[lane]) * P.max_seqs + it.seq_idx) * P.hq + it.head;
-    old = atomicAdd(P.row_done + row, static_cast<int>(it.n_pages));
+struct FinishSmem {
+  float acc[kWarps][D];
+  float2 ml[kWarps];
+  int32_t ready[2];
+  int32_t dead;
+};
+
+// Adds to a row's page counter: releases the partials that the CTA's workers stored (they are ordered
+// before by the CTA's barrier), and the CTA that completes the count acquires everybody's.
+__device__ __forceinline__ int count_pages(int32_t* counter, int n) {
+  int old;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(old) : "l"(counter), "r"(n) : "memory");
+  return old;
+}
+
+template <int D>
+__device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, const CtaDesc& cta, bool dead, int warp, int lane) {
+  constexpr int VPL = D / 32;
+  if (!P.fused_merge) return;
+  if (dead && lane == 0) F.dead = 1;
+  __syncthreads();   // every worker's partial rows are stored
+  if (F.dead) return;
+  const int layer = P.layer_begin, rows = P.heads_per_item_dim, hpi = P.heads_per_item;
+  if (warp < 2) {   // the rows at the ends: are they complete?
+    const EndRow& e = cta.end[warp];
+    int ready = e.here == e.total;
+    if (e.here == 0) {
+      ready = 0;
+    } else if (!ready) {
+      if (lane == 0) {
+        ready = count_pages(P.row_done + e.counter, e.here) + e.here == e.total;
+        if (ready) P.row_done[e.counter] = 0;   // for the next step
+      }
+    }
+    if (lane == 0) F.ready[warp] = ready;
   }
-  for (int x = 0; x < it.n_cons; ++x) {
-    if (!((it.finish >> x) & 1)) continue;
-    const int before = __shfl_sync(0xffffffffu, old, x);
-    if (before + it.n_pages != total) continue;
-    __threadfence();
-    const size_t row = (static_cast<size_t>(it.v_layer[x]) * P.max_seqs + it.seq_idx) * P.hq + it.head;
-    if (lane == 0) P.row_done[row] = 0;   // ready for the next step
-    for (int h = 0; h < it.n_heads; ++h) merge_row<D>(P, it.v_layer[x], it.seq_idx, it.head + h, sq, lane, -1);
+  const int n_inner = max(0, cta.row_last - cta.row_first - 1) * hpi;
+  // first the rows between the ends, one warp per output row; then the ends that this CTA completed,
+  // where several warps share an output row if there are fewer rows than warps
+  RowSum<D> r;
+  int share = 1, o = kWarps - 1 - warp, n_out = n_inner, si = 0, head = 0, first_ready = 1;
+#pragma unroll 1
+  for (int phase = 0;; ++phase) {
+#pragma unroll 1
+    for (; o < n_out; o += kWarps) {
+      int nv, nt;
+      if (phase == 0) {
+        const int row = cta.row_first + 1 + o / hpi, h = o % hpi;
+        si = row / rows;
+        const int u = row - si * rows, n_sub = (P.group + hpi - 1) / hpi, kv_head = u / n_sub, sub = u - kv_head * n_sub;
+        if (sub * hpi + h >= P.group) continue;   // (a slice of the group with fewer heads)
+        head = kv_head * P.group + sub * hpi + h;
+        const uint32_t both = __ldcg(P.row_pieces + static_cast<size_t>(P.launch_index) * P.max_seqs * rows + row);
+        nv = both & 0xffffu, nt = both >> 16;
+      } else {
+        const int out = share > 1 ? warp / share : o, h = out % hpi;
+        const EndRow& e = cta.end[out >= first_ready * hpi];
+        if (h >= e.n_heads) continue;
+        si = e.si, head = e.head + h, nv = e.nv, nt = e.nt;
+      }
+      sum_partials<D>(P, (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots, head, nv, nt, P.slots_per_stream,
+                      share > 1 ? warp % share : 0, share, lane, r);
+      if (share > 1) break;
+      store_row<D>(P, layer, si, head, r, lane);
+    }
+    if (phase == 1) break;
+    __syncthreads();
+    first_ready = F.ready[0];
+    n_out = (first_ready + F.ready[1]) * hpi;
+    if (n_out == 0) return;
+    share = max(1, kWarps / n_out);
+    o = share == 1 ? warp : (warp / share < n_out ? n_out - 1 : n_out);   // (sharing: one round, output row warp / share)
   }
+  if (share == 1) return;
+  // (only rows of one query head come here: with a query group there are more output rows than warps)
+  const int row = warp / share;
+  if (row < n_out) {
+#pragma unroll
+    for (int e = 0; e < VPL; ++e) F.acc[warp][lane * VPL + e] = r.acc[e];
+    if (lane == 0) F.ml[warp] = make_float2(r.m, r.l);
+  }
+  __syncthreads();
+  if (row >= n_out) return;
+  // every thread of the row's warps weighs their sums for some of the elements
+  float w[kWarps], m = -INFINITY, l = 0.f;
+#pragma unroll
+  for (int x = 0; x < kWarps; ++x)
+    if (x < share && F.ml[row * share + x].y > 0.f) m = fmaxf(m, F.ml[row * share + x].x);
+#pragma unroll
+  for (int x = 0; x < kWarps; ++x) {
+    const float2 ml = x < share ? F.ml[row * share + x] : make_float2(0.f, 0.f);
+    w[x] = ml.y > 0.f ? exp2f(ml.x - m) : 0.f;   // (no partial, or empty ones: nothing)
+    if (w[x] > 0.f) l = fmaf(ml.y, w[x], l);
+  }
+  const float inv = 1.f / l;
+  const size_t orow = (static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head;
+  for (int d = 2 * ((warp - row * share) * 32 + lane); d < D; d += 64 * share) {
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+    for (int x = 0; x < kWarps; ++x) {
+      if (x < share && w[x] > 0.f) {
+        a0 = fmaf(F.acc[row * share + x][d], w[x], a0);
+        a1 = fmaf(F.acc[row * share + x][d + 1], w[x], a1);
+      }
+    }
+    *reinterpret_cast<uint32_t*>(P.out + orow * D + d) =
+        f32_to_bf16_rne(a0 * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(a1 * inv)) << 16);
+  }
+  if (P.lse != nullptr && lane == 0 && warp == row * share) P.lse[orow] = (m + log2f(l)) * 0.6931471805599453f;
 }
 
 }  // namespace

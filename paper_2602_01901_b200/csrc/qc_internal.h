@@ -11,7 +11,10 @@ namespace qc {
 constexpr int kPage = 16;      // tokens per page
 constexpr int kMaxCons = 4;    // V streams (output layers) one K sweep can feed
 constexpr int kMaxChunkPages = 32;
-constexpr int kAttendWarps = 12;   // independent workers (warps) per attention CTA; one CTA per SM
+constexpr int kAttendWarps = 6;        // independent workers (warps) per attention CTA
+constexpr int kAttendCtasPerSm = 2;    // attention CTAs an SM holds: while the last CTAs of a launch run, those of the
+                                       // next one start in the halves of SMs that the launch has left
+constexpr int kWorkersPerSm = kAttendWarps * kAttendCtasPerSm;
 
 // flags of Job / Item
 constexpr uint8_t kFlagShared = 1;      // one query scores for every consumer (same weights)
@@ -32,12 +35,8 @@ struct Job {
   uint8_t q_layer[kMaxCons];
   uint8_t skip_new;   // bit x: consumer x leaves out the stream's last key (the step's new token, whose
                       // value row of that layer does not exist yet when the sweep runs)
-  uint8_t finish;     // bit x: consumer x's output rows are complete once this launch's sweeps of them are
-                      // done, so the worker that delivers a row's last partial merges it (no merge launch);
-                      // kFinishOwnStream: only this job's stream contributes to those rows in this launch
-  uint8_t pad[2];
+  uint8_t pad[3];
 };
-constexpr uint8_t kFinishOwnStream = 0x10;
 static_assert(sizeof(Job) == 16, "Job layout");
 
 // One position of the launch plan: a job plus how many visual-stream and text-stream jobs
@@ -59,7 +58,7 @@ struct __align__(16) Item {
   uint16_t head, slot;
   uint16_t first_page, n_pages;
   uint16_t n_valid_last;
-  uint8_t skip_new, finish;     // as in Job
+  uint8_t skip_new, pad0;       // skip_new as in Job
   uint8_t n_heads, pad1;        // query heads head .. head + n_heads - 1 share a KV head (head / group); 1 without GQA
   uint16_t n_pieces;            // static partition, the piece with a row's first page: pieces of the row; else 0
 };
@@ -89,26 +88,49 @@ struct Patch {
 struct LaunchDesc {
   int32_t pos_begin, pos_end;
   int32_t part_q, part_k, part_vw, part_workers, part_row_cost;
-  int32_t merge_wide;   // a row of the launch may leave more than four partial rows of its visual stream
+  int32_t part_wpc;     // workers per CTA
+  int32_t part_wv, part_wt;   // tiles per page summed over the launch's visual / text jobs
+  int32_t layer;        // the one layer whose output rows the launch completes, or -1
+  int32_t fused_merge;  // 1: it merges them itself
+  int32_t vis_launch, text_launch;   // launches whose sweeps left that layer's visual / text partials (an earlier one
+                                     // for what a follower shares with its leader)
+  int32_t pad[2];
 };
-static_assert(sizeof(LaunchDesc) == 32, "LaunchDesc layout");
+static_assert(sizeof(LaunchDesc) == 64, "LaunchDesc layout");
 constexpr int kMaxPlanLaunches = 128;   // launches of a step that can be planned ahead (a launch per layer fits)
 constexpr int kPlanWorkers = 2048;      // worker descriptors kept per launch
 struct LaunchList {
   LaunchDesc launch[kMaxPlanLaunches];
 };
 
-// Where a worker of a statically partitioned launch starts: its first item, the page ids of that
-// item's first two pages (K stream, then the V stream of each consumer) so that the first tiles
-// can be requested at once, and the cursor from which its later items follow.  Written for every
-// launch of a step by one kernel when the step begins; a worker then starts from one 160-byte read.
+// Where a worker of a statically partitioned launch starts: its first two items, the page ids of the
+// first item's first two pages (K stream, then the V stream of each consumer) so that the first
+// tiles can be requested at once, and the cursor from which its later items follow.  Written for
+// every launch of a step by one kernel when the step begins; a worker then starts from one read.
 struct __align__(16) WorkerDesc {
-  Item item;                        // n_pages == 0: the worker has no work
+  Item item[2];                     // n_pages == 0: the worker has no work / no second item
   int32_t pids[1 + kMaxCons][2];
   int32_t pad[2];
   int32_t cursor[20];               // a RangeCursor
 };
-static_assert(sizeof(WorkerDesc) == 160, "WorkerDesc layout");
+static_assert(sizeof(WorkerDesc) == 192, "WorkerDesc layout");
+
+// What a CTA of a launch that merges its own rows needs to know about them, planned like the
+// worker descriptors.  A row is (listed sequence, query head or query group), numbered
+// sequence index * rows per sequence + row.
+struct EndRow {                     // the first or the last row that the CTA's tiles fall into
+  int32_t here, total;              // pages of the row in this CTA / in the launch
+  int32_t counter;                  // its page counter in row_done
+  int32_t si, head, n_heads;        // listed sequence, query heads
+  int32_t nv, nt;                   // partial rows of the visual / the text stream
+};
+struct __align__(16) CtaDesc {
+  EndRow end[2];                    // end[1].here == 0: the first row is the only one
+  int32_t row_first, row_last;
+  int32_t pad[2];
+};
+static_assert(sizeof(CtaDesc) == 80, "CtaDesc layout");
+constexpr int kPlanCtas = 512;      // CTA descriptors kept per launch
 
 // Kernel parameter block.
 struct Params {
@@ -133,8 +155,11 @@ struct Params {
   uint16_t* row_slots;     // [n_layers][max_seqs][hq][2]: partial rows the visual / the text sweep left for an
                            // output row (static partition only)
   const WorkerDesc* wdesc; // [launches of the step][kPlanWorkers] planned ahead, or null: workers find their own start
-  int32_t* row_done;       // [n_layers][max_seqs][hq]: pages of an output row swept so far in the current launch
-                           // (the worker that completes the count merges the row and resets it)
+  const CtaDesc* cdesc;    // [launches of the step][kPlanCtas], planned with wdesc
+  uint32_t* row_pieces;    // [launches of the step][max_seqs * items per chunk]: partial rows of a row's visual stream
+                           // (low half) and text stream, planned with wdesc
+  int32_t* row_done;       // [n_layers][max_seqs][hq]: pages of a row swept so far in the current launch by the CTAs
+                           // that share it (the CTA that completes the count merges the row and resets it)
   int64_t n_pool_pages;    // bound for page ids (reads never leave the pool)
   int32_t n_layers, hq, hkv, d, group, max_seqs, max_pages, max_slots, chunk_pages;
   int32_t heads_per_item_dim;   // work items per (chunk, sequence): hq, or with GQA hkv * ceil(group / 8)
@@ -154,21 +179,23 @@ struct Params {
   int32_t launch_index;              // which work counter that launch uses
   int32_t layer_begin, layer_end;    // range handled by one merge launch
   // static partition of an attention launch: the launch's work, counted in tiles in the order
-  // plan position -> listed sequence -> row (head or query group) -> page, is cut into part_vw
+  // listed sequence -> row (head or query group) -> plan position -> page, is cut into part_vw
   // ranges of part_q tiles; worker w takes ranges w * part_k .. w * part_k + part_k - 1.  A page
   // belongs to the range its first tile falls into.
   int32_t part_static;               // 0: items are claimed from the list
   int32_t part_vw, part_k, part_workers;
-  int32_t part_q, part_tiles;        // tiles per range; tiles of the launch
+  int32_t part_q;                    // tiles per range
+  int32_t part_wpc;                  // workers per CTA
+  int32_t part_wv, part_wt;          // tiles per page summed over the launch's visual / text jobs
+  int32_t fused_merge;               // the launch merges the output rows of its layer (layer_begin) itself
+  int32_t planned_pieces;            // the numbers of partial rows of its layer's output rows are in row_pieces
   int32_t part_row_cost;             // what a row counts for besides its pages, in tiles
-  int32_t tp_v, tp_t;                // pages of the visual / text streams, summed over the listed sequences
   int32_t pos_begin, pos_end;        // plan positions of the launch
   int32_t slots_per_stream;          // partial-row slots of one stream of an output row (text slots start here)
   int32_t fold_append;               // in-order schedule: the new token's k/v rows (and an ordinary layer's q for the
                                      // Q Cache) are taken from the step's inputs by the attention worker (or the
                                      // merge warp) that meets the end of the layer's text stream, which also stores
                                      // them: no append launch, nothing of a layer is touched before its own launch
-  int32_t merge_wide;                // merge: rows may have more than four partial rows of the visual stream
   int32_t debug_drop_tile;           // test hook: every worker of an attention launch leaves out the copy of its first
                                      // tile and waits for it with a short limit (nothing in flight, nothing faults)
   int32_t extra_key_leader;          // merge only, >= 0: the rows also take the step's new token as one more key,
@@ -178,7 +205,7 @@ struct Params {
 // launchers (qc_kernels.cu); all asynchronous on `stream`
 cudaError_t launch_setup(const Params& p, const StepInline* inl, cudaStream_t stream);
 cudaError_t launch_append(const Params& p, cudaStream_t stream);
-cudaError_t launch_plan(const Params& p, const LaunchList& list, int n_launches, cudaStream_t stream);   // writes p.wdesc
+cudaError_t launch_plan(const Params& p, const LaunchList& list, int n_launches, cudaStream_t stream);   // writes p.wdesc, p.cdesc, p.row_pieces
 cudaError_t launch_attend(const Params& p, int n_sms, cudaStream_t stream);      // one query head per item
 cudaError_t launch_attend_tc(const Params& p, int n_sms, cudaStream_t stream);   // query-group items (GQA)
 cudaError_t launch_merge(const Params& p, cudaStream_t stream);

@@ -130,8 +130,7 @@ __global__ void setup_kernel(const __grid_constant__ Params P, const __grid_cons
     it.n_valid_last = static_cast<uint16_t>(last ? len - (total_pages - 1) * kPage : kPage);
     it.n_heads = static_cast<uint8_t>(min(hpi, P.group - sub * hpi));
     it.skip_new = jb.skip_new;
-    it.finish = jb.finish;
-    it.pad1 = 0;
+    it.pad0 = it.pad1 = 0;
     it.n_pieces = 0;
     P.items[item_base + t] = it;
   }
@@ -153,20 +152,106 @@ __global__ void append_kernel(const __grid_constant__ Params P) {
 // plan: where every worker of every statically partitioned launch of the step starts
 // ------------------------------------------------------------------------------------------
 
-__global__ void plan_kernel(const __grid_constant__ Params P, const __grid_constant__ LaunchList list) {
+// Three kinds of threads, by block: one per worker (where it starts), one per CTA (the rows at the
+// ends of its stretch) and one per row (its numbers of partials), for every launch of the step.
+// All of it is integer arithmetic on the sequence descriptors, which a block keeps in shared memory
+// (a search in them would otherwise be five dependent reads for a batch of 32).
+constexpr int kPlanBlock = 128;
+constexpr int kPlanSeqs = 128;    // descriptors kept in shared memory; longer lists are read from global memory
+__global__ void __launch_bounds__(kPlanBlock) plan_kernel(const __grid_constant__ Params P, const __grid_constant__ LaunchList list,
+                                                          int cta_blocks) {
+  __shared__ StepSeq seqs[kPlanSeqs];
   pdl_wait();   // the page tables and the sequence descriptors are final
-  const int g = blockIdx.y, wid = blockIdx.x * blockDim.x + threadIdx.x;
-  const LaunchDesc L = list.launch[g];
-  if (wid >= kPlanWorkers) return;
+  const int g = blockIdx.y;
+  const LaunchDesc& L = list.launch[g];
+  PartView V = part_view(P, L);
+  if (P.n_seqs <= kPlanSeqs) {
+    for (int i = threadIdx.x; i < 2 * P.n_seqs; i += kPlanBlock)
+      reinterpret_cast<uint4*>(seqs)[i] = reinterpret_cast<const uint4*>(P.seqs)[i];
+    __syncthreads();
+    V.seqs = seqs;
+  }
+  // numbers of partial rows that launch G leaves for row (si, u) of `layer`, of the streams it sweeps
+  auto count_pieces = [&](const PartView& G, const StepSeq& sq, int si, int u, int layer, int& nv, int& nt) {
+    int32_t r0 = seq_base(G, sq.pre_v, sq.pre_t, si) + u * row_tiles(G, sq.len_vis, sq.len_text);
+    for (int pos = G.pos_begin; pos < G.pos_end; ++pos) {
+      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(G.plan + pos));
+      const Job& job = *reinterpret_cast<const Job*>(&raw);
+      const int w = job_tiles_per_page(job), pages = pages_of(job.stream ? sq.len_vis : sq.len_text);
+      r0 += G.row_cost;
+      const int n = pages > 0 ? (r0 + w * (pages - 1)) / G.q - r0 / G.q + 1 : 0;
+      for (int x = 0; x < job.n_cons; ++x)
+        if (job.v_layer[x] == layer) (job.stream ? nv : nt) = n;
+      r0 += w * pages;
+    }
+  };
+  auto row_counts = [&](const StepSeq& sq, int si, int u, int& nv, int& nt) {
+    nv = nt = 0;
+    int unused;
+    count_pieces(V, sq, si, u, L.layer, nv, nt);
+    if (L.vis_launch != g) count_pieces(part_view(P, list.launch[L.vis_launch]), sq, si, u, L.layer, nv, unused);
+    if (L.text_launch != g) count_pieces(part_view(P, list.launch[L.text_launch]), sq, si, u, L.layer, unused, nt);
+  };
+
+  constexpr int kWorkerBlocks = kPlanWorkers / kPlanBlock;
+  if (blockIdx.x >= kWorkerBlocks) {
+    if (L.layer < 0) return;
+    int id = (blockIdx.x - kWorkerBlocks) * kPlanBlock + threadIdx.x;
+    if (blockIdx.x >= kWorkerBlocks + cta_blocks) {   // ---- rows
+      id -= cta_blocks * kPlanBlock;
+      if (id >= P.n_seqs * V.rows) return;
+      const int si = id / V.rows, u = id - si * V.rows;
+      int nv, nt;
+      row_counts(V.seqs[si], si, u, nv, nt);
+      P.row_pieces[static_cast<size_t>(g) * P.max_seqs * V.rows + id] = static_cast<uint32_t>(nv) | (static_cast<uint32_t>(nt) << 16);
+      return;
+    }
+    // ---- CTAs
+    if (!L.fused_merge || id * L.part_wpc >= L.part_workers) return;
+    const int32_t per_cta = L.part_wpc * V.k;
+    const int32_t a = id * per_cta * V.q, b = min((id + 1) * per_cta, V.vw) * V.q;   // the CTA's tiles
+    CtaDesc d;
+    d.pad[0] = d.pad[1] = 0;
+    for (int e = 0; e < 2; ++e) {
+      EndRow& r = d.end[e];
+      int si, u;
+      StepSeq sq;
+      int32_t r0 = find_row(V, e == 0 ? a : b - 1, si, u, sq);
+      (e == 0 ? d.row_first : d.row_last) = si * V.rows + u;
+      r.here = r.total = 0;
+      for (int pos = V.pos_begin; pos < V.pos_end; ++pos) {
+        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(V.plan + pos));
+        const Job& job = *reinterpret_cast<const Job*>(&raw);
+        const int w = job_tiles_per_page(job), pages = pages_of(job.stream ? sq.len_vis : sq.len_text);
+        r0 += V.row_cost;
+        auto before = [&](int32_t t) { return t <= r0 ? 0 : min(pages, (t - r0 + w - 1) / w); };   // pages that start before tile t
+        r.here += before(b) - before(a);
+        r.total += pages;
+        r0 += w * pages;
+      }
+      const int hpi = V.heads_per_item, n_sub = (V.group + hpi - 1) / hpi;
+      const int kv_head = u / n_sub, sub = u - kv_head * n_sub;
+      r.si = si;
+      r.head = kv_head * V.group + sub * hpi;
+      r.n_heads = min(hpi, V.group - sub * hpi);
+      r.counter = (L.layer * P.max_seqs + si) * P.hq + r.head;
+      row_counts(sq, si, u, r.nv, r.nt);
+    }
+    if (d.row_last == d.row_first) d.end[1].here = 0;
+    uint4* out = reinterpret_cast<uint4*>(const_cast<CtaDesc*>(P.cdesc) + static_cast<size_t>(g) * kPlanCtas + id);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) out[i] = reinterpret_cast<const uint4*>(&d)[i];
+    return;
+  }
+
+  // ---- workers
+  const int wid = blockIdx.x * kPlanBlock + threadIdx.x;
   WorkerDesc* out = const_cast<WorkerDesc*>(P.wdesc) + static_cast<size_t>(g) * kPlanWorkers + wid;
-  PartView V = part_view(P);
-  V.pos_begin = L.pos_begin, V.pos_end = L.pos_end;
-  V.q = L.part_q, V.k = L.part_k, V.vw = L.part_vw, V.row_cost = L.part_row_cost;
   WorkerDesc d;
-  d.item.n_pages = 0;
+  d.item[0].n_pages = d.item[1].n_pages = 0;
   RangeCursor c;
-  if (wid < L.part_workers && cursor_init_scalar(c, V, wid) && cursor_next(c, V, d.item)) {
-    const Item& it = d.item;
+  if (wid < L.part_workers && cursor_init(c, V, wid) && cursor_next(c, V, d.item[0])) {
+    const Item& it = d.item[0];
     for (int j = 0; j < 2; ++j) {
       const int pg = it.first_page + min(j, it.n_pages - 1);
       d.pids[0][j] = P.table[table_row(P, it.k_layer, it.stream, it.seq_id) + pg];
@@ -174,19 +259,20 @@ __global__ void plan_kernel(const __grid_constant__ Params P, const __grid_const
         d.pids[1 + x][j] = x < it.n_cons ? P.table[table_row(P, it.v_layer[x], 2 + it.stream, it.seq_id) + pg] : 0;
     }
     d.pad[0] = d.pad[1] = 0;
+    if (!cursor_next(c, V, d.item[1])) d.item[1].n_pages = 0;
     *reinterpret_cast<RangeCursor*>(d.cursor) = c;
   } else {
-    d.item.n_pages = 0;
+    d.item[0].n_pages = 0;
   }
   const uint4* src = reinterpret_cast<const uint4*>(&d);
   uint4* dst = reinterpret_cast<uint4*>(out);
-  if (d.item.n_pages == 0) {   // no work: an all-zero item says so
+  if (d.item[0].n_pages == 0) {   // no work: an all-zero item says so
     dst[0] = make_uint4(0, 0, 0, 0);
     dst[1] = make_uint4(0, 0, 0, 0);
     return;
   }
 #pragma unroll
-  for (int i = 0; i < 10; ++i) dst[i] = src[i];
+  for (int i = 0; i < 12; ++i) dst[i] = src[i];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -263,25 +349,28 @@ template <int D, int NQ, int NV, int MODE = 0, bool SKIP = false, bool FOLD = fa
 __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* ctx, uint32_t ring, uint64_t* full,
                                              const Params& P, int lane) {
   auto ctx_of = [ctx](int k) -> const ItemPages& { return ctx[k % kCtxSlots].ip; };
-  constexpr int EPL = D / 8;    // elements of a row held by one lane
+  constexpr int EP2 = D / 16;   // element pairs of a row held by one lane
   constexpr int LPR = D / 64;   // 16-byte loads per lane per row
   const WarpCtx<D>& c = ctx[st.cons_k % kCtxSlots];
   const int kg = lane >> 3;     // which of 4 keys of a pass
   const int c8 = lane & 7;      // which 16-byte chunk of the row (and of its second half)
+  const uint32_t lane_off = kg * (D * 2) + c8 * 16;   // this lane's first chunk of a pass's rows
 
-  float qf[NQ][EPL];
+  // The arithmetic on elements runs on pairs (fma.rn.f32x2): half the instructions, same fp32 results.
+  float2 qf[NQ][EP2];
 #pragma unroll
   for (int x = 0; x < NQ; ++x) {
 #pragma unroll
     for (int j = 0; j < LPR; ++j) {
       const uint4 raw = c.qraw[x][c8 + 8 * j];
-      bf16x8_to_f32(raw, &qf[x][8 * j]);
+      bf16x8_to_f32x2(raw, &qf[x][4 * j]);
     }
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) qf[x][e] *= P.scale_log2;
+    for (int e = 0; e < EP2; ++e) qf[x][e] = mul2(qf[x][e], make_float2(P.scale_log2, P.scale_log2));
   }
 
-  float m[NQ], l[NQ], acc[NV][EPL];
+  float m[NQ], l[NQ];
+  float2 acc[NV][EP2];
 #pragma unroll
   for (int x = 0; x < NQ; ++x) {
     m[x] = -INFINITY;
@@ -290,7 +379,7 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
 #pragma unroll
   for (int v = 0; v < NV; ++v)
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) acc[v][e] = 0.f;
+    for (int e = 0; e < EP2; ++e) acc[v][e] = make_float2(0.f, 0.f);
 
   const int n_pages = c.ip.item.n_pages;
   const int n_valid_last = c.ip.item.n_valid_last;
@@ -323,14 +412,14 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
       }
     } else {
       // ---- K tile: scores of 16 keys
-      const uint8_t* tile = static_cast<const uint8_t*>(__cvta_shared_to_generic(wait_tile<D>(st, ring, full, P, lane)));
+      const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
       if (st.dead) break;
       if (kMayFold && pg == new_pg) {
         // the new token's k row comes from the step's input: into the tile, and into the pool for later steps
         const Item& it = c.ip.item;
         if (lane < D / 8) {
           const uint4 val = c.ip.new_k[lane];
-          reinterpret_cast<uint4*>(const_cast<uint8_t*>(tile) + (nvalid - 1) * (D * 2))[lane] = val;
+          sts128(tile + (nvalid - 1) * (D * 2) + lane * 16, val);
           const int pid = c.ip.pages[0][pg];
           if (static_cast<uint32_t>(pid) < static_cast<uint64_t>(P.n_pool_pages))
             reinterpret_cast<uint4*>(P.pool + ((static_cast<size_t>(pid) * P.hkv + c.ip.kv_head) * kPage + (nvalid - 1)) * D)[lane] = val;
@@ -339,24 +428,23 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
             reinterpret_cast<uint4*>(P.qcache + ((static_cast<size_t>(it.k_layer) * P.max_seqs + it.seq_id) * P.hq + it.head) * D)[lane] =
                 c.qraw[0][lane];
         }
+        fence_proxy_async();   // these generic-proxy writes precede the slot's next asynchronous refill
         __syncwarp();
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = 4 * i + kg;
-        const uint4* row = reinterpret_cast<const uint4*>(tile + r * (D * 2));
-        float kf[EPL];
+        float2 kf[EP2];
 #pragma unroll
-        for (int j = 0; j < LPR; ++j) bf16x8_to_f32(row[c8 + 8 * j], &kf[8 * j]);
+        for (int j = 0; j < LPR; ++j) bf16x8_to_f32x2(lds128(tile + lane_off + i * (4 * D * 2) + j * 128), &kf[4 * j]);
 #pragma unroll
         for (int x = 0; x < NQ; ++x) {
-          float a0 = 0.f, a1 = 0.f;
+          float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < EPL; e += 2) {
-            a0 = fmaf(kf[e], qf[x][e], a0);
-            a1 = fmaf(kf[e + 1], qf[x][e + 1], a1);
+          for (int e = 0; e < EP2; e += 2) {
+            a0 = fma2(kf[e], qf[x][e], a0);
+            a1 = fma2(kf[e + 1], qf[x][e + 1], a1);
           }
-          p[x][i] = a0 + a1;
+          p[x][i] = (a0.x + a1.x) + (a0.y + a1.y);
         }
       }
       release_tile<kRing>(st);
@@ -379,11 +467,11 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
       tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
       tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
       const float m_new = fmaxf(m[x], tmax);
-      const float corr = exp2f(m[x] - m_new);
+      const float corr = ex2_approx(m[x] - m_new);
       float psum = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        p[x][i] = exp2f(p[x][i] - m_new);
+        p[x][i] = ex2_approx(p[x][i] - m_new);
         psum += p[x][i];
       }
       l[x] = l[x] * corr + psum;
@@ -403,7 +491,7 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
         for (int v = 0; v < NV; ++v) {
           if (NQ == 1 || v == x) {
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[v][e] *= corr;
+            for (int e = 0; e < EP2; ++e) acc[v][e] = mul2(acc[v][e], make_float2(corr, corr));
           }
         }
       }
@@ -411,7 +499,7 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
     // ---- V tiles: weighted sums for each consumer
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const uint8_t* tile = static_cast<const uint8_t*>(__cvta_shared_to_generic(wait_tile<D>(st, ring, full, P, lane)));
+      const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
       if (st.dead) break;
       const int nvalid_v = (SKIP && skip_here && pg == n_pages - 1) ? nvalid - static_cast<int>((skip_mask >> v) & 1u) : nvalid;
       if (kMayFold && pg == new_pg && nvalid_v == nvalid) {
@@ -422,25 +510,29 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
                                 ? c.ip.new_v[lane]
                                 : reinterpret_cast<const uint4*>(
                                       P.v + ((static_cast<size_t>(it.v_layer[v]) * P.n_seqs + it.seq_idx) * P.hkv + c.ip.kv_head) * D)[lane];
-          reinterpret_cast<uint4*>(const_cast<uint8_t*>(tile) + (nvalid - 1) * (D * 2))[lane] = val;
+          sts128(tile + (nvalid - 1) * (D * 2) + lane * 16, val);
           const int pid = c.ip.pages[1 + v][pg];
           if (static_cast<uint32_t>(pid) < static_cast<uint64_t>(P.n_pool_pages))
             reinterpret_cast<uint4*>(P.pool + ((static_cast<size_t>(pid) * P.hkv + c.ip.kv_head) * kPage + (nvalid - 1)) * D)[lane] = val;
         }
+        fence_proxy_async();
         __syncwarp();
       }
+      auto add_row = [&](int i) {
+        float2 vf[EP2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = 4 * i + kg;
-        if (r < nvalid_v) {
-          const uint4* row = reinterpret_cast<const uint4*>(tile + r * (D * 2));
-          float vf[EPL];
+        for (int j = 0; j < LPR; ++j) bf16x8_to_f32x2(lds128(tile + lane_off + i * (4 * D * 2) + j * 128), &vf[4 * j]);
+        const float pv = p[NQ == 1 ? 0 : v][i];
 #pragma unroll
-          for (int j = 0; j < LPR; ++j) bf16x8_to_f32(row[c8 + 8 * j], &vf[8 * j]);
-          const float pv = p[NQ == 1 ? 0 : v][i];
+        for (int e = 0; e < EP2; ++e) acc[v][e] = fma2(vf[e], make_float2(pv, pv), acc[v][e]);
+      };
+      if (nvalid_v == kPage) {
 #pragma unroll
-          for (int e = 0; e < EPL; ++e) acc[v][e] = fmaf(pv, vf[e], acc[v][e]);
-        }
+        for (int i = 0; i < 4; ++i) add_row(i);
+      } else {   // (rows past the end hold whatever the pool held: a zero weight does not cancel a NaN)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (4 * i + kg < nvalid_v) add_row(i);
       }
       release_tile<kRing>(st);
       fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
@@ -461,9 +553,11 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-      acc[v][e] += __shfl_xor_sync(0xffffffffu, acc[v][e], 8);
-      acc[v][e] += __shfl_xor_sync(0xffffffffu, acc[v][e], 16);
+    for (int e = 0; e < EP2; ++e) {
+      acc[v][e].x += __shfl_xor_sync(0xffffffffu, acc[v][e].x, 8);
+      acc[v][e].y += __shfl_xor_sync(0xffffffffu, acc[v][e].y, 8);
+      acc[v][e].x += __shfl_xor_sync(0xffffffffu, acc[v][e].x, 16);
+      acc[v][e].y += __shfl_xor_sync(0xffffffffu, acc[v][e].y, 16);
     }
   }
   if (kg == 0) {
@@ -476,23 +570,23 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
 #pragma unroll
       for (int j = 0; j < LPR; ++j) {
         float4* d4 = reinterpret_cast<float4*>(dst + 64 * j + 8 * c8);
-        d4[0] = make_float4(acc[v][8 * j + 0], acc[v][8 * j + 1], acc[v][8 * j + 2], acc[v][8 * j + 3]);
-        d4[1] = make_float4(acc[v][8 * j + 4], acc[v][8 * j + 5], acc[v][8 * j + 6], acc[v][8 * j + 7]);
+        d4[0] = make_float4(acc[v][4 * j + 0].x, acc[v][4 * j + 0].y, acc[v][4 * j + 1].x, acc[v][4 * j + 1].y);
+        d4[1] = make_float4(acc[v][4 * j + 2].x, acc[v][4 * j + 2].y, acc[v][4 * j + 3].x, acc[v][4 * j + 3].y);
       }
       const bool skipping = SKIP && ((skip_mask >> v) & 1u);
       if (c8 == 0) P.part_ml[row] = make_float2(m[NQ == 1 ? 0 : v], skipping ? l_skip : l[NQ == 1 ? 0 : v]);
     }
   }
-  finish_rows<D>(P, c.ip, lane);
 }
 
 // A worker's life: take items (claimed from the list, or the pieces of its static ranges), keep
 // the tile ring full across item boundaries, process each item.  While item k is processed the
 // ring already fetches tiles of item k + 1 and the context of item k + 2 (descriptor, page ids,
 // queries) arrives by asynchronous copies.
+// False if a wait ran out.
 template <int D, bool STATIC>
-__device__ __forceinline__ void attend_worker(const Params& P, WarpCtx<D>* ctx, uint32_t ring, uint64_t* full,
-                                              RangeCursor* cursor, int32_t* stage, int wid, int lane) {
+__device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, uint32_t ring, uint64_t* full,
+                                              RangeCursor* cursor, int32_t* stage, CtaDesc* cta, int wid, int lane) {
   auto ctx_of = [ctx](int k) -> const ItemPages& { return ctx[k % kCtxSlots].ip; };
   WorkerState st;
   worker_init(st, 0);
@@ -506,62 +600,79 @@ __device__ __forceinline__ void attend_worker(const Params& P, WarpCtx<D>* ctx, 
     it = load_item(P, idx);
     return true;
   };
-  // ---- ahead of the wait for the previous kernel: the first items and their page ids (from the
+  // ---- ahead of the wait for the previous kernel: the first two items and their page ids (from the
   // launch plan, the step descriptors and the page tables, all written before that kernel
   // started), and the first tiles unless they could hold a new token that an earlier launch of the
-  // step stores (with the folded append the worker patches the new token's row itself)
+  // step stores (with the folded append the worker patches the new token's row itself).  After it,
+  // only the layer's inputs.
   Item first;
-  if (STATIC && P.wdesc != nullptr) {
-    // planned ahead: one read gives the first item, its first page ids and the cursor
-    if (wid >= P.part_workers) return;
-    if (!load_worker_desc(P, wid, ctx[0].ip, cursor, stage, lane)) return;
-    first = ctx[0].ip.item;
+  bool more;
+  if (STATIC) {
+    bool any = wid >= 0 && wid < P.part_workers;
+    if (P.wdesc != nullptr) {
+      // planned ahead: one read gives the first two items, the first page ids and the cursor
+      any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, cta, lane);
+      if (any) first = ctx[0].ip.item;
+    } else {
+      RangeCursor c;
+      any = any && cursor_init(c, part_view(P), wid);
+      if (lane == 0) *cursor = c;
+      __syncwarp();
+      any = any && take();
+      if (any) {
+        first = it;
+        begin_item_pages(ctx[0].ip, P, first, lane);
+        cp_async_wait_all();
+        __syncwarp();
+      }
+    }
+    if (!any) {
+      pdl_wait();   // (a warp without work may still merge)
+      return true;
+    }
     st.n_my = 1;
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRing);
     if (early_tiles) fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
-    begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
-  } else {
-    if (STATIC) {
-      if (wid >= P.part_workers) return;
-      RangeCursor c;
-      const bool any = cursor_init(c, part_view(P), wid, lane);
-      if (lane == 0) *cursor = c;
-      __syncwarp();
-      if (!any) return;
+    if (P.wdesc != nullptr) {
+      begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
+      it = ctx[1].ip.item;
+      more = it.n_pages > 0;
     } else {
-      pdl_wait();   // the item list and the work counter are the previous kernel's
-      pdl_launch_dependents();
-      issued = claim_issue(P, lane);
+      more = take();
     }
-    if (!take()) return;
-    begin_item_pages(ctx[0].ip, P, it, lane);
+    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    pdl_wait();
+    pdl_launch_dependents();
+  } else {
+    pdl_wait();   // the item list and the work counter are the previous kernel's
+    pdl_launch_dependents();
+    issued = claim_issue(P, lane);
+    if (!take()) return true;
     first = it;
+    begin_item_pages(ctx[0].ip, P, first, lane);
     cp_async_wait_all();
     __syncwarp();
     st.n_my = 1;
-    const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRing);
-    if (early_tiles) fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
+    fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
+    issued = claim_issue(P, lane);
   }
-  if (STATIC) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
-  // ---- this layer's inputs; the rest of the first tiles; the second item's context while they fly
   begin_queries<D>(ctx[0], P, first, lane);
   begin_new_rows(ctx[0].ip, P, first, lane, D);
-  fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
-  if (STATIC) record_row_slots(P, first, lane);
-  if (!STATIC) issued = claim_issue(P, lane);
-  bool more = take();
+  if (!STATIC) {
+    more = take();
+    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+  }
+  cp_async_commit_group();
   if (more) {
-    begin_item_pages(ctx[1].ip, P, it, lane);
     begin_queries<D>(ctx[1], P, it, lane);
     begin_new_rows(ctx[1].ip, P, it, lane, D);
-    if (STATIC) record_row_slots(P, it, lane);
   }
-  cp_async_wait_all();
+  cp_async_commit_group();   // the second item's inputs are waited for when the first item is done
+  if (STATIC) cp_async_wait_group<1>();
+  else cp_async_wait_all();
   __syncwarp();
   if (more) st.n_my = 2;
+  fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
   bool pending = false;   // a context is being filled for item st.n_my
   if (!STATIC && more) issued = claim_issue(P, lane);
 
@@ -576,7 +687,6 @@ __device__ __forceinline__ void attend_worker(const Params& P, WarpCtx<D>* ctx, 
         begin_item_pages(ctx[(k + 2) % kCtxSlots].ip, P, it, lane);
         begin_queries<D>(ctx[(k + 2) % kCtxSlots], P, it, lane);
         begin_new_rows(ctx[(k + 2) % kCtxSlots].ip, P, it, lane, D);
-        if (STATIC) record_row_slots(P, it, lane);
         pending = true;
       }
     }
@@ -598,10 +708,11 @@ __device__ __forceinline__ void attend_worker(const Params& P, WarpCtx<D>* ctx, 
     else if (nc == 3) process_item<D, 3, 3>(st, ctx, ring, full, P, lane);
     else process_item<D, 4, 4>(st, ctx, ring, full, P, lane);
     if (st.dead) break;
-    if (pending) {   // the context of item k + 2 has had this item's time to arrive
+    if (STATIC) record_row_slots(P, cur, lane);
+    if (k + 1 < st.n_my) {   // the contexts of items k + 1 and k + 2 have had this item's time to arrive
       cp_async_wait_all();
       __syncwarp();
-      st.n_my = k + 3;
+      if (pending) st.n_my = k + 3;
       pending = false;
     }
     st.cons_k = k + 1;
@@ -611,15 +722,18 @@ __device__ __forceinline__ void attend_worker(const Params& P, WarpCtx<D>* ctx, 
     cp_async_wait_all();
     drain_ring<kRing>(st, full, P.debug_drop_tile ? kDebugSpinLimit : kSpinLimit);
   }
+  return !st.dead;
 }
 
 template <int D, bool STATIC>
-__global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_constant__ Params P) {
+__global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_kernel(const __grid_constant__ Params P) {
   constexpr uint32_t kTile = kPage * D * 2;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t full_all[kWarps][kRing];
   __shared__ __align__(16) RangeCursor cursors[kWarps];
   __shared__ __align__(16) int32_t stages[kWarps][12];
+  __shared__ __align__(16) FinishSmem<D> finish;
+  __shared__ CtaDesc cta;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t ring = smem_u32(smem) + static_cast<uint32_t>(warp) * kRing * kTile;
@@ -630,148 +744,30 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     for (int s = 0; s < kRing; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
   }
+  if (threadIdx.x == 0) finish.dead = 0;
   __syncthreads();
 
-  attend_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], worker_index(P, warp, kWarps), lane);
+  const bool ok = attend_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], &cta, worker_index(P, warp), lane);
+  if (STATIC) finish_cta<D>(P, finish, cta, !ok, warp, lane);
 }
 
 // ------------------------------------------------------------------------------------------
 // merge: log-sum-exp combination of the partials of one (layer, sequence, head) per warp
 // ------------------------------------------------------------------------------------------
 
-// One warp per (layer, sequence, head).  Under the static partition the numbers of partial rows
-// are themselves data the attention kernel wrote, so the generic merge needs three dependent
-// rounds of loads (counts, then (max, sum) pairs, then rows).  When a row has at most 16 partials
-// per stream (the common case: a launch per layer leaves a handful) everything is requested in
-// one round instead: the counts, the pairs of the first 16 slots of either stream (lanes 0..15 /
-// 16..31) and the rows that a guess at the counts names (up to 4 or 16 of the visual stream, 4 of the
-// text stream); what the counts then rule out is ignored, rows beyond those take one more round
-// (eight visual rows in the first round were measured slower: rows never written are not in the
-// L2).  The step's sequence descriptor is read ahead of the wait for the
-// attention kernel (it was written when the step began).
-// NVIS = 0: the general path alone (few registers: a launch per step merges every layer's rows);
-// NVIS = 4 / 16: the one-round path with up to NVIS visual rows in the first round (the host knows
-// from the partition whether a row of the launch can leave more than four).
-template <int D, int NVIS>
+// One warp per (layer, sequence, head).  What it reads besides the partials (the sequence's
+// descriptor, the numbers of partials where they are planned, page ids) was written when the step
+// began and is read ahead of the wait for the attention kernel, so that one round of reads is left.
+template <int D>
 __global__ void merge_kernel(const __grid_constant__ Params P) {
-  constexpr int VPL = D / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_layers = P.layer_end - P.layer_begin;
   const int idx = blockIdx.x * (blockDim.x >> 5) + warp;
-  const bool live = idx < n_layers * P.n_seqs * P.hq;
-  const int head = idx % P.hq;
-  const int si = (idx / P.hq) % P.n_seqs;
-  const int layer = P.layer_begin + idx / (P.hq * P.n_seqs);
-  StepSeq sq{};
-  if (live) sq = P.seqs[si];
-  const size_t row = (static_cast<size_t>(layer) * P.max_seqs + si) * P.hq + head;
-  // A guess at the row's piece counts, read while the attention kernel may still run: its workers
-  // record the counts when they start a row, and the entry keeps the previous step's counts until
-  // then, which are nearly always the same.  The guess only decides which rows the first round of
-  // loads asks for (rows never written are not in the L2); the counts used are read after the wait.
-  uint32_t guess = 0;
-  if (NVIS > 0 && live) guess = __ldcg(reinterpret_cast<const uint32_t*>(P.row_slots + 2 * row));
-  pdl_wait();
-  pdl_launch_dependents();
-  if (!live) return;
-  if (NVIS == 0) {
-    merge_row<D>(P, layer, si, head, sq, lane, P.extra_key_leader);
+  if (idx >= n_layers * P.n_seqs * P.hq) {
+    pdl_wait();
     return;
   }
-  constexpr int NV1 = NVIS > 0 ? NVIS : 1;   // visual rows of the first round
-  const int S = P.slots_per_stream;
-  const size_t base = (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots;
-  const uint32_t both = __ldcg(reinterpret_cast<const uint32_t*>(P.row_slots + 2 * row));
-  const int my_slot = lane < 16 ? lane : S + lane - 16;
-  float2 my_ml = make_float2(-INFINITY, 0.f);
-  if ((lane & 15) < S) my_ml = __ldcg(P.part_ml + (base + my_slot) * P.hq + head);
-  const int gv = min(min(static_cast<int>(guess & 0xffffu), NV1), S), gt = min(static_cast<int>(guess >> 16), 4);
-  float v[NV1 + 4][VPL];   // rows of visual slots 0..NV1-1 and text slots 0..3, as far as the guess goes
-#pragma unroll
-  for (int u = 0; u < NV1 + 4; ++u) {
-    const int s = u < NV1 ? u : S + u - NV1;
-    const float* src = P.part_acc + ((base + s) * P.hq + head) * D + lane * VPL;
-    if ((u < NV1 ? u : u - NV1) < (u < NV1 ? gv : gt)) {
-      if (VPL == 4) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(src));
-        v[u][0] = a.x, v[u][1] = a.y, v[u][2 % VPL] = a.z, v[u][3 % VPL] = a.w;
-      } else {
-        const float2 a = __ldcg(reinterpret_cast<const float2*>(src));
-        v[u][0] = a.x, v[u][1] = a.y;
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < VPL; ++e) v[u][e] = 0.f;
-    }
-  }
-  const int nv = sq.len_vis > 0 ? static_cast<int>(both & 0xffffu) : 0;
-  const int nt = static_cast<int>(both >> 16);
-  if (nv > 16 || nt > 16 || min(nv, NV1) > gv || min(nt, 4) > gt) {   // more pieces than guessed (or than this path holds)
-    merge_row<D>(P, layer, si, head, sq, lane, -1);
-    return;
-  }
-  const bool mine = lane < 16 ? lane < nv : lane - 16 < nt;
-  if (!mine) my_ml = make_float2(-INFINITY, 0.f);
-  float mmax = my_ml.x;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-  const float my_w = my_ml.y > 0.f ? exp2f(my_ml.x - mmax) : 0.f;   // (an empty partial counts for nothing)
-  float lsum = my_ml.y * my_w;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-  float acc[VPL];
-#pragma unroll
-  for (int e = 0; e < VPL; ++e) acc[e] = 0.f;
-#pragma unroll
-  for (int u = 0; u < NV1 + 4; ++u) {
-    const float w = __shfl_sync(0xffffffffu, my_w, u < NV1 ? u : 16 + u - NV1);   // lanes 0..15: visual slots, 16..: text slots
-    if (w > 0.f) {
-#pragma unroll
-      for (int e = 0; e < VPL; ++e) acc[e] = fmaf(v[u][e], w, acc[e]);
-    }
-  }
-  // rows beyond the first round's (visual rows past NV1, text rows past four): the rest of a stream
-  // in one more round of loads
-#pragma unroll 1
-  for (int t = (NV1 >= 16 ? 1 : 0); t < 2; ++t) {
-    const int n = t ? nt : nv, first = t ? 4 : NV1;
-    if (n <= first) continue;
-    float r[12][VPL];
-#pragma unroll
-    for (int u = 0; u < 12; ++u) {
-      const int s = first + u;
-      const float* src = P.part_acc + ((base + (t ? S : 0) + (s < n ? s : 0)) * P.hq + head) * D + lane * VPL;
-      if (VPL == 4) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(src));
-        r[u][0] = a.x, r[u][1] = a.y, r[u][2 % VPL] = a.z, r[u][3 % VPL] = a.w;
-      } else {
-        const float2 a = __ldcg(reinterpret_cast<const float2*>(src));
-        r[u][0] = a.x, r[u][1] = a.y;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 12; ++u) {
-      const int s = first + u;
-      const float w = __shfl_sync(0xffffffffu, my_w, (t ? 16 : 0) + (s & 15));
-      if (s < n && w > 0.f) {
-#pragma unroll
-        for (int e = 0; e < VPL; ++e) acc[e] = fmaf(r[u][e], w, acc[e]);
-      }
-    }
-  }
-  const float inv = 1.f / lsum;
-  const size_t orow = ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head);
-  uint16_t* dst = P.out + orow * D + lane * VPL;
-  if (VPL == 4) {
-    uint2 o;
-    o.x = f32_to_bf16_rne(acc[0] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[1] * inv)) << 16);
-    o.y = f32_to_bf16_rne(acc[2 % VPL] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[3 % VPL] * inv)) << 16);
-    *reinterpret_cast<uint2*>(dst) = o;
-  } else {
-    const uint32_t o = f32_to_bf16_rne(acc[0] * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(acc[1] * inv)) << 16);
-    *reinterpret_cast<uint32_t*>(dst) = o;
-  }
-  if (P.lse != nullptr && lane == 0) P.lse[orow] = (mmax + log2f(lsum)) * 0.6931471805599453f;
+  merge_row<D>(P, P.layer_begin + idx / (P.hq * P.n_seqs), (idx / P.hq) % P.n_seqs, idx % P.hq, lane);
 }
 
 template <int D>
@@ -785,15 +781,20 @@ constexpr int attend_smem_bytes() {
 // launchers
 // ------------------------------------------------------------------------------------------
 
+namespace {
+template <typename K>
+cudaError_t configure_attend(K kernel, int smem) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+}  // namespace
+
 cudaError_t configure_kernels(int* attend_smem) {
-  cudaError_t e = cudaFuncSetAttribute(attend_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       attend_smem_bytes<128>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attend_smem_bytes<128>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, attend_smem_bytes<64>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attend_smem_bytes<64>());
+  cudaError_t e = configure_attend(attend_kernel<128, false>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<128, true>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, false>, attend_smem_bytes<64>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, true>, attend_smem_bytes<64>());
   if (attend_smem) *attend_smem = attend_smem_bytes<128>();
   return e;
 }
@@ -808,7 +809,17 @@ cudaError_t launch_setup(const Params& p, const StepInline* inl, cudaStream_t st
 
 cudaError_t launch_plan(const Params& p, const LaunchList& list, int n_launches, cudaStream_t stream) {
   if (n_launches <= 0) return cudaSuccess;
-  return launch_pdl(plan_kernel, dim3(kPlanWorkers / 128, n_launches), dim3(128), 0, stream, p, list);
+  int ctas = 0;
+  bool rows = false;
+  for (int g = 0; g < n_launches; ++g) {
+    const LaunchDesc& l = list.launch[g];
+    if (l.fused_merge) ctas = max(ctas, (l.part_workers + l.part_wpc - 1) / l.part_wpc);
+    rows = rows || l.layer >= 0;
+  }
+  const int cta_blocks = (ctas + kPlanBlock - 1) / kPlanBlock;
+  const int row_blocks = rows ? (p.n_seqs * p.heads_per_item_dim + kPlanBlock - 1) / kPlanBlock : 0;
+  return launch_pdl(plan_kernel, dim3(kPlanWorkers / kPlanBlock + cta_blocks + row_blocks, n_launches), dim3(kPlanBlock), 0, stream, p,
+                    list, cta_blocks);
 }
 
 cudaError_t launch_append(const Params& p, cudaStream_t stream) {
@@ -819,8 +830,8 @@ cudaError_t launch_append(const Params& p, cudaStream_t stream) {
 cudaError_t launch_attend(const Params& p, int n_sms, cudaStream_t stream) {
   const int n_items = p.item_end - p.item_begin;
   if (!p.part_static && n_items <= 0) return cudaSuccess;
-  // static ranges: worker w is warp w / grid of CTA w % grid, so a launch with few workers still uses every SM
-  const int grid = min(n_sms, ((p.part_static ? p.part_workers : n_items) + kWarps - 1) / kWarps);
+  const int grid = p.part_static ? (p.part_workers + p.part_wpc - 1) / p.part_wpc
+                                 : min(n_sms * kAttendCtasPerSm, (n_items + kWarps - 1) / kWarps);
   if (p.d == 128) {
     if (p.part_static)
       return launch_pdl(attend_kernel<128, true>, dim3(grid), dim3(kThreads), attend_smem_bytes<128>(), stream, p);
@@ -837,16 +848,8 @@ cudaError_t launch_merge(const Params& p, cudaStream_t stream) {
   const int warps_per_block = 8;
   const int blocks = (n + warps_per_block - 1) / warps_per_block;
   const dim3 grid(blocks), block(warps_per_block * 32);
-  // the one-round path needs the recorded piece counts of the static partition and no extra key
-  const bool one_round = p.part_static && p.extra_key_leader < 0 && p.slots_per_stream >= 4;
-  if (p.d == 128) {
-    if (!one_round) return launch_pdl(merge_kernel<128, 0>, grid, block, 0, stream, p);
-    if (p.merge_wide) return launch_pdl(merge_kernel<128, 16>, grid, block, 0, stream, p);
-    return launch_pdl(merge_kernel<128, 4>, grid, block, 0, stream, p);
-  }
-  if (!one_round) return launch_pdl(merge_kernel<64, 0>, grid, block, 0, stream, p);
-  if (p.merge_wide) return launch_pdl(merge_kernel<64, 16>, grid, block, 0, stream, p);
-  return launch_pdl(merge_kernel<64, 4>, grid, block, 0, stream, p);
+  if (p.d == 128) return launch_pdl(merge_kernel<128>, grid, block, 0, stream, p);
+  return launch_pdl(merge_kernel<64>, grid, block, 0, stream, p);
 }
 
 cudaError_t launch_prefill_scatter(const Params& p, const int32_t* tok_seq, const int32_t* tok_stream,

@@ -36,7 +36,6 @@ struct SeqState {
 struct LaunchGroup {
   int job_begin, job_end, layer_begin, layer_end;
   int extra_key_leader;   // >= 0: the merge of these layers adds the step's new token (in-order schedule, GLA followers)
-  bool needs_merge;       // some output row of these layers is not merged by the attention kernel itself
   int wv, wt;             // tiles per page summed over the launch's visual / text jobs
   int w_min, w_max;       // smallest / largest tiles per page of a job of the launch
   int w_max_v, w_max_t;   // largest tiles per page among its visual / text jobs
@@ -53,7 +52,7 @@ struct OpenStep {
 };
 
 struct Layout {   // byte offsets into the workspace
-  size_t table, layer_flags, layer_kind, leader, jobs, plan, qcache, part_acc, part_ml, logits, items, step, err, counters, row_slots, row_done, wdesc, stage_q,
+  size_t table, layer_flags, layer_kind, leader, jobs, plan, qcache, part_acc, part_ml, logits, items, step, err, counters, row_slots, row_done, wdesc, cdesc, row_pieces, stage_q,
       stage_k, stage_v, stage_out, stage_lse, tok, total;
   size_t step_seqs, step_patches, step_bytes;   // offsets inside the step block
 };
@@ -121,12 +120,13 @@ struct qc_cache {
   std::vector<int> inorder_extra_key;             // per layer: the leader whose new token the merge adds, or -1
   int slots_per_stream = 0;
   int static_partition = -1;      // -1: static ranges when a step is several launches; 0 never; 1 always
-  bool fused_merge = false;       // the worker that delivers an output row's last partial merges it (no merge launch)
+  bool fused_merge = true;        // small launches of one layer merge their output rows themselves (no merge launch)
   bool fold_append = true;        // in-order schedule: new rows are taken and stored by the layer's own launch
   bool plan_ahead = true;         // one kernel per step works out where every worker of every launch starts
   int static_row_cost = 4;        // tiles a row counts for besides its pages (a worker's cost of one more item)
-  int static_min_tiles = 6;       // a static range is at least this long when the launch has the work for it
-                                  // (measured on launches of one layer: 3..8 equal, 12 and 16 slower)
+  int static_min_tiles = 1;       // a static range is at least this long when the launch has the work for it
+                                  // (and at least a page of the heaviest job).  Small launches want every
+                                  // worker there is: batch 1, 1 024 launches: 6 12.7 ms, 3 11.5, 1 11.0
   int text_streams_per_seq = 0;        // pages a sequence needs when its text crosses a page
 
   // pinned staging ring for step descriptors
@@ -207,7 +207,6 @@ void build_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vector<std::p
         j.stream = static_cast<uint8_t>(stream);
         j.n_cons = static_cast<uint8_t>(std::min(kMaxCons, e - first));
         j.flags = kFlagShared;
-        j.finish = static_cast<uint8_t>((1u << j.n_cons) - 1);   // a block's launch sweeps both streams of all its layers
         for (int x = 0; x < j.n_cons; ++x) {
           j.v_layer[x] = static_cast<uint8_t>(first + x);
           j.q_layer[x] = static_cast<uint8_t>(c);
@@ -223,7 +222,6 @@ void build_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vector<std::p
         j.stream = static_cast<uint8_t>(stream);
         j.n_cons = static_cast<uint8_t>(std::min(max_own, e - first));
         j.flags = (j.n_cons == 1) ? kFlagShared : 0;
-        j.finish = static_cast<uint8_t>((1u << j.n_cons) - 1);
         for (int x = 0; x < j.n_cons; ++x) {
           j.v_layer[x] = static_cast<uint8_t>(first + x);
           j.q_layer[x] = static_cast<uint8_t>(first + x);
@@ -238,7 +236,6 @@ void build_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vector<std::p
         j.stream = static_cast<uint8_t>(stream);
         j.n_cons = 1;
         j.flags = kFlagShared;
-        j.finish = 1;
         j.v_layer[0] = static_cast<uint8_t>(x);
         j.q_layer[0] = static_cast<uint8_t>(x);
         jobs.push_back(j);
@@ -283,7 +280,6 @@ void build_layer_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vector<
       j.stream = static_cast<uint8_t>(stream);
       j.n_cons = 1;
       j.flags = kFlagShared;
-      j.finish = 1;   // the layer's launch sweeps both of its streams
       j.v_layer[0] = static_cast<uint8_t>(l);
       j.q_layer[0] = static_cast<uint8_t>(l);
       j.k_layer = static_cast<uint8_t>(l);
@@ -323,13 +319,12 @@ void build_inorder_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vecto
     const int c = l;
     int e = l + 1;
     while (e < N && cfg->layer_kind[e] == QC_LAYER_LAZY) ++e;
-    auto own = [&](int layer, int k_layer, int stream, bool only_stream) {
+    auto own = [&](int layer, int k_layer, int stream) {
       Job j{};
       j.k_layer = static_cast<uint8_t>(k_layer);
       j.stream = static_cast<uint8_t>(stream);
       j.n_cons = 1;
       j.flags = kFlagShared;
-      j.finish = static_cast<uint8_t>(1 | (only_stream ? kFinishOwnStream : 0));
       j.v_layer[0] = static_cast<uint8_t>(layer);
       j.q_layer[0] = static_cast<uint8_t>(layer);
       jobs.push_back(j);
@@ -345,7 +340,6 @@ void build_inorder_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vecto
           j.v_layer[x] = static_cast<uint8_t>(first + x);
           j.q_layer[x] = static_cast<uint8_t>(c);
           if (skip_new && first + x != c) j.skip_new |= static_cast<uint8_t>(1u << x);
-          if (first + x == c) j.finish |= static_cast<uint8_t>(1u << x);   // the followers' rows are completed later
         }
         jobs.push_back(j);
       }
@@ -353,11 +347,11 @@ void build_inorder_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vecto
     // the leader's launch
     int job0 = static_cast<int>(jobs.size());
     if (cfg->lazy_mode == QC_MODE_VLA_EQ8 || e - c == 1) {
-      own(c, c, 1, false);
-      own(c, c, 0, false);
+      own(c, c, 1);
+      own(c, c, 0);
     } else if (cfg->lazy_mode == QC_MODE_VLA_QC) {
       shared(1, false);
-      own(c, c, 0, false);
+      own(c, c, 0);
     } else {
       shared(1, false);
       shared(0, true);
@@ -367,10 +361,10 @@ void build_inorder_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vecto
     for (int f = c + 1; f < e; ++f) {
       job0 = static_cast<int>(jobs.size());
       if (cfg->lazy_mode == QC_MODE_VLA_EQ8) {
-        own(f, c, 1, false);
-        own(f, f, 0, false);
+        own(f, c, 1);
+        own(f, f, 0);
       } else if (cfg->lazy_mode == QC_MODE_VLA_QC) {
-        own(f, f, 0, true);   // the visual partials are there already
+        own(f, f, 0);   // the visual partials are there already
       } else {
         extra_key[f] = c;
       }
@@ -402,6 +396,9 @@ int compute_sizes(const qc_config* cfg, Sizes* s) {
   // most kMaxChunkPages page ids); tiles per page differ by at most 5x between the jobs of a launch
   // (1 .. 1 + kMaxCons), so max_pages / 3 + 2 slots always leave room for a q within both bounds
   s->slots_per_stream = std::max((s->max_pages + s->chunk_pages - 1) / s->chunk_pages, (s->max_pages + 2) / 3 + 2);
+  // a cache for few sequences may cut a row finer, down to one page per worker
+  const int group = s->hq / s->hkv, rows = cfg->max_seqs * (group > 1 ? s->hkv * ((group + 7) / 8) : s->hq);
+  s->slots_per_stream = std::max(s->slots_per_stream, std::min(s->max_pages + 2, kPlanWorkers / rows + 2));
   s->max_slots = 2 * s->slots_per_stream;
   s->page_bytes = static_cast<size_t>(s->hkv) * kPage * s->D * 2;
   if (cfg->page_size == 0)
@@ -456,6 +453,8 @@ int compute_sizes(const qc_config* cfg, Sizes* s) {
   L.row_slots = take(N * S * s->hq * 2 * sizeof(uint16_t));
   L.row_done = take(N * S * s->hq * sizeof(int32_t));
   L.wdesc = take(std::min<size_t>(N, kMaxPlanLaunches) * kPlanWorkers * sizeof(WorkerDesc));
+  L.cdesc = take(std::min<size_t>(N, kMaxPlanLaunches) * kPlanCtas * sizeof(CtaDesc));
+  L.row_pieces = take(std::min<size_t>(N, kMaxPlanLaunches) * S * s->hq * sizeof(uint32_t));
   L.stage_q = take(N * S * s->hq * s->D * 2);
   L.stage_k = take(N * S * s->hkv * s->D * 2);
   L.stage_v = take(N * S * s->hkv * s->D * 2);
@@ -492,6 +491,8 @@ Params base_params(const qc_cache* c) {
   p.work_counter = reinterpret_cast<int32_t*>(c->ws + c->lay.counters);
   p.row_slots = reinterpret_cast<uint16_t*>(c->ws + c->lay.row_slots);
   p.row_done = reinterpret_cast<int32_t*>(c->ws + c->lay.row_done);
+  p.cdesc = reinterpret_cast<const CtaDesc*>(c->ws + c->lay.cdesc);
+  p.row_pieces = reinterpret_cast<uint32_t*>(c->ws + c->lay.row_pieces);
   p.slots_per_stream = c->slots_per_stream;
   p.extra_key_leader = -1;
   p.n_pool_pages = c->n_pool_pages;
@@ -632,14 +633,9 @@ int rebuild_plan(qc_cache* c, int per_launch) {
     const int begin = static_cast<int>(c->plan.size());
     g.wv = g.wt = g.w_max = g.w_max_v = g.w_max_t = 0;
     g.w_min = 1 << 20;
-    std::vector<bool> finished(c->cfg.n_layers, false);
     for (int j : order) {
       const int vb = c->plan_vis_before.back(), tb = c->plan_text_before.back();
-      Job job = jobs[j];
-      if (!c->fused_merge) job.finish = 0;
-      for (int x = 0; x < job.n_cons; ++x)
-        if ((job.finish >> x) & 1) finished[job.v_layer[x]] = true;
-      c->plan.push_back(PlanJob{job, vb, tb, g.wv, g.wt});
+      c->plan.push_back(PlanJob{jobs[j], vb, tb, g.wv, g.wt});
       c->plan_vis_before.push_back(vb + (jobs[j].stream ? 1 : 0));
       c->plan_text_before.push_back(tb + (jobs[j].stream ? 0 : 1));
       const int w = tiles_per_page(jobs[j]);
@@ -649,8 +645,6 @@ int rebuild_plan(qc_cache* c, int per_launch) {
       g.w_min = std::min(g.w_min, w);
       g.w_max = std::max(g.w_max, w);
     }
-    g.needs_merge = false;
-    for (int l = g.layer_begin; l < g.layer_end; ++l) g.needs_merge = g.needs_merge || !finished[l];
     c->groups.push_back(g);
     c->group_pos.emplace_back(begin, static_cast<int>(c->plan.size()));
   }
@@ -747,10 +741,8 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   c->group = s.hq / s.hkv;
   c->heads_per_item = c->group > 1 ? 8 : 1;
   // what one more item costs a worker, in tiles: a query-group item fetches its query fragments when it
-  // starts and leaves up to eight partial rows (measured on launches of one layer: 4 resp. 12 best,
-  // with ranges of at least 6 resp. 4 tiles)
+  // starts and leaves up to eight partial rows (measured on launches of one layer: 4 resp. 12 best)
   c->static_row_cost = c->group > 1 ? 12 : 4;
-  c->static_min_tiles = c->group > 1 ? 4 : 6;
   c->items_per_chunk = c->group > 1 ? s.hkv * ((c->group + 7) / 8) : s.hq;
   c->paged = cfg->page_size == 16;
   c->max_pages = s.max_pages;
@@ -1139,9 +1131,12 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     p.part_vw = one.part_vw;
     p.part_workers = one.part_workers;
     p.part_row_cost = one.part_row_cost;
-    p.merge_wide = one.merge_wide;
-    p.part_tiles = 0;
+    p.part_wpc = one.part_wpc;
+    p.part_wv = one.part_wv;
+    p.part_wt = one.part_wt;
   }
+  p.fused_merge = use_static ? launches.launch[gi].fused_merge : 0;
+  p.planned_pieces = use_static && launches.launch[gi].layer >= 0 ? 1 : 0;
   if (wait_in) QC_CUDA(cudaStreamWaitEvent(stream, wait_in, 0));
   if (append_first) {
     QC_CUDA(launch_append(p, stream));   // this group's layers only
@@ -1160,19 +1155,14 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     evl = &c->ev_launch[2 * c->ev_launches++];
     QC_CUDA(cudaEventRecord(evl[0], stream));
   }
-  if (!has_work) {
-    // (a GLA follower of the in-order schedule: its merge does everything)
-  } else if (c->group > 1) {
-    QC_CUDA(launch_attend_tc(p, c->ctx->n_sms, stream));
-  } else {
-    QC_CUDA(launch_attend(p, c->ctx->n_sms, stream));
-  }
+  // (a GLA follower of the in-order schedule has nothing to sweep: its merge does everything)
+  if (has_work) QC_CUDA(c->group > 1 ? launch_attend_tc(p, c->ctx->n_sms, stream) : launch_attend(p, c->ctx->n_sms, stream));
   if (evl) QC_CUDA(cudaEventRecord(evl[1], stream));
   if (ev && gi + 1 == c->groups.size()) QC_CUDA(cudaEventRecord(ev[2], stream));
-  if (c->groups[gi].needs_merge) QC_CUDA(launch_merge(p, stream));
+  if (!p.fused_merge) QC_CUDA(launch_merge(p, stream));
   if (record_done) QC_CUDA(cudaEventRecord(record_done, stream));
   c->attend_launches += has_work ? 1 : 0;
-  c->kernel_launches += (has_work ? 1 : 0) + (c->groups[gi].needs_merge ? 1 : 0);
+  c->kernel_launches += (has_work ? 1 : 0) + (p.fused_merge ? 0 : 1);
   return QC_OK;
 }
 
@@ -1236,7 +1226,7 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     // step, a long stream cut small also means many partial rows per output row for every one of
     // those launches' merges: beyond 24 rows the chunk is doubled as long as one and a half items
     // per worker remain.
-    const int64_t workers = static_cast<int64_t>(c->ctx->n_sms) * kAttendWarps * static_cast<int64_t>(c->groups.size());
+    const int64_t workers = static_cast<int64_t>(c->ctx->n_sms) * kWorkersPerSm * static_cast<int64_t>(c->groups.size());
     auto items_at = [&](int cp, int* max_slots) {
       int64_t cv = 0, ct = 0;
       int slots = 0;
@@ -1305,7 +1295,7 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   // faster (config 2, five blocks per launch: 0.89 against 1.05 ms per step; two blocks: 1.04
   // against 1.12).  Tile offsets are 32-bit.
   if (c->static_partition < 0) {
-    const int64_t workers = static_cast<int64_t>(c->ctx->n_sms) * kAttendWarps;
+    const int64_t workers = static_cast<int64_t>(c->ctx->n_sms) * kWorkersPerSm;
     for (const LaunchGroup& g : c->groups) {
       const int64_t tiles = static_cast<int64_t>(c->items_per_chunk) * (g.wv * tp_v + g.wt * tp_t);
       if (tiles > workers * 60 * std::max(1, g.w_min)) use_static = false;
@@ -1351,8 +1341,6 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   p.n_pos = use_static ? 0 : n_pos;   // static ranges need no item list
   p.n_items = n_items;
   p.part_static = use_static ? 1 : 0;
-  p.tp_v = static_cast<int32_t>(tp_v);
-  p.tp_t = static_cast<int32_t>(tp_t);
   p.n_patches = n_patches;
   p.tot_v = static_cast<int32_t>(tot_v);
   p.tot_t = static_cast<int32_t>(tot_t);
@@ -1365,6 +1353,9 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   p.fold_append = fold ? 1 : 0;
   p.fused_append = (n_patches == 0 && !pipe && !open_only && !fold) ? 1 : 0;
 
+  const bool planned = use_static && c->plan_ahead && c->groups.size() <= static_cast<size_t>(kMaxPlanLaunches) &&
+                       c->groups.size() <= static_cast<size_t>(std::min(c->cfg.n_layers, kMaxPlanLaunches)) &&
+                       c->ctx->n_sms * kWorkersPerSm <= kPlanWorkers;
   // static partition of every launch of the step (part_workers == 0: the launch has nothing to sweep)
   auto partition_of = [&](size_t gi) {
     const LaunchGroup& g = c->groups[gi];
@@ -1373,6 +1364,14 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     L.pos_begin = pb;
     L.pos_end = pe;
     L.part_row_cost = c->static_row_cost;
+    L.layer = -1;
+    if (planned && g.layer_end - g.layer_begin == 1) {
+      L.layer = g.layer_begin;
+      bool vis = false, text = false;   // swept here?
+      for (int pos = pb; pos < pe; ++pos) (c->plan[pos].job.stream ? vis : text) = true;
+      L.vis_launch = vis ? static_cast<int32_t>(gi) : c->leader[L.layer];
+      L.text_launch = text ? static_cast<int32_t>(gi) : c->leader[L.layer];
+    }
     const int64_t kv_tiles = static_cast<int64_t>(c->items_per_chunk) * (g.wv * tp_v + g.wt * tp_t);
     if (kv_tiles <= 0) return L;
     const int64_t T = kv_tiles + static_cast<int64_t>(c->items_per_chunk) * c->static_row_cost * n_seqs * (pe - pb);
@@ -1382,9 +1381,9 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     const int64_t row_max = std::max<int64_t>(static_cast<int64_t>(pmax_v) * g.w_max_v,
                                               static_cast<int64_t>(pmax_t) * g.w_max_t);
     const int64_t q_max = 30LL * w_lo;
-    int64_t q_min = std::max<int64_t>(2LL * g.w_max, (row_max + c->slots_per_stream - 3) / (c->slots_per_stream - 2));
+    int64_t q_min = std::max<int64_t>(g.w_max, (row_max + c->slots_per_stream - 3) / (c->slots_per_stream - 2));
     q_min = std::max<int64_t>(q_min, std::min<int64_t>(c->static_min_tiles, q_max / 2));
-    const int64_t W = static_cast<int64_t>(c->ctx->n_sms) * kAttendWarps;
+    const int64_t W = static_cast<int64_t>(c->ctx->n_sms) * kWorkersPerSm;
     int64_t k = 1, q;
     if (T > W * q_max) {   // several ranges per worker, each as long as a piece may be
       k = (T + W * q_max - 1) / (W * q_max);
@@ -1397,13 +1396,21 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     L.part_k = static_cast<int32_t>(k);
     L.part_workers = static_cast<int32_t>((vw + k - 1) / k);
     L.part_q = static_cast<int32_t>(q);
-    L.merge_wide = (static_cast<int64_t>(pmax_v) * g.w_max_v + q - 1) / q + 1 > 4 ? 1 : 0;
+    // few workers are spread over the chip rather than packed into few CTAs (batch 1: 13.2 against 13.5 ms)
+    const int n_ctas = c->ctx->n_sms * kAttendCtasPerSm;
+    L.part_wpc = std::min(kAttendWarps, std::max(1, (L.part_workers + n_ctas - 1) / n_ctas));
+    L.part_wv = g.wv;
+    L.part_wt = g.wt;
+    // Who merges the rows of a launch of one layer: with one query head per row, the launch itself
+    // (one merged row per query head is little work next to a launch of its own: 11.87 -> 10.28 ms for
+    // 1 024 such launches at batch 1, 33.0 -> 32.3 for 512 of 100 MB each); with query groups, whose every
+    // partial is seven or eight rows, a merge launch over the whole chip (the other way 19.1 -> 20.4
+    // for 896 launches at batch 32).
+    if (L.layer >= 0 && c->fused_merge && c->group == 1)
+      L.fused_merge = (L.part_workers + L.part_wpc - 1) / L.part_wpc <= kPlanCtas;
     return L;
   };
   LaunchList launches;
-  const bool planned = use_static && c->plan_ahead && c->groups.size() <= static_cast<size_t>(kMaxPlanLaunches) &&
-                       c->groups.size() <= static_cast<size_t>(std::min(c->cfg.n_layers, kMaxPlanLaunches)) &&
-                       c->ctx->n_sms * kAttendWarps <= kPlanWorkers;
   if (use_static)
     for (size_t gi = 0; gi < c->groups.size() && gi < static_cast<size_t>(kMaxPlanLaunches); ++gi)
       launches.launch[gi] = partition_of(gi);
@@ -1711,7 +1718,6 @@ int32_t qc_set_option(qc_cache* c, const char* key, int64_t value) {
   }
   if (k == "fused_merge") {   // 0: partial rows are merged by a launch of their own
     c->fused_merge = value != 0;
-    c->plan_dirty = true;
     return QC_OK;
   }
   if (k == "static_partition") {

@@ -1,0 +1,71 @@
+"""Attention launches that merge their own output rows, at the shapes where the split of a row decides
+which code runs: rows spread over many thread blocks (one or few sequences), many rows inside one
+block (short sequences), a row whose visual partials an earlier launch left, blocks of more layers
+than one sweep feeds."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from oracle.lazy_attention import LazyAttentionOracle
+from paper_2602_01901_b200 import binding as qc
+from paper_2602_01901_b200 import workloads as W
+from paper_2602_01901_b200.session import Session, bits_of
+from parity_util import assert_close, f64
+
+pytestmark = pytest.mark.gpu
+
+# head_dim, heads, lengths (text, visual) per sequence
+SHAPES = {
+    "one_long_row_per_head": (128, 1, [(40, 2500)]),
+    "rows_over_several_blocks": (64, 3, [(700, 900), (33, 1200)]),
+    "many_rows_in_a_block": (128, 2, [(1 + i % 19, (7 * i) % 40) for i in range(23)]),
+    "no_visual_tokens": (64, 4, [(15, 0), (16, 0), (17, 0)]),
+}
+
+
+def _dev(a, device):
+    return torch.from_numpy(a.astype(np.int16)).view(torch.bfloat16).to(device).contiguous()
+
+
+@pytest.mark.parametrize("mode", [qc.QC_MODE_VLA_QC, qc.QC_MODE_VLA_EQ8, qc.QC_MODE_GLA], ids=["qc", "eq8", "gla"])
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+def test_rows_merged_by_the_attention_launch(shape, mode):
+    head_dim, heads, lens = SHAPES[shape]
+    layer_kind = [0, 1, 1, 1, 1, 1, 0]   # a block of six layers (two sweeps), a layer alone
+    n, b, steps = len(layer_kind), len(lens), 3
+    longest = max(t + v for t, v in lens)
+    w = W.Workload(95, "row_merge", n, heads, heads, head_dim, 16, b, 1, longest, longest, 1, steps, tuple(range(1, 6)))
+    o = LazyAttentionOracle(n, heads, heads, head_dim, layer_kind, mode, n_seqs=b)
+    sessions = [Session(n, heads, heads, head_dim, layer_kind, max_seqs=b, max_tokens_per_seq=longest + steps,
+                        n_pages=2 * n * sum((t + steps + 31) // 16 + (v + 15) // 16 for t, v in lens), lazy_mode=mode,
+                        poison_pool=True) for _ in range(2)]
+    sessions[1].set_option("fused_merge", 0)
+    for s in sessions:
+        s.set_option("in_order_launches", 1)
+    for i, (text, vis) in enumerate(lens):
+        _, k, v = W.prefill_kv_np(w, i)
+        k, v = k[:, :text + vis], v[:, :text + vis]
+        kind = np.array([0] * text + [1] * vis, np.uint8)
+        for s in sessions:
+            s.prefill_append([i], [text + vis], kind, _dev(k, s.device), _dev(v, s.device))
+        o.prefill_append(i, kind.tolist(), f64(k), f64(v))
+    outs = [torch.empty((n, b, heads, head_dim), dtype=torch.bfloat16, device=s.device) for s in sessions]
+    lses = [torch.empty((n, b, heads), dtype=torch.float32, device=s.device) for s in sessions]
+    for step in range(steps):
+        qn, kn, vn = W.decode_qkv_np(w, step)
+        for s, out, lse in zip(sessions, outs, lses):
+            s.decode_step(list(range(b)), _dev(qn, s.device), _dev(kn, s.device), _dev(vn, s.device), out, lse)
+        for i in range(b):
+            ref, ref_lse = o.decode_step(i, f64(qn[:, i]), f64(kn[:, i]), f64(vn[:, i]))
+            for l in range(n):
+                for out, lse in zip(outs, lses):
+                    assert_close(bits_of(out)[l, i], ref[l], f"{shape} step {step} seq {i} layer {l}")
+                    assert np.max(np.abs(lse.cpu().numpy()[l, i] - ref_lse[l])) <= 2e-3
+    launches = [s.stats().kernel_launches for s in sessions]
+    assert launches[0] < launches[1]   # the rows were merged without launches of their own
+    for s in sessions:
+        assert s.stats().device_error == 0
+        s.close()
