@@ -229,9 +229,9 @@ struct PrefillMaps {
   CUtensorMap q, k, v, out;
 };
 cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, const uint8_t* layer_kind_dev,
-                                  const uint8_t* leader_dev, const void* q, const void* k, const void* v, void* out,
+                                  const uint8_t* leader_dev, const int* leader, const void* q, const void* k, const void* v, void* out,
                                   int32_t n_tokens, int32_t gla, const PrefillMaps* maps,
-                                  const uint8_t* tile_code_dev, int32_t seq_id, int32_t n0_text, int32_t n0_vis,
+                                  const uint8_t* tile_code_dev, const uint8_t* tile_code, int32_t seq_id, int32_t n0_text, int32_t n0_vis,
                                   const PrefillPass* passes_dev, int32_t n_single, int32_t n_shared,
                                   int32_t pair_min_tokens, cudaStream_t stream);   // qc_prefill.cu; maps null or head_dim 64 = mma.sync kernel
 cudaError_t configure_prefill_kernels();

@@ -18,6 +18,8 @@ namespace {
 constexpr int kBM = 64;   // query rows per CTA
 constexpr int kBN = 64;   // keys per tile
 constexpr int kPrefillThreads = 128;
+constexpr int kMaxLayers = 128;
+constexpr int kCodeTiles = 256;   // tiles whose codes travel as kernel arguments
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -43,6 +45,10 @@ struct PrefillArgs {
   CUtensorMap tmap_pool;   // the paged pool as a 2-D tensor [pages * hkv * 16 rows][D], box 16 rows x 64 elements
   int64_t n_pool_pages;    // bound for page ids read from the table
   const uint8_t* tile_code;    // [ceil(T / 64)] device: 0 = the 64-token tile is all text, 1 = all visual, 2 = mixed
+  // what a CTA needs before its first copy, as kernel arguments: each layer's block leader (itself if
+  // it is ordinary), and the codes of the first tiles, two bits each
+  uint8_t lead_of[kMaxLayers];
+  uint32_t code_bits[kCodeTiles / 16];
   const uint16_t* q;     // [n_layers][T][hq][D]
   const uint16_t* k;     // [n_layers][T][hkv][D]
   const uint16_t* v;     // [n_layers][T][hkv][D]
@@ -520,8 +526,8 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
   }
   const int layer = v_layer[0];   // decides where Q and K come from; with NV > 1 all consumers share that
   const int kvh = head / A.group;
-  const bool lazy = A.layer_kind[layer] != 0;
-  const int lead = A.leader[layer];
+  const int lead = A.lead_of[layer];
+  const bool lazy = lead != layer;
   const bool gla = A.gla != 0;
   const int m0 = qt * kTM;
   const int row = m0 + threadIdx.x;                 // a softmax thread's query row
@@ -532,22 +538,176 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
   const int n_cached = ct_text + ct_vis;
   const int n_ktiles = n_cached + min((A.T + kTN - 1) / kTN, (m0 + kTM + kTN - 1) / kTN);
 
-  if (threadIdx.x == 0) {
-    mbar_init(&bar_s[0], 1);
-    mbar_init(&bar_s[1], 1);
-    mbar_init(&bar_q, 2);
-    mbar_init(&bar_e, kTM);
-    mbar_init(&bar_r, 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&bar_k[b], 1);
-      mbar_init(&bar_v[b], n_cons);
-      mbar_init(&bar_o[b], 1);
-      mbar_init(&bar_p[b], kTM);
+  // Fetch key tile (is_k) or value tile kt into `dst`; completion is one phase of `bar`.
+  // `which`: 0 = 64 query rows (tile index kt counts 64-row tiles), 1 = key tile, 2 = value tile.
+  // The 64 rows go to `dst` and `dst + half` (the two 64-column halves).
+  auto code_of = [&](int kt) -> int {   // of a VLA lazy layer
+    return kt < kCodeTiles ? (A.code_bits[kt >> 4] >> (2 * (kt & 15))) & 3 : A.tile_code[kt];
+  };
+  const int k_text_layer = (CACHED && A.n0_text && !(A.layer_flags[layer] & kLayerOwnsTextK)) ? lead : layer;
+  // Where cached tile kt of the key (which = 1) or value (which = 2) sequence lives: source layer,
+  // stream, first token and the stream's length.
+  auto cached_tile = [&](int which, int kt, int& src, int& stream, int& ord0, int& n_valid) {
+    if (kt < ct_text) {
+      src = which == 1 ? k_text_layer : layer, stream = which == 1 ? 0 : 2, ord0 = kt * kTN, n_valid = A.n0_text;
+    } else {
+      src = which == 1 ? (lazy ? lead : layer) : layer, stream = which == 1 ? 1 : 3;
+      ord0 = (kt - ct_text) * kTN, n_valid = A.n0_vis;
     }
-    fence_mbar_init();
-    failed = 0;
-  }
-  if (warp == 4) {   // the score warp owns the TMEM allocation
+  };
+  // Lanes 0..3 read the page ids of a cached tile's four pages (0 where the page holds no token).
+  auto load_page_ids = [&](int which, int kt) -> int {
+    int src, stream, ord0, n_valid, pid = 0;
+    cached_tile(which, kt, src, stream, ord0, n_valid);
+    if (lane < 4 && ord0 + 16 * lane < n_valid) {
+      const size_t trow = ((static_cast<size_t>(src) * 4 + stream) * A.max_seqs + A.seq_id) * A.max_pages;
+      pid = A.table[trow + ord0 / 16 + lane];
+    }
+    return pid;
+  };
+  // Fetch cached tile kt: 64 tokens of one stream of (source layer, this sequence) from the paged
+  // pool, as four pages.  A page that is full arrives by two tensor-map copies; the rows of a
+  // page that is not (the stream's last page, or pages past its end) are gathered or zeroed by
+  // the lanes, since their pool rows may hold anything and a zero weight does not cancel a NaN.
+  int ahead_tile[2] = {-1, -1}, ahead_pid[2] = {0, 0};   // page ids requested one tile ahead, per which
+  auto fetch_cached = [&](int which, int kt, uint32_t dst, uint32_t half, uint64_t* bar) {
+    int src, stream, ord0, n_valid;
+    cached_tile(which, kt, src, stream, ord0, n_valid);
+    int pid = ahead_tile[which - 1] == kt ? ahead_pid[which - 1] : load_page_ids(which, kt);
+    if (kt + 1 < n_cached) {   // the next tile's ids travel while this tile is fetched and consumed
+      ahead_tile[which - 1] = kt + 1;
+      ahead_pid[which - 1] = load_page_ids(which, kt + 1);
+    }
+    if (static_cast<uint32_t>(pid) >= static_cast<uint64_t>(A.n_pool_pages)) {   // never read outside the pool
+      atomicMax(err, kErrBadPage);
+      pid = 0;
+    }
+    int n_full = 0;
+    bool gathered = false;
+#pragma unroll
+    for (int pg = 0; pg < 4; ++pg) {
+      const int p_id = __shfl_sync(0xffffffffu, pid, pg);
+      const int n_tok = min(16, max(0, n_valid - (ord0 + 16 * pg)));
+      if (n_tok == 16) {
+        ++n_full;
+        continue;
+      }
+      gathered = true;
+      for (int e = lane; e < 16 * (kTD / 8); e += 32) {
+        const int r = 16 * pg + (e >> 4), c = e & 15;
+        const uint32_t d = dst + (c >> 3) * half + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+        if ((e >> 4) < n_tok) {
+          cp_async16(d, A.pool + ((static_cast<size_t>(p_id) * A.hkv + kvh) * 16 + (e >> 4)) * kTD + c * 8);
+        } else {
+          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0u) : "memory");
+        }
+      }
+    }
+    if (gathered) {
+      cp_async_commit();
+      cp_async_wait<0>();
+      fence_proxy_async();
+      __syncwarp();
+    }
+    if (n_full == 0) {
+      if (lane == 0) mbar_arrive(bar);
+      return;
+    }
+    if (lane == 0) mbar_expect_tx(bar, n_full * 4096);
+#pragma unroll
+    for (int pg = 0; pg < 4; ++pg) {
+      const int p_id = __shfl_sync(0xffffffffu, pid, pg);
+      if (n_valid - (ord0 + 16 * pg) >= 16 && lane == 0) {
+        const int32_t row = (p_id * A.hkv + kvh) * 16;
+        tensor_g2s_2d(dst + pg * 2048, &A.tmap_pool, 0, row, bar);
+        tensor_g2s_2d(dst + half + pg * 2048, &A.tmap_pool, 64, row, bar);
+      }
+    }
+  };
+  // `which`: 0 = 64 query rows (kt counts 64-row tiles of the prompt), 1 = key tile kt, 2 = value
+  // tile kt of the CTA's tile sequence (cached tiles first).
+  auto fetch_tile = [&](int which, int kt, uint32_t dst, uint32_t half, uint64_t* bar, int v_src = -1) {
+    if (which != 0) {
+      if (CACHED && kt < n_cached) {
+        fetch_cached(which, kt, dst, half, bar);
+        return;
+      }
+      kt -= n_cached;   // a tile of new tokens
+    }
+    int src = (which == 2 && v_src >= 0) ? v_src : layer;
+    bool mixed = false;
+    if (which != 2 && lazy && kt * kTN < A.T) {   // queries and keys of a lazy layer: the leader's for visual rows
+      if (gla) {
+        src = lead;
+      } else {
+        const int code = code_of(kt);
+        mixed = code == 2;
+        src = code == 1 ? lead : layer;
+      }
+    }
+    if (!mixed) {
+      if (lane == 0) {
+        const void* tm = which == 0 ? static_cast<const void*>(&A.tmap_q)
+                                    : (which == 1 ? static_cast<const void*>(&A.tmap_k) : static_cast<const void*>(&A.tmap_v));
+        const int h = which == 0 ? head : kvh;
+        mbar_expect_tx(bar, kKV);
+        tensor_g2s_3d(dst, tm, 0, h, src * A.T + kt * kTN, bar);
+        tensor_g2s_3d(dst + half, tm, 64, h, src * A.T + kt * kTN, bar);
+      }
+    } else {   // rows of two layers: gather with 16-byte copies (64 rows x 16 chunks over 32 lanes)
+      const uint16_t* from = which == 0 ? A.q : A.k;
+      const int heads = which == 0 ? A.hq : A.hkv, h = which == 0 ? head : kvh;
+      for (int e = lane; e < kTN * (kTD / 8); e += 32) {
+        const int r = e >> 4, c = e & 15, t = kt * kTN + r;
+        const uint32_t d = dst + (c >> 3) * half + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+        if (t < A.T) {
+          const int l = A.kind[t] ? lead : layer;
+          cp_async16(d, from + ((static_cast<size_t>(l) * A.T + t) * heads + h) * kTD + c * 8);
+        } else {
+          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0u) : "memory");
+        }
+      }
+      cp_async_commit();
+      cp_async_wait<0>();
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar);
+    }
+  };
+  auto fetch_values = [&](int kt) {   // one tile per consumer; bar_v[kt & 1] counts them all
+    const int b = kt & 1;
+#pragma unroll
+    for (int x = 0; x < NV; ++x)
+      if (x < n_cons) fetch_tile(2, kt, sV + (2 * x + b) * kKV, kTN * 128, &bar_v[b], v_layer[x]);
+  };
+  if (warp == 5) {
+    // The load warp sets the barriers up and requests the first tiles at once; the other warps
+    // first touch them after the CTA's barrier, by which time the copies are on their way.
+    if (lane == 0) {
+      mbar_init(&bar_s[0], 1);
+      mbar_init(&bar_s[1], 1);
+      mbar_init(&bar_q, 2);
+      mbar_init(&bar_e, kTM);
+      mbar_init(&bar_r, 1);
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&bar_k[b], 1);
+        mbar_init(&bar_v[b], n_cons);
+        mbar_init(&bar_o[b], 1);
+        mbar_init(&bar_p[b], kTM);
+      }
+      fence_mbar_init();
+      failed = 0;
+    }
+    __syncwarp();
+    fetch_tile(0, 2 * qt, sQ, kTM * 128, &bar_q);
+    fetch_tile(1, 0, sK, kTN * 128, &bar_k[0]);
+    fetch_tile(0, 2 * qt + 1, sQ + kTN * 128, kTM * 128, &bar_q);
+    fetch_values(0);
+    if (n_ktiles > 1) {
+      fetch_tile(1, 1, sK + kKV, kTN * 128, &bar_k[1]);
+      fetch_values(1);
+    }
+  } else if (warp == 4) {   // the score warp owns the TMEM allocation
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
                  "r"(kCols)
                  : "memory");
@@ -564,152 +724,6 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
 
   if (warp >= 4) {
     // ------------------------------------------------------------------ tile fetch + product issue
-    // Fetch key tile (is_k) or value tile kt into `dst`; completion is one phase of `bar`.
-    // `which`: 0 = 64 query rows (tile index kt counts 64-row tiles), 1 = key tile, 2 = value tile.
-    // The 64 rows go to `dst` and `dst + half` (the two 64-column halves).
-    // The tile codes of a VLA lazy layer, read once: lane i holds tiles i, i + 32, i + 64.
-    uint32_t codes[3] = {0u, 0u, 0u};
-    if (warp == 5 && lazy && !gla) {
-      const int n_tiles = (A.T + kTN - 1) / kTN;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        if (lane + 32 * i < n_tiles) codes[i] = A.tile_code[lane + 32 * i];
-    }
-    auto code_of = [&](int kt) -> int {   // whole warp
-      if (kt >= 96) return A.tile_code[kt];
-      const uint32_t c = kt < 32 ? codes[0] : (kt < 64 ? codes[1] : codes[2]);
-      return static_cast<int>(__shfl_sync(0xffffffffu, c, kt & 31));
-    };
-    const int k_text_layer = (CACHED && A.n0_text && !(A.layer_flags[layer] & kLayerOwnsTextK)) ? lead : layer;
-    // Where cached tile kt of the key (which = 1) or value (which = 2) sequence lives: source layer,
-    // stream, first token and the stream's length.
-    auto cached_tile = [&](int which, int kt, int& src, int& stream, int& ord0, int& n_valid) {
-      if (kt < ct_text) {
-        src = which == 1 ? k_text_layer : layer, stream = which == 1 ? 0 : 2, ord0 = kt * kTN, n_valid = A.n0_text;
-      } else {
-        src = which == 1 ? (lazy ? lead : layer) : layer, stream = which == 1 ? 1 : 3;
-        ord0 = (kt - ct_text) * kTN, n_valid = A.n0_vis;
-      }
-    };
-    // Lanes 0..3 read the page ids of a cached tile's four pages (0 where the page holds no token).
-    auto load_page_ids = [&](int which, int kt) -> int {
-      int src, stream, ord0, n_valid, pid = 0;
-      cached_tile(which, kt, src, stream, ord0, n_valid);
-      if (lane < 4 && ord0 + 16 * lane < n_valid) {
-        const size_t trow = ((static_cast<size_t>(src) * 4 + stream) * A.max_seqs + A.seq_id) * A.max_pages;
-        pid = A.table[trow + ord0 / 16 + lane];
-      }
-      return pid;
-    };
-    // Fetch cached tile kt: 64 tokens of one stream of (source layer, this sequence) from the paged
-    // pool, as four pages.  A page that is full arrives by two tensor-map copies; the rows of a
-    // page that is not (the stream's last page, or pages past its end) are gathered or zeroed by
-    // the lanes, since their pool rows may hold anything and a zero weight does not cancel a NaN.
-    int ahead_tile[2] = {-1, -1}, ahead_pid[2] = {0, 0};   // page ids requested one tile ahead, per which
-    auto fetch_cached = [&](int which, int kt, uint32_t dst, uint32_t half, uint64_t* bar) {
-      int src, stream, ord0, n_valid;
-      cached_tile(which, kt, src, stream, ord0, n_valid);
-      int pid = ahead_tile[which - 1] == kt ? ahead_pid[which - 1] : load_page_ids(which, kt);
-      if (kt + 1 < n_cached) {   // the next tile's ids travel while this tile is fetched and consumed
-        ahead_tile[which - 1] = kt + 1;
-        ahead_pid[which - 1] = load_page_ids(which, kt + 1);
-      }
-      if (static_cast<uint32_t>(pid) >= static_cast<uint64_t>(A.n_pool_pages)) {   // never read outside the pool
-        atomicMax(err, kErrBadPage);
-        pid = 0;
-      }
-      int n_full = 0;
-      bool gathered = false;
-#pragma unroll
-      for (int pg = 0; pg < 4; ++pg) {
-        const int p_id = __shfl_sync(0xffffffffu, pid, pg);
-        const int n_tok = min(16, max(0, n_valid - (ord0 + 16 * pg)));
-        if (n_tok == 16) {
-          ++n_full;
-          continue;
-        }
-        gathered = true;
-        for (int e = lane; e < 16 * (kTD / 8); e += 32) {
-          const int r = 16 * pg + (e >> 4), c = e & 15;
-          const uint32_t d = dst + (c >> 3) * half + r * 128 + (((c & 7) ^ (r & 7)) << 4);
-          if ((e >> 4) < n_tok) {
-            cp_async16(d, A.pool + ((static_cast<size_t>(p_id) * A.hkv + kvh) * 16 + (e >> 4)) * kTD + c * 8);
-          } else {
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0u) : "memory");
-          }
-        }
-      }
-      if (gathered) {
-        cp_async_commit();
-        cp_async_wait<0>();
-        fence_proxy_async();
-        __syncwarp();
-      }
-      if (n_full == 0) {
-        if (lane == 0) mbar_arrive(bar);
-        return;
-      }
-      if (lane == 0) mbar_expect_tx(bar, n_full * 4096);
-#pragma unroll
-      for (int pg = 0; pg < 4; ++pg) {
-        const int p_id = __shfl_sync(0xffffffffu, pid, pg);
-        if (n_valid - (ord0 + 16 * pg) >= 16 && lane == 0) {
-          const int32_t row = (p_id * A.hkv + kvh) * 16;
-          tensor_g2s_2d(dst + pg * 2048, &A.tmap_pool, 0, row, bar);
-          tensor_g2s_2d(dst + half + pg * 2048, &A.tmap_pool, 64, row, bar);
-        }
-      }
-    };
-    // `which`: 0 = 64 query rows (kt counts 64-row tiles of the prompt), 1 = key tile kt, 2 = value
-    // tile kt of the CTA's tile sequence (cached tiles first).
-    auto fetch_tile = [&](int which, int kt, uint32_t dst, uint32_t half, uint64_t* bar, int v_src = -1) {
-      if (which != 0) {
-        if (CACHED && kt < n_cached) {
-          fetch_cached(which, kt, dst, half, bar);
-          return;
-        }
-        kt -= n_cached;   // a tile of new tokens
-      }
-      int src = (which == 2 && v_src >= 0) ? v_src : layer;
-      bool mixed = false;
-      if (which != 2 && lazy && kt * kTN < A.T) {   // queries and keys of a lazy layer: the leader's for visual rows
-        if (gla) {
-          src = lead;
-        } else {
-          const int code = code_of(kt);
-          mixed = code == 2;
-          src = code == 1 ? lead : layer;
-        }
-      }
-      if (!mixed) {
-        if (lane == 0) {
-          const void* tm = which == 0 ? static_cast<const void*>(&A.tmap_q)
-                                      : (which == 1 ? static_cast<const void*>(&A.tmap_k) : static_cast<const void*>(&A.tmap_v));
-          const int h = which == 0 ? head : kvh;
-          mbar_expect_tx(bar, kKV);
-          tensor_g2s_3d(dst, tm, 0, h, src * A.T + kt * kTN, bar);
-          tensor_g2s_3d(dst + half, tm, 64, h, src * A.T + kt * kTN, bar);
-        }
-      } else {   // rows of two layers: gather with 16-byte copies (64 rows x 16 chunks over 32 lanes)
-        const uint16_t* from = which == 0 ? A.q : A.k;
-        const int heads = which == 0 ? A.hq : A.hkv, h = which == 0 ? head : kvh;
-        for (int e = lane; e < kTN * (kTD / 8); e += 32) {
-          const int r = e >> 4, c = e & 15, t = kt * kTN + r;
-          const uint32_t d = dst + (c >> 3) * half + r * 128 + (((c & 7) ^ (r & 7)) << 4);
-          if (t < A.T) {
-            const int l = A.kind[t] ? lead : layer;
-            cp_async16(d, from + ((static_cast<size_t>(l) * A.T + t) * heads + h) * kTD + c * 8);
-          } else {
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0u) : "memory");
-          }
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar);
-      }
-    };
     bool ok = true;
     auto wait_on = [&](uint64_t* bar, uint32_t& phase) {   // warp-uniform bounded wait
       if (ok && !__all_sync(0xffffffffu, mbar_try_wait(bar, phase)))   // usually complete at the first look
@@ -823,20 +837,6 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
       // The two streams advance independently (the products complete in the order S, S, PV, S, PV, ...),
       // so the warp polls both barriers without blocking on either.
       uint32_t ph_s[2] = {0, 0}, ph_o[2] = {0, 0};
-      fetch_tile(0, 2 * qt, sQ, kTM * 128, &bar_q);
-      fetch_tile(1, 0, sK, kTN * 128, &bar_k[0]);
-      fetch_tile(0, 2 * qt + 1, sQ + kTN * 128, kTM * 128, &bar_q);
-      auto fetch_values = [&](int kt) {   // one tile per consumer; bar_v[kt & 1] counts them all
-        const int b = kt & 1;
-#pragma unroll
-        for (int x = 0; x < NV; ++x)
-          if (x < n_cons) fetch_tile(2, kt, sV + (2 * x + b) * kKV, kTN * 128, &bar_v[b], v_layer[x]);
-      };
-      fetch_values(0);
-      if (n_ktiles > 1) {
-        fetch_tile(1, 1, sK + kKV, kTN * 128, &bar_k[1]);
-        fetch_values(1);
-      }
       int k_next = 2, v_next = 2;
       uint32_t idle = 0;
       while ((k_next < n_ktiles || v_next < n_ktiles) && ok) {
@@ -910,8 +910,10 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
       }
       float mx[4] = {p[0], p[1], p[2], p[3]};
 #pragma unroll
-      for (int j = 4; j < kTN; ++j) mx[j & 3] = fmaxf(mx[j & 3], p[j]);
-      const float m_tile = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * A.scale_log2;   // the scale is positive
+      for (int j = 4; j < kTN - 4; j += 2) mx[(j >> 1) & 3] = max3(mx[(j >> 1) & 3], p[j], p[j + 1]);
+      mx[0] = max3(mx[0], p[kTN - 4], p[kTN - 3]);
+      mx[1] = max3(mx[1], p[kTN - 2], p[kTN - 1]);
+      const float m_tile = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * A.scale_log2;   // the scale is positive
       float corr = 1.f;
       if (m_tile > m_ref + kRescaleThreshold || m_ref == -INFINITY) {
         if (m_tile != -INFINITY) {
@@ -920,13 +922,17 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
         }
       }
       const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-      float ps[4] = {0.f, 0.f, 0.f, 0.f};
+      // scale, exponential and sum of two scores at a time: the softmax threads are short of issue
+      // slots, not of special-function throughput
+      float2 ps[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-      for (int j = 0; j < kTN; ++j) {
-        p[j] = ex2_approx(fmaf(p[j], A.scale_log2, neg_m));
-        ps[j & 3] += p[j];
+      for (int j = 0; j < kTN; j += 2) {
+        const float2 x = fma2(make_float2(p[j], p[j + 1]), make_float2(A.scale_log2, A.scale_log2), make_float2(neg_m, neg_m));
+        p[j] = ex2_approx(x.x);
+        p[j + 1] = ex2_approx(x.y);
+        ps[(j >> 1) & 1] = add2(ps[(j >> 1) & 1], make_float2(p[j], p[j + 1]));
       }
-      l_sum = l_sum * corr + ((ps[0] + ps[1]) + (ps[2] + ps[3]));
+      l_sum = l_sum * corr + ((ps[0].x + ps[0].y) + (ps[1].x + ps[1].y));
       if (kt > 0 && __any_sync(0xffffffffu, corr != 1.f)) {   // rare: move the accumulator to the new reference
         // PV(kt-1) -- and with it every earlier value product -- must be done: phase (kt-1)/2 of its barrier
         ok = bounded_wait(&bar_o[(kt - 1) & 1], ((kt - 1) >> 1) & 1) && !failed;
@@ -1494,9 +1500,9 @@ cudaError_t configure_prefill_kernels() {
 }
 
 cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, const uint8_t* layer_kind_dev,
-                                  const uint8_t* leader_dev, const void* q, const void* k, const void* v, void* out,
+                                  const uint8_t* leader_dev, const int* leader, const void* q, const void* k, const void* v, void* out,
                                   int32_t T, int32_t gla, const PrefillMaps* maps,
-                                  const uint8_t* tile_code_dev, int32_t seq_id, int32_t n0_text, int32_t n0_vis,
+                                  const uint8_t* tile_code_dev, const uint8_t* tile_code, int32_t seq_id, int32_t n0_text, int32_t n0_vis,
                                   const PrefillPass* passes_dev, int32_t n_single, int32_t n_shared,
                                   int32_t pair_min_tokens, cudaStream_t stream) {
   if (T <= 0) return cudaSuccess;
@@ -1531,6 +1537,8 @@ cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, cons
     a.tmap_v = maps->v;
     a.tmap_o = maps->out;
     a.tile_code = tile_code_dev;
+    for (int l = 0; l < p.n_layers; ++l) a.lead_of[l] = static_cast<uint8_t>(leader[l]);
+    for (int i = 0; i < min(kCodeTiles, (T + 63) / 64); ++i) a.code_bits[i >> 4] |= static_cast<uint32_t>(tile_code[i]) << (2 * (i & 15));
     const dim3 grid5((T + kTM - 1) / kTM, p.hq, p.n_layers);
     // prompts that start a sequence, from pair_min_tokens on: two query tiles per CTA, 128-key tiles
     const bool pair = pair_min_tokens > 0 && T >= pair_min_tokens;

@@ -1019,9 +1019,9 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
     ev = &c->ev_prefill[2 * c->ev_prefill_calls];
     QC_CUDA(cudaEventRecord(ev[0], stream));
   }
-  QC_CUDA(launch_prefill_attend(p, kind_dev, c->ws + c->lay.layer_kind, c->ws + c->lay.leader, q_dev, k_dev, v_dev,
+  QC_CUDA(launch_prefill_attend(p, kind_dev, c->ws + c->lay.layer_kind, c->ws + c->lay.leader, c->leader.data(), q_dev, k_dev, v_dev,
                                 out_dev, n_tokens, c->cfg.lazy_mode == QC_MODE_GLA ? 1 : 0, tc5 ? &maps : nullptr,
-                                codes_dev, seq_id, n0_text, n0_vis, (tc5 && share) ? passes_dev : nullptr,
+                                codes_dev, codes.data(), seq_id, n0_text, n0_vis, (tc5 && share) ? passes_dev : nullptr,
                                 c->prefill_n_single, c->prefill_n_shared, c->prefill_pair_min_tokens, stream));
   const bool shared_run = tc5 && share;
   if (ev) {
