@@ -376,7 +376,7 @@ __device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, ui
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRingTc);
     if (early_tiles) fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
     if (P.wdesc != nullptr) {
-      begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
+      if (first.n_pages > 2) begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
       it = ctx[1].ip.item;
       more = it.n_pages > 0;
     } else {

@@ -743,6 +743,7 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   // what one more item costs a worker, in tiles: a query-group item fetches its query fragments when it
   // starts and leaves up to eight partial rows (measured on launches of one layer: 4 resp. 12 best)
   c->static_row_cost = c->group > 1 ? 12 : 4;
+  c->static_min_tiles = c->group > 1 ? 4 : 1;
   c->items_per_chunk = c->group > 1 ? s.hkv * ((c->group + 7) / 8) : s.hq;
   c->paged = cfg->page_size == 16;
   c->max_pages = s.max_pages;
@@ -1381,7 +1382,10 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     const int64_t row_max = std::max<int64_t>(static_cast<int64_t>(pmax_v) * g.w_max_v,
                                               static_cast<int64_t>(pmax_t) * g.w_max_t);
     const int64_t q_max = 30LL * w_lo;
-    int64_t q_min = std::max<int64_t>(g.w_max, (row_max + c->slots_per_stream - 3) / (c->slots_per_stream - 2));
+    // at least a page of the heaviest job, with query groups two (each of a row's pieces then is seven or
+    // eight partial rows to merge: batch 1, 160 launches: one page 2.93 ms, two 2.45; batch 8 2.36 / 2.12)
+    int64_t q_min = std::max<int64_t>(c->group > 1 ? 2 * g.w_max : g.w_max,
+                                      (row_max + c->slots_per_stream - 3) / (c->slots_per_stream - 2));
     q_min = std::max<int64_t>(q_min, std::min<int64_t>(c->static_min_tiles, q_max / 2));
     const int64_t W = static_cast<int64_t>(c->ctx->n_sms) * kWorkersPerSm;
     int64_t k = 1, q;
@@ -1401,12 +1405,12 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     L.part_wpc = std::min(kAttendWarps, std::max(1, (L.part_workers + n_ctas - 1) / n_ctas));
     L.part_wv = g.wv;
     L.part_wt = g.wt;
-    // Who merges the rows of a launch of one layer: with one query head per row, the launch itself
-    // (one merged row per query head is little work next to a launch of its own: 11.87 -> 10.28 ms for
-    // 1 024 such launches at batch 1, 33.0 -> 32.3 for 512 of 100 MB each); with query groups, whose every
-    // partial is seven or eight rows, a merge launch over the whole chip (the other way 19.1 -> 20.4
-    // for 896 launches at batch 32).
-    if (L.layer >= 0 && c->fused_merge && c->group == 1)
+    // Who merges the rows of a launch of one layer.  With one query head per row and at most two rows per
+    // CTA the launch itself: 8 layers, 20 steps, merge launch -> own merge: 64 rows of 3 000 keys 3.97 ->
+    // 3.61 ms, 224 of 800 3.46 -> 3.40, 512 of 576 5.77 -> 5.81, 1 024 of 120 5.12 -> 5.21 (and 1 024 launches
+    // at batch 1 11.87 -> 10.28).  With query groups, whose every partial is seven or eight rows, a merge
+    // launch over the whole chip (896 launches at batch 32: 19.1, the other way 20.4).
+    if (L.layer >= 0 && c->fused_merge && c->group == 1 && static_cast<int64_t>(n_seqs) * c->hq <= 2LL * n_ctas)
       L.fused_merge = (L.part_workers + L.part_wpc - 1) / L.part_wpc <= kPlanCtas;
     return L;
   };
