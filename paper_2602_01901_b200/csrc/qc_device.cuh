@@ -90,6 +90,15 @@ __device__ __forceinline__ void tensor_g2s_2d(uint32_t dst_smem, const void* tma
       : "memory");
 }
 
+__device__ __forceinline__ void tensor_g2s_3d(uint32_t dst_smem, const void* tmap, int32_t x, int32_t y, int32_t z,
+                                              uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+          "r"(dst_smem),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+      : "memory");
+}
+
 // Asynchronous global -> shared copies of 4 or 16 bytes (no registers held while in flight);
 // cp_async_wait_all() waits for the calling thread's own copies.
 __device__ __forceinline__ void cp_async_4(void* dst_smem, const void* src) {

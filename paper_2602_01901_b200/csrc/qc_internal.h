@@ -209,9 +209,15 @@ cudaError_t launch_plan(const Params& p, const LaunchList& list, int n_launches,
 cudaError_t launch_attend(const Params& p, int n_sms, cudaStream_t stream);      // one query head per item
 cudaError_t launch_attend_tc(const Params& p, int n_sms, cudaStream_t stream);   // query-group items (GQA)
 cudaError_t launch_merge(const Params& p, cudaStream_t stream);
-cudaError_t launch_prefill_scatter(const Params& p, const int32_t* tok_seq, const int32_t* tok_stream,
-                                   const int32_t* tok_ord, int32_t n_tokens, int32_t tok_stride,
-                                   int32_t tok_offset, cudaStream_t stream);
+// Up to 16 consecutive tokens of one sequence and stream that go to one page.
+struct __align__(16) StoreSeg {
+  int32_t seq, ord;   // sequence; first token's ordinal in its stream, the stream in the top bit
+  int32_t tok, n;     // first token in the caller's tensors, tokens
+};
+static_assert(sizeof(StoreSeg) == 16, "StoreSeg layout");
+// k, v: the caller's tensors as {d, heads, n_layers * n_tokens}, box {d, 1, 16}; segs: device
+cudaError_t launch_prefill_store(const Params& p, const CUtensorMap& k, const CUtensorMap& v, const StoreSeg* segs, int32_t n_segs,
+                                 int32_t n_tokens, int blocks, cudaStream_t stream);
 // Tensor maps of one prompt for the tcgen05 prefill kernel: q, k, v as 3-D tensors
 // {128, heads, n_layers * T} read in boxes of 64 tokens x one head x 64 elements, and the output
 // as a 4-D tensor {128, hq, T, n_layers} written in boxes of 128 tokens x one head x 64 elements

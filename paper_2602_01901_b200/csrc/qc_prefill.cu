@@ -122,6 +122,13 @@ __device__ __forceinline__ void stage_cached(uint32_t smem, const PrefillArgs& A
   }
 }
 
+// The kernels below may start while the kernel before them in the stream still stores the prompt's
+// K/V rows, of which they read nothing.  Whatever comes after them may: their last block ends after
+// that kernel.
+__device__ __forceinline__ void wait_for_stores() {
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
+}
+
 template <int D>
 __global__ void __launch_bounds__(kPrefillThreads) prefill_attend_kernel(const PrefillArgs A) {
   constexpr int KS = D / 16;   // k-steps of the score product
@@ -299,6 +306,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_attend_kernel(const P
         *reinterpret_cast<uint32_t*>(dst + 8 * i) = pack_bf16x2(o[i][2 * r] * inv, o[i][2 * r + 1] * inv);
     }
   }
+  wait_for_stores();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -435,15 +443,6 @@ __device__ __forceinline__ uint32_t mbar_test_wait(uint64_t* bar, uint32_t parit
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void tensor_g2s_3d(uint32_t dst_smem, const void* tmap, int32_t x, int32_t y, int32_t z,
-                                              uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-          "r"(dst_smem),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-      : "memory");
 }
 
 __device__ __forceinline__ void tensor_s2g_4d(const void* tmap, uint32_t src_smem, int32_t x, int32_t y, int32_t z, int32_t w) {
@@ -1033,6 +1032,7 @@ __global__ void __launch_bounds__(NV > 1 ? kTc5Threads + 32 : kTc5Threads, NV > 
   if (warp == 4) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
   }
+  wait_for_stores();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1448,6 +1448,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   if (warp == 8) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
+  wait_for_stores();
 }
 
 constexpr int kSharedPassLayers = kPrefillSharedLayers;   // 3 x 128 + 2 x 64 columns = all of tensor memory
@@ -1533,35 +1534,30 @@ cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, cons
     // prompts that start a sequence, from pair_min_tokens on: two query tiles per CTA, 128-key tiles
     const bool pair = pair_min_tokens > 0 && T >= pair_min_tokens;
     const dim3 gridp((T + 2 * kTM - 1) / (2 * kTM), p.hq, p.n_layers);
-    if (n0_text + n0_vis > 0) {
-      prefill_attend_tcgen05_kernel<true, 1><<<grid5, kTc5Threads, prefill_tcgen05_smem_bytes(), stream>>>(a, p.err);
-    } else if (passes_dev && n_shared > 0) {
+    if (n0_text + n0_vis > 0)
+      return launch_pdl(prefill_attend_tcgen05_kernel<true, 1>, grid5, dim3(kTc5Threads), prefill_tcgen05_smem_bytes(), stream, a, p.err);
+    if (passes_dev && n_shared > 0) {
       // the layers that share nothing, then the shared-score passes (passes_dev lists them in that order)
       a.passes = passes_dev;
-      if (n_single > 0 && pair) {
-        const dim3 g1(gridp.x, gridp.y, n_single);
-        prefill_attend_pair_kernel<<<g1, kPairThreads, prefill_pair_smem_bytes(), stream>>>(a, p.err);
-      } else if (n_single > 0) {
-        const dim3 g1(grid5.x, grid5.y, n_single);
-        prefill_attend_tcgen05_kernel<false, 1><<<g1, kTc5Threads, prefill_tcgen05_smem_bytes(), stream>>>(a, p.err);
-      }
+      cudaError_t e = cudaSuccess;
+      if (n_single > 0 && pair)
+        e = launch_pdl(prefill_attend_pair_kernel, dim3(gridp.x, gridp.y, n_single), dim3(kPairThreads), prefill_pair_smem_bytes(), stream, a,
+                       p.err);
+      else if (n_single > 0)
+        e = launch_pdl(prefill_attend_tcgen05_kernel<false, 1>, dim3(grid5.x, grid5.y, n_single), dim3(kTc5Threads),
+                       prefill_tcgen05_smem_bytes(), stream, a, p.err);
+      if (e != cudaSuccess) return e;
       a.passes = passes_dev + n_single;
-      const dim3 g3(grid5.x, grid5.y, n_shared);
-      prefill_attend_tcgen05_kernel<false, kSharedPassLayers>
-          <<<g3, kTc5Threads + 32, prefill_tcgen05_smem_bytes(kSharedPassLayers), stream>>>(a, p.err);
-    } else if (pair) {
-      prefill_attend_pair_kernel<<<gridp, kPairThreads, prefill_pair_smem_bytes(), stream>>>(a, p.err);
-    } else {
-      prefill_attend_tcgen05_kernel<false, 1><<<grid5, kTc5Threads, prefill_tcgen05_smem_bytes(), stream>>>(a, p.err);
+      return launch_pdl(prefill_attend_tcgen05_kernel<false, kSharedPassLayers>, dim3(grid5.x, grid5.y, n_shared), dim3(kTc5Threads + 32),
+                        prefill_tcgen05_smem_bytes(kSharedPassLayers), stream, a, p.err);
     }
-    return cudaGetLastError();
+    if (pair)
+      return launch_pdl(prefill_attend_pair_kernel, gridp, dim3(kPairThreads), prefill_pair_smem_bytes(), stream, a, p.err);
+    return launch_pdl(prefill_attend_tcgen05_kernel<false, 1>, grid5, dim3(kTc5Threads), prefill_tcgen05_smem_bytes(), stream, a, p.err);
   }
   const dim3 grid((T + kBM - 1) / kBM, p.hq, p.n_layers);
-  if (p.d == 128)
-    prefill_attend_kernel<128><<<grid, kPrefillThreads, prefill_smem_bytes<128>(), stream>>>(a);
-  else
-    prefill_attend_kernel<64><<<grid, kPrefillThreads, prefill_smem_bytes<64>(), stream>>>(a);
-  return cudaGetLastError();
+  if (p.d == 128) return launch_pdl(prefill_attend_kernel<128>, grid, dim3(kPrefillThreads), prefill_smem_bytes<128>(), stream, a);
+  return launch_pdl(prefill_attend_kernel<64>, grid, dim3(kPrefillThreads), prefill_smem_bytes<64>(), stream, a);
 }
 
 }  // namespace qc

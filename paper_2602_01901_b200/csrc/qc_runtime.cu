@@ -18,7 +18,11 @@ namespace {
 
 constexpr int kStageSlots = 8;       // pinned step-descriptor ring
 constexpr int kMaxProfileSteps = 16384;
-constexpr int kPrefillBatchTokens = 1 << 16;
+constexpr int kPinnedPromptTokens = 1 << 16;   // longer prompts' kinds are uploaded from where they are
+constexpr size_t kStoreSegs = 1 << 14;          // runs of tokens per launch of the kernel that stores prompt rows
+constexpr size_t kPromptBytes = 786432;   // a prompt's kinds, tile codes and passes
+constexpr int kStoreBlocksBeside = 1, kStoreBlocksAlone = 7;   // blocks per SM of the kernel that stores prompt rows
+constexpr int kStageTableSeqs = 4;   // sequences whose page-table rows go through pinned memory
 // Shared-score passes run one CTA per SM (three accumulators fill tensor memory); that pays once
 // a CTA has enough key tiles: measured -16 % / -10 % call time at 2048 / 3008 tokens, +4 % / +9 %
 // at 1120 / 675.
@@ -53,7 +57,7 @@ struct OpenStep {
 
 struct Layout {   // byte offsets into the workspace
   size_t table, layer_flags, layer_kind, leader, jobs, plan, qcache, part_acc, part_ml, logits, items, step, err, counters, row_slots, row_done, wdesc, cdesc, row_pieces, stage_q,
-      stage_k, stage_v, stage_out, stage_lse, tok, total;
+      stage_k, stage_v, stage_out, stage_lse, tok, prompt, total;
   size_t step_seqs, step_patches, step_bytes;   // offsets inside the step block
 };
 
@@ -131,6 +135,8 @@ struct qc_cache {
 
   // pinned staging ring for step descriptors
   uint8_t* pinned = nullptr;
+  uint8_t* prompt_stage = nullptr;    // pinned: what a prompt call uploads (made by the first one)
+  cudaEvent_t prompt_staged = nullptr;
   int32_t* err_host = nullptr;        // mapped host word the kernels mirror the device error word into
   int32_t* err_host_dev = nullptr;    // its device address
   int debug_drop_tile = 0;
@@ -460,7 +466,8 @@ int compute_sizes(const qc_config* cfg, Sizes* s) {
   L.stage_v = take(N * S * s->hkv * s->D * 2);
   L.stage_out = take(N * S * s->hq * s->D * 2);
   L.stage_lse = take(N * S * s->hq * sizeof(float));
-  L.tok = take(static_cast<size_t>(kPrefillBatchTokens) * 3 * sizeof(int32_t));
+  L.tok = take(std::max(kStoreSegs * sizeof(StoreSeg), 3 * S * sizeof(int32_t)));
+  L.prompt = take(kPromptBytes);
   L.total = off;
   return QC_OK;
 }
@@ -556,6 +563,21 @@ int make_prompt_tensor_map(CUtensorMap* out, const void* base, int n_layers, int
   const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
                          elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? QC_OK : QC_ERR_CUDA;
+}
+
+// A prompt's K or V rows [n_rows][heads][d] bf16 as a 3-D tensor {d, heads, n_rows}: a box is 16 rows
+// of one head, in row order (what a page holds of a head).
+int make_rows_tensor_map(CUtensorMap* out, const void* base, int64_t n_rows, int heads, int d) {
+  EncodeFn enc = tensor_map_encoder();
+  if (!enc) return QC_ERR_CUDA;
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(heads), static_cast<cuuint64_t>(n_rows)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * 2, static_cast<cuuint64_t>(heads) * d * 2};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(d), 1, kPage};
+  const cuuint32_t elem_strides[3] = {1, 1, 1};
+  const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem_strides,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? QC_OK : QC_ERR_CUDA;
 }
 
@@ -858,6 +880,8 @@ int32_t qc_free(qc_ctx* ctx, qc_cache* cache) {
     if (cache->copy_out) cudaStreamDestroy(cache->copy_out);
     for (cudaEvent_t e : cache->ev_prefill) cudaEventDestroy(e);
     if (cache->pinned) cudaFreeHost(cache->pinned);
+    if (cache->prompt_stage) cudaFreeHost(cache->prompt_stage);
+    if (cache->prompt_staged) cudaEventDestroy(cache->prompt_staged);
     if (cache->err_host) cudaFreeHost(cache->err_host);
     delete cache;
   }
@@ -865,8 +889,24 @@ int32_t qc_free(qc_ctx* ctx, qc_cache* cache) {
   return QC_OK;
 }
 
-int32_t qc_prefill_append(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const int32_t* n_tokens,
-                          const uint8_t* kind, const void* k_dev, const void* v_dev) {
+}  // extern "C"
+
+namespace {
+
+// What qc_prefill_attend uploads for its kernel, along with the routing of the tokens.
+struct PromptUpload {
+  const uint8_t* codes;
+  size_t n_codes;
+  const std::vector<PrefillPass>* passes;   // null: none
+};
+inline size_t codes_at(size_t n_tokens) { return align_up(n_tokens, 256); }
+inline size_t passes_at(size_t n_tokens, size_t n_codes) { return codes_at(n_tokens) + align_up(n_codes, 256); }
+
+// The body of qc_prefill_append.  Everything that is uploaded goes ahead of the kernel that stores
+// the rows, through pinned memory, so that nothing stands between that kernel and the prompt's
+// attention, which runs beside it.
+int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const int32_t* n_tokens, const uint8_t* kind,
+                     const void* k_dev, const void* v_dev, const PromptUpload* up) {
   if (!c || n_seqs < 0 || (n_seqs > 0 && (!seq_ids || !n_tokens))) return QC_ERR_INVALID_ARG;
   if (c->open.active) return QC_ERR_STATE;   // a decode step is open
   if (n_seqs == 0) return QC_OK;
@@ -909,12 +949,19 @@ int32_t qc_prefill_append(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, c
   QC_CUDA(cudaSetDevice(c->ctx->device));
   cudaStream_t stream = c->ctx->stream;
 
-  // ---- commit: pages (sequence -> layer -> stream order), token routing
-  std::vector<int32_t> tok_seq(total), tok_stream(total), tok_ord(total);
-  int64_t t0 = 0;
+  // ---- what can still fail without a change: the tensor maps of the caller's rows
+  CUtensorMap map_k, map_v;
+  if (total > 0) {
+    if (static_cast<int64_t>(N) * total > 0x7fffffffLL) return QC_ERR_INVALID_ARG;   // rows are counted in 31 bits
+    if (make_rows_tensor_map(&map_k, k_dev, N * total, c->hkv, c->D) != QC_OK || make_rows_tensor_map(&map_v, v_dev, N * total, c->hkv, c->D) != QC_OK)
+      return QC_ERR_CUDA;
+  }
+  // ---- commit: pages (sequence -> layer -> stream order)
+  std::vector<int32_t> at_t(n_seqs), at_v(n_seqs);   // where each sequence's new tokens start in its streams
   for (int i = 0; i < n_seqs; ++i) {
     const int s = seq_ids[i];
     SeqState& st = c->seqs[s];
+    at_t[i] = st.len_text, at_v[i] = st.len_vis;
     if (c->paged) {
       const int have_t = pages_for(st.len_text), have_v = pages_for(st.len_vis);
       const int dt = pages_for(st.len_text + add_t[i]) - have_t;
@@ -923,40 +970,106 @@ int32_t qc_prefill_append(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, c
         for (int sm = 0; sm < 4; ++sm)
           if (owns(c, l, sm)) grow_stream(c, l, sm, s, (sm & 1) ? have_v : have_t, (sm & 1) ? dv : dt, nullptr);
     }
-    int ot = st.len_text, ov = st.len_vis;
-    for (int t = 0; t < n_tokens[i]; ++t) {
-      const bool vis = kind[t0 + t] == QC_KIND_VISUAL;
-      tok_seq[t0 + t] = s;
-      tok_stream[t0 + t] = vis ? 1 : 0;
-      tok_ord[t0 + t] = vis ? ov++ : ot++;
-    }
-    st.len_text = ot;
-    st.len_vis = ov;
+    st.len_text += add_t[i];
+    st.len_vis += add_v[i];
     st.active = true;
-    t0 += n_tokens[i];
   }
-  // the whole host mirror goes to the device (prefill is not the hot path)
-  if (c->paged)
+  if (!c->prompt_stage) {   // runs of tokens | prompt | page-table rows
+    const size_t bytes = kStoreSegs * sizeof(StoreSeg) + 2 * static_cast<size_t>(kPinnedPromptTokens) +
+                         static_cast<size_t>(kStageTableSeqs) * N * 4 * c->max_pages * sizeof(int32_t);
+    QC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->prompt_stage), bytes, cudaHostAllocDefault));
+    QC_CUDA(cudaEventCreateWithFlags(&c->prompt_staged, cudaEventDisableTiming));
+  } else {
+    QC_CUDA(cudaEventSynchronize(c->prompt_staged));   // the last call's copies have run
+  }
+  StoreSeg* segs = reinterpret_cast<StoreSeg*>(c->prompt_stage);
+  uint8_t* prompt = c->prompt_stage + kStoreSegs * sizeof(StoreSeg);
+  int32_t* rows = reinterpret_cast<int32_t*>(prompt + 2 * static_cast<size_t>(kPinnedPromptTokens));
+  // page tables: the listed sequences' rows, or the whole host mirror
+  if (c->paged && n_seqs <= kStageTableSeqs) {
+    const size_t row = c->max_pages * sizeof(int32_t);
+    for (int i = 0; i < n_seqs; ++i, rows += static_cast<size_t>(N) * 4 * c->max_pages) {
+      for (int r = 0; r < 4 * N; ++r)
+        std::memcpy(rows + static_cast<size_t>(r) * c->max_pages, c->table.data() + trow(c, 0, r, seq_ids[i]), row);
+      QC_CUDA(cudaMemcpy2DAsync(c->ws + c->lay.table + static_cast<size_t>(seq_ids[i]) * row, c->cfg.max_seqs * row, rows, row, row,
+                                static_cast<size_t>(N) * 4, cudaMemcpyHostToDevice, stream));
+    }
+  } else if (c->paged) {
     QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.table, c->table.data(), c->table.size() * sizeof(int32_t),
                             cudaMemcpyHostToDevice, stream));
+  }
+  if (up) {   // (one sequence)
+    uint8_t* dev = c->ws + c->lay.prompt;
+    const size_t n_kinds = static_cast<size_t>(total);
+    if (total <= kPinnedPromptTokens) {
+      std::memcpy(prompt, kind, n_kinds);
+      std::memcpy(prompt + codes_at(n_kinds), up->codes, up->n_codes);
+      size_t bytes = passes_at(n_kinds, up->n_codes);
+      if (up->passes) {
+        std::memcpy(prompt + bytes, up->passes->data(), up->passes->size() * sizeof(PrefillPass));
+        bytes += up->passes->size() * sizeof(PrefillPass);
+      }
+      QC_CUDA(cudaMemcpyAsync(dev, prompt, bytes, cudaMemcpyHostToDevice, stream));
+    } else {   // (pageable memory: the copies return when it has been read)
+      QC_CUDA(cudaMemcpyAsync(dev, kind, n_kinds, cudaMemcpyHostToDevice, stream));
+      QC_CUDA(cudaMemcpyAsync(dev + codes_at(n_kinds), up->codes, up->n_codes, cudaMemcpyHostToDevice, stream));
+      if (up->passes)
+        QC_CUDA(cudaMemcpyAsync(dev + passes_at(n_kinds, up->n_codes), up->passes->data(), up->passes->size() * sizeof(PrefillPass),
+                                cudaMemcpyHostToDevice, stream));
+    }
+  }
+  QC_CUDA(cudaEventRecord(c->prompt_staged, stream));
   Params p = base_params(c);
   p.k = static_cast<const uint16_t*>(k_dev);
   p.v = static_cast<const uint16_t*>(v_dev);
-  int32_t* tok_dev = reinterpret_cast<int32_t*>(c->ws + c->lay.tok);
-  for (int64_t off = 0; off < total; off += kPrefillBatchTokens) {
-    const int n = static_cast<int>(std::min<int64_t>(kPrefillBatchTokens, total - off));
-    QC_CUDA(cudaMemcpyAsync(tok_dev, tok_seq.data() + off, n * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
-    QC_CUDA(cudaMemcpyAsync(tok_dev + kPrefillBatchTokens, tok_stream.data() + off, n * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, stream));
-    QC_CUDA(cudaMemcpyAsync(tok_dev + 2 * kPrefillBatchTokens, tok_ord.data() + off, n * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, stream));
+  StoreSeg* segs_dev = reinterpret_cast<StoreSeg*>(c->ws + c->lay.tok);
+  // runs of tokens, a batch at a time; beside the attention of the prompt the stores get one block per
+  // SM, alone as many as fit
+  size_t n = 0;
+  int64_t tok = 0;
+  bool used = false;   // the staging area holds runs that are being copied
+  auto flush = [&]() -> int32_t {
+    QC_CUDA(cudaMemcpyAsync(segs_dev, segs, n * sizeof(StoreSeg), cudaMemcpyHostToDevice, stream));
+    QC_CUDA(cudaEventRecord(c->prompt_staged, stream));
     c->kernel_launches++;
-    QC_CUDA(launch_prefill_scatter(p, tok_dev, tok_dev + kPrefillBatchTokens, tok_dev + 2 * kPrefillBatchTokens, n,
-                                   static_cast<int32_t>(total), static_cast<int32_t>(off), stream));
-    // the host vectors and the device token arrays are reused by the next batch
-    QC_CUDA(cudaStreamSynchronize(stream));
+    QC_CUDA(launch_prefill_store(p, map_k, map_v, segs_dev, static_cast<int32_t>(n), static_cast<int32_t>(total),
+                                 c->ctx->n_sms * (up ? kStoreBlocksBeside : kStoreBlocksAlone), stream));
+    n = 0;
+    used = true;
+    return QC_OK;
+  };
+  for (int i = 0; i < n_seqs; ++i) {
+    for (int t = 0; t < n_tokens[i];) {
+      const uint8_t kd = kind[tok + t];
+      int& at = kd == QC_KIND_VISUAL ? at_v[i] : at_t[i];
+      int len = 1;
+      while (t + len < n_tokens[i] && kind[tok + t + len] == kd && (at + len) % kPage != 0) ++len;
+      if (used && n == 0) QC_CUDA(cudaEventSynchronize(c->prompt_staged));
+      segs[n++] = StoreSeg{seq_ids[i], static_cast<int32_t>(static_cast<uint32_t>(at) | (kd == QC_KIND_VISUAL ? 0x80000000u : 0u)),
+                           static_cast<int32_t>(tok + t), len};
+      at += len;
+      t += len;
+      if (n == kStoreSegs) {
+        const int32_t st = flush();
+        if (st != QC_OK) return st;
+      }
+    }
+    tok += n_tokens[i];
+  }
+  if (n > 0) {
+    const int32_t st = flush();
+    if (st != QC_OK) return st;
   }
   return QC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int32_t qc_prefill_append(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const int32_t* n_tokens,
+                          const uint8_t* kind, const void* k_dev, const void* v_dev) {
+  return store_prompt(c, n_seqs, seq_ids, n_tokens, kind, k_dev, v_dev, nullptr);
 }
 
 int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const uint8_t* kind, const void* q_dev,
@@ -970,10 +1083,8 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
   // tokens the sequence holds already (an earlier prompt chunk, generated tokens) precede the new ones
   const int n0_text = c->seqs[seq_id].active ? c->seqs[seq_id].len_text : 0;
   const int n0_vis = c->seqs[seq_id].active ? c->seqs[seq_id].len_vis : 0;
-  const size_t tok_bytes = static_cast<size_t>(kPrefillBatchTokens) * 3 * sizeof(int32_t);   // kinds, tile codes, passes
-  if (align_up(n_tokens, 256) + align_up((n_tokens + 63) / 64, 256) + c->prefill_passes.size() * sizeof(PrefillPass) >
-      tok_bytes)
-    return QC_ERR_INVALID_ARG;
+  const int n_tiles = (n_tokens + 63) / 64;
+  if (passes_at(n_tokens, n_tiles) + c->prefill_passes.size() * sizeof(PrefillPass) > kPromptBytes) return QC_ERR_INVALID_ARG;
   // what can fail without touching the cache comes first: the tensor maps over the caller's tensors
   PrefillMaps maps;
   const bool tc5 = c->prefill_tcgen05 && c->D == 128 && (c->pool_map_ok || n0_text + n0_vis == 0);
@@ -984,29 +1095,23 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
         make_output_tensor_map(&maps.out, out_dev, c->cfg.n_layers, n_tokens, c->hq) != QC_OK)
       return QC_ERR_CUDA;
   }
-  // store K/V: this validates the rest and leaves the cache unchanged on an error
-  int st = qc_prefill_append(c, 1, &seq_id, &n_tokens, kind, k_dev, v_dev);
-  if (st != QC_OK) return st;
-  cudaStream_t stream = c->ctx->stream;
-  uint8_t* kind_dev = c->ws + c->lay.tok;   // free again: qc_prefill_append has waited for its copies
   // per 64-token tile: all text, all visual or mixed (the tcgen05 kernel fetches unmixed tiles whole)
-  const int n_tiles = (n_tokens + 63) / 64;
   std::vector<uint8_t> codes(n_tiles);
   for (int i = 0; i < n_tiles; ++i) {
     int nv = 0, n = std::min(64, n_tokens - 64 * i);
     for (int t = 0; t < n; ++t) nv += kind[64 * i + t] == QC_KIND_VISUAL;
     codes[i] = nv == 0 ? 0 : (nv == n ? 1 : 2);
   }
-  uint8_t* codes_dev = kind_dev + align_up(n_tokens, 256);
-  QC_CUDA(cudaMemcpyAsync(kind_dev, kind, n_tokens, cudaMemcpyHostToDevice, stream));
-  QC_CUDA(cudaMemcpyAsync(codes_dev, codes.data(), n_tiles, cudaMemcpyHostToDevice, stream));
-  PrefillPass* passes_dev = reinterpret_cast<PrefillPass*>(codes_dev + align_up(n_tiles, 256));
   const bool share = c->prefill_n_shared > 0 && n0_text + n0_vis == 0 &&
                      (c->prefill_shared == 2 || (c->prefill_shared == 1 && n_tokens >= kPrefillShareMinTokens));
-  if (share)
-    QC_CUDA(cudaMemcpyAsync(passes_dev, c->prefill_passes.data(), c->prefill_passes.size() * sizeof(PrefillPass),
-                            cudaMemcpyHostToDevice, stream));
-  QC_CUDA(cudaStreamSynchronize(stream));   // `kind` is the caller's host memory
+  // store K/V: this validates the rest and leaves the cache unchanged on an error
+  const PromptUpload up{codes.data(), codes.size(), share ? &c->prefill_passes : nullptr};
+  const int st = store_prompt(c, 1, &seq_id, &n_tokens, kind, k_dev, v_dev, &up);
+  if (st != QC_OK) return st;
+  cudaStream_t stream = c->ctx->stream;
+  const uint8_t* kind_dev = c->ws + c->lay.prompt;
+  const uint8_t* codes_dev = kind_dev + codes_at(n_tokens);
+  const PrefillPass* passes_dev = reinterpret_cast<const PrefillPass*>(kind_dev + passes_at(n_tokens, n_tiles));
   const Params p = base_params(c);
   cudaEvent_t* ev = nullptr;
   if (c->profile && c->ev_prefill_calls < kMaxProfileSteps) {

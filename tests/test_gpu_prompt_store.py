@@ -1,0 +1,69 @@
+"""Prompt rows in their pages: runs of tokens that start and end anywhere in a page, several sequences in
+one call, more runs than one launch takes."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2602_01901_b200 import binding as qc
+from paper_2602_01901_b200.session import Session, bits_of
+
+pytestmark = pytest.mark.gpu
+
+
+def _rows(s, n, lens, heads, kinds, k, v, layers):
+    """Every stored row of the named layers against the tensors that were handed over."""
+    at, kb, vb = 0, bits_of(k), bits_of(v)
+    for seq, kind in enumerate(kinds):
+        for stream, name in ((0, 0), (1, 1)):
+            tokens = [at + t for t in range(len(kind)) if kind[t] == name]
+            for layer in layers:
+                for h in range(heads):
+                    for i in {0, 1, 15, 16, 17, len(tokens) // 2, len(tokens) - 1} & set(range(len(tokens))):
+                        what = (seq, stream, layer, h, i)
+                        assert np.array_equal(s.read_row(layer, 2 + stream, seq, lens[seq][stream] + i, h), vb[layer, tokens[i], h]), what
+                        if layer == 0:   # (a lazy layer keeps no visual K)
+                            assert np.array_equal(s.read_row(layer, stream, seq, lens[seq][stream] + i, h), kb[layer, tokens[i], h]), what
+        at += len(kind)
+
+
+@pytest.mark.parametrize("head_dim,q_heads,kv_heads", [(128, 2, 2), (64, 4, 1), (128, 7, 1)])
+def test_runs_of_any_alignment(head_dim, q_heads, kv_heads):
+    rng = np.random.default_rng(7)
+    n = 2
+    s = Session(n, q_heads, kv_heads, head_dim, [0, 1], max_seqs=3, max_tokens_per_seq=256, n_pages=2 * n * 3 * 32,
+                lazy_mode=qc.QC_MODE_VLA_QC, poison_pool=True)
+    lens = [[0, 0] for _ in range(3)]
+    patterns = [
+        [[0] * 5, [1] * 16, [0, 1] * 20],                                  # one run, one page, a run per token
+        [[1] * 33 + [0] * 15, [0] * 16 + [1] * 1, [0, 0, 1] * 11],
+        [rng.integers(0, 2, 61).tolist(), [0], rng.integers(0, 2, 40).tolist()],
+    ]
+    for call in patterns:   # each call continues the sequences of the one before
+        kinds = [np.array(x, np.uint8) for x in call]
+        total = sum(len(x) for x in kinds)
+        k, v = (torch.randn(n, total, kv_heads, head_dim, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+        s.prefill_append([0, 1, 2], [len(x) for x in kinds], np.concatenate(kinds), k, v)
+        _rows(s, n, lens, kv_heads, kinds, k, v, range(n))
+        for i, x in enumerate(kinds):
+            lens[i][0] += int((x == 0).sum())
+            lens[i][1] += int((x == 1).sum())
+    assert s.stats().device_error == 0
+    s.close()
+
+
+def test_more_runs_than_one_launch_takes():
+    t = 33000   # one token per run: the runs of three launches
+    s = Session(1, 1, 1, 64, [0], max_seqs=1, max_tokens_per_seq=t, n_pages=2 * (t // 16 + 8), poison_pool=True)
+    kind = np.arange(t, dtype=np.int64) % 2
+    k, v = (torch.randn(1, t, 1, 64, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+    s.prefill_append([0], [t], kind.astype(np.uint8), k, v)
+    kb, vb = bits_of(k), bits_of(v)
+    for i in list(range(0, t // 2, 997)) + [8190, 8191, 8192, 8193, t // 2 - 1]:
+        for stream in (0, 1):
+            assert np.array_equal(s.read_row(0, stream, 0, i, 0), kb[0, 2 * i + stream, 0])
+            assert np.array_equal(s.read_row(0, 2 + stream, 0, i, 0), vb[0, 2 * i + stream, 0])
+    assert s.stats().device_error == 0
+    s.close()
