@@ -342,11 +342,13 @@ __global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant
     any = find(u, x);   // (its reads overlap the copy)
     uint32_t done = 0;
     for (uint32_t spin = 0; !done && spin < kSpinLimit; ++spin) done = mbar_try_wait(&full[lane], phase);
-    phase ^= 1u;
     if (!done) {
       report_error(P.err, P.err_host, kErrTimeout);
+      // the copy still writes into this block's shared memory: a bounded chance to land
+      for (uint32_t spin = 0; !done && spin < kSpinLimit; ++spin) done = mbar_try_wait(&full[lane], phase);
       break;
     }
+    phase ^= 1u;
     uint16_t* dst = P.pool + ((static_cast<size_t>(now.pid) * P.hkv + now.head) * kPage + now.slot) * D;
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(buf), "r"(now.bytes) : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
