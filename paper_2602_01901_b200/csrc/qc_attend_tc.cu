@@ -325,10 +325,9 @@ __device__ __forceinline__ void process_item_tc(WorkerState& st, const TcCtx* ct
 // the tile ring full across item boundaries, process each item.  While item k is processed the
 // ring already fetches tiles of item k + 1 and the context of item k + 2 (descriptor, page ids)
 // arrives by asynchronous copies.
-// False if a wait ran out.
 template <int D, bool STATIC>
-__device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, uint32_t ring, uint64_t* full,
-                                                 RangeCursor* cursor, int32_t* stage, CtaDesc* cta, int wid, int lane) {
+__device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, uint32_t ring, uint64_t* full,
+                                                 RangeCursor* cursor, int32_t* stage, int wid, int lane) {
   auto ctx_of = [ctx](int k) -> const ItemPages& { return ctx[k % kCtxSlots].ip; };
   WorkerState st;
   worker_init(st, 0);
@@ -353,7 +352,7 @@ __device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, ui
     bool any = wid >= 0 && wid < P.part_workers;
     if (P.wdesc != nullptr) {
       // planned ahead: one read gives the first two items, the first page ids and the cursor
-      any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, cta, lane);
+      any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, nullptr, lane);
       if (any) first = ctx[0].ip.item;
     } else {
       RangeCursor c;
@@ -369,8 +368,8 @@ __device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, ui
       }
     }
     if (!any) {
-      pdl_wait();   // (a warp without work may still merge)
-      return true;
+      pdl_wait();
+      return;
     }
     st.n_my = 1;
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRingTc);
@@ -389,7 +388,7 @@ __device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, ui
     pdl_wait();   // the item list and the work counter are the previous kernel's
     pdl_launch_dependents();
     issued = claim_issue(P, lane);
-    if (!take()) return true;
+    if (!take()) return;
     first = it;
     begin_item_pages(ctx[0].ip, P, first, lane);
     cp_async_wait_all();
@@ -459,7 +458,6 @@ __device__ __forceinline__ bool attend_tc_worker(const Params& P, TcCtx* ctx, ui
     cp_async_wait_all();
     drain_ring<kRingTc>(st, full, P.debug_drop_tile ? kDebugSpinLimit : kSpinLimit);
   }
-  return !st.dead;
 }
 
 template <int D, bool STATIC>
@@ -469,8 +467,6 @@ __global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_tc_kernel(c
   __shared__ __align__(8) uint64_t full_all[kWarps][kRingTc];
   __shared__ __align__(16) RangeCursor cursors[kWarps];
   __shared__ __align__(16) int32_t stages[kWarps][12];
-  __shared__ __align__(16) FinishSmem<D> finish;
-  __shared__ CtaDesc cta;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // swizzled tiles must sit on 1024-byte boundaries
@@ -484,11 +480,9 @@ __global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_tc_kernel(c
     for (int s = 0; s < kRingTc; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
   }
-  if (threadIdx.x == 0) finish.dead = 0;
   __syncthreads();
 
-  const bool ok = attend_tc_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], &cta, worker_index(P, warp), lane);
-  if (STATIC) finish_cta<D>(P, finish, cta, !ok, warp, lane);
+  attend_tc_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], worker_index(P, warp), lane);
 }
 
 template <int D>

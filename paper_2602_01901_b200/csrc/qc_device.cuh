@@ -923,7 +923,7 @@ __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, in
 }
 
 // ------------------------------------------------------------------------------------------
-// merge by the attention launch itself (static partition, launches of one layer)
+// merge by the attention launch itself (static partition, launches of one layer, no query groups)
 // ------------------------------------------------------------------------------------------
 //
 // A CTA's workers own one stretch of the launch's tiles, ordered by output row.  When they are done,
@@ -957,7 +957,7 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
   if (dead && lane == 0) F.dead = 1;
   __syncthreads();   // every worker's partial rows are stored
   if (F.dead) return;
-  const int layer = P.layer_begin, rows = P.heads_per_item_dim, hpi = P.heads_per_item;
+  const int layer = P.layer_begin, rows = P.heads_per_item_dim;   // (one row per query head)
   if (warp < 2) {   // the rows at the ends: are they complete?
     const EndRow& e = cta.end[warp];
     int ready = e.here == e.total;
@@ -971,9 +971,9 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
     }
     if (lane == 0) F.ready[warp] = ready;
   }
-  const int n_inner = max(0, cta.row_last - cta.row_first - 1) * hpi;
+  const int n_inner = max(0, cta.row_last - cta.row_first - 1);
   // first the rows between the ends, one warp per output row; then the ends that this CTA completed,
-  // where several warps share an output row if there are fewer rows than warps
+  // where several warps share an output row
   RowSum<D> r;
   int share = 1, o = kWarps - 1 - warp, n_out = n_inner, si = 0, head = 0, first_ready = 1;
 #pragma unroll 1
@@ -982,18 +982,13 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
     for (; o < n_out; o += kWarps) {
       int nv, nt;
       if (phase == 0) {
-        const int row = cta.row_first + 1 + o / hpi, h = o % hpi;
-        si = row / rows;
-        const int u = row - si * rows, n_sub = (P.group + hpi - 1) / hpi, kv_head = u / n_sub, sub = u - kv_head * n_sub;
-        if (sub * hpi + h >= P.group) continue;   // (a slice of the group with fewer heads)
-        head = kv_head * P.group + sub * hpi + h;
+        const int row = cta.row_first + 1 + o;
+        si = row / rows, head = row - si * rows;
         const uint32_t both = __ldcg(P.row_pieces + static_cast<size_t>(P.launch_index) * P.max_seqs * rows + row);
         nv = both & 0xffffu, nt = both >> 16;
       } else {
-        const int out = share > 1 ? warp / share : o, h = out % hpi;
-        const EndRow& e = cta.end[out >= first_ready * hpi];
-        if (h >= e.n_heads) continue;
-        si = e.si, head = e.head + h, nv = e.nv, nt = e.nt;
+        const EndRow& e = cta.end[(share > 1 ? warp / share : o) >= first_ready];
+        si = e.si, head = e.head, nv = e.nv, nt = e.nt;
       }
       sum_partials<D>(P, (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots, head, nv, nt, P.slots_per_stream,
                       share > 1 ? warp % share : 0, share, lane, r);
@@ -1003,13 +998,11 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
     if (phase == 1) break;
     __syncthreads();
     first_ready = F.ready[0];
-    n_out = (first_ready + F.ready[1]) * hpi;
+    n_out = first_ready + F.ready[1];
     if (n_out == 0) return;
-    share = max(1, kWarps / n_out);
-    o = share == 1 ? warp : (warp / share < n_out ? n_out - 1 : n_out);   // (sharing: one round, output row warp / share)
+    share = kWarps / n_out;
+    o = warp / share < n_out ? n_out - 1 : n_out;   // (one round, output row warp / share)
   }
-  if (share == 1) return;
-  // (only rows of one query head come here: with a query group there are more output rows than warps)
   const int row = warp / share;
   if (row < n_out) {
 #pragma unroll

@@ -121,7 +121,7 @@ static_assert(sizeof(WorkerDesc) == 192, "WorkerDesc layout");
 struct EndRow {                     // the first or the last row that the CTA's tiles fall into
   int32_t here, total;              // pages of the row in this CTA / in the launch
   int32_t counter;                  // its page counter in row_done
-  int32_t si, head, n_heads;        // listed sequence, query heads
+  int32_t si, head, pad;            // listed sequence, query head
   int32_t nv, nt;                   // partial rows of the visual / the text stream
 };
 struct __align__(16) CtaDesc {

@@ -229,12 +229,10 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(const __grid_constant_
         r.total += pages;
         r0 += w * pages;
       }
-      const int hpi = V.heads_per_item, n_sub = (V.group + hpi - 1) / hpi;
-      const int kv_head = u / n_sub, sub = u - kv_head * n_sub;
       r.si = si;
-      r.head = kv_head * V.group + sub * hpi;
-      r.n_heads = min(hpi, V.group - sub * hpi);
-      r.counter = (L.layer * P.max_seqs + si) * P.hq + r.head;
+      r.head = u;   // (no query groups: a row per query head)
+      r.pad = 0;
+      r.counter = (L.layer * P.max_seqs + si) * P.hq + u;
       row_counts(sq, si, u, r.nv, r.nt);
     }
     if (d.row_last == d.row_first) d.end[1].here = 0;
