@@ -973,9 +973,13 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
   }
   const int n_inner = max(0, cta.row_last - cta.row_first - 1);
   // first the rows between the ends, one warp per output row; then the ends that this CTA completed,
-  // where several warps share an output row
+  // half of the warps each: which CTA completes a row, and whether it completes one or two, depends
+  // on the run, so neither may decide the order in which the row's partials are added
+  constexpr int kShare = kWarps / 2;
+  static_assert(2 * kShare == kWarps, "two end rows share the warps");
+  const int end = warp / kShare;
   RowSum<D> r;
-  int share = 1, o = kWarps - 1 - warp, n_out = n_inner, si = 0, head = 0, first_ready = 1;
+  int o = kWarps - 1 - warp, n_out = n_inner, si = 0, head = 0;
 #pragma unroll 1
   for (int phase = 0;; ++phase) {
 #pragma unroll 1
@@ -987,56 +991,54 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
         const uint32_t both = __ldcg(P.row_pieces + static_cast<size_t>(P.launch_index) * P.max_seqs * rows + row);
         nv = both & 0xffffu, nt = both >> 16;
       } else {
-        const EndRow& e = cta.end[(share > 1 ? warp / share : o) >= first_ready];
+        const EndRow& e = cta.end[o];
         si = e.si, head = e.head, nv = e.nv, nt = e.nt;
       }
       sum_partials<D>(P, (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots, head, nv, nt, P.slots_per_stream,
-                      share > 1 ? warp % share : 0, share, lane, r);
-      if (share > 1) break;
+                      phase ? warp % kShare : 0, phase ? kShare : 1, lane, r);
+      if (phase == 1) break;
       store_row<D>(P, layer, si, head, r, lane);
     }
     if (phase == 1) break;
     __syncthreads();
-    first_ready = F.ready[0];
-    n_out = first_ready + F.ready[1];
-    if (n_out == 0) return;
-    share = kWarps / n_out;
-    o = warp / share < n_out ? n_out - 1 : n_out;   // (one round, output row warp / share)
+    if (!F.ready[0] && !F.ready[1]) return;
+    o = end;
+    n_out = F.ready[end] ? end + 1 : 0;   // (at most one round)
   }
-  const int row = warp / share;
-  if (row < n_out) {
+  if (n_out > 0) {
 #pragma unroll
     for (int e = 0; e < VPL; ++e) F.acc[warp][lane * VPL + e] = r.acc[e];
     if (lane == 0) F.ml[warp] = make_float2(r.m, r.l);
   }
   __syncthreads();
-  if (row >= n_out) return;
+  if (n_out == 0) return;
   // every thread of the row's warps weighs their sums for some of the elements
-  float w[kWarps], m = -INFINITY, l = 0.f;
+  const int w0 = end * kShare;
+  float w[kShare], m = -INFINITY, l = 0.f;
 #pragma unroll
-  for (int x = 0; x < kWarps; ++x)
-    if (x < share && F.ml[row * share + x].y > 0.f) m = fmaxf(m, F.ml[row * share + x].x);
+  for (int x = 0; x < kShare; ++x)
+    if (F.ml[w0 + x].y > 0.f) m = fmaxf(m, F.ml[w0 + x].x);
 #pragma unroll
-  for (int x = 0; x < kWarps; ++x) {
-    const float2 ml = x < share ? F.ml[row * share + x] : make_float2(0.f, 0.f);
+  for (int x = 0; x < kShare; ++x) {
+    const float2 ml = F.ml[w0 + x];
     w[x] = ml.y > 0.f ? exp2f(ml.x - m) : 0.f;   // (no partial, or empty ones: nothing)
     if (w[x] > 0.f) l = fmaf(ml.y, w[x], l);
   }
   const float inv = 1.f / l;
   const size_t orow = (static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head;
-  for (int d = 2 * ((warp - row * share) * 32 + lane); d < D; d += 64 * share) {
+  for (int d = 2 * ((warp - w0) * 32 + lane); d < D; d += 64 * kShare) {
     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
-    for (int x = 0; x < kWarps; ++x) {
-      if (x < share && w[x] > 0.f) {
-        a0 = fmaf(F.acc[row * share + x][d], w[x], a0);
-        a1 = fmaf(F.acc[row * share + x][d + 1], w[x], a1);
+    for (int x = 0; x < kShare; ++x) {
+      if (w[x] > 0.f) {
+        a0 = fmaf(F.acc[w0 + x][d], w[x], a0);
+        a1 = fmaf(F.acc[w0 + x][d + 1], w[x], a1);
       }
     }
     *reinterpret_cast<uint32_t*>(P.out + orow * D + d) =
         f32_to_bf16_rne(a0 * inv) | (static_cast<uint32_t>(f32_to_bf16_rne(a1 * inv)) << 16);
   }
-  if (P.lse != nullptr && lane == 0 && warp == row * share) P.lse[orow] = (m + log2f(l)) * 0.6931471805599453f;
+  if (P.lse != nullptr && lane == 0 && warp == w0) P.lse[orow] = (m + log2f(l)) * 0.6931471805599453f;
 }
 
 }  // namespace

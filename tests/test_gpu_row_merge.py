@@ -69,3 +69,38 @@ def test_rows_merged_by_the_attention_launch(shape, mode):
     for s in sessions:
         assert s.stats().device_error == 0
         s.close()
+
+
+@pytest.mark.parametrize("shape", ["one_long_row_per_head", "rows_over_several_blocks"])
+def test_the_same_step_gives_the_same_bits(shape):
+    """Which block completes a row that several blocks share, and how many rows it completes, differs
+    from run to run; the bits of the output may not."""
+    head_dim, _, lens = SHAPES[shape]
+    heads, b = 16, len(lens)
+    layer_kind = [0, 1, 0, 1]
+    n, longest = len(layer_kind), max(t + v for t, v in lens)
+    s = Session(n, heads, heads, head_dim, layer_kind, max_seqs=b, max_tokens_per_seq=longest + 1,
+                n_pages=2 * n * sum((t + 32) // 16 + (v + 15) // 16 for t, v in lens))
+    s.set_option("in_order_launches", 1)
+    gen = torch.Generator(device=s.device).manual_seed(3)
+
+    def normal(*size):
+        return torch.randn(size, generator=gen, device=s.device, dtype=torch.bfloat16)
+
+    total = sum(t + v for t, v in lens)
+    kind = np.concatenate([np.repeat(np.array([0, 1], np.uint8), (t, v)) for t, v in lens])
+    k, v = normal(n, total, heads, head_dim), normal(n, total, heads, head_dim)
+    qkv = [normal(n, b, heads, head_dim) for _ in range(3)]
+    out, lse = torch.empty_like(qkv[0]), torch.empty((n, b, heads), dtype=torch.float32, device=s.device)
+    first = None
+    for run in range(60):
+        s.prefill_append(list(range(b)), [t + v_ for t, v_ in lens], kind, k, v)
+        s.decode_step(list(range(b)), *qkv, out, lse)
+        got = (out.view(torch.int16).clone(), lse.view(torch.int32).clone())
+        if first is None:
+            first = got
+        assert torch.equal(got[0], first[0]) and torch.equal(got[1], first[1]), f"run {run} differs from the first"
+        for i in range(b):
+            qc.qc_free_seq(s.cache, i)
+    assert s.stats().device_error == 0
+    s.close()
