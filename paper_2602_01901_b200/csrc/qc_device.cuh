@@ -792,14 +792,16 @@ __device__ __forceinline__ void sum_partials(const Params& P, size_t base, int h
         if (s0 + u < cnt) load_elems<VPL>(v[u], acc0 + static_cast<size_t>(slot_of(c0 + (s0 + u) * step)) * acc_stride);
     };
     request(0);
-    float m_new = ml.y > 0.f ? ml.x : -INFINITY;   // (a sweep that left out its only key has an empty partial)
+    // A sweep that left out its only key has an empty partial (sum 0, weight 0).  A sum that is not a number
+    // has weight 0 too, but makes the row's sum, and with it the row, not a number.
+    float m_new = ml.y > 0.f ? ml.x : -INFINITY;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
     m_new = fmaxf(m_new, r.m);
-    if (m_new == -INFINITY) continue;
-    const float corr = exp2f(r.m - m_new);
-    const float w = ml.y > 0.f ? exp2f(ml.x - m_new) : 0.f;
-    float ls = ml.y > 0.f ? ml.y * w : 0.f;
+    const float ref = m_new == -INFINITY ? 0.f : m_new;   // (nothing that counts so far)
+    const float corr = exp2f(r.m - ref);
+    const float w = ml.y > 0.f ? exp2f(ml.x - ref) : 0.f;
+    float ls = ml.y * w;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
     r.m = m_new;
@@ -1022,7 +1024,7 @@ __device__ __forceinline__ void finish_cta(const Params& P, FinishSmem<D>& F, co
   for (int x = 0; x < kShare; ++x) {
     const float2 ml = F.ml[w0 + x];
     w[x] = ml.y > 0.f ? exp2f(ml.x - m) : 0.f;   // (no partial, or empty ones: nothing)
-    if (w[x] > 0.f) l = fmaf(ml.y, w[x], l);
+    l = fmaf(ml.y, w[x], l);                     // (a sum that is not a number stays one)
   }
   const float inv = 1.f / l;
   const size_t orow = (static_cast<size_t>(layer) * P.n_seqs + si) * P.hq + head;

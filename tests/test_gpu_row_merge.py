@@ -104,3 +104,33 @@ def test_the_same_step_gives_the_same_bits(shape):
             qc.qc_free_seq(s.cache, i)
     assert s.stats().device_error == 0
     s.close()
+
+
+@pytest.mark.parametrize("options", [{}, {"in_order_launches": 1}, {"in_order_launches": 1, "fused_merge": 0}],
+                         ids=["one_launch", "own_merge", "merge_launch"])
+@pytest.mark.parametrize("q_heads,kv_heads", [(4, 4), (8, 2)])
+def test_a_key_that_is_not_a_number_reaches_every_row_it_belongs_to(q_heads, kv_heads, options):
+    """Softmax over a score that is not a number is not a number: a partial result that holds one may not be
+    left out of the row, however many finite ones there are beside it."""
+    n, b, text, vis, d, at, kv = 2, 2, 20, 700, 128, 333, 1
+    s = Session(n, q_heads, kv_heads, d, [0, 1], max_seqs=b, max_tokens_per_seq=vis, n_pages=2 * n * b * 50)
+    for key, value in options.items():
+        s.set_option(key, value)
+    gen = torch.Generator(device=s.device).manual_seed(5)
+
+    def normal(*size):
+        return torch.randn(size, generator=gen, device=s.device, dtype=torch.bfloat16)
+
+    kind = np.array([0] * text + [1] * vis, np.uint8)
+    k, v = normal(n, b * (text + vis), kv_heads, d), normal(n, b * (text + vis), kv_heads, d)
+    k[0, text + at, kv, 7] = float("nan")   # the leader's, sequence 0, a visual token: its follower scores it too
+    s.prefill_append([0, 1], [text + vis] * b, np.concatenate([kind] * b), k, v)
+    q, kn, vn = normal(n, b, q_heads, d), normal(n, b, kv_heads, d), normal(n, b, kv_heads, d)
+    out = torch.empty_like(q)
+    s.decode_step([0, 1], q, kn, vn, out)
+    group = q_heads // kv_heads
+    hit = torch.zeros(n, b, q_heads, dtype=torch.bool, device=s.device)
+    hit[:, 0, kv * group:(kv + 1) * group] = True
+    assert torch.equal(torch.isnan(out).all(-1), hit) and torch.equal(torch.isnan(out).any(-1), hit)
+    assert s.stats().device_error == 0
+    s.close()
