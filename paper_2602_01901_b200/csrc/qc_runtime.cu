@@ -18,9 +18,8 @@ namespace {
 
 constexpr int kStageSlots = 8;       // pinned step-descriptor ring
 constexpr int kMaxProfileSteps = 16384;
-constexpr int kPinnedPromptTokens = 1 << 16;   // longer prompts' kinds are uploaded from where they are
 constexpr size_t kStoreSegs = 1 << 14;          // runs of tokens per launch of the kernel that stores prompt rows
-constexpr size_t kPromptBytes = 786432;   // a prompt's kinds, tile codes and passes
+constexpr size_t kPromptBytes = 786432;   // a prompt's kinds, tile codes and passes, on the device and in pinned memory
 constexpr int kStoreBlocksBeside = 1, kStoreBlocksAlone = 7;   // blocks per SM of the kernel that stores prompt rows
 constexpr int kStageTableSeqs = 4;   // sequences whose page-table rows go through pinned memory
 // Shared-score passes run one CTA per SM (three accumulators fill tensor memory); that pays once
@@ -975,7 +974,7 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     st.active = true;
   }
   if (!c->prompt_stage) {   // runs of tokens | prompt | page-table rows
-    const size_t bytes = kStoreSegs * sizeof(StoreSeg) + 2 * static_cast<size_t>(kPinnedPromptTokens) +
+    const size_t bytes = kStoreSegs * sizeof(StoreSeg) + kPromptBytes +
                          static_cast<size_t>(kStageTableSeqs) * N * 4 * c->max_pages * sizeof(int32_t);
     QC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->prompt_stage), bytes, cudaHostAllocDefault));
     QC_CUDA(cudaEventCreateWithFlags(&c->prompt_staged, cudaEventDisableTiming));
@@ -984,7 +983,7 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   }
   StoreSeg* segs = reinterpret_cast<StoreSeg*>(c->prompt_stage);
   uint8_t* prompt = c->prompt_stage + kStoreSegs * sizeof(StoreSeg);
-  int32_t* rows = reinterpret_cast<int32_t*>(prompt + 2 * static_cast<size_t>(kPinnedPromptTokens));
+  int32_t* rows = reinterpret_cast<int32_t*>(prompt + kPromptBytes);
   // page tables: the listed sequences' rows, or the whole host mirror
   if (c->paged && n_seqs <= kStageTableSeqs) {
     const size_t row = c->max_pages * sizeof(int32_t);
@@ -998,25 +997,16 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.table, c->table.data(), c->table.size() * sizeof(int32_t),
                             cudaMemcpyHostToDevice, stream));
   }
-  if (up) {   // (one sequence)
-    uint8_t* dev = c->ws + c->lay.prompt;
+  if (up) {   // (one sequence; qc_prefill_attend has checked that it fits)
     const size_t n_kinds = static_cast<size_t>(total);
-    if (total <= kPinnedPromptTokens) {
-      std::memcpy(prompt, kind, n_kinds);
-      std::memcpy(prompt + codes_at(n_kinds), up->codes, up->n_codes);
-      size_t bytes = passes_at(n_kinds, up->n_codes);
-      if (up->passes) {
-        std::memcpy(prompt + bytes, up->passes->data(), up->passes->size() * sizeof(PrefillPass));
-        bytes += up->passes->size() * sizeof(PrefillPass);
-      }
-      QC_CUDA(cudaMemcpyAsync(dev, prompt, bytes, cudaMemcpyHostToDevice, stream));
-    } else {   // (pageable memory: the copies return when it has been read)
-      QC_CUDA(cudaMemcpyAsync(dev, kind, n_kinds, cudaMemcpyHostToDevice, stream));
-      QC_CUDA(cudaMemcpyAsync(dev + codes_at(n_kinds), up->codes, up->n_codes, cudaMemcpyHostToDevice, stream));
-      if (up->passes)
-        QC_CUDA(cudaMemcpyAsync(dev + passes_at(n_kinds, up->n_codes), up->passes->data(), up->passes->size() * sizeof(PrefillPass),
-                                cudaMemcpyHostToDevice, stream));
+    std::memcpy(prompt, kind, n_kinds);
+    std::memcpy(prompt + codes_at(n_kinds), up->codes, up->n_codes);
+    size_t bytes = passes_at(n_kinds, up->n_codes);
+    if (up->passes) {
+      std::memcpy(prompt + bytes, up->passes->data(), up->passes->size() * sizeof(PrefillPass));
+      bytes += up->passes->size() * sizeof(PrefillPass);
     }
+    QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.prompt, prompt, bytes, cudaMemcpyHostToDevice, stream));
   }
   QC_CUDA(cudaEventRecord(c->prompt_staged, stream));
   Params p = base_params(c);

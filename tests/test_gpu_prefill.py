@@ -276,3 +276,34 @@ def test_prefill_attend_continues_a_cached_sequence(mode, head_dim, group):
             assert_close(got2[l, t0:t0 + 64], ref[l, T1 + 3 + t0: T1 + 3 + t0 + 64], f"second chunk layer {l} tokens {t0}..")
     assert s.stats().device_error == 0
     s.close()
+
+
+def test_kinds_of_a_long_prompt_are_consumed_by_the_call():
+    """`kind` belongs to the caller again when the call returns, also when it is page-locked, the prompt is longer
+    than 65 536 tokens and the stream is still busy with earlier work: the array is overwritten at once.
+    Runs of 1 to 200 tokens, so tiles of all three codes, far past the ones that travel as arguments."""
+    import ctypes
+
+    T, D = 66001, 128
+    s = Session(2, 1, 1, D, [0, 1], max_seqs=2, max_tokens_per_seq=T, n_pages=4 * 2 * (T // 16 + 3))
+    gen = torch.Generator(device=s.device).manual_seed(11)
+    q, k, v = (torch.randn(2, T, 1, D, generator=gen, device=s.device, dtype=torch.bfloat16) for _ in range(3))
+    out = torch.empty_like(q)
+    s.prefill_attend(1, [0] * 5, *(x[:, :5].contiguous() for x in (q, k, v, out)))   # (what a first call sets up)
+    rng = np.random.default_rng(12)
+    runs = rng.integers(1, 201, T)
+    kind = np.repeat(np.arange(T) % 2, runs)[:T].astype(np.uint8)
+    pinned = torch.from_numpy(kind.copy()).pin_memory()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)   # the stream is busy for a tenth of a second
+    qc._check(qc.load().qc_prefill_attend(s.cache, 0, T, ctypes.cast(pinned.data_ptr(), ctypes.POINTER(ctypes.c_uint8)),
+                                          *(ctypes.c_void_p(x.data_ptr()) for x in (q, k, v, out))), "qc_prefill_attend")
+    pinned.fill_(1).sub_(torch.from_numpy(kind))   # every kind the other one
+    vis = torch.from_numpy(kind != 0).to(s.device)
+    key = torch.where(vis[:, None], k[0, :, 0], k[1, :, 0]).double()
+    for t in (0, 63, 64, 8191, 16383, 16384, 16448, 30000, 65535, 65536, T - 1, *rng.integers(0, T, 20).tolist()):
+        query = q[0 if kind[t] else 1, t, 0].double()
+        want = torch.softmax(key[:t + 1] @ query * D ** -0.5, 0) @ v[1, :t + 1, 0].double()
+        assert_close(bits_of(out[1, t, 0]), want.cpu().numpy(), f"token {t}")
+    assert s.stats().device_error == 0
+    s.close()
