@@ -22,8 +22,9 @@
  *   - "dev" pointers are CUDA device pointers on the context's device; "host" pointers are
  *     ordinary host memory.  All device memory is owned by the caller: the pool and the
  *     workspace are handed in at qc_alloc_cache and must outlive the cache.  The library
- *     allocates no device memory.  It owns the qc_ctx / qc_cache host objects and a few KiB of
- *     pinned host memory per cache.
+ *     allocates no device memory.  It owns the qc_ctx / qc_cache host objects and, per
+ *     cache and from qc_alloc_cache on, 2 MiB of pinned host memory for what prompt calls upload
+ *     and eight copies of a step's descriptors (32 bytes per sequence, 16 per layer and sequence).
  *   - Kernels are launched asynchronously on the stream given to qc_init.  Device pointers
  *     passed to a call must stay valid until that stream has executed the call.  Host arrays
  *     (seq_ids, n_tokens, kind) are consumed before the call returns.

@@ -21,7 +21,11 @@ constexpr int kMaxProfileSteps = 16384;
 constexpr size_t kStoreSegs = 1 << 14;          // runs of tokens per launch of the kernel that stores prompt rows
 constexpr size_t kPromptBytes = 786432;   // a prompt's kinds, tile codes and passes, on the device and in pinned memory
 constexpr int kStoreBlocksBeside = 1, kStoreBlocksAlone = 7;   // blocks per SM of the kernel that stores prompt rows
-constexpr int kStageTableSeqs = 4;   // sequences whose page-table rows go through pinned memory
+// Page tables of a prompt call: a small mirror goes to the device whole, in one copy; otherwise the used ids of up
+// to four listed sequences in a copy each, as far as they fit; otherwise the whole mirror as it is.
+constexpr size_t kStageTableBytes = 1 << 20, kSmallTableBytes = 1 << 17;
+constexpr int kStageTableSeqs = 4;
+constexpr size_t kPromptStageBytes = kStoreSegs * sizeof(StoreSeg) + kPromptBytes + kStageTableBytes;
 // Shared-score passes run one CTA per SM (three accumulators fill tensor memory); that pays once
 // a CTA has enough key tiles: measured -16 % / -10 % call time at 2048 / 3008 tokens, +4 % / +9 %
 // at 1120 / 675.
@@ -134,7 +138,7 @@ struct qc_cache {
 
   // pinned staging ring for step descriptors
   uint8_t* pinned = nullptr;
-  uint8_t* prompt_stage = nullptr;    // pinned: what a prompt call uploads (made by the first one)
+  uint8_t* prompt_stage = nullptr;    // pinned: what a prompt call uploads (runs of tokens | prompt | page-table rows)
   cudaEvent_t prompt_staged = nullptr;
   int32_t* err_host = nullptr;        // mapped host word the kernels mirror the device error word into
   int32_t* err_host_dev = nullptr;    // its device address
@@ -835,6 +839,8 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
                           cudaHostAllocDefault) == cudaSuccess;
   for (int i = 0; ok && i < kStageSlots; ++i)
     ok = cudaEventCreateWithFlags(&c->stage_done[i], cudaEventDisableTiming) == cudaSuccess;
+  ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->prompt_stage), kPromptStageBytes, cudaHostAllocDefault) == cudaSuccess &&
+       cudaEventCreateWithFlags(&c->prompt_staged, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->err_host), 64, cudaHostAllocMapped) == cudaSuccess;
   if (ok) {
     *c->err_host = 0;
@@ -955,6 +961,7 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     if (make_rows_tensor_map(&map_k, k_dev, N * total, c->hkv, c->D) != QC_OK || make_rows_tensor_map(&map_v, v_dev, N * total, c->hkv, c->D) != QC_OK)
       return QC_ERR_CUDA;
   }
+  QC_CUDA(cudaEventSynchronize(c->prompt_staged));   // the last call's copies from the staging area have run
   // ---- commit: pages (sequence -> layer -> stream order)
   std::vector<int32_t> at_t(n_seqs), at_v(n_seqs);   // where each sequence's new tokens start in its streams
   for (int i = 0; i < n_seqs; ++i) {
@@ -973,29 +980,28 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     st.len_vis += add_v[i];
     st.active = true;
   }
-  if (!c->prompt_stage) {   // runs of tokens | prompt | page-table rows
-    const size_t bytes = kStoreSegs * sizeof(StoreSeg) + kPromptBytes +
-                         static_cast<size_t>(kStageTableSeqs) * N * 4 * c->max_pages * sizeof(int32_t);
-    QC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->prompt_stage), bytes, cudaHostAllocDefault));
-    QC_CUDA(cudaEventCreateWithFlags(&c->prompt_staged, cudaEventDisableTiming));
-  } else {
-    QC_CUDA(cudaEventSynchronize(c->prompt_staged));   // the last call's copies have run
-  }
   StoreSeg* segs = reinterpret_cast<StoreSeg*>(c->prompt_stage);
   uint8_t* prompt = c->prompt_stage + kStoreSegs * sizeof(StoreSeg);
   int32_t* rows = reinterpret_cast<int32_t*>(prompt + kPromptBytes);
-  // page tables: the listed sequences' rows, or the whole host mirror
-  if (c->paged && n_seqs <= kStageTableSeqs) {
-    const size_t row = c->max_pages * sizeof(int32_t);
-    for (int i = 0; i < n_seqs; ++i, rows += static_cast<size_t>(N) * 4 * c->max_pages) {
-      for (int r = 0; r < 4 * N; ++r)
-        std::memcpy(rows + static_cast<size_t>(r) * c->max_pages, c->table.data() + trow(c, 0, r, seq_ids[i]), row);
-      QC_CUDA(cudaMemcpy2DAsync(c->ws + c->lay.table + static_cast<size_t>(seq_ids[i]) * row, c->cfg.max_seqs * row, rows, row, row,
-                                static_cast<size_t>(N) * 4, cudaMemcpyHostToDevice, stream));
+  if (c->paged) {
+    const size_t row = c->max_pages * sizeof(int32_t), table_bytes = c->table.size() * sizeof(int32_t);
+    int used = 1;   // page ids of the longest listed stream
+    for (int i = 0; i < n_seqs; ++i)
+      used = std::max(used, std::max(pages_for(c->seqs[seq_ids[i]].len_text), pages_for(c->seqs[seq_ids[i]].len_vis)));
+    const size_t width = used * sizeof(int32_t), n_rows = static_cast<size_t>(N) * 4;
+    if (table_bytes <= kSmallTableBytes) {
+      std::memcpy(rows, c->table.data(), table_bytes);
+      QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.table, rows, table_bytes, cudaMemcpyHostToDevice, stream));
+    } else if (n_seqs <= kStageTableSeqs && n_seqs * n_rows * width <= kStageTableBytes) {
+      for (int i = 0; i < n_seqs; ++i, rows += n_rows * used) {
+        for (size_t r = 0; r < n_rows; ++r)
+          std::memcpy(rows + r * used, c->table.data() + trow(c, 0, static_cast<int>(r), seq_ids[i]), width);
+        QC_CUDA(cudaMemcpy2DAsync(c->ws + c->lay.table + static_cast<size_t>(seq_ids[i]) * row, c->cfg.max_seqs * row, rows, width,
+                                  width, n_rows, cudaMemcpyHostToDevice, stream));
+      }
+    } else {
+      QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.table, c->table.data(), table_bytes, cudaMemcpyHostToDevice, stream));
     }
-  } else if (c->paged) {
-    QC_CUDA(cudaMemcpyAsync(c->ws + c->lay.table, c->table.data(), c->table.size() * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, stream));
   }
   if (up) {   // (one sequence; qc_prefill_attend has checked that it fits)
     const size_t n_kinds = static_cast<size_t>(total);

@@ -67,3 +67,32 @@ def test_more_runs_than_one_launch_takes():
             assert np.array_equal(s.read_row(0, 2 + stream, 0, i, 0), vb[0, 2 * i + stream, 0])
     assert s.stats().device_error == 0
     s.close()
+
+
+def _mapped_kib():
+    with open("/proc/self/status") as f:
+        return int(next(line for line in f if line.startswith("VmSize")).split()[1])
+
+
+def test_prompt_calls_take_no_host_memory():
+    """What a prompt call needs is there when the cache is: a call that had to allocate could fail after the
+    sequence's pages were taken.  Long sequences, whose page tables are large."""
+    def session():
+        return Session(8, 1, 1, 64, [0, 1] * 4, max_seqs=2, max_tokens_per_seq=(1 << 20) - 16, n_pages=400)
+
+    kind = np.array([0] * 5 + [1] * 40, np.uint8)
+    x = [torch.randn(8, 45, 1, 64, dtype=torch.bfloat16, device="cuda") for _ in range(4)]
+    warm = session()   # (loads the kernels)
+    warm.prefill_attend(0, kind, *x)
+    s = session()
+    torch.cuda.synchronize()
+    before = _mapped_kib()
+    s.prefill_attend(0, kind, *x)
+    s.prefill_append([1], [45], kind, x[1], x[2])
+    torch.cuda.synchronize()
+    assert _mapped_kib() - before < 4096
+    for seq in (0, 1):   # (of each table row only the ids in use travel)
+        assert np.array_equal(s.read_row(7, qc.QC_STREAM_V_VISUAL, seq, 39, 0), bits_of(x[2])[7, 44, 0])
+    assert s.stats().device_error == 0
+    warm.close()
+    s.close()
