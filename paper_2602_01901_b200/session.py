@@ -49,16 +49,29 @@ class Session:
                    split_tokens=split_tokens, device=device, poison_pool=poison_pool)
 
     # ---- calls --------------------------------------------------------------------------
+    # Calls are enqueued on the stream that was current when the session was made and return at once.
+    # The prompt calls tell the allocator that their tensors are in use there, so that they can be
+    # dropped under any stream; and what prefill_append reads may be overwritten from the current
+    # stream right after the call, whichever that is.
+    def _in_use(self, *tensors):
+        for t in tensors:
+            t.record_stream(self.stream)
+
     def prefill_append(self, seq_ids: Sequence[int], n_tokens: Sequence[int], kind, k: torch.Tensor, v: torch.Tensor):
         assert k.dtype == torch.bfloat16 and v.dtype == torch.bfloat16 and k.is_contiguous() and v.is_contiguous()
         qc.qc_prefill_append(self.cache, list(seq_ids), list(n_tokens), bytes(bytearray(np.asarray(kind, np.uint8))),
                              k.data_ptr(), v.data_ptr())
+        self._in_use(k, v)
+        current = torch.cuda.current_stream(self.device)
+        if current != self.stream:
+            current.wait_stream(self.stream)
 
     def prefill_attend(self, seq_id: int, kind, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, out: torch.Tensor):
         for t in (q, k, v, out):
             assert t.dtype == torch.bfloat16 and t.is_contiguous()
         qc.qc_prefill_attend(self.cache, seq_id, bytes(bytearray(np.asarray(kind, np.uint8))), q.data_ptr(),
                              k.data_ptr(), v.data_ptr(), out.data_ptr())
+        self._in_use(q, k, v, out)
 
     def decode_step(self, seq_ids, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, out: torch.Tensor,
                     lse: Optional[torch.Tensor] = None):

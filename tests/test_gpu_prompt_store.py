@@ -70,8 +70,15 @@ def test_more_runs_than_one_launch_takes():
 
 
 def _mapped_kib():
-    with open("/proc/self/status") as f:
-        return int(next(line for line in f if line.startswith("VmSize")).split()[1])
+    """Readable and writable memory of this process (address space that is only reserved does not count)."""
+    total = 0
+    with open("/proc/self/maps") as f:
+        for line in f:
+            span, perms = line.split()[:2]
+            if perms.startswith("rw"):
+                first, last = (int(x, 16) for x in span.split("-"))
+                total += (last - first) // 1024
+    return total
 
 
 def test_prompt_calls_take_no_host_memory():
@@ -95,4 +102,33 @@ def test_prompt_calls_take_no_host_memory():
         assert np.array_equal(s.read_row(7, qc.QC_STREAM_V_VISUAL, seq, 39, 0), bits_of(x[2])[7, 44, 0])
     assert s.stats().device_error == 0
     warm.close()
+    s.close()
+
+
+@pytest.mark.parametrize("reuse", ["dropped", "overwritten"])
+def test_rows_may_be_reused_from_another_stream(reuse):
+    """The caller's tensors live on a stream of their own, and the session's is still busy when the call
+    returns: neither dropping them nor writing to them on that stream reaches the rows being stored."""
+    t, heads, d = 300, 8, 128
+    s = Session(2, heads, heads, d, [0, 1], max_seqs=2, max_tokens_per_seq=t, n_pages=8 * 2 * (t // 16 + 2))
+    kind = np.array([0] * 30 + [1] * (t - 30), np.uint8)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        k, v = (torch.randn(2, t, heads, d, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+        want = bits_of(v)
+        side.synchronize()
+        s.prefill_append([1], [t], kind, k, v)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s.stream):
+            torch.cuda._sleep(200_000_000)   # a tenth of a second
+        s.prefill_append([0], [t], kind, k, v)
+        if reuse == "dropped":
+            del k, v
+            others = [torch.full((2, t, heads, d), 3.0, device=s.device, dtype=torch.bfloat16) for _ in range(4)]
+        else:
+            k.fill_(3.0), v.fill_(3.0)
+    torch.cuda.synchronize()
+    for i in (0, 100, t - 31):
+        assert np.array_equal(s.read_row(1, qc.QC_STREAM_V_VISUAL, 0, i, 5), want[1, 30 + i, 5])
+    assert s.stats().device_error == 0
     s.close()
