@@ -215,9 +215,20 @@ struct __align__(16) StoreSeg {
   int32_t tok, n;     // first token in the caller's tensors, tokens
 };
 static_assert(sizeof(StoreSeg) == 16, "StoreSeg layout");
-// k, v: the caller's tensors as {d, heads, n_layers * n_tokens}, box {d, 1, 16}; segs: device
-cudaError_t launch_prefill_store(const Params& p, const CUtensorMap& k, const CUtensorMap& v, const StoreSeg* segs, int32_t n_segs,
-                                 int32_t n_tokens, int blocks, cudaStream_t stream);
+// Runs by length: a run of up to 16, 8, 4, 2 or 1 tokens is fetched 1, 2, 4, 8 or 16 heads at a time, so that a
+// box always has 16 rows of which more than half are wanted.
+constexpr int kStoreKinds = 5;
+inline int store_kind(int n) { return n > 8 ? 0 : n > 4 ? 1 : n > 2 ? 2 : n > 1 ? 3 : 4; }
+struct StoreMaps {
+  CUtensorMap k[kStoreKinds], v[kStoreKinds];   // the caller's tensors as {d, n_layers * n_tokens, heads}, box {d, 16 >> kind, 1 << kind}
+};
+// segs: device, ordered by kind; first[i]: the first one of kind i, first[kStoreKinds]: their number
+struct StoreList {
+  const StoreSeg* segs;
+  int32_t first[kStoreKinds + 1];
+  int32_t n_tokens;
+};
+cudaError_t launch_prefill_store(const Params& p, const StoreMaps& maps, const StoreList& list, int blocks, cudaStream_t stream);
 // Tensor maps of one prompt for the tcgen05 prefill kernel: q, k, v as 3-D tensors
 // {128, heads, n_layers * T} read in boxes of 64 tokens x one head x 64 elements, and the output
 // as a 4-D tensor {128, hq, T, n_layers} written in boxes of 128 tokens x one head x 64 elements

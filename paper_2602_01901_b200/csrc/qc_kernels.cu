@@ -278,10 +278,11 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(const __grid_constant_
 // ------------------------------------------------------------------------------------------
 
 // Stores prompt tokens' K/V rows into their pages.  A unit is what one page receives of one run of
-// tokens (StoreSeg: up to 16 consecutive tokens of one stream) for one layer, tensor and head: rows
-// strided in the caller's tensor, contiguous in the page.  A tensor-map copy brings 16 rows into
-// shared memory and a bulk copy writes the valid ones out, so no data passes through registers; a
-// lane of the block's one warp owns one buffer and walks its own units.
+// tokens (StoreSeg: up to 16 consecutive tokens of one stream) for one layer, tensor and group of heads: rows
+// strided in the caller's tensor, contiguous per head in the page.  A tensor-map copy brings 16 rows into
+// shared memory -- 16 tokens of one head, or fewer tokens of more heads where the run is short -- and a bulk
+// copy per head writes the valid ones out, so no data passes through registers; a lane of the block's one warp
+// owns one buffer and walks its own units.
 // The next kernel in the stream may start while this one runs: the prompt's attention reads the
 // caller's tensors and pages stored earlier, nothing of what is stored here (it waits for this
 // kernel before it ends).  One block per SM (28 KB of shared memory) fits beside two blocks of the
@@ -289,11 +290,13 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(const __grid_constant_
 // Per call, rows passing through registers in a launch ahead of the attention -> this: 675 tokens, 32
 // layers 451 -> 343 us; 4 352 tokens 5.94 -> 5.47 ms; alone, 32 prompts of 1 120 tokens with 4 heads 1.62 ->
 // 0.63 ms, 8 of 3 008 with 32 heads 3.79 -> 3.31 ms (6.8 TB/s).
+// Tokens that alternate between text and visual (a run is one token), 32 layers x 32 heads, storing alone / with the
+// attention: with 16 rows of one head fetched for every run 0.32 / 1.50 ms at 675 tokens, 1.58 / 7.17 at 3 008; by the
+// length of the run 0.17 / 0.57 and 0.55 / 5.31 (through registers 0.17 / 0.65 and 0.56 / 5.74).
 constexpr int kStoreLanes = 7;
 template <int D>
-__global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tmap_k,
-                                                           const __grid_constant__ CUtensorMap tmap_v, const StoreSeg* segs, int32_t n_segs,
-                                                           int32_t n_tokens) {
+__global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant__ Params P, const __grid_constant__ StoreMaps maps,
+                                                           const __grid_constant__ StoreList list) {
   constexpr uint32_t kTile = kPage * D * 2;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t full[kStoreLanes];
@@ -303,23 +306,37 @@ __global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant
   mbar_init(&full[lane], 1);
   fence_mbar_init();
   const uint32_t buf = smem_u32(smem) + lane * kTile;
-  const uint32_t n_units = static_cast<uint32_t>(n_segs) * P.hkv * P.n_layers * 2, stride = gridDim.x * kStoreLanes;
+  // units per (layer, tensor): runs of one kind after those of another, groups of heads fastest
+  uint32_t before[kStoreKinds + 1];
+  before[0] = 0;
+#pragma unroll
+  for (int i = 0; i < kStoreKinds; ++i)
+    before[i + 1] = before[i] + static_cast<uint32_t>(list.first[i + 1] - list.first[i]) * ((P.hkv + (1 << i) - 1) >> i);
+  const uint32_t per_tensor = before[kStoreKinds], n_units = per_tensor * P.n_layers * 2, stride = gridDim.x * kStoreLanes;
   struct Unit {
-    int32_t head, row, pid, slot, bytes;
+    int32_t head, heads, row, pid, slot, bytes, kind;
     bool value;
   };
   // the lane's next unit at or after u that is stored at all
   auto find = [&](uint32_t& u, Unit& x) -> bool {
     for (; u < n_units; u += stride) {
-      const uint32_t a = u / P.hkv, b = a / n_segs, layer = b >> 1;   // head fastest, then segment, tensor, layer
-      const StoreSeg sg = segs[a - b * n_segs];
+      const uint32_t b = u / per_tensor, r = u - b * per_tensor, layer = b >> 1;
+      int kind = 0;
+      uint32_t base = 0;
+#pragma unroll
+      for (int i = 1; i < kStoreKinds; ++i)
+        if (r >= before[i]) kind = i, base = before[i];
+      const uint32_t groups = (P.hkv + (1 << kind) - 1) >> kind, run = (r - base) / groups;
+      const StoreSeg sg = list.segs[list.first[kind] + run];
       const int stream = sg.ord < 0, ord = sg.ord & 0x7fffffff;
       x.value = b & 1;
       const uint8_t lf = P.layer_flags[layer];
       // K of a lazy layer: visual rows are never kept; text rows only where the mode keeps them
       if (!x.value && !((lf & kLayerWritesQCache) || (stream == 0 && (lf & kLayerOwnsTextK)))) continue;
-      x.head = u - a * P.hkv;
-      x.row = layer * n_tokens + sg.tok;
+      x.kind = kind;
+      x.head = static_cast<int>(r - base - run * groups) << kind;
+      x.heads = min(1 << kind, P.hkv - x.head);
+      x.row = layer * list.n_tokens + sg.tok;
       x.pid = P.table[table_row(P, layer, (x.value ? 2 : 0) + stream, sg.seq) + ord / kPage];
       x.slot = ord % kPage;
       x.bytes = sg.n * (D * 2);
@@ -334,7 +351,7 @@ __global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant
   while (any) {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the buffer's last rows have been read
     mbar_expect_tx(&full[lane], kTile);
-    tensor_g2s_3d(buf, x.value ? &tmap_v : &tmap_k, 0, x.head, x.row, &full[lane]);
+    tensor_g2s_3d(buf, x.value ? &maps.v[x.kind] : &maps.k[x.kind], 0, x.row, x.head, &full[lane]);
     const Unit now = x;
     u += stride;
     any = find(u, x);   // (its reads overlap the copy)
@@ -348,7 +365,9 @@ __global__ void __launch_bounds__(32) prefill_store_kernel(const __grid_constant
     }
     phase ^= 1u;
     uint16_t* dst = P.pool + ((static_cast<size_t>(now.pid) * P.hkv + now.head) * kPage + now.slot) * D;
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(buf), "r"(now.bytes) : "memory");
+    for (int h = 0; h < now.heads; ++h, dst += kPage * D)
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(buf + h * (kTile >> now.kind)), "r"(now.bytes)
+                   : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -901,12 +920,11 @@ cudaError_t launch_merge(const Params& p, cudaStream_t stream) {
   return launch_pdl(merge_kernel<64>, grid, block, 0, stream, p);
 }
 
-cudaError_t launch_prefill_store(const Params& p, const CUtensorMap& k, const CUtensorMap& v, const StoreSeg* segs, int32_t n_segs,
-                                 int32_t n_tokens, int blocks, cudaStream_t stream) {
-  if (n_segs <= 0) return cudaSuccess;
+cudaError_t launch_prefill_store(const Params& p, const StoreMaps& maps, const StoreList& list, int blocks, cudaStream_t stream) {
+  if (list.first[kStoreKinds] <= 0) return cudaSuccess;
   const int smem = kStoreLanes * kPage * p.d * 2;
-  if (p.d == 128) prefill_store_kernel<128><<<blocks, 32, smem, stream>>>(p, k, v, segs, n_segs, n_tokens);
-  else prefill_store_kernel<64><<<blocks, 32, smem, stream>>>(p, k, v, segs, n_segs, n_tokens);
+  if (p.d == 128) prefill_store_kernel<128><<<blocks, 32, smem, stream>>>(p, maps, list);
+  else prefill_store_kernel<64><<<blocks, 32, smem, stream>>>(p, maps, list);
   return cudaGetLastError();
 }
 

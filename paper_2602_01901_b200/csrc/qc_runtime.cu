@@ -569,14 +569,14 @@ int make_prompt_tensor_map(CUtensorMap* out, const void* base, int n_layers, int
   return r == CUDA_SUCCESS ? QC_OK : QC_ERR_CUDA;
 }
 
-// A prompt's K or V rows [n_rows][heads][d] bf16 as a 3-D tensor {d, heads, n_rows}: a box is 16 rows
-// of one head, in row order (what a page holds of a head).
-int make_rows_tensor_map(CUtensorMap* out, const void* base, int64_t n_rows, int heads, int d) {
+// A prompt's K or V rows [n_rows][heads][d] bf16 as a 3-D tensor {d, n_rows, heads}: a box of the given kind is 16 rows
+// in all, those of one head side by side and in row order (what a page holds of a head).
+int make_rows_tensor_map(CUtensorMap* out, const void* base, int64_t n_rows, int heads, int d, int kind) {
   EncodeFn enc = tensor_map_encoder();
   if (!enc) return QC_ERR_CUDA;
-  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(heads), static_cast<cuuint64_t>(n_rows)};
-  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * 2, static_cast<cuuint64_t>(heads) * d * 2};
-  const cuuint32_t box[3] = {static_cast<cuuint32_t>(d), 1, kPage};
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(n_rows), static_cast<cuuint64_t>(heads)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(heads) * d * 2, static_cast<cuuint64_t>(d) * 2};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(d), static_cast<cuuint32_t>(kPage >> kind), 1u << kind};
   const cuuint32_t elem_strides[3] = {1, 1, 1};
   const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem_strides,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -955,11 +955,13 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   cudaStream_t stream = c->ctx->stream;
 
   // ---- what can still fail without a change: the tensor maps of the caller's rows
-  CUtensorMap map_k, map_v;
+  StoreMaps maps;
   if (total > 0) {
     if (static_cast<int64_t>(N) * total > 0x7fffffffLL) return QC_ERR_INVALID_ARG;   // rows are counted in 31 bits
-    if (make_rows_tensor_map(&map_k, k_dev, N * total, c->hkv, c->D) != QC_OK || make_rows_tensor_map(&map_v, v_dev, N * total, c->hkv, c->D) != QC_OK)
-      return QC_ERR_CUDA;
+    for (int i = 0; i < kStoreKinds; ++i)
+      if (make_rows_tensor_map(&maps.k[i], k_dev, N * total, c->hkv, c->D, i) != QC_OK ||
+          make_rows_tensor_map(&maps.v[i], v_dev, N * total, c->hkv, c->D, i) != QC_OK)
+        return QC_ERR_CUDA;
   }
   QC_CUDA(cudaEventSynchronize(c->prompt_staged));   // the last call's copies from the staging area have run
   // ---- commit: pages (sequence -> layer -> stream order)
@@ -1019,17 +1021,24 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   p.k = static_cast<const uint16_t*>(k_dev);
   p.v = static_cast<const uint16_t*>(v_dev);
   StoreSeg* segs_dev = reinterpret_cast<StoreSeg*>(c->ws + c->lay.tok);
-  // runs of tokens, a batch at a time; beside the attention of the prompt the stores get one block per
-  // SM, alone as many as fit
+  // runs of tokens, a batch at a time, by kind; beside the attention of the prompt the stores get one block
+  // per SM, alone as many as fit
+  std::vector<StoreSeg> runs[kStoreKinds];
   size_t n = 0;
   int64_t tok = 0;
   bool used = false;   // the staging area holds runs that are being copied
   auto flush = [&]() -> int32_t {
+    if (used) QC_CUDA(cudaEventSynchronize(c->prompt_staged));
+    StoreList list{segs_dev, {0}, static_cast<int32_t>(total)};
+    for (int i = 0; i < kStoreKinds; ++i) {
+      std::copy(runs[i].begin(), runs[i].end(), segs + list.first[i]);
+      list.first[i + 1] = list.first[i] + static_cast<int32_t>(runs[i].size());
+      runs[i].clear();
+    }
     QC_CUDA(cudaMemcpyAsync(segs_dev, segs, n * sizeof(StoreSeg), cudaMemcpyHostToDevice, stream));
     QC_CUDA(cudaEventRecord(c->prompt_staged, stream));
     c->kernel_launches++;
-    QC_CUDA(launch_prefill_store(p, map_k, map_v, segs_dev, static_cast<int32_t>(n), static_cast<int32_t>(total),
-                                 c->ctx->n_sms * (up ? kStoreBlocksBeside : kStoreBlocksAlone), stream));
+    QC_CUDA(launch_prefill_store(p, maps, list, c->ctx->n_sms * (up ? kStoreBlocksBeside : kStoreBlocksAlone), stream));
     n = 0;
     used = true;
     return QC_OK;
@@ -1040,12 +1049,11 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
       int& at = kd == QC_KIND_VISUAL ? at_v[i] : at_t[i];
       int len = 1;
       while (t + len < n_tokens[i] && kind[tok + t + len] == kd && (at + len) % kPage != 0) ++len;
-      if (used && n == 0) QC_CUDA(cudaEventSynchronize(c->prompt_staged));
-      segs[n++] = StoreSeg{seq_ids[i], static_cast<int32_t>(static_cast<uint32_t>(at) | (kd == QC_KIND_VISUAL ? 0x80000000u : 0u)),
-                           static_cast<int32_t>(tok + t), len};
+      runs[store_kind(len)].push_back(StoreSeg{seq_ids[i], static_cast<int32_t>(static_cast<uint32_t>(at) | (kd == QC_KIND_VISUAL ? 0x80000000u : 0u)),
+                                               static_cast<int32_t>(tok + t), len});
       at += len;
       t += len;
-      if (n == kStoreSegs) {
+      if (++n == kStoreSegs) {
         const int32_t st = flush();
         if (st != QC_OK) return st;
       }

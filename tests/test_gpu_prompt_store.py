@@ -132,3 +132,57 @@ def test_rows_may_be_reused_from_another_stream(reuse):
         assert np.array_equal(s.read_row(1, qc.QC_STREAM_V_VISUAL, 0, i, 5), want[1, 30 + i, 5])
     assert s.stats().device_error == 0
     s.close()
+
+
+@pytest.mark.parametrize("head_dim,q_heads,kv_heads", [(128, 17, 17), (64, 10, 5)])
+def test_runs_of_every_length(head_dim, q_heads, kv_heads):
+    """Runs of 1 to 17 tokens: fetched a few or many heads at a time, with heads left over in the last group."""
+    n = 2
+    kinds = [np.concatenate([np.full(i, i % 2, np.uint8) for i in range(1, 18)]),
+             np.concatenate([np.full(1 + (5 * i) % 9, i % 2, np.uint8) for i in range(40)])]
+    s = Session(n, q_heads, kv_heads, head_dim, [0, 1], max_seqs=2, max_tokens_per_seq=256, n_pages=2 * n * 2 * 32,
+                lazy_mode=qc.QC_MODE_VLA_QC, poison_pool=True)
+    total = sum(len(x) for x in kinds)
+    k, v = (torch.randn(n, total, kv_heads, head_dim, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+    s.prefill_append([0, 1], [len(x) for x in kinds], np.concatenate(kinds), k, v)
+    at, kb, vb = 0, bits_of(k), bits_of(v)
+    for seq, kind in enumerate(kinds):
+        for stream in (0, 1):
+            tokens = [at + t for t in range(len(kind)) if kind[t] == stream]
+            for h in {0, 1, 3, 4, 7, 8, 15, 16} & set(range(kv_heads)):
+                for i, t in enumerate(tokens):
+                    assert np.array_equal(s.read_row(1, 2 + stream, seq, i, h), vb[1, t, h]), (seq, stream, h, i)
+                    assert np.array_equal(s.read_row(0, stream, seq, i, h), kb[0, t, h]), (seq, stream, h, i)
+        at += len(kind)
+    assert s.stats().device_error == 0
+    s.close()
+
+
+def _best_ms(call, runs=8):
+    best = float("inf")
+    for _ in range(runs):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        e[0].record()
+        call()
+        e[1].record()
+        torch.cuda.synchronize()
+        best = min(best, e[0].elapsed_time(e[1]))
+    return best
+
+
+def test_alternating_tokens_cost_about_what_runs_do():
+    """One token of text, one visual, and so on: 16 times as many runs of as many rows.  (Measured 1.1 times the
+    time of two long runs with the rows stored one by one, 3.2 times with 16 rows fetched for each run.)"""
+    t, n, heads, d = 3008, 8, 32, 128
+    s = Session(n, heads, heads, d, [0, 1] * 4, max_seqs=1, max_tokens_per_seq=t, n_pages=2 * n * (t // 16 + 3))
+    k, v = (torch.randn(n, t, heads, d, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+
+    def stored(kind):
+        s.prefill_append([0], [t], kind, k, v)
+        qc.qc_free_seq(s.cache, 0)
+
+    half = np.repeat(np.array([0, 1], np.uint8), t // 2)
+    alternating = np.tile(np.array([0, 1], np.uint8), t // 2)
+    assert _best_ms(lambda: stored(alternating)) < 2 * _best_ms(lambda: stored(half))
+    s.close()
