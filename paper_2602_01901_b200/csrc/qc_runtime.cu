@@ -903,6 +903,7 @@ struct PromptUpload {
   const uint8_t* codes;
   size_t n_codes;
   const std::vector<PrefillPass>* passes;   // null: none
+  bool beside;   // the attention runs beside the stores (it does not with an event between them)
 };
 inline size_t codes_at(size_t n_tokens) { return align_up(n_tokens, 256); }
 inline size_t passes_at(size_t n_tokens, size_t n_codes) { return codes_at(n_tokens) + align_up(n_codes, 256); }
@@ -1038,7 +1039,7 @@ int32_t store_prompt(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     QC_CUDA(cudaMemcpyAsync(segs_dev, segs, n * sizeof(StoreSeg), cudaMemcpyHostToDevice, stream));
     QC_CUDA(cudaEventRecord(c->prompt_staged, stream));
     c->kernel_launches++;
-    QC_CUDA(launch_prefill_store(p, maps, list, c->ctx->n_sms * (up ? kStoreBlocksBeside : kStoreBlocksAlone), stream));
+    QC_CUDA(launch_prefill_store(p, maps, list, c->ctx->n_sms * (up && up->beside ? kStoreBlocksBeside : kStoreBlocksAlone), stream));
     n = 0;
     used = true;
     return QC_OK;
@@ -1109,7 +1110,8 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
   const bool share = c->prefill_n_shared > 0 && n0_text + n0_vis == 0 &&
                      (c->prefill_shared == 2 || (c->prefill_shared == 1 && n_tokens >= kPrefillShareMinTokens));
   // store K/V: this validates the rest and leaves the cache unchanged on an error
-  const PromptUpload up{codes.data(), codes.size(), share ? &c->prefill_passes : nullptr};
+  const bool timed = c->profile && c->ev_prefill_calls < kMaxProfileSteps;
+  const PromptUpload up{codes.data(), codes.size(), share ? &c->prefill_passes : nullptr, !timed};
   const int st = store_prompt(c, 1, &seq_id, &n_tokens, kind, k_dev, v_dev, &up);
   if (st != QC_OK) return st;
   cudaStream_t stream = c->ctx->stream;
@@ -1118,7 +1120,7 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
   const PrefillPass* passes_dev = reinterpret_cast<const PrefillPass*>(kind_dev + passes_at(n_tokens, n_tiles));
   const Params p = base_params(c);
   cudaEvent_t* ev = nullptr;
-  if (c->profile && c->ev_prefill_calls < kMaxProfileSteps) {
+  if (timed) {
     if (static_cast<int>(c->ev_prefill.size()) < 2 * (c->ev_prefill_calls + 1)) {
       for (int i = 0; i < 2; ++i) {
         cudaEvent_t e;

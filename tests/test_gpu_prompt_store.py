@@ -186,3 +186,30 @@ def test_alternating_tokens_cost_about_what_runs_do():
     alternating = np.tile(np.array([0, 1], np.uint8), t // 2)
     assert _best_ms(lambda: stored(alternating)) < 2 * _best_ms(lambda: stored(half))
     s.close()
+
+
+def test_a_timed_prompt_call_stores_at_full_speed():
+    """With "profile" the attention kernel has an event in front of it, so the stores run alone: what a call
+    takes beyond that kernel is about what qc_prefill_append takes."""
+    t, n, heads, d = 3008, 8, 32, 128
+    s = Session(n, heads, heads, d, [0, 1] * 4, max_seqs=1, max_tokens_per_seq=t, n_pages=2 * n * (t // 16 + 3))
+    q, k, v = (torch.randn(n, t, heads, d, device=s.device, dtype=torch.bfloat16) for _ in range(3))
+    out = torch.empty_like(q)
+    kind = np.repeat(np.array([0, 1], np.uint8), t // 2)
+
+    def stored():
+        s.prefill_append([0], [t], kind, k, v)
+        qc.qc_free_seq(s.cache, 0)
+
+    def attended():
+        s.prefill_attend(0, kind, q, k, v, out)
+        qc.qc_free_seq(s.cache, 0)
+
+    alone = _best_ms(stored)
+    s.set_option("profile", 1)
+    rest = []
+    for _ in range(6):
+        call = _best_ms(attended, 1)
+        rest.append(call - s.profile().prefill_attend_ms)
+    assert min(rest) < 1.35 * alone
+    s.close()
