@@ -332,13 +332,12 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
   WorkerState st;
   worker_init(st, 0);
   st.drop_next = P.debug_drop_tile != 0;   // (test hook)
-  Item it;
   int issued = 0;
-  auto take = [&]() -> bool {   // the next item into `it`
-    if (STATIC) return cursor_step(cursor, P, it, lane);
+  auto take = [&](ItemPages& slot) -> bool {   // the next item into a context slot
+    if (STATIC) return cursor_step(cursor, P, slot, lane);
     const int idx = claim_take(P, issued);
     if (idx < 0) return false;
-    it = load_item(P, idx);
+    load_item(slot, P, idx, lane);
     return true;
   };
   // ---- ahead of the wait for the previous kernel: the first two items and their page ids (from the
@@ -346,23 +345,20 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
   // started), and the first tiles unless they could hold a new token that an earlier launch of the
   // step stores (with the folded append the worker patches the new token's row itself).  After it,
   // only the layer's inputs.
-  Item first;
   bool more;
   if (STATIC) {
     bool any = wid >= 0 && wid < P.part_workers;
     if (P.wdesc != nullptr) {
       // planned ahead: one read gives the first two items, the first page ids and the cursor
       any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, nullptr, lane);
-      if (any) first = ctx[0].ip.item;
     } else {
       RangeCursor c;
       any = any && cursor_init(c, part_view(P), wid);
       if (lane == 0) *cursor = c;
       __syncwarp();
-      any = any && take();
+      any = any && take(ctx[0].ip);
       if (any) {
-        first = it;
-        begin_item_pages(ctx[0].ip, P, first, lane);
+        begin_item_pages(ctx[0].ip, P, lane);
         cp_async_wait_all();
         __syncwarp();
       }
@@ -372,39 +368,38 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
       return;
     }
     st.n_my = 1;
+    const Item& first = ctx[0].ip.item;
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRingTc);
     if (early_tiles) fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
     if (P.wdesc != nullptr) {
-      if (first.n_pages > 2) begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
-      it = ctx[1].ip.item;
-      more = it.n_pages > 0;
+      if (first.n_pages > 2) begin_item_pages(ctx[0].ip, P, lane);   // the whole page list, while the tiles fly
+      more = ctx[1].ip.item.n_pages > 0;
     } else {
-      more = take();
+      more = take(ctx[1].ip);
     }
-    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    if (more) begin_item_pages(ctx[1].ip, P, lane);
     pdl_wait();
     pdl_launch_dependents();
   } else {
     pdl_wait();   // the item list and the work counter are the previous kernel's
     pdl_launch_dependents();
     issued = claim_issue(P, lane);
-    if (!take()) return;
-    first = it;
-    begin_item_pages(ctx[0].ip, P, first, lane);
+    if (!take(ctx[0].ip)) return;
+    begin_item_pages(ctx[0].ip, P, lane);
     cp_async_wait_all();
     __syncwarp();
     st.n_my = 1;
     fill_ring<D, kRingTc, true>(st, ctx_of, ring, full, P, lane);
     issued = claim_issue(P, lane);
   }
-  begin_new_rows(ctx[0].ip, P, first, lane, D);
+  begin_new_rows(ctx[0].ip, P, lane, D);
   if (!STATIC) {
-    more = take();
-    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    more = take(ctx[1].ip);
+    if (more) begin_item_pages(ctx[1].ip, P, lane);
   }
   cp_async_commit_group();
   if (more) {
-    begin_new_rows(ctx[1].ip, P, it, lane, D);
+    begin_new_rows(ctx[1].ip, P, lane, D);
   }
   cp_async_commit_group();   // the second item's inputs are waited for when the first item is done
   if (STATIC) cp_async_wait_group<1>();
@@ -421,17 +416,18 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
     const bool shared = cur.flags & kFlagShared;
     if (more) {
       // the third slot is free (it held the item before this one): start filling it with the item after next
-      more = take();
+      ItemPages& next = ctx[(k + 2) % kCtxSlots].ip;
+      more = take(next);
       if (more) {
-        begin_item_pages(ctx[(k + 2) % kCtxSlots].ip, P, it, lane);
-        begin_new_rows(ctx[(k + 2) % kCtxSlots].ip, P, it, lane, D);
+        begin_item_pages(next, P, lane);
+        begin_new_rows(next, P, lane, D);
         pending = true;
       }
     }
     if (!STATIC && more) issued = claim_issue(P, lane);   // answered by the time the next item starts
     if (nc == 1 && (cur.flags & kFlagReadLogits)) process_item_tc<D, 1, 1, 2>(st, ctx, ring, full, P, lane);
     else if (nc == 1 && (cur.flags & kFlagWriteLogits)) process_item_tc<D, 1, 1, 1>(st, ctx, ring, full, P, lane);
-    else if (shared && cur.skip_new) {
+    else if (shared && P.any_skip) {
       if (nc == 1) process_item_tc<D, 1, 1, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 2) process_item_tc<D, 1, 2, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 3) process_item_tc<D, 1, 3, 0, true>(st, ctx, ring, full, P, lane);
@@ -493,11 +489,16 @@ constexpr int attend_tc_smem_bytes() {
 }  // namespace
 
 namespace {
+// Shared memory for as many blocks as an SM holds of the kernel, and no more: the rest is L1 cache.
 template <typename K>
 cudaError_t configure_attend(K kernel, int smem) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  cudaFuncAttributes a;
+  e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  const int need = kAttendCtasPerSm * (smem + static_cast<int>(a.sharedSizeBytes) + 1024), all = 228 * 1024;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, min(100, (100 * need + all - 1) / all));
 }
 }  // namespace
 

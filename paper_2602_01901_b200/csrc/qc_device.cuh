@@ -421,14 +421,10 @@ __device__ __forceinline__ void drain_ring(WorkerState& st, uint64_t* full, uint
 // already fetches) and the one after, which is being filled by asynchronous copies meanwhile.
 constexpr int kCtxSlots = 3;
 
-// Start filling a context slot with an item and the page ids of its K stream and V streams
+// Start filling a context slot that holds an item with the page ids of its K stream and V streams
 // (asynchronous copies; cp_async_wait_all() + __syncwarp() completes them).
-__device__ __forceinline__ void begin_item_pages(ItemPages& c, const Params& P, const Item& it, int lane) {
-  __syncwarp();   // the slot's previous item is no longer read
-  if (lane == 0) {
-    c.item = it;
-    c.kv_head = it.head / P.group;
-  }
+__device__ __forceinline__ void begin_item_pages(ItemPages& c, const Params& P, int lane) {
+  const Item& it = c.item;
   if (lane < it.n_pages) {
     cp_async_4(&c.pages[0][lane], P.table + table_row(P, it.k_layer, it.stream, it.seq_id) + it.first_page + lane);
     for (int x = 0; x < it.n_cons; ++x)
@@ -437,19 +433,21 @@ __device__ __forceinline__ void begin_item_pages(ItemPages& c, const Params& P, 
   }
 }
 
-// Fetch an item's descriptor from the item list.
-__device__ __forceinline__ Item load_item(const Params& P, int item_idx) {
-  const uint4* ip = reinterpret_cast<const uint4*>(P.items + item_idx);
-  uint4 a = __ldg(ip), b = __ldg(ip + 1);
-  Item it;
-  reinterpret_cast<uint4*>(&it)[0] = a;
-  reinterpret_cast<uint4*>(&it)[1] = b;
-  return it;
+// Fetch an item's descriptor from the item list into a context slot.  (Items live in shared memory only: a
+// variable whose arrays are indexed at run time is local memory, and what twelve warps have of that does not stay
+// in the L1 cache beside the tiles.)
+__device__ __forceinline__ void load_item(ItemPages& c, const Params& P, int item_idx, int lane) {
+  __syncwarp();   // the slot's previous item is no longer read
+  if (lane < 2) reinterpret_cast<uint4*>(&c.item)[lane] = __ldg(reinterpret_cast<const uint4*>(P.items + item_idx) + lane);
+  __syncwarp();
+  if (lane == 0) c.kv_head = c.item.head / P.group;
 }
 
 // Items of a launch are handed out in list order (heaviest first, so the work left at the end
-// comes in small pieces).  A claim is an atomic increment issued by lane 0 whose result is only
-// looked at one item later, so its latency never stalls the tile pipeline.
+// comes in small pieces).  A claim is an atomic increment by lane 0.  It is issued when an item ends and
+// looked at when the next one begins; issued an item ahead, its result is one more register across the
+// page loops, which have none to spare (one-launch steps, us per layer: 12 sequences of 1 300 keys 32.8 -> 31.3 with the
+// claim at the end, 4 of 4 200 36.0 -> 35.1, 30 of 260 13.7 -> 13.4).
 __device__ __forceinline__ int claim_issue(const Params& P, int lane) {
   int idx = 0;
   if (lane == 0) idx = atomicAdd(P.work_counter + P.launch_index, 1);
@@ -661,13 +659,21 @@ __device__ __forceinline__ bool cursor_next(RangeCursor& c, const PartView& V, I
   }
 }
 
-// One step of a worker's cursor, kept in shared memory between items.  Warp-uniform.
-__device__ __forceinline__ bool cursor_step(RangeCursor* slot, const Params& P, Item& it, int lane) {
+// One step of a worker's cursor, kept in shared memory between items: the next item into a context slot.
+// Warp-uniform.
+__device__ __forceinline__ bool cursor_step(RangeCursor* cursor, const Params& P, ItemPages& slot, int lane) {
   __syncwarp();
-  RangeCursor c = *slot;
+  RangeCursor c = *cursor;
+  Item it;
   const bool ok = cursor_next(c, part_view(P), it);
   __syncwarp();
-  if (lane == 0) *slot = c;
+  if (lane == 0) {
+    *cursor = c;
+    if (ok) {
+      slot.item = it;
+      slot.kv_head = it.head / P.group;
+    }
+  }
   __syncwarp();
   return ok;
 }
@@ -684,7 +690,8 @@ __device__ __forceinline__ int first_taker(const Item& it) {   // first consumer
     if (!((it.skip_new >> x) & 1)) return x;
   return -1;
 }
-__device__ __forceinline__ void begin_new_rows(ItemPages& c, const Params& P, const Item& it, int lane, int d) {
+__device__ __forceinline__ void begin_new_rows(ItemPages& c, const Params& P, int lane, int d) {
+  const Item& it = c.item;
   if (!(P.fold_append && it.stream == 0 && (it.flags & kFlagStreamEnd))) return;
   const int n_vec = d / 8, kv_head = it.head / P.group;
   if (lane < n_vec)
@@ -719,7 +726,7 @@ __device__ __forceinline__ bool load_worker_desc(const Params& P, int wid, ItemP
   __syncwarp();
   if (c0.item.n_pages == 0) return false;
   if (lane < 2 * (1 + kMaxCons)) c0.pages[lane >> 1][lane & 1] = stage[lane];
-  if (lane == 0) c0.kv_head = c0.item.head / P.group;
+  if (lane == 0) c0.kv_head = c0.item.head / P.group, c1.kv_head = c1.item.head / P.group;
   __syncwarp();
   return true;
 }

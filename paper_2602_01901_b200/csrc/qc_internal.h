@@ -187,6 +187,8 @@ struct Params {
   int32_t part_q;                    // tiles per range
   int32_t part_wpc;                  // workers per CTA
   int32_t part_wv, part_wt;          // tiles per page summed over the launch's visual / text jobs
+  int32_t any_skip;                  // some item of the launch leaves out the step's new token for a consumer
+  int32_t any_own;                   // some item of the launch scores for several consumers with a query each
   int32_t fused_merge;               // the launch merges the output rows of its layer (layer_begin) itself
   int32_t planned_pieces;            // the numbers of partial rows of its layer's output rows are in row_pieces
   int32_t part_row_cost;             // what a row counts for besides its pages, in tiles

@@ -387,7 +387,8 @@ struct WarpCtx {
 
 // Start fetching the raw queries of the item in a context slot (asynchronous copies).
 template <int D>
-__device__ __forceinline__ void begin_queries(WarpCtx<D>& c, const Params& P, const Item& it, int lane) {
+__device__ __forceinline__ void begin_queries(WarpCtx<D>& c, const Params& P, int lane) {
+  const Item& it = c.ip.item;
   const int nq = (it.flags & kFlagShared) ? 1 : it.n_cons;
   if (lane < D / 8) {
     for (int x = 0; x < nq; ++x) {
@@ -467,38 +468,59 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
 
   constexpr bool kMayFold = FOLD || SKIP;
   const int new_pg = (kMayFold && holds_new_token(P, c.ip.item, n_pages - 1)) ? n_pages - 1 : -1;   // folded append: page of the new token
+  float p[NQ][4];
   for (int pg = 0; pg < n_pages && !st.dead; ++pg) {
     const int nvalid = (pg == n_pages - 1) ? n_valid_last : kPage;
-    float p[NQ][4];
-    if (MODE == 2) {
-      // ---- scores of 16 keys from the logit cache; the next page's are requested now
+    // softmax step of the page's 16 scores
+    auto weigh = [&]() {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) p[0][i] = lg_next[i];
-      if (pg + 1 < n_pages) {
+      for (int x = 0; x < NQ; ++x) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) lg_next[i] = lg[(pg + 1) * kPage + 4 * i + kg];
-      }
-    } else {
-      // ---- K tile: scores of 16 keys
-      const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
-      if (st.dead) break;
-      if (kMayFold && pg == new_pg) {
-        // the new token's k row comes from the step's input: into the tile, and into the pool for later steps
-        const Item& it = c.ip.item;
-        if (lane < D / 8) {
-          const uint4 val = c.ip.new_k[lane];
-          sts128(tile + (nvalid - 1) * (D * 2) + lane * 16, val);
-          const int pid = c.ip.pages[0][pg];
-          if (static_cast<uint32_t>(pid) < static_cast<uint64_t>(P.n_pool_pages))
-            reinterpret_cast<uint4*>(P.pool + ((static_cast<size_t>(pid) * P.hkv + c.ip.kv_head) * kPage + (nvalid - 1)) * D)[lane] = val;
-          // an ordinary layer's query goes to the Q Cache
-          if (it.q_layer[0] == it.k_layer && !((it.flags >> kFlagCachedShift) & 1) && (P.layer_flags[it.k_layer] & kLayerWritesQCache))
-            reinterpret_cast<uint4*>(P.qcache + ((static_cast<size_t>(it.k_layer) * P.max_seqs + it.seq_id) * P.hq + it.head) * D)[lane] =
-                c.qraw[0][lane];
+        for (int i = 0; i < 4; ++i) {
+          float s = p[x][i];
+          if (MODE != 2) {
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            s += __shfl_xor_sync(0xffffffffu, s, 4);
+          }
+          if (MODE == 1 && c8 == 0 && 4 * i + kg < nvalid) lg[pg * kPage + 4 * i + kg] = s;
+          p[x][i] = (4 * i + kg < nvalid) ? s : -INFINITY;
         }
-        fence_proxy_async();   // these generic-proxy writes precede the slot's next asynchronous refill
-        __syncwarp();
+        float tmax = fmaxf(fmaxf(p[x][0], p[x][1]), fmaxf(p[x][2], p[x][3]));
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
+        const float m_new = fmaxf(m[x], tmax);
+        const float corr = ex2_approx(m[x] - m_new);
+        float psum = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          p[x][i] = ex2_approx(p[x][i] - m_new);
+          psum += p[x][i];
+        }
+        l[x] = l[x] * corr + psum;
+        if (SKIP) {
+          float psum_skip = psum;
+          if (skip_here && pg == n_pages - 1) {
+            const int r_new = nvalid - 1;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (4 * i + kg == r_new) psum_skip -= p[x][i];
+          }
+          l_skip = l_skip * corr + psum_skip;
+        }
+        m[x] = m_new;
+        if (corr != 1.f) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            if (NQ == 1 || v == x) {
+#pragma unroll
+              for (int e = 0; e < EP2; ++e) acc[v][e] = mul2(acc[v][e], make_float2(corr, corr));
+            }
+          }
+        }
       }
+    };
+    auto score = [&](uint32_t tile) {   // K tile: scores of 16 keys
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         float2 kf[EP2];
@@ -515,92 +537,92 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
           p[x][i] = (a0.x + a1.x) + (a0.y + a1.y);
         }
       }
-      release_tile<kRing>(st);
-      fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
-    }
-#pragma unroll
-    for (int x = 0; x < NQ; ++x) {
+    };
+    auto add = [&](uint32_t tile, int v) {   // V tile: weighted sum for consumer v (a constant after unrolling)
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        float s = p[x][i];
-        if (MODE != 2) {
-          s += __shfl_xor_sync(0xffffffffu, s, 1);
-          s += __shfl_xor_sync(0xffffffffu, s, 2);
-          s += __shfl_xor_sync(0xffffffffu, s, 4);
-        }
-        if (MODE == 1 && c8 == 0 && 4 * i + kg < nvalid) lg[pg * kPage + 4 * i + kg] = s;
-        p[x][i] = (4 * i + kg < nvalid) ? s : -INFINITY;
-      }
-      float tmax = fmaxf(fmaxf(p[x][0], p[x][1]), fmaxf(p[x][2], p[x][3]));
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-      const float m_new = fmaxf(m[x], tmax);
-      const float corr = ex2_approx(m[x] - m_new);
-      float psum = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        p[x][i] = ex2_approx(p[x][i] - m_new);
-        psum += p[x][i];
-      }
-      l[x] = l[x] * corr + psum;
-      if (SKIP) {
-        float psum_skip = psum;
-        if (skip_here && pg == n_pages - 1) {
-          const int r_new = nvalid - 1;
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (4 * i + kg == r_new) psum_skip -= p[x][i];
-        }
-        l_skip = l_skip * corr + psum_skip;
-      }
-      m[x] = m_new;
-      if (corr != 1.f) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          if (NQ == 1 || v == x) {
-#pragma unroll
-            for (int e = 0; e < EP2; ++e) acc[v][e] = mul2(acc[v][e], make_float2(corr, corr));
-          }
-        }
-      }
-    }
-    // ---- V tiles: weighted sums for each consumer
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
-      if (st.dead) break;
-      const int nvalid_v = (SKIP && skip_here && pg == n_pages - 1) ? nvalid - static_cast<int>((skip_mask >> v) & 1u) : nvalid;
-      if (kMayFold && pg == new_pg && nvalid_v == nvalid) {
-        // this consumer's new v row, likewise
-        const Item& it = c.ip.item;
-        if (lane < D / 8) {
-          const uint4 val = v == first_taker(it)
-                                ? c.ip.new_v[lane]
-                                : reinterpret_cast<const uint4*>(
-                                      P.v + ((static_cast<size_t>(it.v_layer[v]) * P.n_seqs + it.seq_idx) * P.hkv + c.ip.kv_head) * D)[lane];
-          sts128(tile + (nvalid - 1) * (D * 2) + lane * 16, val);
-          const int pid = c.ip.pages[1 + v][pg];
-          if (static_cast<uint32_t>(pid) < static_cast<uint64_t>(P.n_pool_pages))
-            reinterpret_cast<uint4*>(P.pool + ((static_cast<size_t>(pid) * P.hkv + c.ip.kv_head) * kPage + (nvalid - 1)) * D)[lane] = val;
-        }
-        fence_proxy_async();
-        __syncwarp();
-      }
-      auto add_row = [&](int i) {
         float2 vf[EP2];
 #pragma unroll
         for (int j = 0; j < LPR; ++j) bf16x8_to_f32x2(lds128(tile + lane_off + i * (4 * D * 2) + j * 128), &vf[4 * j]);
         const float pv = p[NQ == 1 ? 0 : v][i];
 #pragma unroll
         for (int e = 0; e < EP2; ++e) acc[v][e] = fma2(vf[e], make_float2(pv, pv), acc[v][e]);
-      };
-      if (nvalid_v == kPage) {
+      }
+    };
+    auto clear_tail = [&](uint32_t tile, int n) {
+      // rows past the end hold whatever the pool held (a zero weight does not cancel a NaN): cleared
+      for (int r = n * (D / 8) + lane; r < kPage * (D / 8); r += 32) sts128(tile + r * 16, make_uint4(0u, 0u, 0u, 0u));
+      fence_proxy_async();   // these generic-proxy writes precede the slot's next asynchronous refill
+      __syncwarp();
+    };
+    if constexpr (NQ > 1) {
+      uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
+      if (st.dead) break;
+      score(tile);
+      release_tile<kRing>(st);
+      fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
+      weigh();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) add_row(i);
-      } else {   // (rows past the end hold whatever the pool held: a zero weight does not cancel a NaN)
+      for (int v = 0; v < NV; ++v) {
+        tile = wait_tile<D>(st, ring, full, P, lane);
+        if (st.dead) break;
+        if (nvalid < kPage) clear_tail(tile, nvalid);
+        add(tile, v);
+        release_tile<kRing>(st);
+        fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
+      }
+      continue;
+    }
+    if (MODE == 2) {
+      // ---- scores of 16 keys from the logit cache; the next page's are requested now
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (4 * i + kg < nvalid_v) add_row(i);
+      for (int i = 0; i < 4; ++i) p[0][i] = lg_next[i];
+      if (pg + 1 < n_pages) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) lg_next[i] = lg[(pg + 1) * kPage + 4 * i + kg];
+      }
+    }
+    // The page's tiles, K (t = 0) and then one V tile per consumer, in one loop: what they have in
+    // common -- wait, new token, release, refill -- stands in the code once.  Workers that go from a
+    // row's visual to its text stream go from one copy of this loop to another, and an SM's twelve
+    // are all somewhere else, so with short rows the size of the code is what a launch waits for.
+    // Unrolled, with a loop of its own for pages that are not full -> this, us per layer, 30 sequences of 260
+    // tokens and 16 heads: 20.0 -> 19.3; GLA in blocks of four 19.8 -> 16.4; 8 of 2 000 tokens in GLA 38.4 -> 35.2.
+#pragma unroll 1
+    for (int t = MODE == 2 ? 1 : 0; t <= NV; ++t) {
+      if (t == 1) weigh();
+      const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
+      if (st.dead) break;
+      const int skips = (SKIP && t > 0 && skip_here && pg == n_pages - 1) ? static_cast<int>((skip_mask >> (t - 1)) & 1u) : 0;
+      if (kMayFold && pg == new_pg && !skips) {
+        // the new token's row comes from the step's input: into the tile, and into the pool for later steps
+        const Item& it = c.ip.item;
+        if (lane < D / 8) {
+          const uint4 val = t == 0 ? c.ip.new_k[lane]
+                            : t - 1 == first_taker(it)
+                                ? c.ip.new_v[lane]
+                                : reinterpret_cast<const uint4*>(
+                                      P.v + ((static_cast<size_t>(it.v_layer[t - 1]) * P.n_seqs + it.seq_idx) * P.hkv + c.ip.kv_head) * D)[lane];
+          sts128(tile + (nvalid - 1) * (D * 2) + lane * 16, val);
+          const int pid = c.ip.pages[t][pg];
+          if (static_cast<uint32_t>(pid) < static_cast<uint64_t>(P.n_pool_pages))
+            reinterpret_cast<uint4*>(P.pool + ((static_cast<size_t>(pid) * P.hkv + c.ip.kv_head) * kPage + (nvalid - 1)) * D)[lane] = val;
+          // an ordinary layer's query goes to the Q Cache
+          if (t == 0 && it.q_layer[0] == it.k_layer && !((it.flags >> kFlagCachedShift) & 1) &&
+              (P.layer_flags[it.k_layer] & kLayerWritesQCache))
+            reinterpret_cast<uint4*>(P.qcache + ((static_cast<size_t>(it.k_layer) * P.max_seqs + it.seq_id) * P.hq + it.head) * D)[lane] =
+                c.qraw[0][lane];
+        }
+        fence_proxy_async();   // these generic-proxy writes precede the slot's next asynchronous refill
+        __syncwarp();
+      }
+      if (t == 0) {
+        score(tile);
+      } else {
+        if (nvalid - skips < kPage) clear_tail(tile, nvalid - skips);
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          if (t == v + 1) add(tile, v);
       }
       release_tile<kRing>(st);
       fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
@@ -652,20 +674,23 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
 // ring already fetches tiles of item k + 1 and the context of item k + 2 (descriptor, page ids,
 // queries) arrives by asynchronous copies.
 // False if a wait ran out.
-template <int D, bool STATIC>
+// OWN: launches with sweeps that score with a query per consumer.  Those sweeps hold up to four queries and
+// four accumulators; in a kernel of their own they do not cost the others registers (with both in one, items in local
+// memory and all of the L1 given to tiles -> now, us per layer: batch 1 10.5 -> 9.7, batch 16 32.7 -> 31.6, 30 short
+// sequences 19.3 -> 17.9; own-query sweeps of four, 12 sequences of 800 keys, 28.4 -> 25.0).
+template <int D, bool STATIC, bool OWN>
 __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, uint32_t ring, uint64_t* full,
                                               RangeCursor* cursor, int32_t* stage, CtaDesc* cta, int wid, int lane) {
   auto ctx_of = [ctx](int k) -> const ItemPages& { return ctx[k % kCtxSlots].ip; };
   WorkerState st;
   worker_init(st, 0);
   st.drop_next = P.debug_drop_tile != 0;   // (test hook)
-  Item it;
   int issued = 0;
-  auto take = [&]() -> bool {   // the next item into `it`
-    if (STATIC) return cursor_step(cursor, P, it, lane);
+  auto take = [&](ItemPages& slot) -> bool {   // the next item into a context slot
+    if (STATIC) return cursor_step(cursor, P, slot, lane);
     const int idx = claim_take(P, issued);
     if (idx < 0) return false;
-    it = load_item(P, idx);
+    load_item(slot, P, idx, lane);
     return true;
   };
   // ---- ahead of the wait for the previous kernel: the first two items and their page ids (from the
@@ -673,23 +698,20 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
   // started), and the first tiles unless they could hold a new token that an earlier launch of the
   // step stores (with the folded append the worker patches the new token's row itself).  After it,
   // only the layer's inputs.
-  Item first;
   bool more;
   if (STATIC) {
     bool any = wid >= 0 && wid < P.part_workers;
     if (P.wdesc != nullptr) {
       // planned ahead: one read gives the first two items, the first page ids and the cursor
       any = any && load_worker_desc(P, wid, ctx[0].ip, ctx[1].ip, cursor, stage, cta, lane);
-      if (any) first = ctx[0].ip.item;
     } else {
       RangeCursor c;
       any = any && cursor_init(c, part_view(P), wid);
       if (lane == 0) *cursor = c;
       __syncwarp();
-      any = any && take();
+      any = any && take(ctx[0].ip);
       if (any) {
-        first = it;
-        begin_item_pages(ctx[0].ip, P, first, lane);
+        begin_item_pages(ctx[0].ip, P, lane);
         cp_async_wait_all();
         __syncwarp();
       }
@@ -699,41 +721,40 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
       return true;
     }
     st.n_my = 1;
+    const Item& first = ctx[0].ip.item;
     const bool early_tiles = P.fold_append || !(first.stream == 0 && (first.flags & kFlagStreamEnd) && first.n_pages <= kRing);
     if (early_tiles) fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
     if (P.wdesc != nullptr) {
-      if (first.n_pages > 2) begin_item_pages(ctx[0].ip, P, first, lane);   // the whole page list, while the tiles fly
-      it = ctx[1].ip.item;
-      more = it.n_pages > 0;
+      if (first.n_pages > 2) begin_item_pages(ctx[0].ip, P, lane);   // the whole page list, while the tiles fly
+      more = ctx[1].ip.item.n_pages > 0;
     } else {
-      more = take();
+      more = take(ctx[1].ip);
     }
-    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    if (more) begin_item_pages(ctx[1].ip, P, lane);
     pdl_wait();
     pdl_launch_dependents();
   } else {
     pdl_wait();   // the item list and the work counter are the previous kernel's
     pdl_launch_dependents();
     issued = claim_issue(P, lane);
-    if (!take()) return true;
-    first = it;
-    begin_item_pages(ctx[0].ip, P, first, lane);
+    if (!take(ctx[0].ip)) return true;
+    begin_item_pages(ctx[0].ip, P, lane);
     cp_async_wait_all();
     __syncwarp();
     st.n_my = 1;
     fill_ring<D, kRing, false>(st, ctx_of, ring, full, P, lane);
     issued = claim_issue(P, lane);
   }
-  begin_queries<D>(ctx[0], P, first, lane);
-  begin_new_rows(ctx[0].ip, P, first, lane, D);
+  begin_queries<D>(ctx[0], P, lane);
+  begin_new_rows(ctx[0].ip, P, lane, D);
   if (!STATIC) {
-    more = take();
-    if (more) begin_item_pages(ctx[1].ip, P, it, lane);
+    more = take(ctx[1].ip);
+    if (more) begin_item_pages(ctx[1].ip, P, lane);
   }
   cp_async_commit_group();
   if (more) {
-    begin_queries<D>(ctx[1], P, it, lane);
-    begin_new_rows(ctx[1].ip, P, it, lane, D);
+    begin_queries<D>(ctx[1], P, lane);
+    begin_new_rows(ctx[1].ip, P, lane, D);
   }
   cp_async_commit_group();   // the second item's inputs are waited for when the first item is done
   if (STATIC) cp_async_wait_group<1>();
@@ -747,21 +768,25 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
   for (int k = 0; k < st.n_my && !st.dead; ++k) {
     const Item& cur = ctx[k % kCtxSlots].ip.item;
     const int nc = cur.n_cons;
-    const bool shared = cur.flags & kFlagShared;
     if (more) {
       // the third slot is free (it held the item before this one): start filling it with the item after next
-      more = take();
+      WarpCtx<D>& next = ctx[(k + 2) % kCtxSlots];
+      more = take(next.ip);
       if (more) {
-        begin_item_pages(ctx[(k + 2) % kCtxSlots].ip, P, it, lane);
-        begin_queries<D>(ctx[(k + 2) % kCtxSlots], P, it, lane);
-        begin_new_rows(ctx[(k + 2) % kCtxSlots].ip, P, it, lane, D);
+        begin_item_pages(next.ip, P, lane);
+        begin_queries<D>(next, P, lane);
+        begin_new_rows(next.ip, P, lane, D);
         pending = true;
       }
     }
-    if (!STATIC && more) issued = claim_issue(P, lane);   // answered by the time the next item starts
-    if (nc == 1 && (cur.flags & kFlagReadLogits)) process_item<D, 1, 1, 2>(st, ctx, ring, full, P, lane);
+    if constexpr (OWN) {
+      if (nc == 1) process_item<D, 1, 1>(st, ctx, ring, full, P, lane);
+      else if (nc == 2) process_item<D, 2, 2>(st, ctx, ring, full, P, lane);
+      else if (nc == 3) process_item<D, 3, 3>(st, ctx, ring, full, P, lane);
+      else process_item<D, 4, 4>(st, ctx, ring, full, P, lane);
+    } else if (nc == 1 && (cur.flags & kFlagReadLogits)) process_item<D, 1, 1, 2>(st, ctx, ring, full, P, lane);
     else if (nc == 1 && (cur.flags & kFlagWriteLogits)) process_item<D, 1, 1, 1>(st, ctx, ring, full, P, lane);
-    else if (shared && cur.skip_new) {
+    else if (P.any_skip) {   // (one copy of the loop per launch here too: GLA leaders of short rows 16.4 -> 14.8 us a layer)
       if (nc == 1) process_item<D, 1, 1, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 2) process_item<D, 1, 2, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 3) process_item<D, 1, 3, 0, true>(st, ctx, ring, full, P, lane);
@@ -769,13 +794,11 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
     }
     else if (nc == 1 && P.fold_append) process_item<D, 1, 1, 0, false, true>(st, ctx, ring, full, P, lane);   // (one code path per launch)
     else if (nc == 1) process_item<D, 1, 1>(st, ctx, ring, full, P, lane);
-    else if (shared && nc == 2) process_item<D, 1, 2>(st, ctx, ring, full, P, lane);
-    else if (shared && nc == 3) process_item<D, 1, 3>(st, ctx, ring, full, P, lane);
-    else if (shared) process_item<D, 1, 4>(st, ctx, ring, full, P, lane);
-    else if (nc == 2) process_item<D, 2, 2>(st, ctx, ring, full, P, lane);
-    else if (nc == 3) process_item<D, 3, 3>(st, ctx, ring, full, P, lane);
-    else process_item<D, 4, 4>(st, ctx, ring, full, P, lane);
+    else if (nc == 2) process_item<D, 1, 2>(st, ctx, ring, full, P, lane);
+    else if (nc == 3) process_item<D, 1, 3>(st, ctx, ring, full, P, lane);
+    else process_item<D, 1, 4>(st, ctx, ring, full, P, lane);
     if (st.dead) break;
+    if (!STATIC && more) issued = claim_issue(P, lane);   // (not held across the page loops, which need the registers)
     if (STATIC) record_row_slots(P, cur, lane);
     if (k + 1 < st.n_my) {   // the contexts of items k + 1 and k + 2 have had this item's time to arrive
       cp_async_wait_all();
@@ -793,7 +816,7 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
   return !st.dead;
 }
 
-template <int D, bool STATIC>
+template <int D, bool STATIC, bool OWN>
 __global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_kernel(const __grid_constant__ Params P) {
   constexpr uint32_t kTile = kPage * D * 2;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -815,7 +838,7 @@ __global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_kernel(cons
   if (threadIdx.x == 0) finish.dead = 0;
   __syncthreads();
 
-  const bool ok = attend_worker<D, STATIC>(P, ctx, ring, full, &cursors[warp], stages[warp], &cta, worker_index(P, warp), lane);
+  const bool ok = attend_worker<D, STATIC, OWN>(P, ctx, ring, full, &cursors[warp], stages[warp], &cta, worker_index(P, warp), lane);
   if (STATIC) finish_cta<D>(P, finish, cta, !ok, warp, lane);
 }
 
@@ -850,19 +873,28 @@ constexpr int attend_smem_bytes() {
 // ------------------------------------------------------------------------------------------
 
 namespace {
+// Shared memory for as many blocks as an SM holds of the kernel, and no more: the rest is L1 cache.
 template <typename K>
 cudaError_t configure_attend(K kernel, int smem) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  cudaFuncAttributes a;
+  e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  const int need = kAttendCtasPerSm * (smem + static_cast<int>(a.sharedSizeBytes) + 1024), all = 228 * 1024;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, min(100, (100 * need + all - 1) / all));
 }
 }  // namespace
 
 cudaError_t configure_kernels(int* attend_smem) {
-  cudaError_t e = configure_attend(attend_kernel<128, false>, attend_smem_bytes<128>());
-  if (e == cudaSuccess) e = configure_attend(attend_kernel<128, true>, attend_smem_bytes<128>());
-  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, false>, attend_smem_bytes<64>());
-  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, true>, attend_smem_bytes<64>());
+  cudaError_t e = configure_attend(attend_kernel<128, false, false>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<128, false, true>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<128, true, false>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<128, true, true>, attend_smem_bytes<128>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, false, false>, attend_smem_bytes<64>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, false, true>, attend_smem_bytes<64>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, true, false>, attend_smem_bytes<64>());
+  if (e == cudaSuccess) e = configure_attend(attend_kernel<64, true, true>, attend_smem_bytes<64>());
   if (attend_smem) *attend_smem = attend_smem_bytes<128>();
   return e;
 }
@@ -900,14 +932,15 @@ cudaError_t launch_attend(const Params& p, int n_sms, cudaStream_t stream) {
   if (!p.part_static && n_items <= 0) return cudaSuccess;
   const int grid = p.part_static ? (p.part_workers + p.part_wpc - 1) / p.part_wpc
                                  : min(n_sms * kAttendCtasPerSm, (n_items + kWarps - 1) / kWarps);
+  auto launch = [&](auto kernel, int smem) { return launch_pdl(kernel, dim3(grid), dim3(kThreads), smem, stream, p); };
   if (p.d == 128) {
-    if (p.part_static)
-      return launch_pdl(attend_kernel<128, true>, dim3(grid), dim3(kThreads), attend_smem_bytes<128>(), stream, p);
-    return launch_pdl(attend_kernel<128, false>, dim3(grid), dim3(kThreads), attend_smem_bytes<128>(), stream, p);
+    const int smem = attend_smem_bytes<128>();
+    if (p.part_static) return p.any_own ? launch(attend_kernel<128, true, true>, smem) : launch(attend_kernel<128, true, false>, smem);
+    return p.any_own ? launch(attend_kernel<128, false, true>, smem) : launch(attend_kernel<128, false, false>, smem);
   }
-  if (p.part_static)
-    return launch_pdl(attend_kernel<64, true>, dim3(grid), dim3(kThreads), attend_smem_bytes<64>(), stream, p);
-  return launch_pdl(attend_kernel<64, false>, dim3(grid), dim3(kThreads), attend_smem_bytes<64>(), stream, p);
+  const int smem = attend_smem_bytes<64>();
+  if (p.part_static) return p.any_own ? launch(attend_kernel<64, true, true>, smem) : launch(attend_kernel<64, true, false>, smem);
+  return p.any_own ? launch(attend_kernel<64, false, true>, smem) : launch(attend_kernel<64, false, false>, smem);
 }
 
 cudaError_t launch_merge(const Params& p, cudaStream_t stream) {

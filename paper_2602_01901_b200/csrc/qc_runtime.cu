@@ -1247,6 +1247,12 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     p.part_wv = one.part_wv;
     p.part_wt = one.part_wt;
   }
+  p.any_skip = p.any_own = 0;
+  for (int pos = pb; pos < pe; ++pos) {
+    const Job& job = c->plan[pos].job;
+    p.any_skip |= job.skip_new ? 1 : 0;
+    p.any_own |= job.n_cons > 1 && !(job.flags & kFlagShared) ? 1 : 0;
+  }
   p.fused_merge = use_static ? launches.launch[gi].fused_merge : 0;
   p.planned_pieces = use_static && launches.launch[gi].layer >= 0 ? 1 : 0;
   if (wait_in) QC_CUDA(cudaStreamWaitEvent(stream, wait_in, 0));

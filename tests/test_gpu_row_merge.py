@@ -134,3 +134,33 @@ def test_a_key_that_is_not_a_number_reaches_every_row_it_belongs_to(q_heads, kv_
     assert torch.equal(torch.isnan(out).all(-1), hit) and torch.equal(torch.isnan(out).any(-1), hit)
     assert s.stats().device_error == 0
     s.close()
+
+
+def test_a_shared_sweep_of_short_rows_is_not_slower_than_sweeps_of_its_own():
+    """Many short sequences: what an item costs beyond its pages decides.  A GLA block moves fewer bytes than
+    the same layers in VLA and has fewer sweeps; its leader's launch once took so much longer per item (its
+    items alternated between two copies of the page loop) that the step was no faster."""
+    n, b, heads, d, text, vis, steps = 10, 30, 16, 128, 110, 150, 8
+    layer_kind = [1 if l >= 2 and (l - 2) % 4 else 0 for l in range(n)]
+    best = {}
+    for mode in (qc.QC_MODE_GLA, qc.QC_MODE_VLA_QC):
+        s = Session(n, heads, heads, d, layer_kind, max_seqs=b, max_tokens_per_seq=vis + 100, n_pages=2 * n * b * 25, lazy_mode=mode)
+        s.set_option("in_order_launches", 1)
+        kind = np.tile(np.array([0] * text + [1] * vis, np.uint8), b)
+        k, v = (torch.randn(n, len(kind), heads, d, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+        s.prefill_append(list(range(b)), [text + vis] * b, kind, k, v)
+        q, kn, vn = (torch.randn(n, b, heads, d, device=s.device, dtype=torch.bfloat16) for _ in range(3))
+        out = torch.empty_like(q)
+        times = []
+        for _ in range(6):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda.synchronize()
+            e[0].record()
+            for _ in range(steps):
+                s.decode_step(list(range(b)), q, kn, vn, out)
+            e[1].record()
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        best[mode] = min(times)
+        s.close()
+    assert best[qc.QC_MODE_GLA] < 0.9 * best[qc.QC_MODE_VLA_QC], best
