@@ -300,8 +300,8 @@ int32_t qc_debug_read_row(qc_cache* cache, int32_t layer, int32_t stream, int32_
  * "static_row_cost" (tuning of those ranges: shortest range, and what one more output row counts
  * for, in 4 KiB tiles), "plan_ahead" (0 = workers locate their ranges themselves instead of reading
  * starting points that one kernel per step works out for every launch), "fused_merge" (1, the default = an
- * attention launch of one layer without query groups merges its output rows itself; 0 = by a merge
- * launch),
+ * attention launch of one layer without query groups merges its output rows itself where the step's launches
+ * are planned ahead and n_seqs * n_q_heads is at most four per SM; 0 = always by a merge launch),
  * "fold_append" (in-order schedule and qc_decode_layer; 1, the default = a layer's new k/v rows and an
  * ordinary layer's q are taken from the inputs and stored by that layer's own launch; 0 = by an
  * append when the step begins, resp. an append launch per layer call),

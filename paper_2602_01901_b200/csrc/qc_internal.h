@@ -40,12 +40,11 @@ struct Job {
 static_assert(sizeof(Job) == 16, "Job layout");
 
 // One position of the launch plan: a job plus how many visual-stream and text-stream jobs
-// precede it in the item list (all launches of a step share one list), and the tiles per page
-// (one K tile unless the scores come from the logit cache, one V tile per consumer) of the
-// visual-stream and text-stream jobs that precede it in its own launch.  Static per cache.
+// precede it in the item list (all launches of a step share one list).  Static per cache.
 struct __align__(16) PlanJob {
   Job job;
-  int32_t vis_before, text_before, wv_before, wt_before;
+  int32_t vis_before, text_before;
+  int32_t pad[2];
 };
 static_assert(sizeof(PlanJob) == 32, "PlanJob layout");
 

@@ -660,7 +660,7 @@ int rebuild_plan(qc_cache* c, int per_launch) {
     g.w_min = 1 << 20;
     for (int j : order) {
       const int vb = c->plan_vis_before.back(), tb = c->plan_text_before.back();
-      c->plan.push_back(PlanJob{jobs[j], vb, tb, g.wv, g.wt});
+      c->plan.push_back(PlanJob{jobs[j], vb, tb, {0, 0}});
       c->plan_vis_before.push_back(vb + (jobs[j].stream ? 1 : 0));
       c->plan_text_before.push_back(tb + (jobs[j].stream ? 0 : 1));
       const int w = tiles_per_page(jobs[j]);
@@ -1500,7 +1500,7 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
                                               static_cast<int64_t>(pmax_t) * g.w_max_t);
     const int64_t q_max = 30LL * w_lo;
     // at least a page of the heaviest job, with query groups two (each of a row's pieces then is seven or
-    // eight partial rows to merge: batch 1, 160 launches: one page 2.93 ms, two 2.45; batch 8 2.36 / 2.12)
+    // eight partial rows to merge: batch 1, 160 launches: one page 2.93 ms, two 2.45; batch 8 2.36 / 2.06)
     int64_t q_min = std::max<int64_t>(c->group > 1 ? 2 * g.w_max : g.w_max,
                                       (row_max + c->slots_per_stream - 3) / (c->slots_per_stream - 2));
     q_min = std::max<int64_t>(q_min, std::min<int64_t>(c->static_min_tiles, q_max / 2));
@@ -1523,9 +1523,9 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     L.part_wv = g.wv;
     L.part_wt = g.wt;
     // Who merges the rows of a launch of one layer.  With one query head per row and at most two rows per
-    // CTA the launch itself: 8 layers, 20 steps, merge launch -> own merge: 64 rows of 3 000 keys 3.97 ->
-    // 3.61 ms, 224 of 800 3.46 -> 3.40, 512 of 576 5.77 -> 5.81, 1 024 of 120 5.12 -> 5.21 (and 1 024 launches
-    // at batch 1 11.87 -> 10.28).  With query groups, whose every partial is seven or eight rows, a merge
+    // CTA (592) the launch itself: 8 layers, time with its own merge over time with a merge launch, rows of 140 / 280 /
+    // 600 / 1 200 keys: 64 rows 1.04 / 0.94 / 0.89 / 0.87, 224 rows 0.99 / 0.97 / 0.96 / 0.97, 480 rows 0.99 / 0.98 / 0.99 / 1.00,
+    // 576 rows 0.99 / 0.99 / 0.99 / 1.00.  With query groups, whose every partial is seven or eight rows, a merge
     // launch over the whole chip (896 launches at batch 32: 19.1, the other way 20.4).
     if (L.layer >= 0 && c->fused_merge && c->group == 1 && static_cast<int64_t>(n_seqs) * c->hq <= 2LL * n_ctas)
       L.fused_merge = (L.part_workers + L.part_wpc - 1) / L.part_wpc <= kPlanCtas;

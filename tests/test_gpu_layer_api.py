@@ -33,6 +33,16 @@ def _dev(a, device):
 @pytest.mark.parametrize("mode", MODES, ids=["vla_qc", "vla_eq8", "gla"])
 @pytest.mark.parametrize("shape", range(len(SHAPES)))
 def test_layer_by_layer_step_matches_the_oracle_and_the_step_call(mode, shape):
+    _layer_by_layer(mode, shape, {})
+
+
+@pytest.mark.parametrize("mode", MODES, ids=["vla_qc", "vla_eq8", "gla"])
+@pytest.mark.parametrize("shape", [0, 1])
+def test_layer_calls_whose_workers_find_their_own_start(mode, shape):
+    _layer_by_layer(mode, shape, {"plan_ahead": 0})
+
+
+def _layer_by_layer(mode, shape, options):
     head_dim, group, layer_kind = SHAPES[shape]
     lazy = tuple(i for i, k in enumerate(layer_kind) if k)
     w = W.Workload(70 + shape, f"layer{shape}", len(layer_kind), 2 * group, 2, head_dim, 16, 3, 5, 150, 150, 22, 20, lazy)
@@ -41,6 +51,8 @@ def test_layer_by_layer_step_matches_the_oracle_and_the_step_call(mode, shape):
     sessions = [Session(w.n_layers, w.n_q_heads, w.n_kv_heads, head_dim, layer_kind, max_seqs=4, max_tokens_per_seq=256,
                         n_pages=w.n_layers * 4 * 3 * 17, lazy_mode=mode, poison_pool=True) for _ in range(2)]
     layered, whole = sessions
+    for key, value in options.items():
+        layered.set_option(key, value)
     for b, sid in enumerate(seq_ids):
         kind, k, v = W.prefill_kv_np(w, b)
         T = trunc[b]

@@ -257,8 +257,8 @@ SCHEDULES = {
     "in_order_short_ranges": [("in_order_launches", 1), ("static_min_tiles", 1), ("static_row_cost", 0)],
     "in_order_costly_rows": [("in_order_launches", 1), ("static_row_cost", 5)],
     "in_order_append_at_step_start": [("in_order_launches", 1), ("fold_append", 0)],
-    "in_order_merge_in_kernel": [("in_order_launches", 1), ("fused_merge", 1)],
-    "one_launch_merge_in_kernel": [("fused_merge", 1)],
+    "in_order_merge_launch": [("in_order_launches", 1), ("fused_merge", 0)],
+    "in_order_unplanned": [("in_order_launches", 1), ("plan_ahead", 0)],
 }
 
 
@@ -310,7 +310,15 @@ def test_schedules_against_the_oracle(mode, case, schedule):
             assert np.array_equal(s.read_row(l, qc.QC_STREAM_K_TEXT, sid, n_text - 1, 1), kn[owner, b, 1])
             if layer_kind[l]:
                 assert np.array_equal(s.read_qcache(l)[sid], qn[leaders[l], b])
-    assert s.stats().device_error == 0
+    st = s.stats()
+    assert st.device_error == 0
+    if schedule in ("in_order", "in_order_merge_launch", "in_order_unplanned"):
+        # who merges: query heads of planned launches their own launch (a GLA follower has none), else a launch of its own
+        planned = schedule != "in_order_unplanned"
+        merges = (st.kernel_launches - 3 - st.attend_launches) // w.decode_steps - (2 if planned else 1)   # 3 prompts; set-up, plan
+        own = schedule == "in_order" and group == 1
+        followers = sum(layer_kind) if mode == qc.QC_MODE_GLA else 0
+        assert merges == (followers if own else w.n_layers)
     s.close()
 
 
