@@ -38,7 +38,7 @@ MODES = {"vla_qc": 0, "vla_eq8": 1, "gla": 2}
 # 181-257 MB for the MHA kernel, 74-107 MB for the GQA kernel).  Every tile is fetched once and the
 # partial rows are written once per piece, so traffic grows in proportion to the K/V bytes swept and a
 # full-size launch's traffic is this ratio times its algorithmic bytes.
-NCU_TRAFFIC_RATIO = {"attend_kernel": 1.028, "attend_tc_kernel": 1.057}
+NCU_TRAFFIC_RATIO = {"attend_kernel": 1.022, "attend_tc_kernel": 1.047}
 
 
 def _peaks():
@@ -499,7 +499,7 @@ def run_gpu(args, rank, world, local_rank):
             "launches_per_step": head["attend_launches_per_step"], "frac_of_nominal_8TBs": head["frac_of_nominal_8TBs"],
             "whole_step_frac": head["whole_step_frac"],
             "note": "achieved = K/V bytes of the attention launches / their summed durations (events around every "
-                    "launch, second pass); whole_step_frac = the same bytes / the profiling-off step time",
+                    "launch, second pass; where query heads are not grouped a launch also merges its output rows); whole_step_frac = the same bytes / the profiling-off step time",
         },
         "e2e": head["e2e"], "gpu_launches": head["gpu_launches"], "clocks": head["clocks"],
         "kv_cache": head["kv_saved"], "one_launch": head["one_launch"],
