@@ -582,13 +582,13 @@ __device__ __forceinline__ void process_item(WorkerState& st, const WarpCtx<D>* 
         for (int i = 0; i < 4; ++i) lg_next[i] = lg[(pg + 1) * kPage + 4 * i + kg];
       }
     }
-    // The page's tiles, K (t = 0) and then one V tile per consumer, in one loop: what they have in
-    // common -- wait, new token, release, refill -- stands in the code once.  Workers that go from a
-    // row's visual to its text stream go from one copy of this loop to another, and an SM's twelve
-    // are all somewhere else, so with short rows the size of the code is what a launch waits for.
-    // Unrolled, with a loop of its own for pages that are not full -> this, us per layer, 30 sequences of 260
-    // tokens and 16 heads: 20.0 -> 19.3; GLA in blocks of four 19.8 -> 16.4; 8 of 2 000 tokens in GLA 38.4 -> 35.2.
-#pragma unroll 1
+    // The page's tiles, K (t = 0) and then one V tile per consumer.  Workers that go from a row's
+    // visual to its text stream go from one copy of this loop to another, and an SM's twelve are all
+    // somewhere else, so with short rows the size of the code is what a launch waits for: a page that
+    // is not full has no loop of its own (30 sequences of 260 tokens, 16 heads, 20.0 -> 19.4 us a layer).  Left
+    // rolled up the loop is smaller still, but its branches cost more: 17.9 against 17.6 us there, batch 16 31.1
+    // / 30.3, one-launch steps of 2 short sequences with 64-wide heads 2.21 / 2.05.
+#pragma unroll
     for (int t = MODE == 2 ? 1 : 0; t <= NV; ++t) {
       if (t == 1) weigh();
       const uint32_t tile = wait_tile<D>(st, ring, full, P, lane);
@@ -786,7 +786,7 @@ __device__ __forceinline__ bool attend_worker(const Params& P, WarpCtx<D>* ctx, 
       else process_item<D, 4, 4>(st, ctx, ring, full, P, lane);
     } else if (nc == 1 && (cur.flags & kFlagReadLogits)) process_item<D, 1, 1, 2>(st, ctx, ring, full, P, lane);
     else if (nc == 1 && (cur.flags & kFlagWriteLogits)) process_item<D, 1, 1, 1>(st, ctx, ring, full, P, lane);
-    else if (P.any_skip) {   // (one copy of the loop per launch here too: GLA leaders of short rows 16.4 -> 14.8 us a layer)
+    else if (P.any_skip) {   // (one copy of the loop per launch here too: GLA blocks of short rows 16.4 -> 14.8 us a layer)
       if (nc == 1) process_item<D, 1, 1, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 2) process_item<D, 1, 2, 0, true>(st, ctx, ring, full, P, lane);
       else if (nc == 3) process_item<D, 1, 3, 0, true>(st, ctx, ring, full, P, lane);
