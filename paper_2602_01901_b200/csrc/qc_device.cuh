@@ -863,6 +863,7 @@ __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, in
     const uint32_t both = __ldcg(P.row_pieces + (static_cast<size_t>(P.launch_index) * P.max_seqs + si) * rows + u);
     nv = both & 0xffffu, nt = both >> 16, text0 = P.slots_per_stream;
   }
+  if (P.row_cluster > 0) nv = 1, nt = 0;
   const int pos = sq.len_text - 1;
   int pid = 0, pid_v = -1;
   if (extra_leader >= 0) {
@@ -875,7 +876,7 @@ __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, in
   }
   pdl_wait();
   pdl_launch_dependents();
-  if (P.part_static && !P.planned_pieces) {
+  if (P.part_static && !P.planned_pieces && P.row_cluster == 0) {
     const size_t row = (static_cast<size_t>(layer) * P.max_seqs + si) * P.hq + head;
     const uint32_t both = __ldcg(reinterpret_cast<const uint32_t*>(P.row_slots + 2 * row));
     nv = sq.len_vis > 0 ? static_cast<int>(both & 0xffffu) : 0;

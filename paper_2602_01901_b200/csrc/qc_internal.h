@@ -199,6 +199,8 @@ struct Params {
                                      // them: no append launch, nothing of a layer is touched before its own launch
   int32_t debug_drop_tile;           // test hook: every worker of an attention launch leaves out the copy of its first
                                      // tile and waits for it with a short limit (nothing in flight, nothing faults)
+  int32_t row_cluster;               // > 0: the step's launches give every output row a cluster of that many CTAs, and what a
+                                     // leader's launch leaves for a follower is one partial row (slot 0)
   int32_t extra_key_leader;          // merge only, >= 0: the rows also take the step's new token as one more key,
                                      // scored by that layer's Q Cache entry and new k (Eq. 6), valued by the own new v
 };
@@ -210,6 +212,16 @@ cudaError_t launch_plan(const Params& p, const LaunchList& list, int n_launches,
 cudaError_t launch_attend(const Params& p, int n_sms, cudaStream_t stream);      // one query head per item
 cudaError_t launch_attend_tc(const Params& p, int n_sms, cudaStream_t stream);   // query-group items (GQA)
 cudaError_t launch_merge(const Params& p, cudaStream_t stream);
+// A layer's sweeps where every output row has a cluster (in-order schedule, qc_rows.cu): at most one over the visual
+// stream, for the layer and the followers that share its scores, and one over the text stream, all with the layer's query.
+struct RowJobs {
+  Job vis, text;
+  int32_t has_vis, has_text;
+  int32_t add_earlier;   // the rows also take what the leader's launch left for the layer
+  int32_t pad;
+};
+cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int cluster, cudaStream_t stream);
+cudaError_t configure_rows_kernels();
 // Up to 16 consecutive tokens of one sequence and stream that go to one page.
 struct __align__(16) StoreSeg {
   int32_t seq, ord;   // sequence; first token's ordinal in its stream, the stream in the top bit

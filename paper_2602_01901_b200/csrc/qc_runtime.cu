@@ -125,6 +125,9 @@ struct qc_cache {
   std::vector<Job> inorder_jobs;                  // in-order schedule (a leader's launch also sweeps its followers' cached V)
   std::vector<std::pair<int, int>> inorder_job_range;
   std::vector<int> inorder_extra_key;             // per layer: the leader whose new token the merge adds, or -1
+  std::vector<RowJobs> row_jobs;                  // per layer, for launches that give every output row a cluster
+  bool rows_fit = false;                          // every layer's sweeps have that form
+  int row_cluster = -1;                           // CTAs per output row: -1 chosen per step, 0 never, n always n
   int slots_per_stream = 0;
   int static_partition = -1;      // -1: static ranges when a step is several launches; 0 never; 1 always
   bool fused_merge = true;        // small launches of one layer merge their output rows themselves (no merge launch)
@@ -380,6 +383,23 @@ void build_inorder_jobs(const qc_config* cfg, std::vector<Job>& jobs, std::vecto
       layer_jobs.emplace_back(job0, static_cast<int>(jobs.size()));
     }
     l = e;
+  }
+}
+
+// The in-order schedule's jobs as launches that give every output row a cluster take them.
+void build_row_jobs(qc_cache* c) {
+  c->row_jobs.assign(c->cfg.n_layers, RowJobs{});
+  c->rows_fit = true;
+  for (int l = 0; l < c->cfg.n_layers; ++l) {
+    RowJobs& r = c->row_jobs[l];
+    for (int j = c->inorder_job_range[l].first; j < c->inorder_job_range[l].second; ++j) {
+      const Job& job = c->inorder_jobs[j];
+      int32_t& has = job.stream ? r.has_vis : r.has_text;
+      c->rows_fit = c->rows_fit && !has && job.v_layer[0] == l && job.q_layer[0] == l;   // (a block of more than kMaxCons layers: two sweeps)
+      has = 1;
+      (job.stream ? r.vis : r.text) = job;
+    }
+    r.add_earlier = r.has_text && !r.has_vis;
   }
 }
 
@@ -722,6 +742,7 @@ int32_t qc_init(int32_t device, void* cuda_stream, qc_ctx** out) {
   int smem = 0, smem_tc = 0;
   QC_CUDA(configure_kernels(&smem));
   QC_CUDA(configure_kernels_tc(&smem_tc));
+  QC_CUDA(configure_rows_kernels());
   QC_CUDA(configure_prefill_kernels());
   if (static_cast<size_t>(std::max(smem, smem_tc)) > prop.sharedMemPerBlockOptin) return QC_ERR_UNSUPPORTED;
   qc_ctx* ctx = new (std::nothrow) qc_ctx();
@@ -800,6 +821,7 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   build_jobs(&c->cfg, c->jobs, c->block_jobs, c->block_layers);
   build_layer_jobs(&c->cfg, c->layer_jobs, c->layer_job_range);
   build_inorder_jobs(&c->cfg, c->inorder_jobs, c->inorder_job_range, c->inorder_extra_key);
+  build_row_jobs(c);
   if (c->cfg.lazy_mode == QC_MODE_GLA) {
     // Eq. 5: every layer of a lazy block attends with the block's first layer's Q and K, so runs
     // of up to three of its layers share one score pass of the prefill kernel
@@ -1247,14 +1269,17 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     p.part_wv = one.part_wv;
     p.part_wt = one.part_wt;
   }
+  const bool by_rows = p.row_cluster > 0;
+  const RowJobs* row_jobs = by_rows ? &c->row_jobs[p.layer_begin] : nullptr;
+  if (by_rows) has_work = row_jobs->has_vis || row_jobs->has_text;
   p.any_skip = p.any_own = 0;
   for (int pos = pb; pos < pe; ++pos) {
     const Job& job = c->plan[pos].job;
     p.any_skip |= job.skip_new ? 1 : 0;
     p.any_own |= job.n_cons > 1 && !(job.flags & kFlagShared) ? 1 : 0;
   }
-  p.fused_merge = use_static ? launches.launch[gi].fused_merge : 0;
-  p.planned_pieces = use_static && launches.launch[gi].layer >= 0 ? 1 : 0;
+  p.fused_merge = by_rows ? has_work : use_static ? launches.launch[gi].fused_merge : 0;
+  p.planned_pieces = !by_rows && use_static && launches.launch[gi].layer >= 0 ? 1 : 0;
   if (wait_in) QC_CUDA(cudaStreamWaitEvent(stream, wait_in, 0));
   if (append_first) {
     QC_CUDA(launch_append(p, stream));   // this group's layers only
@@ -1274,7 +1299,8 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     QC_CUDA(cudaEventRecord(evl[0], stream));
   }
   // (a GLA follower of the in-order schedule has nothing to sweep: its merge does everything)
-  if (has_work) QC_CUDA(c->group > 1 ? launch_attend_tc(p, c->ctx->n_sms, stream) : launch_attend(p, c->ctx->n_sms, stream));
+  if (has_work && by_rows) QC_CUDA(launch_attend_rows(p, *row_jobs, p.row_cluster, stream));
+  else if (has_work) QC_CUDA(c->group > 1 ? launch_attend_tc(p, c->ctx->n_sms, stream) : launch_attend(p, c->ctx->n_sms, stream));
   if (evl) QC_CUDA(cudaEventRecord(evl[1], stream));
   if (ev && gi + 1 == c->groups.size()) QC_CUDA(cudaEventRecord(ev[2], stream));
   if (!p.fused_merge) QC_CUDA(launch_merge(p, stream));
@@ -1282,6 +1308,33 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
   c->attend_launches += has_work ? 1 : 0;
   c->kernel_launches += (has_work ? 1 : 0) + (p.fused_merge ? 0 : 1);
   return QC_OK;
+}
+
+// CTAs that an output row gets in the launches of a step of the in-order schedule, or 0: its launches are cut into
+// tile ranges.  As many as leave one CTA per SM (the next launch then starts in the other half of each SM, and
+// its first tiles have landed when this one ends), twice that where a warp would still have more than six pages.
+// us per layer, tile ranges / 1, 2, 4, 8 CTAs per row (* what the rule takes): 32 rows of 43 pages 9.54 / 10.2, 7.49, 7.00*, 7.74; 32
+// of 188 13.8 / 30.2, 17.4, 12.4, 11.8*; 32 of 50, group of 4, 11.9 / 11.3, 8.67, 8.13*, 9.98; 4 of 71, group of 7, 12.2 / 14.7, 10.1,
+// 8.35, 7.81*; 52 of 131, group of 7, 19.4 / 22.9, 15.8, 15.4*, 23.1; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4; 128 of 71, group of
+// 7, 20.3 / 17.5, 17.9*, 24.0, 43.4; 256 of 188 55.9 / 53.2*, 54.6, 62.2, 83.7; 256 of 130, GLA, 34.4 / 33.0*, 32.8, 36.9, 46.6.  More
+// rows than there are places for CTAs stay with the ranges (512 of 43 30.9 / 31.0, 480 of 17 18.3 / 18.4), and so do batches whose
+// longest row is over 1.6 times the average one: a launch takes as long as its longest row.
+int row_cluster_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids) {
+  if (!c->rows_fit || c->static_partition != -1 || !c->plan_ahead || !c->fused_merge || c->row_cluster == 0) return 0;
+  if (c->row_cluster > 0) return c->row_cluster;
+  const int rows = n_seqs * c->items_per_chunk, slots = c->ctx->n_sms * kAttendCtasPerSm;
+  int64_t pages = 0, longest = 0;
+  for (int i = 0; i < n_seqs; ++i) {
+    const SeqState& st = c->seqs[seq_ids[i]];
+    const int64_t n = pages_for(st.len_vis) + pages_for(st.len_text);
+    pages += n;
+    longest = std::max(longest, n);
+  }
+  if (rows > slots || 5 * longest * n_seqs > 8 * pages) return 0;
+  int n = 8;
+  while (n > 1 && n * rows > c->ctx->n_sms) n /= 2;
+  if (n < 8 && 2 * n * rows <= slots && longest > 36 * n) n *= 2;
+  return n;
 }
 
 int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const void* q_dev, const void* k_dev,
@@ -1471,7 +1524,9 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   p.fold_append = fold ? 1 : 0;
   p.fused_append = (n_patches == 0 && !pipe && !open_only && !fold) ? 1 : 0;
 
-  const bool planned = use_static && c->plan_ahead && c->groups.size() <= static_cast<size_t>(kMaxPlanLaunches) &&
+  // Few output rows: a cluster of CTAs for each, if the options leave the schedule as it comes.
+  p.row_cluster = fold && use_static ? row_cluster_of(c, n_seqs, seq_ids) : 0;
+  const bool planned = use_static && p.row_cluster == 0 && c->plan_ahead && c->groups.size() <= static_cast<size_t>(kMaxPlanLaunches) &&
                        c->groups.size() <= static_cast<size_t>(std::min(c->cfg.n_layers, kMaxPlanLaunches)) &&
                        c->ctx->n_sms * kWorkersPerSm <= kPlanWorkers;
   // static partition of every launch of the step (part_workers == 0: the launch has nothing to sweep)
@@ -1856,6 +1911,11 @@ int32_t qc_set_option(qc_cache* c, const char* key, int64_t value) {
   }
   if (k == "plan_ahead") {
     c->plan_ahead = value != 0;
+    return QC_OK;
+  }
+  if (k == "row_cluster") {
+    if (value < -1 || value > 8) return QC_ERR_INVALID_ARG;
+    c->row_cluster = static_cast<int>(value);
     return QC_OK;
   }
   if (k == "static_row_cost") {
