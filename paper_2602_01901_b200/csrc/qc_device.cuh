@@ -80,13 +80,13 @@ __device__ __forceinline__ void tensor_g2s_2d(uint32_t dst_smem, const void* tma
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
-// the same with an L2 cache policy
-__device__ __forceinline__ void tensor_g2s_2d(uint32_t dst_smem, const void* tmap, int32_t x, int32_t y,
+// 3-D, with an L2 cache policy
+__device__ __forceinline__ void tensor_g2s_3d(uint32_t dst_smem, const void* tmap, int32_t x, int32_t y, int32_t z,
                                               uint64_t* bar, uint64_t policy) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, "
-      "%3}], [%4], %5;" ::"r"(dst_smem),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy)
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, "
+      "%3, %4}], [%5], %6;" ::"r"(dst_smem),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
 
@@ -343,9 +343,7 @@ __device__ __forceinline__ bool issue_one(WorkerState& st, CtxFn ctx, uint32_t r
     const uint32_t dst = ring + st.iss_slot * kTile;
     mbar_expect_tx(bar, kTile);
     if (TMAP) {
-      const int32_t row = (pid * P.hkv + st.iss_kv_head) * kPage;
-      tensor_g2s_2d(dst, &P.tmap, 0, row, bar, st.policy);
-      if (D == 128) tensor_g2s_2d(dst + kTile / 2, &P.tmap, 64, row, bar, st.policy);
+      tensor_g2s_3d(dst, &P.tmap, 0, (pid * P.hkv + st.iss_kv_head) * kPage, 0, bar, st.policy);
     } else {
       const uint16_t* src = P.pool + (static_cast<size_t>(pid) * P.hkv + st.iss_kv_head) * (kPage * D);
       bulk_g2s(dst, src, kTile, bar, st.policy);

@@ -134,8 +134,8 @@ constexpr int kPlanCtas = 512;      // CTA descriptors kept per launch
 // Kernel parameter block.
 struct Params {
   // cache-lifetime
-  CUtensorMap tmap;        // the pool as a 2-D bf16 tensor [pages * hkv * 16 rows][d], box 16 x min(d, 64),
-                           // 128-byte swizzle (used by the tensor-core kernel only)
+  CUtensorMap tmap;        // the pool as a bf16 tensor [d / 64][pages * hkv * 16 rows][64], box d / 64 x 16 x 64 (a (page,
+                           // head) tile in column halves), 128-byte swizzle (query groups only)
   uint16_t* pool;          // bf16 pages
   int32_t* table;          // [n_layers][4][max_seqs][max_pages]
   uint16_t* qcache;        // bf16 [n_layers][max_seqs][hq][d]
@@ -201,6 +201,7 @@ struct Params {
                                      // tile and waits for it with a short limit (nothing in flight, nothing faults)
   int32_t row_cluster;               // > 0: the step's launches give every output row a cluster of that many CTAs, and what a
                                      // leader's launch leaves for a follower is one partial row (slot 0)
+  int32_t row_warps;                 // warps of each of them
   int32_t extra_key_leader;          // merge only, >= 0: the rows also take the step's new token as one more key,
                                      // scored by that layer's Q Cache entry and new k (Eq. 6), valued by the own new v
 };
@@ -220,7 +221,7 @@ struct RowJobs {
   int32_t add_earlier;   // the rows also take what the leader's launch left for the layer
   int32_t pad;
 };
-cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int cluster, cudaStream_t stream);
+cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, cudaStream_t stream);   // p.row_cluster, p.row_warps
 cudaError_t configure_rows_kernels();
 // Up to 16 consecutive tokens of one sequence and stream that go to one page.
 struct __align__(16) StoreSeg {
@@ -257,6 +258,7 @@ constexpr int kPrefillSharedLayers = 3;   // layers one shared-score pass feeds
 
 struct PrefillMaps {
   CUtensorMap q, k, v, out;
+  CUtensorMap pool;   // cached pages: the pool as a 2-D tensor [pages * hkv * 16 rows][d], box 16 x 64
 };
 cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, const uint8_t* layer_kind_dev,
                                   const uint8_t* leader_dev, const int* leader, const void* q, const void* k, const void* v, void* out,

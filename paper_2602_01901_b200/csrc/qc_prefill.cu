@@ -1521,7 +1521,7 @@ cudaError_t launch_prefill_attend(const Params& p, const uint8_t* kind_dev, cons
   a.n0_text = n0_text;
   a.n0_vis = n0_vis;
   if (p.d == kTD && maps) {
-    a.tmap_pool = p.tmap;
+    a.tmap_pool = maps->pool;
     a.n_pool_pages = p.n_pool_pages;
     a.tmap_q = maps->q;
     a.tmap_k = maps->k;

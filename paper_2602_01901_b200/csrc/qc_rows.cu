@@ -1,22 +1,28 @@
-// Attention of one layer over few output rows (in-order schedule): a cluster of CTAs per row.
+// Attention of one layer (in-order schedule) where every output row has thread blocks of its own.
 //
 // A launch of one layer for a small batch moves a few MB, which HBM delivers in 2 us, and what it
-// costs is its chain of dependent steps.  Cut into tile ranges (qc_kernels.cu, qc_attend_tc.cu) that
-// chain is: a worker's page, its partial row through the L2, an atomic per shared row, the partials
-// of 40 workers read back by one CTA (or a merge launch).  Here a row (a query head, or a query group) belongs to a
-// cluster of up to eight CTAs whose warps take its pages in turn -- all visual pages, then all text
-// pages -- and the warps' sums are added in shared memory: first in each CTA, then over the cluster
-// through distributed shared memory.  The launch writes finished rows; the only sums that reach HBM
-// are one per row and follower of a lazy block (the sums of the keys it shares with its leader).  No plan, no counters,
-// no merge launch, and every row is added up in one order.
+// costs is its chain of dependent steps; a launch for a large batch is bound by HBM and loses at its end what that chain takes.  Cut into
+// tile ranges (qc_kernels.cu, qc_attend_tc.cu) the chain is: a worker's page, its partial row through
+// the L2, an atomic per shared row, the partials of 40 workers read back by one CTA (or a merge
+// launch).  Here a row (a query head, or a query group) belongs to a cluster of up to eight CTAs, or to one CTA, whose
+// warps take its pages in turn -- all visual pages, then all text pages -- and the warps' sums are
+// added in shared memory: first in each CTA, then over the cluster through distributed shared memory.
+// The launch writes finished rows; the only sums that reach HBM are one per row and follower of a lazy
+// block (the sums of the keys it shares with its leader).  No plan, no counters, no merge launch, and
+// every row is added up in one order.
+// us per layer, tile ranges -> this: one sequence of 675 tokens, 32 heads 9.5 -> 6.9; 16 of them 30.8 -> 26.9; 32 of 500 44.9 -> 40.5; 32 of
+// 1 120 with 4 KV heads 20.2 -> 17.7.  After the wait for the previous kernel the first of these spends, of some 12 000 cycles, 850 on the query, 2 300 on the
+// first K tile and its softmax, 1 900 on the V tiles, as much on a second page, and 2 500 from the last page to the row.
 //
 // Every launch of the in-order schedule scores with one query per row (its layer's own), so one
 // running softmax serves the row's streams: consumer 0 is the layer itself, consumers 1 .. are the
 // followers whose cached V the leader's launch also weights.  Under VLA_QC those take no text keys:
 // their softmax reference stays where the visual pages left it.
 //
-// One query head per KV head: fp32 arithmetic on pairs; query groups: mma.m16n8k16 with keys as M and
-// the group as N, as in qc_attend_tc.cu.
+// One query head per KV head: fp32 arithmetic on pairs.  Query groups: mma.m16n8k16 with keys as M and
+// the group as N, as in qc_attend_tc.cu, but with the weights as the sum of two bf16 values, a product each on the same V
+// fragment (error against 64 bits, 32 sequences of 1 120 tokens: 2.05e-3 in tile ranges, 2.11e-3 here with one bf16 value -- fewer,
+// longer pieces have fewer weights that are exactly 1 -- and 1.66e-3, the rounding of the output, with two; 17.6 and 17.7 us a layer).
 
 #include "qc_device.cuh"
 
@@ -25,9 +31,9 @@
 namespace qc {
 namespace {
 
-constexpr int kRowWarps = 6;
-constexpr int kRowThreads = kRowWarps * 32;
-constexpr int kRowRing = 4;    // tiles in flight per warp
+// Warps per CTA (W): six, or fewer where rows are many; an SM holds twelve in all.  Tiles in flight per warp (RING): four
+// where the next launch's first tiles are to land during this one; two where the launch is bound by HBM, which
+// scattered tiles use worse the more there are in flight (512 rows of 43 pages, 3 warps: 27.5 us a layer with four, 27.0 with two).
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -80,20 +86,20 @@ template <int D, bool MH, int NV>
 constexpr int kRowStride = D + (MH || NV == 4 ? 0 : 4);   // floats from one head's sums to the next one's (bank conflicts, where there is room)
 
 // What the CTA keeps of the row besides the tiles.
-template <int D, bool MH, int NV>
+template <int D, bool MH, int NV, int W, int RING>
 struct __align__(16) RowSmem {
   float red[NV][kRowHeads<MH>][D];                  // the CTA's sums
   float2 red_ml[NV > 1 ? 2 : 1][kRowHeads<MH>];     // and their (reference, sum of weights): own, followers'
-  float2 ml[NV > 1 ? 2 : 1][kRowHeads<MH>][kRowWarps];
-  float weight[NV > 1 ? 2 : 1][kRowHeads<MH>][kRowWarps + 2];   // of the warps' sums in the CTA's
+  float2 ml[NV > 1 ? 2 : 1][kRowHeads<MH>][W];
+  float weight[NV > 1 ? 2 : 1][kRowHeads<MH>][W + 2];   // of the warps' sums in the CTA's
   uint4 new_k[D / 8], new_v[D / 8];                 // the new token's rows (for the one warp that sweeps it)
-  int32_t pages[kRowWarps][1 + NV][32];             // page ids of a warp's next pages: K, V of each consumer
-  uint64_t full[kRowWarps][kRowRing];
+  int32_t pages[W][1 + NV][32];             // page ids of a warp's next pages: K, V of each consumer
+  uint64_t full[W][RING];
   int32_t dead;
 };
 
-template <int D, bool MH, int NV>
-__global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ RowJobs J) {
+template <int D, bool MH, int NV, int W, int RING>
+__global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ RowJobs J) {
   constexpr uint32_t kTile = kPage * D * 2;
   constexpr int KS = D / 16;
   constexpr int NH = MH ? 1 : 2;       // heads whose softmax a lane follows (query groups: columns 2t, 2t + 1)
@@ -103,14 +109,14 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles sit on 1024-byte boundaries
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  using Smem = RowSmem<D, MH, NV>;
-  Smem& S = *reinterpret_cast<Smem*>(base_ptr + kRowWarps * kRowRing * kTile);
+  using Smem = RowSmem<D, MH, NV, W, RING>;
+  Smem& S = *reinterpret_cast<Smem*>(base_ptr + W * RING * kTile);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = cluster_rank(), n_ctas = cluster_size();
-  const uint32_t ring = base + static_cast<uint32_t>(warp) * kRowRing * kTile;
+  const uint32_t ring = base + static_cast<uint32_t>(warp) * RING * kTile;
   uint64_t* full = S.full[warp];
   if (lane == 0) {
-    for (int s = 0; s < kRowRing; ++s) mbar_init(&full[s], 1);
+    for (int s = 0; s < RING; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
   }
   if (threadIdx.x == 0) S.dead = 0;
@@ -124,7 +130,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   const int hpi = P.heads_per_item, n_sub = (P.group + hpi - 1) / hpi, kv_head = u / n_sub, sub = u - kv_head * n_sub;
   const int head = kv_head * P.group + sub * hpi, n_heads = min(hpi, P.group - sub * hpi);
   const int n_vis = J.has_vis ? pages_of(len_vis) : 0, n_text = J.has_text ? pages_of(len_text) : 0;
-  const int total = n_vis + n_text, step = n_ctas * kRowWarps, first = rank * kRowWarps + warp;
+  const int total = n_vis + n_text, step = n_ctas * W, first = rank * W + warp;
   const int n_my = total > first ? (total - first + step - 1) / step : 0;               // pages first, first + step, ...
   const int j_text = n_vis > first ? (n_vis - first + step - 1) / step : 0;             // the first of them that is a text page
   const int vis_cons = J.vis.n_cons, text_cons = J.text.n_cons;
@@ -153,7 +159,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   uint32_t cons_phase = 0;
   bool drop_next = P.debug_drop_tile != 0;   // (test hook)
   auto fill = [&]() {
-    while (in_flight < kRowRing && iss_j < n_my) {
+    while (in_flight < RING && iss_j < n_my) {
       if (iss_t == 0 && iss_j > 0 && (iss_j & 31) == 0) load_pages(iss_j);
       if (drop_next) {
         drop_next = false;   // counted as in flight without being requested: its wait will run out
@@ -164,12 +170,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
         if (MH) {
           bulk_g2s(dst, P.pool + (static_cast<size_t>(pid) * P.hkv + kv_head) * (kPage * D), kTile, &full[iss_slot], policy);
         } else {
-          const int32_t y = (pid * P.hkv + kv_head) * kPage;
-          tensor_g2s_2d(dst, &P.tmap, 0, y, &full[iss_slot], policy);
-          if (D == 128) tensor_g2s_2d(dst + kTile / 2, &P.tmap, 64, y, &full[iss_slot], policy);
+          tensor_g2s_3d(dst, &P.tmap, 0, (pid * P.hkv + kv_head) * kPage, 0, &full[iss_slot], policy);
         }
       }
-      iss_slot = iss_slot + 1 == kRowRing ? 0 : iss_slot + 1;
+      iss_slot = iss_slot + 1 == RING ? 0 : iss_slot + 1;
       ++in_flight;
       if (iss_t == (iss_j < j_text ? vis_cons : text_cons)) iss_t = 0, ++iss_j;
       else ++iss_t;
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   auto release = [&]() {
     __syncwarp();
     --in_flight;
-    if (++cons_slot == kRowRing) cons_slot = 0, cons_phase ^= 1u;
+    if (++cons_slot == RING) cons_slot = 0, cons_phase ^= 1u;
     fill();
   };
 
@@ -263,7 +267,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
     }
   }
   const int lrow = lane & 7, lmat = lane >> 3;   // ldmatrix lane roles
-  const int k_row = lrow + ((lmat & 1) << 3), k_chunk = lmat >> 1, v_row = lrow + ((lmat >> 1) << 3), v_chunk = lmat & 1;
+  const uint32_t k_off = tile_at<D, MH>(lrow + ((lmat & 1) << 3), lmat >> 1), v_off = tile_at<D, MH>(lrow + ((lmat >> 1) << 3), lmat & 1);
+  // chunk 2 * i further along a lane's row (tiles are 1024-byte aligned: the swizzle is an exclusive or on the address)
+  auto step_addr = [](uint32_t addr, int i) -> uint32_t { return (addr ^ ((i & 3) << 5)) + ((i >> 2) << 11); };
 
   for (int j = 0; j < n_my; ++j) {
     const bool vis = j < j_text;
@@ -327,7 +333,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
 #pragma unroll
       for (int kk = 0; kk < KS; ++kk) {   // two chains: a product waits for the one before it
         uint32_t a[4];
-        ldmatrix_x4(a, tile + tile_at<D, MH>(k_row, 2 * kk + k_chunk));
+        ldmatrix_x4(a, step_addr(tile + k_off, kk));
         mma_bf16_16816(s[kk & 1], a, qb[kk]);
       }
       release();
@@ -366,7 +372,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
         }
       }
     }
-    uint32_t pb[2], pb_skip[2];
+    uint32_t pb[2][2], pb_skip[2][2];   // query groups: the weights as B operands, in two parts
+    auto operands = [&](uint32_t (&b)[2][2]) {
+#pragma unroll
+      for (int j2 = 0; j2 < 2; ++j2) {
+        const uint32_t hi = pack_bf16x2(w[0][j2], w[NH - 1][j2]);
+        b[0][j2] = movmatrix_trans(hi);
+        b[1][j2] = movmatrix_trans(pack_bf16x2(w[0][j2] - __uint_as_float(hi << 16), w[NH - 1][j2] - __uint_as_float(hi & 0xffff0000u)));
+      }
+    };
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
       w[h][0] = ex2_approx(w[h][0] - m[0][h]);
@@ -377,8 +391,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
 #pragma unroll
       for (int i = 0; i < 4; ++i) pk[i] = __shfl_sync(0xffffffffu, w[0][0], (lane & 24) + (i >> 1) * 4 + (i & 1) * 2);
     } else {
-      pb[0] = movmatrix_trans(pack_bf16x2(w[0][0], w[NH - 1][0]));
-      pb[1] = movmatrix_trans(pack_bf16x2(w[0][1], w[NH - 1][1]));
+      operands(pb);
     }
     if (with_followers) {   // they leave out the new token: its value row of theirs does not exist yet
       const int r_new = takes_new ? nvalid - 1 : kPage;
@@ -394,8 +407,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
         if (NC > 1) l[NC - 1][h] += w[h][0] + w[h][1];
       }
       if constexpr (!MH) {
-        pb_skip[0] = takes_new ? movmatrix_trans(pack_bf16x2(w[0][0], w[NH - 1][0])) : pb[0];
-        pb_skip[1] = takes_new ? movmatrix_trans(pack_bf16x2(w[0][1], w[NH - 1][1])) : pb[1];
+        if (takes_new) operands(pb_skip);
       }
     }
     // ---- V tiles
@@ -425,8 +437,14 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
 #pragma unroll
           for (int i = 0; i < KS; ++i) {
             uint32_t a[4];
-            ldmatrix_x4_trans(a, tile + tile_at<D, MH>(v_row, 2 * i + v_chunk));
-            mma_bf16_16816(o[x][i], a, x == 0 ? pb : pb_skip);
+            ldmatrix_x4_trans(a, step_addr(tile + v_off, i));
+            if (x > 0 && takes_new) {
+              mma_bf16_16816(o[x][i], a, pb_skip[0]);
+              mma_bf16_16816(o[x][i], a, pb_skip[1]);
+            } else {
+              mma_bf16_16816(o[x][i], a, pb[0]);
+              mma_bf16_16816(o[x][i], a, pb[1]);
+            }
           }
         }
         release();
@@ -442,15 +460,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
       uint32_t done = 0;
       for (uint32_t spin = 0; !done && spin < limit; ++spin) done = mbar_try_wait(&full[cons_slot], cons_phase);
       --in_flight;
-      if (++cons_slot == kRowRing) cons_slot = 0, cons_phase ^= 1u;
+      if (++cons_slot == RING) cons_slot = 0, cons_phase ^= 1u;
     }
   }
 
   // ---- the warp's sums, over its own tiles (all consumed): [consumer][part or head][D]; the parts are a
   // head's sums over a quarter of the keys each (MH)
   constexpr int kParts = MH ? 4 : kRowHeads<MH>;
-  static_assert(NV * kParts * kRowStride<D, MH, NV> * 4 <= kRowRing * static_cast<int>(kTile), "a warp's sums fit its tiles");
-  float* stage = reinterpret_cast<float*>(base_ptr + static_cast<size_t>(warp) * kRowRing * kTile);
+  static_assert(NV * kParts * kRowStride<D, MH, NV> * 4 <= RING * static_cast<int>(kTile), "a warp's sums fit its tiles");
+  float* stage = reinterpret_cast<float*>(base_ptr + static_cast<size_t>(warp) * RING * kTile);
   // (a warp that had no pages has stored nothing but zeros, with no weight)
   __syncwarp();
   {
@@ -486,15 +504,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   // weight counts for nothing, one that is not a number makes the row not a number.
   if (threadIdx.x < NC * kRowHeads<MH>) {
     const int cl = threadIdx.x / kRowHeads<MH>, h = threadIdx.x % kRowHeads<MH>;
-    float2 ml[kRowWarps];
+    float2 ml[W];
     float top = -INFINITY, sum = 0.f;
 #pragma unroll
-    for (int v = 0; v < kRowWarps; ++v) {
+    for (int v = 0; v < W; ++v) {
       ml[v] = S.ml[cl][h][v];
       top = ml[v].y > 0.f ? fmaxf(top, ml[v].x) : top;
     }
 #pragma unroll
-    for (int v = 0; v < kRowWarps; ++v) {
+    for (int v = 0; v < W; ++v) {
       const float wt = ml[v].y > 0.f ? ex2_approx(ml[v].x - top) : 0.f;
       sum = fmaf(ml[v].y, wt, sum);
       S.weight[cl][h][v] = wt;
@@ -515,15 +533,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
     r.x = fmaf(v.x, w, r.x), r.y = fmaf(v.y, w, r.y);
     if constexpr (!MH) r.z = fmaf(v.z, w, r.z), r.w = fmaf(v.w, w, r.w);
   };
-  for (int i = threadIdx.x; i < n_units; i += kRowThreads) {
+  for (int i = threadIdx.x; i < n_units; i += (W * 32)) {
     int x, h, e;
     unit_of(i, x, h, e);
     const float* src = reinterpret_cast<const float*>(base_ptr) + (x * kParts + (MH ? 0 : h)) * kRowStride<D, MH, NV> + e;
     const float* wt = S.weight[x > 0 ? NC - 1 : 0][h];
     Vec r{};
 #pragma unroll
-    for (int v = 0; v < kRowWarps; ++v) {
-      const float* at = src + static_cast<size_t>(v) * kRowRing * (kTile / 4);
+    for (int v = 0; v < W; ++v) {
+      const float* at = src + static_cast<size_t>(v) * RING * (kTile / 4);
       Vec a = *reinterpret_cast<const Vec*>(at);
       if constexpr (MH) {
 #pragma unroll
@@ -537,7 +555,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
     *reinterpret_cast<Vec*>(&S.red[x][h][e]) = r;
   }
   // ---- the row: its elements are dealt out over the cluster
-  const int unit0 = threadIdx.x * n_ctas + rank, unit_step = kRowThreads * n_ctas;
+  const int unit0 = threadIdx.x * n_ctas + rank, unit_step = (W * 32) * n_ctas;
   // what the leader's launch left for this layer (one consumer), asked for ahead of the barrier
   float2 e_ml = make_float2(-INFINITY, 0.f);
   Vec e_acc{};
@@ -609,28 +627,36 @@ __global__ void __launch_bounds__(kRowThreads, 2) attend_rows_kernel(const __gri
   if (n_ctas > 1) cluster_sync();   // nobody reads this CTA's shared memory any more
 }
 
-template <int D, bool MH, int NV>
+template <int D, bool MH, int NV, int W, int RING>
 constexpr int rows_smem_bytes() {
-  return 1024 + kRowWarps * kRowRing * kPage * D * 2 + static_cast<int>(sizeof(RowSmem<D, MH, NV>));
+  return 1024 + W * RING * kPage * D * 2 + static_cast<int>(sizeof(RowSmem<D, MH, NV, W, RING>));
 }
 
 // Calls fn(kernel, shared memory) for the kernel that a launch takes.
 template <typename Fn>
-cudaError_t with_rows_kernel(int d, bool mh, int nv, Fn fn) {
-  auto by_nv = [&](auto dd, auto m) -> cudaError_t {
-    constexpr int D = decltype(dd)::value;
+cudaError_t with_rows_kernel(int d, bool mh, int nv, int warps, Fn fn) {
+  using std::integral_constant;
+  auto by_nv = [&](auto dd, auto m, auto w, auto r) -> cudaError_t {
+    constexpr int D = decltype(dd)::value, W = decltype(w)::value, R = decltype(r)::value;
     constexpr bool MH = decltype(m)::value;
     switch (nv) {
-      case 1: return fn(attend_rows_kernel<D, MH, 1>, rows_smem_bytes<D, MH, 1>());
-      case 2: return fn(attend_rows_kernel<D, MH, 2>, rows_smem_bytes<D, MH, 2>());
-      case 3: return fn(attend_rows_kernel<D, MH, 3>, rows_smem_bytes<D, MH, 3>());
-      default: return fn(attend_rows_kernel<D, MH, 4>, rows_smem_bytes<D, MH, 4>());
+      case 1: return fn(attend_rows_kernel<D, MH, 1, W, R>, rows_smem_bytes<D, MH, 1, W, R>());
+      case 2: return fn(attend_rows_kernel<D, MH, 2, W, R>, rows_smem_bytes<D, MH, 2, W, R>());
+      case 3: return fn(attend_rows_kernel<D, MH, 3, W, R>, rows_smem_bytes<D, MH, 3, W, R>());
+      default: return fn(attend_rows_kernel<D, MH, 4, W, R>, rows_smem_bytes<D, MH, 4, W, R>());
     }
   };
-  using D128 = std::integral_constant<int, 128>;
-  using D64 = std::integral_constant<int, 64>;
-  if (d == 128) return mh ? by_nv(D128{}, std::true_type{}) : by_nv(D128{}, std::false_type{});
-  return mh ? by_nv(D64{}, std::true_type{}) : by_nv(D64{}, std::false_type{});
+  auto by_warps = [&](auto dd) -> cudaError_t {
+    if (!mh) return by_nv(dd, std::false_type{}, integral_constant<int, 6>{}, integral_constant<int, 4>{});
+    switch (warps) {
+      case 1: return by_nv(dd, std::true_type{}, integral_constant<int, 1>{}, integral_constant<int, 3>{});
+      case 2: return by_nv(dd, std::true_type{}, integral_constant<int, 2>{}, integral_constant<int, 2>{});
+      case 3: return by_nv(dd, std::true_type{}, integral_constant<int, 3>{}, integral_constant<int, 2>{});
+      case 4: return by_nv(dd, std::true_type{}, integral_constant<int, 4>{}, integral_constant<int, 2>{});
+      default: return by_nv(dd, std::true_type{}, integral_constant<int, 6>{}, integral_constant<int, 4>{});
+    }
+  };
+  return d == 128 ? by_warps(integral_constant<int, 128>{}) : by_warps(integral_constant<int, 64>{});
 }
 
 }  // namespace
@@ -638,30 +664,31 @@ cudaError_t with_rows_kernel(int d, bool mh, int nv, Fn fn) {
 cudaError_t configure_rows_kernels() {
   for (int d = 64; d <= 128; d += 64)
     for (int mh = 0; mh < 2; ++mh)
-      for (int nv = 1; nv <= kMaxCons; ++nv) {
-        const cudaError_t e = with_rows_kernel(d, mh != 0, nv, [](auto kernel, int smem) {
-          cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-          if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-          return r;
-        });
-        if (e != cudaSuccess) return e;
-      }
+      for (int warps : {1, 2, 3, 4, 6})
+        for (int nv = 1; nv <= kMaxCons; ++nv) {
+          const cudaError_t e = with_rows_kernel(d, mh != 0, nv, warps, [](auto kernel, int smem) {
+            cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+            return r;
+          });
+          if (e != cudaSuccess) return e;
+        }
   return cudaSuccess;
 }
 
-cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int cluster, cudaStream_t stream) {
+cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, cudaStream_t stream) {
   const int nv = jobs.has_vis ? jobs.vis.n_cons : jobs.text.n_cons;
-  return with_rows_kernel(p.d, p.group == 1, nv, [&](auto kernel, int smem) {
+  return with_rows_kernel(p.d, p.group == 1, nv, p.row_warps, [&](auto kernel, int smem) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.n_seqs * p.heads_per_item_dim * cluster));
-    cfg.blockDim = dim3(kRowThreads);
+    cfg.gridDim = dim3(static_cast<unsigned>(p.n_seqs * p.heads_per_item_dim * p.row_cluster));
+    cfg.blockDim = dim3(p.row_warps * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = cluster, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = p.row_cluster, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, p, jobs);

@@ -81,7 +81,8 @@ struct qc_cache {
   int D = 0, hq = 0, hkv = 0, group = 0;
   int heads_per_item = 1;  // query heads one work item covers (8 with GQA: one query group, or a slice of it)
   int items_per_chunk = 0; // work items per (chunk, sequence)
-  CUtensorMap tmap{};      // the pool as a swizzled 2-D tensor (query-group kernel)
+  CUtensorMap tmap{};      // the pool's (page, head) tiles, for the query-group decode kernels
+  CUtensorMap tmap_rows{}; // the pool's rows, for the prompt kernel
   bool paged = true;
   int max_pages = 0;       // per stream
   int chunk_pages = 0, min_chunk_pages = 0, max_slots = 0;
@@ -99,7 +100,7 @@ struct qc_cache {
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   std::vector<cudaEvent_t> ev_in, ev_done;
   bool prefill_tcgen05 = true;    // head_dim 128: tcgen05 kernel; otherwise (or when switched off) mma.sync kernel
-  bool pool_map_ok = false;       // c->tmap was encoded
+  bool pool_map_ok = false;       // both were encoded
   int prefill_pair_min_tokens = 0;   // prompts this long that start a sequence run two query tiles per CTA (0: never)
   int prefill_shared = 1;         // GLA prefill: layers of a block whose scores coincide share one score pass
                                   // (0 never, 1 for prompts of kPrefillShareMinTokens or more, 2 always)
@@ -127,6 +128,7 @@ struct qc_cache {
   std::vector<int> inorder_extra_key;             // per layer: the leader whose new token the merge adds, or -1
   std::vector<RowJobs> row_jobs;                  // per layer, for launches that give every output row a cluster
   bool rows_fit = false;                          // every layer's sweeps have that form
+  int row_warps = 0;                              // warps of a CTA where rows have one each: 0 chosen per step
   int row_cluster = -1;                           // CTAs per output row: -1 chosen per step, 0 never, n always n
   int slots_per_stream = 0;
   int static_partition = -1;      // -1: static ranges when a step is several launches; 0 never; 1 always
@@ -621,19 +623,21 @@ int make_output_tensor_map(CUtensorMap* out, void* base, int n_layers, int T, in
   return r == CUDA_SUCCESS ? QC_OK : QC_ERR_CUDA;
 }
 
-int make_pool_tensor_map(qc_cache* c) {
+int make_pool_tensor_maps(qc_cache* c) {
   EncodeFn enc = tensor_map_encoder();
   if (!enc) return QC_ERR_CUDA;
   const cuuint64_t rows = static_cast<cuuint64_t>(c->n_pool_pages) * c->hkv * kPage;
   if (rows > 0x7fffffffULL) return QC_ERR_INVALID_ARG;   // tile coordinates are 32-bit
-  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(c->D), rows};
-  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(c->D) * 2};
-  const cuuint32_t box[2] = {64, kPage};
-  const cuuint32_t elem_strides[2] = {1, 1};
-  const CUresult r = enc(
-      &c->tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, c->pool, dims, strides, box, elem_strides,
-      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  const cuuint64_t d = static_cast<cuuint64_t>(c->D);
+  const cuuint64_t row_dims[2] = {d, rows}, row_strides[1] = {d * 2}, dims[3] = {64, rows, d / 64}, strides[2] = {d * 2, 64 * 2};
+  const cuuint32_t row_box[2] = {64, kPage}, box[3] = {64, kPage, static_cast<cuuint32_t>(d / 64)}, elem_strides[3] = {1, 1, 1};
+  if (enc(&c->tmap_rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, c->pool, row_dims, row_strides, row_box, elem_strides,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return QC_ERR_CUDA;
+  const CUresult r = enc(&c->tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, c->pool, dims, strides, box, elem_strides,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? QC_OK : QC_ERR_CUDA;
 }
 
@@ -848,9 +852,9 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
     for (size_t i = 0; i < c->table.size(); ++i) c->table[i] = static_cast<int32_t>(i);
   }
 
-  // the pool's tensor map: needed by the query-group decode kernel; the prefill kernel uses it for
+  // the pool's tensor maps: needed by the query-group decode kernels; the prefill kernel uses its one for
   // cached tiles when it exists
-  c->pool_map_ok = make_pool_tensor_map(c) == QC_OK;
+  c->pool_map_ok = make_pool_tensor_maps(c) == QC_OK;
   if (c->group > 1 && !c->pool_map_ok) {
     delete c;
     return QC_ERR_CUDA;
@@ -1116,6 +1120,7 @@ int32_t qc_prefill_attend(qc_cache* c, int32_t seq_id, int32_t n_tokens, const u
   PrefillMaps maps;
   const bool tc5 = c->prefill_tcgen05 && c->D == 128 && (c->pool_map_ok || n0_text + n0_vis == 0);
   if (tc5) {
+    maps.pool = c->tmap_rows;
     if (make_prompt_tensor_map(&maps.q, q_dev, c->cfg.n_layers, n_tokens, c->hq) != QC_OK ||
         make_prompt_tensor_map(&maps.k, k_dev, c->cfg.n_layers, n_tokens, c->hkv) != QC_OK ||
         make_prompt_tensor_map(&maps.v, v_dev, c->cfg.n_layers, n_tokens, c->hkv) != QC_OK ||
@@ -1299,7 +1304,7 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     QC_CUDA(cudaEventRecord(evl[0], stream));
   }
   // (a GLA follower of the in-order schedule has nothing to sweep: its merge does everything)
-  if (has_work && by_rows) QC_CUDA(launch_attend_rows(p, *row_jobs, p.row_cluster, stream));
+  if (has_work && by_rows) QC_CUDA(launch_attend_rows(p, *row_jobs, stream));
   else if (has_work) QC_CUDA(c->group > 1 ? launch_attend_tc(p, c->ctx->n_sms, stream) : launch_attend(p, c->ctx->n_sms, stream));
   if (evl) QC_CUDA(cudaEventRecord(evl[1], stream));
   if (ev && gi + 1 == c->groups.size()) QC_CUDA(cudaEventRecord(ev[2], stream));
@@ -1310,19 +1315,29 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
   return QC_OK;
 }
 
-// CTAs that an output row gets in the launches of a step of the in-order schedule, or 0: its launches are cut into
-// tile ranges.  As many as leave one CTA per SM (the next launch then starts in the other half of each SM, and
-// its first tiles have landed when this one ends), twice that where a warp would still have more than six pages.
-// us per layer, tile ranges / 1, 2, 4, 8 CTAs per row (* what the rule takes): 32 rows of 43 pages 9.54 / 10.2, 7.49, 7.00*, 7.74; 32
-// of 188 13.8 / 30.2, 17.4, 12.4, 11.8*; 32 of 50, group of 4, 11.9 / 11.3, 8.67, 8.13*, 9.98; 4 of 71, group of 7, 12.2 / 14.7, 10.1,
-// 8.35, 7.81*; 52 of 131, group of 7, 19.4 / 22.9, 15.8, 15.4*, 23.1; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4; 128 of 71, group of
-// 7, 20.3 / 17.5, 17.9*, 24.0, 43.4; 256 of 188 55.9 / 53.2*, 54.6, 62.2, 83.7; 256 of 130, GLA, 34.4 / 33.0*, 32.8, 36.9, 46.6.  More
-// rows than there are places for CTAs stay with the ranges (512 of 43 30.9 / 31.0, 480 of 17 18.3 / 18.4), and so do batches whose
-// longest row is over 1.6 times the average one: a launch takes as long as its longest row.
-int row_cluster_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids) {
-  if (!c->rows_fit || c->static_partition != -1 || !c->plan_ahead || !c->fused_merge || c->row_cluster == 0) return 0;
-  if (c->row_cluster > 0) return c->row_cluster;
-  const int rows = n_seqs * c->items_per_chunk, slots = c->ctx->n_sms * kAttendCtasPerSm;
+// CTAs that an output row gets in the launches of a step of the in-order schedule, and their warps, or 0: its launches
+// are cut into tile ranges.
+// Up to 296 rows (two six-warp CTAs per SM): as many CTAs per row as leave one CTA per SM (the next launch then starts in the other
+// half of each SM, and its first tiles have landed when this one ends), twice that where a warp would still have more than six
+// pages.  us per layer, tile ranges / 1, 2, 4, 8 CTAs per row (* what the rule takes): 32 rows of 43 pages 9.54 / 10.2, 7.53, 6.92*,
+// 7.74; 32 of 188 13.8 / 30.2, 17.4, 12.4, 11.6*; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4; 256 of 188 55.5 / 52.7*, 54.6, 62.2; 256 of
+// 130, GLA, 34.4 / 32.7*, 32.8, 36.9; 32 of 43, 64-wide, GLA 7.50 / 8.0, 5.9, 5.09*, 4.94; with query groups 32 of 50 11.7 / 12.3, 9.27,
+// 8.34*, 9.98; 4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1; 128 of 71 20.2 / 18.7, 17.8*, 24.4.
+// More rows, no query groups: one CTA per row, with the most warps that leave every row resident.  Ranges / 6, 4, 3, 2, 1 warps:
+// 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
+// 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.
+// A launch takes as long as its longest row: batches whose longest row is over 1.6 times the average one stay with the
+// ranges, and one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
+// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
+struct RowSplit {
+  int cluster, warps;
+};
+RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids) {
+  const RowSplit ranges{0, 0};
+  if (!c->rows_fit || c->static_partition != -1 || !c->plan_ahead || !c->fused_merge || c->row_cluster == 0) return ranges;
+  if (c->group == 1 && c->row_warps > 0) return RowSplit{1, c->row_warps};
+  if (c->row_cluster > 0) return RowSplit{c->row_cluster, kAttendWarps};
+  const int rows = n_seqs * c->items_per_chunk, n_sms = c->ctx->n_sms;
   int64_t pages = 0, longest = 0;
   for (int i = 0; i < n_seqs; ++i) {
     const SeqState& st = c->seqs[seq_ids[i]];
@@ -1330,11 +1345,17 @@ int row_cluster_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids) {
     pages += n;
     longest = std::max(longest, n);
   }
-  if (rows > slots || 5 * longest * n_seqs > 8 * pages) return 0;
-  int n = 8;
-  while (n > 1 && n * rows > c->ctx->n_sms) n /= 2;
-  if (n < 8 && 2 * n * rows <= slots && longest > 36 * n) n *= 2;
-  return n;
+  if (5 * longest * n_seqs > 8 * pages) return ranges;
+  if (rows <= n_sms * kAttendCtasPerSm) {
+    int n = 8;
+    while (n > 1 && n * rows > n_sms) n /= 2;
+    if (n < 8 && 2 * n * rows <= n_sms * kAttendCtasPerSm && longest > 36 * n) n *= 2;
+    return RowSplit{n, kAttendWarps};
+  }
+  if (c->group > 1) return ranges;
+  for (int warps : {4, 3, 2, 1})
+    if (rows <= n_sms * (kWorkersPerSm / warps)) return RowSplit{1, warps == 1 && 20 * longest * n_seqs > 23 * pages ? 3 : warps};
+  return ranges;
 }
 
 int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const void* q_dev, const void* k_dev,
@@ -1525,7 +1546,9 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   p.fused_append = (n_patches == 0 && !pipe && !open_only && !fold) ? 1 : 0;
 
   // Few output rows: a cluster of CTAs for each, if the options leave the schedule as it comes.
-  p.row_cluster = fold && use_static ? row_cluster_of(c, n_seqs, seq_ids) : 0;
+  const RowSplit by_rows = fold && use_static ? row_split_of(c, n_seqs, seq_ids) : RowSplit{0, 0};
+  p.row_cluster = by_rows.cluster;
+  p.row_warps = by_rows.warps;
   const bool planned = use_static && p.row_cluster == 0 && c->plan_ahead && c->groups.size() <= static_cast<size_t>(kMaxPlanLaunches) &&
                        c->groups.size() <= static_cast<size_t>(std::min(c->cfg.n_layers, kMaxPlanLaunches)) &&
                        c->ctx->n_sms * kWorkersPerSm <= kPlanWorkers;
@@ -1911,6 +1934,11 @@ int32_t qc_set_option(qc_cache* c, const char* key, int64_t value) {
   }
   if (k == "plan_ahead") {
     c->plan_ahead = value != 0;
+    return QC_OK;
+  }
+  if (k == "row_warps") {
+    if (value != 0 && value != 1 && value != 2 && value != 3 && value != 4 && value != 6) return QC_ERR_INVALID_ARG;
+    c->row_warps = static_cast<int>(value);
     return QC_OK;
   }
   if (k == "row_cluster") {

@@ -17,7 +17,8 @@ from parity_util import assert_close, f64
 
 pytestmark = pytest.mark.gpu
 
-# head_dim, query heads, KV heads, followers per leader, lengths (text, visual) per sequence, CTAs per row
+# head_dim, query heads, KV heads, followers per leader, lengths (text, visual) per sequence, CTAs per row (of six
+# warps) or warps of a row's only CTA
 SHAPES = {
     "a_page_or_two": (128, 2, 2, 1, [(1, 0), (14, 3), (15, 1), (16, 16)], 8),
     "fewer_pages_than_warps": (64, 3, 3, 2, [(30, 65), (47, 0), (33, 17)], 4),
@@ -26,6 +27,10 @@ SHAPES = {
     "group_of_seven": (128, 14, 2, 1, [(31, 300), (15, 129), (64, 0)], 2),
     "group_three_followers": (128, 4, 1, 3, [(47, 500)], 8),
     "group_in_two_slices": (64, 24, 2, 2, [(33, 250), (16, 90)], 5),
+    "four_warps": (128, 2, 2, 1, [(30, 200), (47, 190)], "row_warps 4"),
+    "three_warps": (64, 3, 3, 2, [(33, 17), (16, 95)], "row_warps 3"),
+    "two_warps": (128, 2, 2, 3, [(15, 300), (1, 0)], "row_warps 2"),
+    "one_warp": (128, 2, 2, 1, [(47, 700), (14, 33)], "row_warps 1"),
     "as_chosen": (128, 8, 2, 1, [(35, 400), (50, 380)], -1),
 }
 
@@ -47,7 +52,8 @@ def test_a_cluster_per_row(shape, mode):
     s = Session(n, hq, hkv, head_dim, layer_kind, max_seqs=b + 1, max_tokens_per_seq=longest + steps,
                 n_pages=2 * n * sum((t + steps + 31) // 16 + (v + 15) // 16 for t, v in lens), lazy_mode=mode, poison_pool=True)
     s.set_option("in_order_launches", 1)
-    s.set_option("row_cluster", cluster)
+    option, value = cluster.split() if isinstance(cluster, str) else ("row_cluster", cluster)
+    s.set_option(option, int(value))
     ids = list(range(b, 0, -1))
     for i, (text, vis) in enumerate(lens):
         _, k, v = W.prefill_kv_np(w, i)
