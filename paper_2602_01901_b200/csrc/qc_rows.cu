@@ -22,7 +22,8 @@
 // One query head per KV head: fp32 arithmetic on pairs.  Query groups: mma.m16n8k16 with keys as M and
 // the group as N, as in qc_attend_tc.cu, but with the weights as the sum of two bf16 values, a product each on the same V
 // fragment (error against 64 bits, 32 sequences of 1 120 tokens: 2.05e-3 in tile ranges, 2.11e-3 here with one bf16 value -- fewer,
-// longer pieces have fewer weights that are exactly 1 -- and 1.66e-3, the rounding of the output, with two; 17.6 and 17.7 us a layer).
+// longer pieces have fewer weights that are exactly 1 -- and 1.66e-3, the rounding of the output, with two; 17.9 us a layer with one, 17.7 with two and a
+// single tensor-map copy per tile).
 
 #include "qc_device.cuh"
 
