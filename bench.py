@@ -34,11 +34,11 @@ UNIT = "tokens/s"
 MODES = {"vla_qc": 0, "vla_eq8": 1, "gla": 2}
 
 # (dram__bytes_read.sum + dram__bytes_write.sum) / algorithmic K/V bytes of one attention launch of the
-# in-order schedule, from ncu captures of small cases of the same shapes (first 8 layers: launches of
-# 181-257 MB for the MHA kernel, 74-107 MB for the GQA kernel).  Every tile is fetched once and the
-# partial rows are written once per piece, so traffic grows in proportion to the K/V bytes swept and a
-# full-size launch's traffic is this ratio times its algorithmic bytes.
-NCU_TRAFFIC_RATIO = {"attend_kernel": 1.022, "attend_tc_kernel": 1.047}
+# in-order schedule, from ncu captures of small cases of the same shapes (first 4 layers: launches of
+# 27-253 MB with one query head per KV head, 6-107 MB with query groups; 1.028 for either, over all of
+# them).  Every tile is fetched once, pages that are not full in whole, so traffic grows in proportion
+# to the K/V bytes swept and a full-size launch's traffic is this ratio times its algorithmic bytes.
+NCU_TRAFFIC_RATIO = {"attend_rows_kernel": 1.028}
 
 
 def _peaks():
@@ -343,7 +343,7 @@ def measure_workload(args, w, mode, group, local_rank, world, rank, K, W_, Ke, e
     attention launch for the kernel's own time.  The one-launch schedule (every layer's q/k/v known
     up front, which only a harness has) is reported beside it."""
     peak, peak_kind = _peaks()
-    kernel = "attend_tc_kernel" if w.group > 1 else "attend_kernel"
+    kernel = "attend_rows_kernel"   # the in-order launches of these workloads give every output row its own blocks
     a = _Arms(args, w, mode, group, local_rank, rank * w.batch)
     a.set(IN_ORDER)
     for kv in args.option:
