@@ -70,7 +70,6 @@ __device__ __forceinline__ int32_t peer_load_s32(uint32_t addr) {
   asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Byte offset of 16-byte chunk `chunk` of row `row` in a tile: linear (MH), or as the tensor map's
 // 128-byte swizzle leaves it.
