@@ -661,18 +661,21 @@ cudaError_t with_rows_kernel(int d, bool mh, int nv, int warps, Fn fn) {
 
 }  // namespace
 
-cudaError_t configure_rows_kernels() {
-  for (int d = 64; d <= 128; d += 64)
-    for (int mh = 0; mh < 2; ++mh)
-      for (int warps : {1, 2, 3, 4, 6})
-        for (int nv = 1; nv <= kMaxCons; ++nv) {
-          const cudaError_t e = with_rows_kernel(d, mh != 0, nv, warps, [](auto kernel, int smem) {
-            cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            return r;
-          });
-          if (e != cudaSuccess) return e;
-        }
+// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone).
+cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers) {
+  for (int nv = 1; nv <= kMaxCons; ++nv) {
+    bool used = false;
+    for (const RowJobs& j : layers) used = used || (j.has_vis ? j.vis.n_cons : j.has_text ? j.text.n_cons : 0) == nv;
+    for (int warps : {6, 4, 3, 2, 1}) {
+      if (!used || (group > 1 && warps != 6)) continue;
+      const cudaError_t e = with_rows_kernel(d, group == 1, nv, warps, [](auto kernel, int smem) {
+        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        return r;
+      });
+      if (e != cudaSuccess) return e;
+    }
+  }
   return cudaSuccess;
 }
 

@@ -746,7 +746,6 @@ int32_t qc_init(int32_t device, void* cuda_stream, qc_ctx** out) {
   int smem = 0, smem_tc = 0;
   QC_CUDA(configure_kernels(&smem));
   QC_CUDA(configure_kernels_tc(&smem_tc));
-  QC_CUDA(configure_rows_kernels());
   QC_CUDA(configure_prefill_kernels());
   if (static_cast<size_t>(std::max(smem, smem_tc)) > prop.sharedMemPerBlockOptin) return QC_ERR_UNSUPPORTED;
   qc_ctx* ctx = new (std::nothrow) qc_ctx();
@@ -861,7 +860,8 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   }
 
   cudaStream_t stream = ctx->stream;
-  bool ok = cudaHostAlloc(reinterpret_cast<void**>(&c->pinned), kStageSlots * c->lay.step_bytes,
+  bool ok = !c->rows_fit || configure_rows_kernels(c->D, c->group, c->row_jobs) == cudaSuccess;
+  ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->pinned), kStageSlots * c->lay.step_bytes,
                           cudaHostAllocDefault) == cudaSuccess;
   for (int i = 0; ok && i < kStageSlots; ++i)
     ok = cudaEventCreateWithFlags(&c->stage_done[i], cudaEventDisableTiming) == cudaSuccess;
