@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
     x = MH ? pair : pair / n_heads, h = MH ? 0 : pair - x * n_heads;
   };
   auto mad = [](Vec& r, float w, const Vec& v) {
+    if (!(w > 0.f)) return;   // (no weight times an infinite element would not be a number)
     r.x = fmaf(v.x, w, r.x), r.y = fmaf(v.y, w, r.y);
     if constexpr (!MH) r.z = fmaf(v.z, w, r.z), r.w = fmaf(v.w, w, r.w);
   };
