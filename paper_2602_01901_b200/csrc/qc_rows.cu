@@ -373,10 +373,13 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
       }
     }
     uint32_t pb[2][2], pb_skip[2][2];   // query groups: the weights as B operands, in two parts
+    // The first part is the next bf16 value below the weight and the second what is left, so a weight that is not zero has
+    // two positive parts: an infinite value element stays infinite (times a zero or negative part it would not).
     auto operands = [&](uint32_t (&b)[2][2]) {
+      constexpr float kBelow = 1.f - 0x1p-24f;   // the largest float below 1
 #pragma unroll
       for (int j2 = 0; j2 < 2; ++j2) {
-        const uint32_t hi = pack_bf16x2(w[0][j2], w[NH - 1][j2]);
+        const uint32_t hi = pack_bf16x2_rz(w[0][j2] * kBelow, w[NH - 1][j2] * kBelow);
         b[0][j2] = movmatrix_trans(hi);
         b[1][j2] = movmatrix_trans(pack_bf16x2(w[0][j2] - __uint_as_float(hi << 16), w[NH - 1][j2] - __uint_as_float(hi & 0xffff0000u)));
       }

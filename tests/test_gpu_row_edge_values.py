@@ -80,8 +80,7 @@ def _check_infinite(got, ref):
     assert_close(torch.from_numpy(rest).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16), ref_rest, "finite elements")
 
 
-@pytest.mark.parametrize("split,heads,mode", [c for c in _cases([("row_cluster", 3), ("row_cluster", 5), ("row_warps", 2)])
-                                              if c.values[1][0] == c.values[1][1]])
+@pytest.mark.parametrize("split,heads,mode", _cases([("row_cluster", 3), ("row_cluster", 5), ("row_warps", 2)]))
 def test_an_infinite_value_makes_its_element_infinite_and_no_other(split, heads, mode):
     def change(k, v, text):
         # pages 13 and 25 of the 40: with three, resp. five thread blocks per row they are the last one's
