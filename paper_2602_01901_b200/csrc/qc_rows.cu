@@ -27,6 +27,7 @@
 
 #include "qc_device.cuh"
 
+#include <cfloat>
 #include <type_traits>
 
 namespace qc {
@@ -249,13 +250,15 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
     }
   }
 
-  float m[NC][NH], l[NC][NH];            // softmax references; this lane's parts of the sums of weights
+  // Softmax references and this lane's parts of the sums of weights.  References start at the lowest finite value: the
+  // weight of a score of minus infinity then is zero also in a warp whose first pages hold no other.
+  float m[NC][NH], l[NC][NH];
   float2 acc[MH ? NV : 1][MH ? EP2 : 1];
   float o[MH ? 1 : NV][MH ? 1 : KS][4];
 #pragma unroll
   for (int x = 0; x < NC; ++x)
 #pragma unroll
-    for (int h = 0; h < NH; ++h) m[x][h] = -INFINITY, l[x][h] = 0.f;
+    for (int h = 0; h < NH; ++h) m[x][h] = -FLT_MAX, l[x][h] = 0.f;
 #pragma unroll
   for (int x = 0; x < NV; ++x) {
     if constexpr (MH) {

@@ -89,3 +89,17 @@ def test_an_infinite_value_makes_its_element_infinite_and_no_other(split, heads,
         return k, v
 
     _check_infinite(*_case(split, heads, mode, 640, change))
+
+
+@pytest.mark.parametrize("split,heads,mode", _cases([("row_cluster", 1), ("row_cluster", 2), ("row_cluster", 8), ("row_warps", 1),
+                                                     ("row_warps", 3)]))
+def test_pages_of_keys_that_score_minus_infinity_count_for_nothing(split, heads, mode):
+    def change(k, v, text):
+        # all of the prompt's text and the second and third of 12 visual pages: the first page that some warp meets
+        k[:, :text, :, 0] = -float("inf")
+        k[:, text + 16:text + 48, :, 0] = -float("inf")
+        return k, v
+
+    got, ref = _case(split, heads, mode, 192, change)
+    assert np.isfinite(got).all()
+    assert_close(torch.from_numpy(got).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16), ref, "masked pages")
