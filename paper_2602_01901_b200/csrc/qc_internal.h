@@ -204,6 +204,8 @@ struct Params {
   int32_t row_cluster;               // > 0: the step's launches give every output row a cluster of that many CTAs, and what a
                                      // leader's launch leaves for a follower is one partial row (slot 0)
   int32_t row_warps;                 // warps of each of them
+  int32_t follows_setup;             // the launch directly before wrote the step's descriptors, page-table entries or plan:
+                                     // nothing of them is read ahead of the wait for it
   int32_t extra_key_leader;          // merge only, >= 0: the rows also take the step's new token as one more key,
                                      // scored by that layer's Q Cache entry and new k (Eq. 6), valued by the own new v
 };

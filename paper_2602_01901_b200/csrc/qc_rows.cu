@@ -122,8 +122,10 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
   }
   if (threadIdx.x == 0) S.dead = 0;
 
-  // ---- ahead of the wait for the previous kernel: the row, its page ids and the first tiles (the
-  // sequence descriptors, the page tables and the cached pages were written two or more launches back)
+  // ---- ahead of the wait for the previous kernel: the row, its page ids and the first tiles.  The sequence
+  // descriptors, the page tables and the cached pages were written two or more launches back, but for a step's first
+  // launch, which comes right after the one that writes the first two (its wait is 1 us of the 227 of a step of 32 layers).
+  if (P.follows_setup) pdl_wait();
   const int row = blockIdx.x / n_ctas, rows = P.heads_per_item_dim;
   const int si = row / rows, u = row - si * rows;
   const uint4 sq = *reinterpret_cast<const uint4*>(P.seqs + si);

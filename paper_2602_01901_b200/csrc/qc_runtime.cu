@@ -1261,6 +1261,7 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
   p.pos_begin = pb;
   p.pos_end = pe;
   p.extra_key_leader = c->groups[gi].extra_key_leader;
+  p.follows_setup = gi == 0 && !append_first;   // (an append waits for the set-up before it lets its successor start)
   bool has_work = p.item_end > p.item_begin;
   if (use_static) {   // (a step has at most n_layers <= 127 launches: every one has its entry)
     const LaunchDesc& one = launches.launch[gi];

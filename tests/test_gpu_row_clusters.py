@@ -85,3 +85,48 @@ def test_a_cluster_per_row(shape, mode):
             assert np.array_equal(s.read_qcache(l)[sid], qn[leader[l], i])
     assert s.stats().device_error == 0
     s.close()
+
+
+@pytest.mark.parametrize("entry", ["step", "layers"])
+@pytest.mark.parametrize("hq,hkv", [(4, 4), (8, 2)])
+def test_steps_enqueued_without_a_wait_between_them(hq, hkv, entry):
+    """The first launch of a step comes right after the one that writes the step's descriptors and new page-table
+    entries, in a stack of two layers every second one does: sequences in another order each step, pages that fill up
+    every few steps, nothing that lets one step finish before the next is enqueued."""
+    n, d, b, steps = 2, 128, 4, 48
+    text, vis = [29, 33, 38, 44], [200, 190, 180, 170]
+    s = Session(n, hq, hkv, d, [0, 0], max_seqs=b, max_tokens_per_seq=256, n_pages=2 * n * b * 24, poison_pool=True)
+    s.set_option("in_order_launches", 1)
+    o = LazyAttentionOracle(n, hq, hkv, d, [0, 0], qc.QC_MODE_VLA_QC, n_seqs=b)
+    gen = torch.Generator().manual_seed(21)
+
+    def normal(*size):
+        return torch.randn(size, generator=gen).to(torch.bfloat16)
+
+    for i in range(b):
+        kind = np.array([0] * text[i] + [1] * vis[i], np.uint8)
+        k, v = normal(n, len(kind), hkv, d), normal(n, len(kind), hkv, d)
+        s.prefill_append([i], [len(kind)], kind, k.to(s.device), v.to(s.device))
+        o.prefill_append(i, kind.tolist(), k.double().numpy(), v.double().numpy())
+    q, k, v = normal(steps, n, b, hq, d), normal(steps, n, b, hkv, d), normal(steps, n, b, hkv, d)
+    orders = [torch.randperm(b, generator=gen).tolist() for _ in range(steps)]
+    dq, dk, dv = (t.to(s.device) for t in (q, k, v))
+    out = torch.empty_like(dq)
+    launches = s.stats().kernel_launches
+    torch.cuda._sleep(20_000_000)   # the steps queue up behind this
+    for i in range(steps):
+        if entry == "step":
+            s.decode_step(orders[i], dq[i], dk[i], dv[i], out[i])
+        else:
+            s.decode_begin(orders[i])
+            for l in range(n):
+                s.decode_layer(l, dq[i, l], dk[i, l], dv[i, l], out[i, l])
+    assert s.stats().device_error == 0
+    assert s.stats().kernel_launches - launches == (1 + n) * steps   # set-up and a launch per layer
+    got = bits_of(out)
+    for i in range(steps):
+        for at, seq in enumerate(orders[i]):
+            ref, _ = o.decode_step(seq, *(t[i, :, at].double().numpy() for t in (q, k, v)))
+            for l in range(n):
+                assert_close(got[i, l, at], ref[l], f"step {i} sequence {seq} layer {l}")
+    s.close()
