@@ -347,6 +347,7 @@ __device__ __forceinline__ void attend_tc_worker(const Params& P, TcCtx* ctx, ui
   // only the layer's inputs.
   bool more;
   if (STATIC) {
+    if (P.follows_setup) pdl_wait();   // (a step's first launch: the plan or the descriptors are the previous kernel's)
     bool any = wid >= 0 && wid < P.part_workers;
     if (P.wdesc != nullptr) {
       // planned ahead: one read gives the first two items, the first page ids and the cursor

@@ -120,7 +120,8 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // starts running, the kernel before its predecessor -- and by induction everything earlier in
 // the stream -- has completed: what a kernel does ahead of its own wait may read anything that
 // was written two or more launches back (the attention kernels plan their first work items there,
-// from the launch plan, the step descriptors and the page tables).
+// from the launch plan, the step descriptors and the page tables; a step's first attention launch,
+// right behind the kernel that writes those, waits first).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

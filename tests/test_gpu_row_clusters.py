@@ -88,15 +88,17 @@ def test_a_cluster_per_row(shape, mode):
 
 
 @pytest.mark.parametrize("entry", ["step", "layers"])
+@pytest.mark.parametrize("options", [{}, {"row_cluster": 0}, {"plan_ahead": 0}], ids=["rows", "ranges", "unplanned_ranges"])
 @pytest.mark.parametrize("hq,hkv", [(4, 4), (8, 2)])
-def test_steps_enqueued_without_a_wait_between_them(hq, hkv, entry):
+def test_steps_enqueued_without_a_wait_between_them(hq, hkv, options, entry):
     """The first launch of a step comes right after the one that writes the step's descriptors and new page-table
     entries, in a stack of two layers every second one does: sequences in another order each step, pages that fill up
     every few steps, nothing that lets one step finish before the next is enqueued."""
     n, d, b, steps = 2, 128, 4, 48
     text, vis = [29, 33, 38, 44], [200, 190, 180, 170]
     s = Session(n, hq, hkv, d, [0, 0], max_seqs=b, max_tokens_per_seq=256, n_pages=2 * n * b * 24, poison_pool=True)
-    s.set_option("in_order_launches", 1)
+    for key, value in {"in_order_launches": 1, **options}.items():
+        s.set_option(key, value)
     o = LazyAttentionOracle(n, hq, hkv, d, [0, 0], qc.QC_MODE_VLA_QC, n_seqs=b)
     gen = torch.Generator().manual_seed(21)
 
@@ -122,7 +124,9 @@ def test_steps_enqueued_without_a_wait_between_them(hq, hkv, entry):
             for l in range(n):
                 s.decode_layer(l, dq[i, l], dk[i, l], dv[i, l], out[i, l])
     assert s.stats().device_error == 0
-    assert s.stats().kernel_launches - launches == (1 + n) * steps   # set-up and a launch per layer
+    # set-up, the plan of tile ranges, a launch per layer and the merge launches that these leave
+    merges = 0 if not options or (hq == hkv and "plan_ahead" not in options) else n
+    assert s.stats().kernel_launches - launches == (1 + ("row_cluster" in options) + n + merges) * steps
     got = bits_of(out)
     for i in range(steps):
         for at, seq in enumerate(orders[i]):
