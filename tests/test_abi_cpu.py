@@ -53,6 +53,25 @@ def test_sizes_and_argument_checks_without_a_device(lib):
     assert lib.qc_free(None, None) == qc.QC_OK
 
 
+@pytest.mark.parametrize("bad", [b"0123456789abcdef", "0123456789abcdef", (C.c_uint16 * 8)(), C.c_void_p(64), 64.0],
+                         ids=["bytes", "text", "array", "pointer_object", "float"])
+@pytest.mark.parametrize("at", range(5))
+def test_a_decode_call_takes_no_host_object_for_a_device_pointer(lib, bad, at):
+    pointers = [64, 64, 64, 64, 64]
+    pointers[at] = bad
+    with pytest.raises(TypeError):
+        qc.qc_decode_step(None, [0], *pointers)
+    with pytest.raises(TypeError):
+        qc.qc_decode_layer(None, 0, *pointers)
+    # what is an address is handed on: the missing cache is what is wrong here
+    for good in (64, 0, None, True):
+        pointers[at] = good
+        for call in (lambda: qc.qc_decode_step(None, [0], *pointers), lambda: qc.qc_decode_layer(None, 0, *pointers)):
+            with pytest.raises(qc.QcError) as e:
+                call()
+            assert e.value.status == qc.QC_ERR_INVALID_ARG
+
+
 def test_no_device_means_an_error_status_not_a_fallback(lib):
     import torch
 
