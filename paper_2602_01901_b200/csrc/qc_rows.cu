@@ -27,7 +27,9 @@
 
 #include "qc_device.cuh"
 
+#include <algorithm>
 #include <cfloat>
+#include <climits>
 #include <type_traits>
 
 namespace qc {
@@ -670,16 +672,32 @@ cudaError_t with_rows_kernel(int d, bool mh, int nv, int warps, Fn fn) {
 
 }  // namespace
 
-// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone).
-cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers) {
+// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone), and
+// the clusters of 1, 2, 4 and 8 six-warp CTAs that are resident at once of the one that holds the fewest.
+cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, int (&places)[4]) {
+  for (int& n : places) n = INT_MAX;
   for (int nv = 1; nv <= kMaxCons; ++nv) {
     bool used = false;
     for (const RowJobs& j : layers) used = used || (j.has_vis ? j.vis.n_cons : j.has_text ? j.text.n_cons : 0) == nv;
     for (int warps : {6, 4, 3, 2, 1}) {
       if (!used || (group > 1 && warps != 6)) continue;
-      const cudaError_t e = with_rows_kernel(d, group == 1, nv, warps, [](auto kernel, int smem) {
+      const cudaError_t e = with_rows_kernel(d, group == 1, nv, warps, [&](auto kernel, int smem) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        for (int i = 0; r == cudaSuccess && warps == 6 && i < 4; ++i) {
+          cudaLaunchConfig_t cfg{};
+          cfg.gridDim = dim3(1u << i);
+          cfg.blockDim = dim3(warps * 32);
+          cfg.dynamicSmemBytes = smem;
+          cudaLaunchAttribute attr;
+          attr.id = cudaLaunchAttributeClusterDimension;
+          attr.val.clusterDim.x = 1u << i, attr.val.clusterDim.y = 1, attr.val.clusterDim.z = 1;
+          cfg.attrs = &attr;
+          cfg.numAttrs = 1;
+          int n = 0;
+          r = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+          places[i] = std::min(places[i], n);
+        }
         return r;
       });
       if (e != cudaSuccess) return e;

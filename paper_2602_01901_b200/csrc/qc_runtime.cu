@@ -128,6 +128,7 @@ struct qc_cache {
   std::vector<int> inorder_extra_key;             // per layer: the leader whose new token the merge adds, or -1
   std::vector<RowJobs> row_jobs;                  // per layer, for launches that give every output row a cluster
   bool rows_fit = false;                          // every layer's sweeps have that form
+  int row_places[4] = {};                         // clusters of 1, 2, 4, 8 six-warp CTAs resident at once, fewest over the layers
   int row_warps = 0;                              // warps of a CTA where rows have one each: 0 chosen per step
   int row_cluster = -1;                           // CTAs per output row: -1 chosen per step, 0 never, n always n
   int slots_per_stream = 0;
@@ -860,7 +861,7 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   }
 
   cudaStream_t stream = ctx->stream;
-  bool ok = !c->rows_fit || configure_rows_kernels(c->D, c->group, c->row_jobs) == cudaSuccess;
+  bool ok = !c->rows_fit || configure_rows_kernels(c->D, c->group, c->row_jobs, c->row_places) == cudaSuccess;
   ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->pinned), kStageSlots * c->lay.step_bytes,
                           cudaHostAllocDefault) == cudaSuccess;
   for (int i = 0; ok && i < kStageSlots; ++i)
@@ -1318,12 +1319,20 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 
 // CTAs that an output row gets in the launches of a step of the in-order schedule, and their warps, or 0: its launches
 // are cut into tile ranges.
-// Up to 296 rows (two six-warp CTAs per SM): as many CTAs per row as leave one CTA per SM (the next launch then starts in the other
+// As long as every row's cluster is resident at once (six-warp CTAs fit an SM twice, 296 of them; clusters of two, four and eight
+// 148, 71 and 33 times): as many CTAs per row as leave one CTA per SM (the next launch then starts in the other
 // half of each SM, and its first tiles have landed when this one ends), twice that where a warp would still have more than six
 // pages.  us per layer, tile ranges / 1, 2, 4, 8 CTAs per row (* what the rule takes): 32 rows of 43 pages 9.54 / 10.2, 7.53, 6.92*,
-// 7.74; 32 of 188 13.8 / 30.2, 17.4, 12.4, 11.6*; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4; 256 of 188 55.5 / 52.7*, 54.6, 62.2; 256 of
+// 7.74; 32 of 188 13.8 / 30.2, 17.4, 12.4, 11.6*; 34 of 500 24.2 / 68.3, 37.3, 23.8*, 31.4; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4;
+// 256 of 188 55.5 / 52.7*, 54.6, 62.2; 256 of
 // 130, GLA, 34.4 / 32.7*, 32.8, 36.9; 32 of 43, 64-wide, GLA 7.50 / 8.0, 5.9, 5.09*, 4.94; with query groups 32 of 50 11.7 / 12.3, 9.27,
-// 8.34*, 9.98; 4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1; 128 of 71 20.2 / 18.7, 17.8*, 24.4.
+// 8.34*, 9.98; 4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1; 72 of 190 24.4 / 33.5, 21.8*, 31.0, 38.4;
+// 128 of 71 20.2 / 18.7, 17.8*, 24.4.
+// Query groups of 128-wide heads with two or three followers: their sums and tiles fit an SM once (148, 74, 33 and 15 clusters).  As many
+// CTAs per row as are resident, and ranges where a row's pages are too many for them: blocks of four, VLA_QC, 16 rows of 64 pages 13.5 / 18.6,
+// 12.7, 10.4*, 15.5; 64 of 64 16.1 / 19.1, 13.5*, 18.4; 64 of 190 22.5* / 44.6, 26.4; 128 of 21 13.6 / 11.1*, 15.1; 128 of 64 19.4* / 19.6,
+// 23.6; the same blocks in GLA, 16 of 64 10.4 / 17.6, 11.7, 8.3*, 12.3; 72 of 64 13.5 / 18.0, 12.7*, 20.9; 72 of 190 21.9* / 43.1, 24.7;
+// 80 of 64 13.8* / 18.1, 21.2; 16 of 500 24.0* / 106, 55.8, 30.1, 33.7.
 // More rows, no query groups: one CTA per row, with the most warps that leave every row resident.  Ranges / 6, 4, 3, 2, 1 warps:
 // 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
 // 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.
@@ -1347,10 +1356,17 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     longest = std::max(longest, n);
   }
   if (5 * longest * n_seqs > 8 * pages) return ranges;
-  if (rows <= n_sms * kAttendCtasPerSm) {
+  auto places = [&](int n) { return c->row_places[n == 8 ? 3 : n / 2]; };
+  if (rows <= places(1)) {
     int n = 8;
-    while (n > 1 && n * rows > n_sms) n /= 2;
-    if (n < 8 && 2 * n * rows <= n_sms * kAttendCtasPerSm && longest > 36 * n) n *= 2;
+    if (places(1) > n_sms) {
+      while (n > 1 && n * rows > n_sms) n /= 2;
+      if (n < 8 && rows <= places(2 * n) && longest > 36 * n) n *= 2;
+    } else {
+      while (rows > places(n)) n /= 2;
+      static constexpr int kMostPages[2][4] = {{45, 135, 300, 900}, {0, 85, 270, 900}};
+      if (longest > kMostPages[c->cfg.lazy_mode == QC_MODE_GLA][n == 8 ? 3 : n / 2]) return ranges;
+    }
     return RowSplit{n, kAttendWarps};
   }
   if (c->group > 1) return ranges;

@@ -1,0 +1,65 @@
+"""How the launches of a step are cut is chosen from the numbers of rows and pages: a choice that is slower than
+the library's other way of cutting the same step is a wrong choice.  Sizes where the places for thread blocks run
+out, or where a few rows are most of the work."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2602_01901_b200 import binding as qc
+from paper_2602_01901_b200.session import Session
+
+pytestmark = pytest.mark.gpu
+
+
+def _us_per_layer(s, n, b, steps=16):
+    """Best of three runs of `steps` steps, microseconds per layer."""
+    q = torch.randn(n, b, s.hq, s.d, device=s.device, dtype=torch.bfloat16)
+    k = torch.randn(n, b, s.hkv, s.d, device=s.device, dtype=torch.bfloat16)
+    out, ids, best = torch.empty_like(q), list(range(b)), float("inf")
+    for _ in range(3):
+        for _ in range(3):
+            s.decode_step(ids, q, k, k, out)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        torch.cuda._sleep(3_000_000)   # the steps queue up behind this
+        e[0].record()
+        for _ in range(steps):
+            s.decode_step(ids, q, k, k, out)
+        e[1].record()
+        torch.cuda.synchronize()
+        best = min(best, e[0].elapsed_time(e[1]) * 1e3 / steps / n)
+    return best
+
+
+def _not_slower_than_ranges(hq, hkv, d, layer_kind, mode, lens, margin=1.12):
+    n, b = len(layer_kind), len(lens)
+    s = Session(n, hq, hkv, d, layer_kind, max_seqs=b, max_tokens_per_seq=max(map(max, lens)) + 256,
+                n_pages=2 * n * sum(t // 16 + v // 16 + 12 for t, v in lens), lazy_mode=mode)
+    s.set_option("in_order_launches", 1)
+    for i, (text, vis) in enumerate(lens):
+        k = torch.randn(n, text + vis, hkv, d, device=s.device, dtype=torch.bfloat16)
+        s.prefill_append([i], [text + vis], np.array([0] * text + [1] * vis, np.uint8), k, k)
+    took = {}
+    for cluster in (-1, 0):
+        s.set_option("row_cluster", cluster)
+        took[cluster] = _us_per_layer(s, n, b)
+    assert s.stats().device_error == 0
+    s.close()
+    assert took[-1] <= margin * took[0], f"as chosen {took[-1]:.1f} us a layer, in tile ranges {took[0]:.1f}"
+
+
+BLOCKS_OF_4, BLOCKS_OF_2 = [0, 1, 1, 1] * 2, [0, 1] * 2
+
+
+@pytest.mark.parametrize("hq,hkv,block,mode,batch,tokens", [
+    (28, 4, BLOCKS_OF_4, qc.QC_MODE_GLA, 4, 1000),     # 16 rows: clusters of eight are resident fifteen times
+    (28, 4, BLOCKS_OF_4, qc.QC_MODE_VLA_QC, 20, 1000),   # 80 rows, one thread block per SM
+    (32, 8, BLOCKS_OF_4, qc.QC_MODE_GLA, 20, 1000),    # 160 rows, more than places
+    (28, 4, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, 18, 3000),   # 72 rows: clusters of four are resident 71 times
+    (34, 34, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, 1, 8000),   # 34 rows: clusters of eight are resident 33 times
+])
+def test_rows_get_no_more_thread_blocks_than_are_resident(hq, hkv, block, mode, batch, tokens):
+    _not_slower_than_ranges(hq, hkv, 128, block, mode, [(60, tokens - 60)] * batch)
