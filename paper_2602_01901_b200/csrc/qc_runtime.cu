@@ -1328,6 +1328,10 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // 130, GLA, 34.4 / 32.7*, 32.8, 36.9; 32 of 43, 64-wide, GLA 7.50 / 8.0, 5.9, 5.09*, 4.94; with query groups 32 of 50 11.7 / 12.3, 9.27,
 // 8.34*, 9.98; 4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1; 72 of 190 24.4 / 33.5, 21.8*, 31.0, 38.4;
 // 128 of 71 20.2 / 18.7, 17.8*, 24.4.
+// Few rows, eight CTAs each, leave SMs idle, and ranges are the better the longer the rows are; that they pay for it in merges of hundreds of
+// partials per row decides where: one query head, VLA, 4 rows of 1 000 pages 21.7 / 21.3*, of 1 880 24.7* / 35.2, 8 of 500 17.1 / 14.1*, of
+// 1 000 19.9 / 21.7*, of 1 880 26.4* / 35.7; GLA blocks of four, 8 of 1 000 24.4 / 18.0*, of 1 880 29.6 / 30.6*; query groups, VLA, 4 of 1 000
+// 45.3 / 25.1*, of 2 000 48.8 / 42.9*, of 3 760 55.8* / 74.7.
 // Query groups of 128-wide heads with two or three followers: their sums and tiles fit an SM once (148, 74, 33 and 15 clusters).  As many
 // CTAs per row as are resident, and ranges where a row's pages are too many for them: blocks of four, VLA_QC, 16 rows of 64 pages 13.5 / 18.6,
 // 12.7, 10.4*, 15.5; 64 of 64 16.1 / 19.1, 13.5*, 18.4; 64 of 190 22.5* / 44.6, 26.4; 128 of 21 13.6 / 11.1*, 15.1; 128 of 64 19.4* / 19.6,
@@ -1362,6 +1366,7 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     if (places(1) > n_sms) {
       while (n > 1 && n * rows > n_sms) n /= 2;
       if (n < 8 && rows <= places(2 * n) && longest > 36 * n) n *= 2;
+      if (8 * rows <= n_sms && longest > ((c->cfg.lazy_mode == QC_MODE_GLA) == (c->group > 1) ? 1000 : 2000)) return ranges;
     } else {
       while (rows > places(n)) n /= 2;
       static constexpr int kMostPages[2][4] = {{45, 135, 300, 900}, {0, 85, 270, 900}};

@@ -63,3 +63,8 @@ BLOCKS_OF_4, BLOCKS_OF_2 = [0, 1, 1, 1] * 2, [0, 1] * 2
 ])
 def test_rows_get_no_more_thread_blocks_than_are_resident(hq, hkv, block, mode, batch, tokens):
     _not_slower_than_ranges(hq, hkv, 128, block, mode, [(60, tokens - 60)] * batch)
+
+
+@pytest.mark.parametrize("heads,d,tokens", [(8, 128, 32000), (4, 64, 32000), (2, 128, 48000)])
+def test_a_few_very_long_rows_use_the_whole_chip(heads, d, tokens):
+    _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(100, tokens)])
