@@ -128,6 +128,7 @@ struct qc_cache {
   std::vector<int> inorder_extra_key;             // per layer: the leader whose new token the merge adds, or -1
   std::vector<RowJobs> row_jobs;                  // per layer, for launches that give every output row a cluster
   bool rows_fit = false;                          // every layer's sweeps have that form
+  int text_launches = 0, no_launches = 0;         // layers whose launch sweeps the text alone, that have no sweep
   int row_places[4] = {};                         // clusters of 1, 2, 4, 8 six-warp CTAs resident at once, fewest over the layers
   int row_warps = 0;                              // warps of a CTA where rows have one each: 0 chosen per step
   int row_cluster = -1;                           // CTAs per output row: -1 chosen per step, 0 never, n always n
@@ -403,6 +404,8 @@ void build_row_jobs(qc_cache* c) {
       (job.stream ? r.vis : r.text) = job;
     }
     r.add_earlier = r.has_text && !r.has_vis;
+    c->text_launches += r.add_earlier;
+    c->no_launches += !r.has_text && !r.has_vis;
   }
 }
 
@@ -1341,7 +1344,8 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
 // 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.
 // A launch takes as long as its longest row: batches whose longest row is over 1.6 times the average one stay with the
-// ranges, and one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
+// ranges.  Followers that sweep the text alone are launches of their own in this: sequences of as many tokens, one with 3 000 of text and seven
+// with 16, 54.9* / 65.1; 16 of 600 or 16 28.8* / 29.5 (query groups lose more to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  And one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
 // 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
 struct RowSplit {
   int cluster, warps;
@@ -1352,14 +1356,17 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   if (c->group == 1 && c->row_warps > 0) return RowSplit{1, c->row_warps};
   if (c->row_cluster > 0) return RowSplit{c->row_cluster, kAttendWarps};
   const int rows = n_seqs * c->items_per_chunk, n_sms = c->ctx->n_sms;
-  int64_t pages = 0, longest = 0;
+  int64_t pages = 0, longest = 0, pages_t = 0, longest_t = 0;   // of a row in a launch; in one that sweeps the text alone
   for (int i = 0; i < n_seqs; ++i) {
     const SeqState& st = c->seqs[seq_ids[i]];
-    const int64_t n = pages_for(st.len_vis) + pages_for(st.len_text);
+    const int64_t t = pages_for(st.len_text), n = pages_for(st.len_vis) + t;
     pages += n;
+    pages_t += t;
     longest = std::max(longest, n);
+    longest_t = std::max(longest_t, t);
   }
-  if (5 * longest * n_seqs > 8 * pages) return ranges;
+  const int text_launches = c->group > 1 ? 0 : c->text_launches, launches = c->group > 1 ? 1 : c->cfg.n_layers - c->no_launches - text_launches;
+  if (5 * n_seqs * (launches * longest + text_launches * longest_t) > 8 * (launches * pages + text_launches * pages_t)) return ranges;
   auto places = [&](int n) { return c->row_places[n == 8 ? 3 : n / 2]; };
   if (rows <= places(1)) {
     int n = 8;

@@ -68,3 +68,7 @@ def test_rows_get_no_more_thread_blocks_than_are_resident(hq, hkv, block, mode, 
 @pytest.mark.parametrize("heads,d,tokens", [(8, 128, 32000), (4, 64, 32000), (2, 128, 48000)])
 def test_a_few_very_long_rows_use_the_whole_chip(heads, d, tokens):
     _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(100, tokens)])
+
+
+def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges():
+    _not_slower_than_ranges(32, 32, 128, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(3000, 16)] + [(16, 3000)] * 7)
