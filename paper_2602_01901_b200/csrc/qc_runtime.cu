@@ -409,6 +409,9 @@ void build_row_jobs(qc_cache* c) {
   }
 }
 
+int default_row_cost(const qc_cache* c) { return c->group > 1 ? 12 : 4; }
+int default_min_tiles(const qc_cache* c) { return c->group > 1 ? 4 : 1; }
+
 struct Sizes {
   int D, hq, hkv, max_pages, chunk_pages, max_slots, slots_per_stream;
   int64_t n_pool_pages;
@@ -795,8 +798,8 @@ int32_t qc_alloc_cache(qc_ctx* ctx, const qc_config* cfg, void* pool_dev, size_t
   c->heads_per_item = c->group > 1 ? 8 : 1;
   // what one more item costs a worker, in tiles: a query-group item fetches its query fragments when it
   // starts and leaves up to eight partial rows (measured on launches of one layer: 4 resp. 12 best)
-  c->static_row_cost = c->group > 1 ? 12 : 4;
-  c->static_min_tiles = c->group > 1 ? 4 : 1;
+  c->static_row_cost = default_row_cost(c);
+  c->static_min_tiles = default_min_tiles(c);
   c->items_per_chunk = c->group > 1 ? s.hkv * ((c->group + 7) / 8) : s.hq;
   c->paged = cfg->page_size == 16;
   c->max_pages = s.max_pages;
@@ -1352,7 +1355,9 @@ struct RowSplit {
 };
 RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids) {
   const RowSplit ranges{0, 0};
-  if (!c->rows_fit || c->static_partition != -1 || !c->plan_ahead || !c->fused_merge || c->row_cluster == 0) return ranges;
+  if (!c->rows_fit || c->static_partition != -1 || !c->plan_ahead || !c->fused_merge || c->row_cluster == 0 ||
+      c->static_row_cost != default_row_cost(c) || c->static_min_tiles != default_min_tiles(c))
+    return ranges;
   if (c->group == 1 && c->row_warps > 0) return RowSplit{1, c->row_warps};
   if (c->row_cluster > 0) return RowSplit{c->row_cluster, kAttendWarps};
   const int rows = n_seqs * c->items_per_chunk, n_sms = c->ctx->n_sms;

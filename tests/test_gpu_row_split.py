@@ -72,3 +72,27 @@ def test_a_few_very_long_rows_use_the_whole_chip(heads, d, tokens):
 
 def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges():
     _not_slower_than_ranges(32, 32, 128, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(3000, 16)] + [(16, 3000)] * 7)
+
+
+@pytest.mark.parametrize("hq,hkv", [(4, 4), (8, 2)])
+@pytest.mark.parametrize("key,value", [("static_min_tiles", 7), ("static_row_cost", 9), ("static_partition", 1), ("plan_ahead", 0),
+                                       ("fused_merge", 0), ("fold_append", 0), ("row_cluster", 0)])
+def test_an_option_of_the_tile_ranges_is_answered_by_tile_ranges(key, value, hq, hkv):
+    n, b = 4, 2
+    s = Session(n, hq, hkv, 128, [0, 1, 0, 1], max_seqs=b, max_tokens_per_seq=400, n_pages=2 * n * b * 30)
+    s.set_option("in_order_launches", 1)
+    k = torch.randn(n, 330 * b, hkv, 128, device=s.device, dtype=torch.bfloat16)
+    s.prefill_append([0, 1], [330] * b, np.array(([0] * 30 + [1] * 300) * b, np.uint8), k, k)
+    q, out = (torch.randn(n, b, hq, 128, device=s.device, dtype=torch.bfloat16) for _ in range(2))
+    new = torch.randn(n, b, hkv, 128, device=s.device, dtype=torch.bfloat16)
+
+    def launches():
+        before = s.stats().kernel_launches
+        s.decode_step([0, 1], q, new, new, out)
+        return s.stats().kernel_launches - before
+
+    assert launches() == 1 + n     # set-up, and a launch that finishes its rows for each layer
+    s.set_option(key, value)
+    assert launches() > 1 + n      # a plan, an append or merges besides
+    assert s.stats().device_error == 0
+    s.close()
