@@ -857,20 +857,24 @@ __device__ __forceinline__ void store_row(const Params& P, int layer, int si, in
 // lengths; launches of one layer under the static partition have them planned; otherwise the
 // sweeps recorded them.  P.extra_key_leader >= 0 adds the step's new token as one more key (rows of
 // a GLA follower under the in-order schedule; Eq. 6).
-template <int D>
+// ROWS: the step's rows had thread blocks of their own, what there is is one partial row from the leader's launch (an
+// instantiation of its own: with both in one, two turns of 8 steps of a 64-wide GLA stack took 1 272 us, now 1 223, and a step of
+// two layers with claimed items 14.6 us, now 14.45).
+template <int D, bool ROWS>
 __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, int head, int lane) {
   constexpr int VPL = D / 32;
   const size_t base = (static_cast<size_t>(layer) * P.max_seqs + si) * P.max_slots;
   const int kvh = head / P.group, extra_leader = P.extra_key_leader;
   const StepSeq sq = P.seqs[si];
   int nv = sq.ncv, nt = sq.n_slots - sq.ncv, text0 = sq.ncv;
-  if (P.planned_pieces) {
+  if (ROWS) {
+    nv = 1, nt = 0;
+  } else if (P.planned_pieces) {
     const int hpi = P.heads_per_item, n_sub = (P.group + hpi - 1) / hpi, rows = P.heads_per_item_dim;
     const int u = kvh * n_sub + (head - kvh * P.group) / hpi;
     const uint32_t both = __ldcg(P.row_pieces + (static_cast<size_t>(P.launch_index) * P.max_seqs + si) * rows + u);
     nv = both & 0xffffu, nt = both >> 16, text0 = P.slots_per_stream;
   }
-  if (P.row_cluster > 0) nv = 1, nt = 0;
   const int pos = sq.len_text - 1;
   int pid = 0, pid_v = -1;
   if (extra_leader >= 0) {
@@ -887,7 +891,7 @@ __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, in
     l2_prefetch(P.v + ((static_cast<size_t>(layer) * P.n_seqs + si) * P.hkv + kvh) * D + lane * 64);
   pdl_wait();
   pdl_launch_dependents();
-  if (P.part_static && !P.planned_pieces && P.row_cluster == 0) {
+  if (!ROWS && P.part_static && !P.planned_pieces) {
     const size_t row = (static_cast<size_t>(layer) * P.max_seqs + si) * P.hq + head;
     const uint32_t both = __ldcg(reinterpret_cast<const uint32_t*>(P.row_slots + 2 * row));
     nv = sq.len_vis > 0 ? static_cast<int>(both & 0xffffu) : 0;

@@ -850,7 +850,7 @@ __global__ void __launch_bounds__(kThreads, kAttendCtasPerSm) attend_kernel(cons
 // One warp per (layer, sequence, head).  What it reads besides the partials (the sequence's
 // descriptor, the numbers of partials where they are planned, page ids) was written when the step
 // began and is read ahead of the wait for the attention kernel, so that one round of reads is left.
-template <int D>
+template <int D, bool ROWS>
 __global__ void merge_kernel(const __grid_constant__ Params P) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_layers = P.layer_end - P.layer_begin;
@@ -859,7 +859,7 @@ __global__ void merge_kernel(const __grid_constant__ Params P) {
     pdl_wait();
     return;
   }
-  merge_row<D>(P, P.layer_begin + idx / (P.hq * P.n_seqs), (idx / P.hq) % P.n_seqs, idx % P.hq, lane);
+  merge_row<D, ROWS>(P, P.layer_begin + idx / (P.hq * P.n_seqs), (idx / P.hq) % P.n_seqs, idx % P.hq, lane);
 }
 
 template <int D>
@@ -950,8 +950,11 @@ cudaError_t launch_merge(const Params& p, cudaStream_t stream) {
   const int warps_per_block = 8;
   const int blocks = (n + warps_per_block - 1) / warps_per_block;
   const dim3 grid(blocks), block(warps_per_block * 32);
-  if (p.d == 128) return launch_pdl(merge_kernel<128>, grid, block, 0, stream, p);
-  return launch_pdl(merge_kernel<64>, grid, block, 0, stream, p);
+  if (p.d == 128)
+    return p.row_cluster > 0 ? launch_pdl(merge_kernel<128, true>, grid, block, 0, stream, p)
+                             : launch_pdl(merge_kernel<128, false>, grid, block, 0, stream, p);
+  return p.row_cluster > 0 ? launch_pdl(merge_kernel<64, true>, grid, block, 0, stream, p)
+                           : launch_pdl(merge_kernel<64, false>, grid, block, 0, stream, p);
 }
 
 cudaError_t launch_prefill_store(const Params& p, const StoreMaps& maps, const StoreList& list, int blocks, cudaStream_t stream) {
