@@ -225,7 +225,7 @@ struct RowJobs {
   int32_t add_earlier;   // the rows also take what the leader's launch left for the layer
   int32_t pad;
 };
-cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, cudaStream_t stream);   // p.row_cluster, p.row_warps
+cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int n_sms, cudaStream_t stream);   // p.row_cluster, p.row_warps
 cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, int (&places)[4]);
 // Up to 16 consecutive tokens of one sequence and stream that go to one page.
 struct __align__(16) StoreSeg {

@@ -1312,7 +1312,7 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
     QC_CUDA(cudaEventRecord(evl[0], stream));
   }
   // (a GLA follower of the in-order schedule has nothing to sweep: its merge does everything)
-  if (has_work && by_rows) QC_CUDA(launch_attend_rows(p, *row_jobs, stream));
+  if (has_work && by_rows) QC_CUDA(launch_attend_rows(p, *row_jobs, c->ctx->n_sms, stream));
   else if (has_work) QC_CUDA(c->group > 1 ? launch_attend_tc(p, c->ctx->n_sms, stream) : launch_attend(p, c->ctx->n_sms, stream));
   if (evl) QC_CUDA(cudaEventRecord(evl[1], stream));
   if (ev && gi + 1 == c->groups.size()) QC_CUDA(cudaEventRecord(ev[2], stream));

@@ -60,6 +60,7 @@ BLOCKS_OF_4, BLOCKS_OF_2 = [0, 1, 1, 1] * 2, [0, 1] * 2
     (32, 8, BLOCKS_OF_4, qc.QC_MODE_GLA, 20, 1000),    # 160 rows, more than places
     (28, 4, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, 18, 3000),   # 72 rows: clusters of four are resident 71 times
     (34, 34, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, 1, 8000),   # 34 rows: clusters of eight are resident 33 times
+    (40, 40, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, 32, 300),   # 1 280 rows of one warp: an SM holds eight clusters at most
 ])
 def test_rows_get_no_more_thread_blocks_than_are_resident(hq, hkv, block, mode, batch, tokens):
     _not_slower_than_ranges(hq, hkv, 128, block, mode, [(60, tokens - 60)] * batch)
