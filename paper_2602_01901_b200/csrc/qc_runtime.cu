@@ -1346,9 +1346,15 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // More rows, no query groups: one CTA per row, with the most warps that leave every row resident.  Ranges / 6, 4, 3, 2, 1 warps:
 // 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
 // 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.
-// A launch takes as long as its longest row: batches whose longest row is over 1.6 times the average one stay with the
-// ranges.  Followers that sweep the text alone are launches of their own in this: sequences of as many tokens, one with 3 000 of text and seven
-// with 16, 54.9* / 65.1; 16 of 600 or 16 28.8* / 29.5 (query groups lose more to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  And one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
+// A launch takes as long as its longest row.  Batches whose longest row is over 1.6 times the average one stay with the
+// ranges, and so do those where it has more pages than the average one by what a launch's start and end are worth: 32 for each
+// six-warp CTA of a row (half of that for 64-wide heads), 50 for rows of fewer warps, 64 for query groups.  Ranges / rows, by pages more than the average:
+// 256 rows of 188 pages 31 45.5 / 44.8*; 240 of 251 38 68.4* / 70.3, 64 61.3* / 66.2; 480 of 251 35 86.3 / 82.6*, 58 78.1* / 78.6;
+// 384 of 188 42 61.3 / 58.8*; 64-wide, 240 of 251 46 33.2* / 34.9, 112 of 501 74 32.4* / 35.4; query groups, 240 of 251
+// 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6.
+// Followers that sweep the text alone are launches of their own in both: sequences of as many tokens, one with 3 000 of text and
+// seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 (query groups lose more
+// to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  One warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
 // 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
 struct RowSplit {
   int cluster, warps;
@@ -1370,9 +1376,14 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     longest = std::max(longest, n);
     longest_t = std::max(longest_t, t);
   }
-  const int text_launches = c->group > 1 ? 0 : c->text_launches, launches = c->group > 1 ? 1 : c->cfg.n_layers - c->no_launches - text_launches;
-  if (5 * n_seqs * (launches * longest + text_launches * longest_t) > 8 * (launches * pages + text_launches * pages_t)) return ranges;
+  // pages of the longest row, summed over the step's launches, and of all rows
+  const int64_t text_launches = c->group > 1 ? 0 : c->text_launches;
+  const int64_t launches = c->group > 1 ? 1 : c->cfg.n_layers - c->no_launches - text_launches;
+  const int64_t worst = launches * longest + text_launches * longest_t, all = launches * pages + text_launches * pages_t;
+  if (5 * worst * n_seqs > 8 * all) return ranges;
   auto places = [&](int n) { return c->row_places[n == 8 ? 3 : n / 2]; };
+  RowSplit split = ranges;
+  int64_t most = 50;   // pages that the longest row may have more than the average one
   if (rows <= places(1)) {
     int n = 8;
     if (places(1) > n_sms) {
@@ -1384,12 +1395,15 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
       static constexpr int kMostPages[2][4] = {{45, 135, 300, 900}, {0, 85, 270, 900}};
       if (longest > kMostPages[c->cfg.lazy_mode == QC_MODE_GLA][n == 8 ? 3 : n / 2]) return ranges;
     }
-    return RowSplit{n, kAttendWarps};
+    split = RowSplit{n, kAttendWarps};
+    most = c->group > 1 ? 64 : n * c->D / 4;
+  } else if (c->group == 1) {
+    for (int warps : {1, 2, 3, 4})
+      if (rows <= n_sms * (kWorkersPerSm / warps)) split = RowSplit{1, warps};
+    if (split.warps == 1 && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
   }
-  if (c->group > 1) return ranges;
-  for (int warps : {4, 3, 2, 1})
-    if (rows <= n_sms * (kWorkersPerSm / warps)) return RowSplit{1, warps == 1 && 20 * longest * n_seqs > 23 * pages ? 3 : warps};
-  return ranges;
+  if (worst * n_seqs - all > most * n_seqs * (launches + text_launches)) return ranges;
+  return split;
 }
 
 int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const void* q_dev, const void* k_dev,

@@ -71,6 +71,15 @@ def test_a_few_very_long_rows_use_the_whole_chip(heads, d, tokens):
     _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(100, tokens)])
 
 
+@pytest.mark.parametrize("heads,d,lens", [
+    (16, 128, [(18, 4000), (4000, 18)] * 7),
+    (16, 64, [(60, int(7900 * f)) for f in (1, .62, .75, .68, .97, .88, .71, .82)]),
+    (16, 128, [(60, int(3900 * (1 - 0.035 * i))) for i in range(15)]),
+], ids=["text_of_half_the_batch", "64_wide", "six_tenths_to_one"])
+def test_rows_that_are_longer_than_others_by_many_pages(heads, d, lens):
+    _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens, margin=1.05)
+
+
 def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges():
     _not_slower_than_ranges(32, 32, 128, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(3000, 16)] + [(16, 3000)] * 7)
 
