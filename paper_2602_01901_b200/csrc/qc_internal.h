@@ -226,7 +226,11 @@ struct RowJobs {
   int32_t pad;
 };
 cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int n_sms, cudaStream_t stream);   // p.row_cluster, p.row_warps
-cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, int (&places)[4]);
+struct RowPlaces {           // what is resident at once, fewest over a cache's layers
+  int clusters[4] = {};      // clusters of 1, 2, 4, 8 six-warp CTAs
+  int per_sm[5] = {};        // CTAs of 1 .. 4 warps per SM, without query groups
+};
+cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, RowPlaces& places);
 // Up to 16 consecutive tokens of one sequence and stream that go to one page.
 struct __align__(16) StoreSeg {
   int32_t seq, ord;   // sequence; first token's ordinal in its stream, the stream in the top bit

@@ -35,7 +35,7 @@
 namespace qc {
 namespace {
 
-// Warps per CTA (W): six, or fewer where rows are many; an SM holds twelve in all.  Tiles in flight per warp (RING): four
+// Warps per CTA (W): six, or fewer where rows are many; an SM holds twelve in all (64-wide heads sixteen).  Tiles in flight per warp (RING): four
 // where the next launch's first tiles are to land during this one; two where the launch is bound by HBM, which
 // scattered tiles use worse the more there are in flight (512 rows of 43 pages, 3 warps: 27.5 us a layer with four, 27.0 with two).
 
@@ -672,10 +672,11 @@ cudaError_t with_rows_kernel(int d, bool mh, int nv, int warps, Fn fn) {
 
 }  // namespace
 
-// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone), and
-// the clusters of 1, 2, 4 and 8 six-warp CTAs that are resident at once of the one that holds the fewest.
-cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, int (&places)[4]) {
-  for (int& n : places) n = INT_MAX;
+// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone), and what
+// is resident of the one that fits least.
+cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, RowPlaces& places) {
+  for (int& n : places.clusters) n = INT_MAX;
+  for (int& n : places.per_sm) n = INT_MAX;
   for (int nv = 1; nv <= kMaxCons; ++nv) {
     bool used = false;
     for (const RowJobs& j : layers) used = used || (j.has_vis ? j.vis.n_cons : j.has_text ? j.text.n_cons : 0) == nv;
@@ -684,6 +685,11 @@ cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>&
       const cudaError_t e = with_rows_kernel(d, group == 1, nv, warps, [&](auto kernel, int smem) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        int n = 0;
+        if (r == cudaSuccess && warps < 6) {
+          r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, warps * 32, smem);
+          places.per_sm[warps] = std::min(places.per_sm[warps], n);
+        }
         for (int i = 0; r == cudaSuccess && warps == 6 && i < 4; ++i) {
           cudaLaunchConfig_t cfg{};
           cfg.gridDim = dim3(1u << i);
@@ -694,9 +700,8 @@ cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>&
           attr.val.clusterDim.x = 1u << i, attr.val.clusterDim.y = 1, attr.val.clusterDim.z = 1;
           cfg.attrs = &attr;
           cfg.numAttrs = 1;
-          int n = 0;
           r = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-          places[i] = std::min(places[i], n);
+          places.clusters[i] = std::min(places.clusters[i], n);
         }
         return r;
       });

@@ -129,7 +129,7 @@ struct qc_cache {
   std::vector<RowJobs> row_jobs;                  // per layer, for launches that give every output row a cluster
   bool rows_fit = false;                          // every layer's sweeps have that form
   int text_launches = 0, no_launches = 0;         // layers whose launch sweeps the text alone, that have no sweep
-  int row_places[4] = {};                         // clusters of 1, 2, 4, 8 six-warp CTAs resident at once, fewest over the layers
+  RowPlaces row_places;                           // thread blocks of such launches that are resident at once
   int row_warps = 0;                              // warps of a CTA where rows have one each: 0 chosen per step
   int row_cluster = -1;                           // CTAs per output row: -1 chosen per step, 0 never, n always n
   int slots_per_stream = 0;
@@ -1345,7 +1345,9 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // 80 of 64 13.8* / 18.1, 21.2; 16 of 500 24.0* / 106, 55.8, 30.1, 33.7.
 // More rows, no query groups: one CTA per row, with the most warps that leave every row resident.  Ranges / 6, 4, 3, 2, 1 warps:
 // 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
-// 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.
+// 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.  64-wide
+// heads, of which an SM holds more: 480 of 63 25.2 / 25.7, 20.2*, 23.1, 27.5, 43.8; 640 of 63 32.2 / 37.4, 37.0, 25.3*, 31.0, 47.6; 900 of 63
+// 40.8 / 48.7, 40.1, 46.8, 34.0*, 48.2; 640 of 19, GLA blocks of four (fewer again), 12.9 / 13.7, 11.8, 13.4, 10.2*, 14.3.
 // A launch takes as long as its longest row.  Batches whose longest row is over 1.6 times the average one stay with the
 // ranges, and so do those where it has more pages than the average one by what a launch's start and end are worth: 32 for each
 // six-warp CTA of a row (half of that for 64-wide heads), 50 for rows of fewer warps, 64 for query groups.  Ranges / rows, by pages more than the average:
@@ -1354,8 +1356,9 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6.
 // Followers that sweep the text alone are launches of their own in both: sequences of as many tokens, one with 3 000 of text and
 // seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 (query groups lose more
-// to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  One warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
-// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
+// to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  Up to 1 184 rows one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
+// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; beyond that blocks of three run in a third wave: 1 280 of 4 to 6 pages 20.6 / 27.7, 21.3, 19.2,
+// 16.4, 15.7*, of 10 to 32 42.2 / 45.7, 40.0, 40.2, 40.4, 39.3*; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
 struct RowSplit {
   int cluster, warps;
 };
@@ -1381,7 +1384,7 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   const int64_t launches = c->group > 1 ? 1 : c->cfg.n_layers - c->no_launches - text_launches;
   const int64_t worst = launches * longest + text_launches * longest_t, all = launches * pages + text_launches * pages_t;
   if (5 * worst * n_seqs > 8 * all) return ranges;
-  auto places = [&](int n) { return c->row_places[n == 8 ? 3 : n / 2]; };
+  auto places = [&](int n) { return c->row_places.clusters[n == 8 ? 3 : n / 2]; };
   RowSplit split = ranges;
   int64_t most = 50;   // pages that the longest row may have more than the average one
   if (rows <= places(1)) {
@@ -1399,8 +1402,8 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     most = c->group > 1 ? 64 : n * c->D / 4;
   } else if (c->group == 1) {
     for (int warps : {1, 2, 3, 4})
-      if (rows <= n_sms * (kWorkersPerSm / warps)) split = RowSplit{1, warps};
-    if (split.warps == 1 && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
+      if (rows <= n_sms * (warps == 1 ? kWorkersPerSm : c->row_places.per_sm[warps])) split = RowSplit{1, warps};
+    if (split.warps == 1 && rows <= 8 * n_sms && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
   }
   if (worst * n_seqs - all > most * n_seqs * (launches + text_launches)) return ranges;
   return split;

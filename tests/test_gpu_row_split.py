@@ -34,7 +34,7 @@ def _us_per_layer(s, n, b, steps=16):
     return best
 
 
-def _not_slower_than_ranges(hq, hkv, d, layer_kind, mode, lens, margin=1.12):
+def _not_slower_than_ranges(hq, hkv, d, layer_kind, mode, lens, margin=1.12, other=("row_cluster", 0)):
     n, b = len(layer_kind), len(lens)
     s = Session(n, hq, hkv, d, layer_kind, max_seqs=b, max_tokens_per_seq=max(map(max, lens)) + 256,
                 n_pages=2 * n * sum(t // 16 + v // 16 + 12 for t, v in lens), lazy_mode=mode)
@@ -42,13 +42,12 @@ def _not_slower_than_ranges(hq, hkv, d, layer_kind, mode, lens, margin=1.12):
     for i, (text, vis) in enumerate(lens):
         k = torch.randn(n, text + vis, hkv, d, device=s.device, dtype=torch.bfloat16)
         s.prefill_append([i], [text + vis], np.array([0] * text + [1] * vis, np.uint8), k, k)
-    took = {}
-    for cluster in (-1, 0):
-        s.set_option("row_cluster", cluster)
-        took[cluster] = _us_per_layer(s, n, b)
+    chosen = _us_per_layer(s, n, b)
+    s.set_option(*other)
+    us = _us_per_layer(s, n, b)
     assert s.stats().device_error == 0
     s.close()
-    assert took[-1] <= margin * took[0], f"as chosen {took[-1]:.1f} us a layer, in tile ranges {took[0]:.1f}"
+    assert chosen <= margin * us, f"as chosen {chosen:.1f} us a layer, with {other[0]} {other[1]} {us:.1f}"
 
 
 BLOCKS_OF_4, BLOCKS_OF_2 = [0, 1, 1, 1] * 2, [0, 1] * 2
@@ -64,6 +63,14 @@ BLOCKS_OF_4, BLOCKS_OF_2 = [0, 1, 1, 1] * 2, [0, 1] * 2
 ])
 def test_rows_get_no_more_thread_blocks_than_are_resident(hq, hkv, block, mode, batch, tokens):
     _not_slower_than_ranges(hq, hkv, 128, block, mode, [(60, tokens - 60)] * batch)
+
+
+@pytest.mark.parametrize("heads,d,lens,warps", [
+    (30, 64, [(60, 940)] * 30, 2),                                            # 900 rows: an SM holds eight blocks of two warps
+    (40, 128, [(20 + i % 30, 5 + 7 * i % 41) for i in range(32)], 1),         # 1 280 uneven rows: blocks of three warps in a third wave
+], ids=["64_wide", "uneven"])
+def test_rows_of_many_sequences_get_the_warps_that_are_resident(heads, d, lens, warps):
+    _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens, other=("row_warps", warps))
 
 
 @pytest.mark.parametrize("heads,d,tokens", [(8, 128, 32000), (4, 64, 32000), (2, 128, 48000)])
