@@ -1337,7 +1337,9 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // Few rows, eight CTAs each, leave SMs idle, and ranges are the better the longer the rows are; that they pay for it in merges of hundreds of
 // partials per row decides where: one query head, VLA, 4 rows of 1 000 pages 21.7 / 21.3*, of 1 880 24.7* / 35.2, 8 of 500 17.1 / 14.1*, of
 // 1 000 19.9 / 21.7*, of 1 880 26.4* / 35.7; GLA blocks of four, 8 of 1 000 24.4 / 18.0*, of 1 880 29.6 / 30.6*; query groups, VLA, 4 of 1 000
-// 45.3 / 25.1*, of 2 000 48.8 / 42.9*, of 3 760 55.8* / 74.7.
+// 45.3 / 25.1*, of 2 000 48.8 / 42.9*, of 3 760 55.8* / 74.7; 64-wide heads, 16 of 500 14.1 / 13.4*, of 606 15.2* / 16.8.  Of 64-wide heads ranges
+// are also the better for long rows where some SMs have two CTAs and most have one: 40 of 660 19.2* / 24.4, 48 of 500 20.3* / 21.0, of 250
+// 14.4 / 13.7*, 56 of 500 22.1 / 21.3*, 80 of 313 19.0* / 20.6, 96 of 198 19.5* / 21.6, 112 of 251 22.1 / 21.1*.
 // Query groups of 128-wide heads with two or three followers: their sums and tiles fit an SM once (148, 74, 33 and 15 clusters).  As many
 // CTAs per row as are resident, and ranges where a row's pages are too many for them: blocks of four, VLA_QC, 16 rows of 64 pages 13.5 / 18.6,
 // 12.7, 10.4*, 15.5; 64 of 64 16.1 / 19.1, 13.5*, 18.4; 64 of 190 22.5* / 44.6, 26.4; 128 of 21 13.6 / 11.1*, 15.1; 128 of 64 19.4* / 19.6,
@@ -1357,7 +1359,8 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // Followers that sweep the text alone are launches of their own in both: sequences of as many tokens, one with 3 000 of text and
 // seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 (query groups lose more
 // to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  Up to 1 184 rows one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
-// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; beyond that blocks of three run in a third wave: 1 280 of 4 to 6 pages 20.6 / 27.7, 21.3, 19.2,
+// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; beyond that, where long rows are left to ranges (1 280 of 32 42.2 / 39.3*, of 63 78.3 / 77.6*, of 80
+// 131* / 141), blocks of three run in a third wave: 1 280 of 4 to 6 pages 20.6 / 27.7, 21.3, 19.2,
 // 16.4, 15.7*, of 10 to 32 42.2 / 45.7, 40.0, 40.2, 40.4, 39.3*; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
 struct RowSplit {
   int cluster, warps;
@@ -1392,7 +1395,9 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     if (places(1) > n_sms) {
       while (n > 1 && n * rows > n_sms) n /= 2;
       if (n < 8 && rows <= places(2 * n) && longest > 36 * n) n *= 2;
-      if (8 * rows <= n_sms && longest > ((c->cfg.lazy_mode == QC_MODE_GLA) == (c->group > 1) ? 1000 : 2000)) return ranges;
+      const int few = (c->D == 64 ? 600 : 1000) * ((c->cfg.lazy_mode == QC_MODE_GLA) == (c->group > 1) ? 1 : 2);
+      if (8 * rows <= n_sms && longest > few) return ranges;
+      if (c->D == 64 && c->group == 1 && n * rows > n_sms && 10 * n * rows < 7 * places(1) && longest > 80 * n) return ranges;
     } else {
       while (rows > places(n)) n /= 2;
       static constexpr int kMostPages[2][4] = {{45, 135, 300, 900}, {0, 85, 270, 900}};
@@ -1403,6 +1408,7 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   } else if (c->group == 1) {
     for (int warps : {1, 2, 3, 4})
       if (rows <= n_sms * (warps == 1 ? kWorkersPerSm : c->row_places.per_sm[warps])) split = RowSplit{1, warps};
+    if (rows > 8 * n_sms && longest > 64) return ranges;
     if (split.warps == 1 && rows <= 8 * n_sms && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
   }
   if (worst * n_seqs - all > most * n_seqs * (launches + text_launches)) return ranges;

@@ -73,6 +73,16 @@ def test_rows_of_many_sequences_get_the_warps_that_are_resident(heads, d, lens, 
     _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens, other=("row_warps", warps))
 
 
+@pytest.mark.parametrize("heads,d,batch,tokens,block,mode", [
+    (40, 64, 1, 10400, BLOCKS_OF_2, qc.QC_MODE_VLA_EQ8),    # clusters of four on 160 of 296 places
+    (32, 64, 3, 3140, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),     # of two on 192
+    (16, 64, 1, 9700, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),     # of eight on 128
+    (40, 128, 32, 1240, BLOCKS_OF_4, qc.QC_MODE_VLA_EQ8),   # a warp for each of 1 280 rows
+])
+def test_long_rows_on_part_of_the_chip(heads, d, batch, tokens, block, mode):
+    _not_slower_than_ranges(heads, heads, d, block, mode, [(100, tokens - 100)] * batch, margin=1.05)
+
+
 @pytest.mark.parametrize("heads,d,tokens", [(8, 128, 32000), (4, 64, 32000), (2, 128, 48000)])
 def test_a_few_very_long_rows_use_the_whole_chip(heads, d, tokens):
     _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(100, tokens)])
