@@ -1357,8 +1357,8 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
 // 384 of 188 42 61.3 / 58.8*; 64-wide, 240 of 251 46 33.2* / 34.9, 112 of 501 74 32.4* / 35.4; query groups, 240 of 251
 // 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6.
 // Followers that sweep the text alone are launches of their own in both: sequences of as many tokens, one with 3 000 of text and
-// seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 (query groups lose more
-// to ranges than that: 32 of 1 500 or 16 23.9 / 22.1*).  Up to 1 184 rows one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
+// seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 With query groups
+// they count for the second only: 32 of 1 500 or 16 23.9 / 22.1*, 64-wide, five of 8 800, text in two of them, 27.2* / 34.0.  Up to 1 184 rows one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
 // 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; beyond that, where long rows are left to ranges (1 280 of 32 42.2 / 39.3*, of 63 78.3 / 77.6*, of 80
 // 131* / 141), blocks of three run in a third wave: 1 280 of 4 to 6 pages 20.6 / 27.7, 21.3, 19.2,
 // 16.4, 15.7*, of 10 to 32 42.2 / 45.7, 40.0, 40.2, 40.4, 39.3*; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
@@ -1383,10 +1383,9 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     longest_t = std::max(longest_t, t);
   }
   // pages of the longest row, summed over the step's launches, and of all rows
-  const int64_t text_launches = c->group > 1 ? 0 : c->text_launches;
-  const int64_t launches = c->group > 1 ? 1 : c->cfg.n_layers - c->no_launches - text_launches;
+  const int64_t text_launches = c->text_launches, launches = c->cfg.n_layers - c->no_launches - text_launches;
   const int64_t worst = launches * longest + text_launches * longest_t, all = launches * pages + text_launches * pages_t;
-  if (5 * worst * n_seqs > 8 * all) return ranges;
+  if (5 * longest * n_seqs > 8 * pages || (c->group == 1 && 5 * worst * n_seqs > 8 * all)) return ranges;
   auto places = [&](int n) { return c->row_places.clusters[n == 8 ? 3 : n / 2]; };
   RowSplit split = ranges;
   int64_t most = 50;   // pages that the longest row may have more than the average one

@@ -97,8 +97,12 @@ def test_rows_that_are_longer_than_others_by_many_pages(heads, d, lens):
     _not_slower_than_ranges(heads, heads, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens, margin=1.05)
 
 
-def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges():
-    _not_slower_than_ranges(32, 32, 128, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, [(3000, 16)] + [(16, 3000)] * 7)
+@pytest.mark.parametrize("hq,hkv,d,lens", [
+    (32, 32, 128, [(3000, 16)] + [(16, 3000)] * 7),
+    (32, 8, 64, [(26, 8800), (8800, 26)] * 2 + [(26, 8800)]),
+])
+def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges(hq, hkv, d, lens):
+    _not_slower_than_ranges(hq, hkv, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens)
 
 
 @pytest.mark.parametrize("hq,hkv", [(4, 4), (8, 2)])
