@@ -1686,7 +1686,7 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
     return L;
   };
   LaunchList launches;
-  if (use_static)
+  if (use_static && p.row_cluster == 0)
     for (size_t gi = 0; gi < c->groups.size() && gi < static_cast<size_t>(kMaxPlanLaunches); ++gi)
       launches.launch[gi] = partition_of(gi);
   p.wdesc = planned ? reinterpret_cast<const WorkerDesc*>(c->ws + c->lay.wdesc) : nullptr;
