@@ -25,7 +25,7 @@ def _workload(group, index):
     return W.Workload(index, f"err{index}", 3, 2 * group, 2, 128, 16, 2, 5, 100, 100, 22, 6, (1,))
 
 
-@pytest.mark.parametrize("schedule", ["one_launch", "in_order"])
+@pytest.mark.parametrize("schedule", ["one_launch", "in_order", "in_order_ranges"])
 @pytest.mark.parametrize("group", [1, 4], ids=["mha_kernel", "gqa_kernel"])
 def test_a_wait_that_runs_out_is_reported_and_nothing_hangs(schedule, group):
     w = _workload(group, 80 + group)
@@ -34,15 +34,20 @@ def test_a_wait_that_runs_out_is_reported_and_nothing_hangs(schedule, group):
     def fresh():
         s = Session.for_workload(w)
         s.prefill_workload(w)
-        if schedule == "in_order":
+        if schedule != "one_launch":
             s.set_option("in_order_launches", 1)
+        if schedule == "in_order_ranges":   # as it comes, every row of this batch has thread blocks of its own
+            s.set_option("row_cluster", 0)
         return s
 
     s = fresh()
     out = torch.empty((w.n_layers, w.batch, w.n_q_heads, w.head_dim), dtype=torch.bfloat16, device=s.device)
     q, k, v = W.decode_qkv_torch(w, 0, s.device)
+    launches = s.stats().kernel_launches
     s.decode_step(ids, q, k, v, out)
     assert s.stats().device_error == 0
+    if schedule != "one_launch":
+        assert (s.stats().kernel_launches - launches == 1 + w.n_layers) == (schedule == "in_order")
     s.set_option("debug_drop_tile", 1)
     q, k, v = W.decode_qkv_torch(w, 1, s.device)
     s.decode_step(ids, q, k, v, out)                      # enqueued; the kernel gives up on the device

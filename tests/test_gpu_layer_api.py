@@ -1,6 +1,6 @@
 """qc_decode_begin / qc_decode_layer: a decode step issued layer by layer, each call with only that
 layer's q/k/v (separately allocated tensors, so that nothing of another layer is within reach),
-against the fp64 oracle and against qc_decode_step on a twin cache.  Ragged batch, all modes, MHA
+against the fp64 oracle and against qc_decode_step on a twin cache.  Ragged and even batches, all modes, MHA
 and GQA shapes, blocks with several followers, pages that fill up during the steps."""
 
 import numpy as np
@@ -42,11 +42,20 @@ def test_layer_calls_whose_workers_find_their_own_start(mode, shape):
     _layer_by_layer(mode, shape, {"plan_ahead": 0})
 
 
-def _layer_by_layer(mode, shape, options):
+@pytest.mark.parametrize("mode", MODES, ids=["vla_qc", "vla_eq8", "gla"])
+@pytest.mark.parametrize("shape", [0, 1, 2])
+def test_layer_calls_whose_rows_have_thread_blocks_of_their_own(mode, shape):
+    layered = _layer_by_layer(mode, shape, {}, trunc=(177, 168, 150))   # (the batch above is too uneven for them)
+    assert set(layered) == {1 + len(SHAPES[shape][2])}   # a step: set-up, and a launch that finishes its rows for each layer
+
+
+def _layer_by_layer(mode, shape, options, trunc=(177, 9, 70)):
+    """Returns the kernels launched by every step's calls."""
     head_dim, group, layer_kind = SHAPES[shape]
     lazy = tuple(i for i, k in enumerate(layer_kind) if k)
     w = W.Workload(70 + shape, f"layer{shape}", len(layer_kind), 2 * group, 2, head_dim, 16, 3, 5, 150, 150, 22, 20, lazy)
-    trunc, seq_ids = [w.n_prompt, 9, 70], [2, 0, 3]
+    seq_ids = [2, 0, 3]
+    assert w.n_prompt == 177
     o = LazyAttentionOracle(w.n_layers, w.n_q_heads, w.n_kv_heads, head_dim, layer_kind, mode, n_seqs=3)
     sessions = [Session(w.n_layers, w.n_q_heads, w.n_kv_heads, head_dim, layer_kind, max_seqs=4, max_tokens_per_seq=256,
                         n_pages=w.n_layers * 4 * 3 * 17, lazy_mode=mode, poison_pool=True) for _ in range(2)]
@@ -64,9 +73,11 @@ def _layer_by_layer(mode, shape, options):
         o.prefill_append(b, kind.tolist(), f64(k), f64(v))
     dev = layered.device
     out_whole = torch.empty((w.n_layers, 3, w.n_q_heads, head_dim), dtype=torch.bfloat16, device=dev)
+    launches = []
     for step in range(w.decode_steps):
         qn, kn, vn = W.decode_qkv_np(w, step)
         whole.decode_step(seq_ids, _dev(qn, dev), _dev(kn, dev), _dev(vn, dev), out_whole)
+        before = layered.stats().kernel_launches
         layered.decode_begin(seq_ids)
         outs, lses = [], []
         for l in range(w.n_layers):
@@ -77,6 +88,7 @@ def _layer_by_layer(mode, shape, options):
             outs.append(out_l)
             lses.append(lse_l)
         torch.cuda.synchronize()
+        launches.append(layered.stats().kernel_launches - before)
         got = np.stack([bits_of(t) for t in outs])
         got_lse = np.stack([t.cpu().numpy() for t in lses])
         ref_whole = f64(bits_of(out_whole))
@@ -97,6 +109,7 @@ def _layer_by_layer(mode, shape, options):
                 assert layered.page_table(l, stream, sid) == whole.page_table(l, stream, sid)
     for s in sessions:
         s.close()
+    return launches
 
 
 def test_an_open_step_refuses_everything_but_its_next_layer():

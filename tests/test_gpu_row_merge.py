@@ -71,9 +71,10 @@ def test_rows_merged_by_the_attention_launch(shape, mode):
         s.close()
 
 
+@pytest.mark.parametrize("row_cluster", [-1, 0], ids=["rows", "ranges"])
 @pytest.mark.parametrize("shape", ["one_long_row_per_head", "rows_over_several_blocks"])
-def test_the_same_step_gives_the_same_bits(shape):
-    """Which block completes a row that several blocks share, and how many rows it completes, differs
+def test_the_same_step_gives_the_same_bits(shape, row_cluster):
+    """Which block completes a row that several blocks share (tile ranges), and how many rows it completes, differs
     from run to run; the bits of the output may not."""
     head_dim, _, lens = SHAPES[shape]
     heads, b = 16, len(lens)
@@ -82,6 +83,7 @@ def test_the_same_step_gives_the_same_bits(shape):
     s = Session(n, heads, heads, head_dim, layer_kind, max_seqs=b, max_tokens_per_seq=longest + 1,
                 n_pages=2 * n * sum((t + 32) // 16 + (v + 15) // 16 for t, v in lens))
     s.set_option("in_order_launches", 1)
+    s.set_option("row_cluster", row_cluster)
     gen = torch.Generator(device=s.device).manual_seed(3)
 
     def normal(*size):
@@ -95,7 +97,9 @@ def test_the_same_step_gives_the_same_bits(shape):
     first = None
     for run in range(60):
         s.prefill_append(list(range(b)), [t + v_ for t, v_ in lens], kind, k, v)
+        launches = s.stats().kernel_launches
         s.decode_step(list(range(b)), *qkv, out, lse)
+        assert s.stats().kernel_launches - launches == n + (1 if row_cluster else 2)   # set-up, with ranges their plan, a launch per layer
         got = (out.view(torch.int16).clone(), lse.view(torch.int32).clone())
         if first is None:
             first = got
@@ -106,8 +110,9 @@ def test_the_same_step_gives_the_same_bits(shape):
     s.close()
 
 
-@pytest.mark.parametrize("options", [{}, {"in_order_launches": 1}, {"in_order_launches": 1, "fused_merge": 0}],
-                         ids=["one_launch", "own_merge", "merge_launch"])
+@pytest.mark.parametrize("options", [{}, {"in_order_launches": 1}, {"in_order_launches": 1, "row_cluster": 0},
+                                     {"in_order_launches": 1, "fused_merge": 0}],
+                         ids=["one_launch", "rows", "own_merge", "merge_launch"])
 @pytest.mark.parametrize("q_heads,kv_heads", [(4, 4), (8, 2)])
 def test_a_key_that_is_not_a_number_reaches_every_row_it_belongs_to(q_heads, kv_heads, options):
     """Softmax over a score that is not a number is not a number: a partial result that holds one may not be
