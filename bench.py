@@ -34,11 +34,12 @@ UNIT = "tokens/s"
 MODES = {"vla_qc": 0, "vla_eq8": 1, "gla": 2}
 
 # (dram__bytes_read.sum + dram__bytes_write.sum) / algorithmic K/V bytes of one attention launch of the
-# in-order schedule, from ncu captures of small cases of the same shapes (first 4 layers: launches of
-# 27-253 MB with one query head per KV head, 6-107 MB with query groups; 1.028 for either, over all of
-# them).  Every tile is fetched once, pages that are not full in whole, so traffic grows in proportion
+# in-order schedule, from ncu captures of small cases of the same shapes (attend_rows_kernel: first 4
+# layers, launches of 27-253 MB with one query head per KV head, 6-107 MB with query groups; 1.028 for
+# either, over all of them; the kernels of tile ranges: first 8 layers, launches of 181-257 MB, resp.
+# 74-107 MB).  Every tile is fetched once, pages that are not full in whole, so traffic grows in proportion
 # to the K/V bytes swept and a full-size launch's traffic is this ratio times its algorithmic bytes.
-NCU_TRAFFIC_RATIO = {"attend_rows_kernel": 1.028}
+NCU_TRAFFIC_RATIO = {"attend_rows_kernel": 1.028, "attend_kernel": 1.022, "attend_tc_kernel": 1.047}
 
 
 def _peaks():
@@ -343,7 +344,6 @@ def measure_workload(args, w, mode, group, local_rank, world, rank, K, W_, Ke, e
     attention launch for the kernel's own time.  The one-launch schedule (every layer's q/k/v known
     up front, which only a harness has) is reported beside it."""
     peak, peak_kind = _peaks()
-    kernel = "attend_rows_kernel"   # the in-order launches of these workloads give every output row its own blocks
     a = _Arms(args, w, mode, group, local_rank, rank * w.batch)
     a.set(IN_ORDER)
     for kv in args.option:
@@ -355,6 +355,9 @@ def measure_workload(args, w, mode, group, local_rank, world, rank, K, W_, Ke, e
         main = a.run(K)
     gpu_launches = int(a.s.stats().kernel_launches - launches0)
     a.check_output()
+    # a step whose rows have thread blocks of their own is the set-up and a launch per layer; one in tile ranges has its plan besides
+    own_blocks = round(main["launches_per_step"]) == 1 + w.n_layers
+    kernel = "attend_rows_kernel" if own_blocks else "attend_tc_kernel" if w.group > 1 else "attend_kernel"
     kp = a.run(min(K, 16), profile=2)           # the kernel's own time, launch by launch
     prof = kp["prof"]
     n_launch = max(1, prof.attend_kernel_launches)
@@ -492,7 +495,7 @@ def run_gpu(args, rank, world, local_rank):
         },
         "roofline": {
             "bound": "hbm", "achieved": head["kernel_gb_per_s"], "peak": peak, "unit": "GB/s", "frac": head["frac"],
-            "traffic": traffic, "traffic_source": "ncu dram bytes of launches of the same kernel and schedule on the first 8 "
+            "traffic": traffic, "traffic_source": "ncu dram bytes of launches of the same kernel and schedule on the first "
                                                   "layers of llava15_7b / qwen2vl_gqa, scaled by the K/V bytes of a launch",
             "peak_kind": f"of {peak_kind}", "kernel": head["kernel"],
             "algorithmic_bytes_per_launch": head["algorithmic_bytes_per_launch"], "avg_launch_ms": head["avg_launch_ms"],
