@@ -304,9 +304,10 @@ int32_t qc_debug_read_row(qc_cache* cache, int32_t layer, int32_t stream, int32_
  * are planned ahead and n_seqs * n_q_heads is at most four per SM; 0 = always by a merge launch),
  * "row_cluster" (in-order schedule and qc_decode_layer, with the options above as they come: CTAs that each
  * output row gets in launches that finish their rows themselves, without plan, partials or merge launch;
- * -1, the default = chosen from the number of rows and their lengths; 0 = never; 1 to 8 = that many, where no
- * lazy block has more than four layers), "row_warps" (the same with one CTA of 1, 2, 3, 4 or 6 warps per row, without
- * query groups; 0, the default = chosen),
+ * -1, the default = chosen from the numbers of rows and pages, among 1, 2, 4 and 8 or tile ranges; 0 = never;
+ * 1 to 8 = that many, where no lazy block has more than four layers and no launch of the step has more than 60
+ * pages of its lightest sweep for every worker; larger steps claim chunk items), "row_warps" (the same with one CTA
+ * of 1, 2, 3, 4 or 6 warps per row, without query groups; 0, the default = chosen),
  * "fold_append" (in-order schedule and qc_decode_layer; 1, the default = a layer's new k/v rows and an
  * ordinary layer's q are taken from the inputs and stored by that layer's own launch; 0 = by an
  * append when the step begins, resp. an append launch per layer call),

@@ -852,14 +852,13 @@ __device__ __forceinline__ void store_row(const Params& P, int layer, int si, in
   if (P.lse != nullptr && lane == 0) P.lse[orow] = (r.m + log2f(r.l)) * 0.6931471805599453f;
 }
 
-// Merge of one output row by a launch of its own (merge_kernel), including the wait for the launch
-// that leaves the last partials.  With claimed items the numbers of partials follow from the stream
-// lengths; launches of one layer under the static partition have them planned; otherwise the
-// sweeps recorded them.  P.extra_key_leader >= 0 adds the step's new token as one more key (rows of
-// a GLA follower under the in-order schedule; Eq. 6).
-// ROWS: the step's rows had thread blocks of their own, what there is is one partial row from the leader's launch (an
-// instantiation of its own: with both in one, two turns of 8 steps of a 64-wide GLA stack took 1 272 us, now 1 223, and a step of
-// two layers with claimed items 14.6 us, now 14.45).
+// Merge of one output row by a launch of its own (merge_kernel), including the wait for the launch that leaves
+// the last partials.  With claimed items the numbers of partials follow from the stream lengths; launches of
+// one layer under the static partition have them planned; otherwise the sweeps recorded them.
+// P.extra_key_leader >= 0 adds the step's new token as one more key (rows of a GLA follower under the in-order
+// schedule; Eq. 6). ROWS: the step's rows had thread blocks of their own, what there is is one partial row from
+// the leader's launch (an instantiation of its own: with both in one, two turns of 8 steps of a 64-wide GLA
+// stack took 1 272 us, now 1 223, and a step of two layers with claimed items 14.6 us, now 14.45).
 template <int D, bool ROWS>
 __device__ __forceinline__ void merge_row(const Params& P, int layer, int si, int head, int lane) {
   constexpr int VPL = D / 32;

@@ -1,29 +1,31 @@
 // Attention of one layer (in-order schedule) where every output row has thread blocks of its own.
 //
-// A launch of one layer for a small batch moves a few MB, which HBM delivers in 2 us, and what it
-// costs is its chain of dependent steps; a launch for a large batch is bound by HBM and loses at its end what that chain takes.  Cut into
-// tile ranges (qc_kernels.cu, qc_attend_tc.cu) the chain is: a worker's page, its partial row through
-// the L2, an atomic per shared row, the partials of 40 workers read back by one CTA (or a merge
-// launch).  Here a row (a query head, or a query group) belongs to a cluster of up to eight CTAs, or to one CTA, whose
-// warps take its pages in turn -- all visual pages, then all text pages -- and the warps' sums are
-// added in shared memory: first in each CTA, then over the cluster through distributed shared memory.
-// The launch writes finished rows; the only sums that reach HBM are one per row and follower of a lazy
-// block (the sums of the keys it shares with its leader).  No plan, no counters, no merge launch, and
-// every row is added up in one order.
-// us per layer, tile ranges -> this: one sequence of 675 tokens, 32 heads 9.5 -> 6.9; 16 of them 30.8 -> 26.9; 32 of 500 44.9 -> 40.5; 32 of
-// 1 120 with 4 KV heads 20.2 -> 17.7.  After the wait for the previous kernel the first of these spends, of some 12 000 cycles, 850 on the query, 2 300 on the
-// first K tile and its softmax, 1 900 on the V tiles, as much on a second page, and 2 500 from the last page to the row.
+// A launch of one layer for a small batch moves a few MB, which HBM delivers in 2 us, and what it costs is its
+// chain of dependent steps; a launch for a large batch is bound by HBM and loses at its end what that chain
+// takes.  Cut into tile ranges (qc_kernels.cu, qc_attend_tc.cu) the chain is: a worker's page, its partial row
+// through the L2, an atomic per shared row, the partials of 40 workers read back by one CTA (or a merge
+// launch).  Here a row (a query head, or a query group) belongs to a cluster of up to eight CTAs, or to one
+// CTA, whose warps take its pages in turn -- all visual pages, then all text pages -- and the warps' sums are
+// added in shared memory: first in each CTA, then over the cluster through distributed shared memory.  The
+// launch writes finished rows; the only sums that reach HBM are one per row and follower of a lazy block (the
+// sums of the keys it shares with its leader).  No plan, no counters, no merge launch, and every row is added
+// up in one order.
+// us per layer, tile ranges -> this: one sequence of 675 tokens, 32 heads 9.5 -> 6.9; 16 of them 30.8 -> 26.9;
+// 32 of 500 44.9 -> 40.5; 32 of 1 120 with 4 KV heads 20.2 -> 17.7.  After the wait for the previous kernel the
+// first of these spends, of some 12 000 cycles, 850 on the query, 2 300 on the first K tile and its softmax,
+// 1 900 on the V tiles, as much on a second page, and 2 500 from the last page to the row.
 //
-// Every launch of the in-order schedule scores with one query per row (its layer's own), so one
-// running softmax serves the row's streams: consumer 0 is the layer itself, consumers 1 .. are the
-// followers whose cached V the leader's launch also weights.  Under VLA_QC those take no text keys:
-// their softmax reference stays where the visual pages left it.
+// Every launch of the in-order schedule scores with one query per row (its layer's own), so one running softmax
+// serves the row's streams: consumer 0 is the layer itself, consumers 1 .. are the followers whose cached V the
+// leader's launch also weights.  Under VLA_QC those take no text keys: their softmax reference stays where the
+// visual pages left it.
 //
-// One query head per KV head: fp32 arithmetic on pairs.  Query groups: mma.m16n8k16 with keys as M and
-// the group as N, as in qc_attend_tc.cu, but with the weights as the sum of two bf16 values, a product each on the same V
-// fragment (error against 64 bits, 32 sequences of 1 120 tokens: 2.05e-3 in tile ranges, 2.11e-3 here with one bf16 value -- fewer,
-// longer pieces have fewer weights that are exactly 1 -- and 1.66e-3, the rounding of the output, with two; 17.9 us a layer with one, 17.7 with two and a
-// single tensor-map copy per tile).
+// One query head per KV head: fp32 arithmetic on pairs.  Query groups: mma.m16n8k16 with keys as M and the
+// group as N, as in qc_attend_tc.cu, but with the weights as the sum of two bf16 values, a product each on the
+// same V fragment (error against 64 bits, 32 sequences of 1 120 tokens: 2.05e-3 in tile ranges, 2.11e-3 here
+// with one bf16 value -- fewer, longer pieces have fewer weights that are exactly 1 -- and 1.66e-3, the
+// rounding of the output, with two; 17.9 us a layer with one, 17.7 with two and a single tensor-map copy per
+// tile).
 
 #include "qc_device.cuh"
 
@@ -35,9 +37,11 @@
 namespace qc {
 namespace {
 
-// Warps per CTA (W): six, or fewer where rows are many; an SM holds twelve in all (64-wide heads sixteen).  Tiles in flight per warp (RING): four
-// where the next launch's first tiles are to land during this one; two where the launch is bound by HBM, which
-// scattered tiles use worse the more there are in flight (512 rows of 43 pages, 3 warps: 27.5 us a layer with four, 27.0 with two).
+// Warps per CTA (W): six, or fewer where rows are many; an SM holds twelve in all (64-wide heads sixteen).  Tiles in
+// flight per warp (RING): four where the next launch's first tiles are to land during this one; two where the
+// launch is bound by HBM, which scattered tiles use worse the more there are in flight (512 rows of 43 pages, 3 warps:
+// 27.5 us a layer with four, 27.0 with two); three for blocks of one warp (two, three, four: 1 024 rows of 19 pages 26.4,
+// 25.9, 25.7; 1 110 of 38 46.5, 45.5, 46.3; 1 440 of 38 57.9, 59.0, 59.7).
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -125,8 +129,9 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
   if (threadIdx.x == 0) S.dead = 0;
 
   // ---- ahead of the wait for the previous kernel: the row, its page ids and the first tiles.  The sequence
-  // descriptors, the page tables and the cached pages were written two or more launches back, but for a step's first
-  // launch, which comes right after the one that writes the first two (its wait is 1 us of the 227 of a step of 32 layers).
+  // descriptors, the page tables and the cached pages were written two or more launches back, but for a step's
+  // first launch, which comes right after the one that writes the first two (its wait is 1 us of the 227 of a
+  // step of 32 layers).
   if (P.follows_setup) pdl_wait();
   const int row = blockIdx.x / n_ctas, rows = P.heads_per_item_dim;
   const int si = row / rows, u = row - si * rows;
@@ -254,8 +259,8 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
     }
   }
 
-  // Softmax references and this lane's parts of the sums of weights.  References start at the lowest finite value: the
-  // weight of a score of minus infinity then is zero also in a warp whose first pages hold no other.
+  // Softmax references and this lane's parts of the sums of weights.  References start at the lowest finite
+  // value: the weight of a score of minus infinity then is zero also in a warp whose first pages hold no other.
   float m[NC][NH], l[NC][NH];
   float2 acc[MH ? NV : 1][MH ? EP2 : 1];
   float o[MH ? 1 : NV][MH ? 1 : KS][4];
@@ -275,7 +280,8 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
   }
   const int lrow = lane & 7, lmat = lane >> 3;   // ldmatrix lane roles
   const uint32_t k_off = tile_at<D, MH>(lrow + ((lmat & 1) << 3), lmat >> 1), v_off = tile_at<D, MH>(lrow + ((lmat >> 1) << 3), lmat & 1);
-  // chunk 2 * i further along a lane's row (tiles are 1024-byte aligned: the swizzle is an exclusive or on the address)
+  // chunk 2 * i further along a lane's row (tiles are 1024-byte aligned: the swizzle is an exclusive or on the
+  // address)
   auto step_addr = [](uint32_t addr, int i) -> uint32_t { return (addr ^ ((i & 3) << 5)) + ((i >> 2) << 11); };
 
   for (int j = 0; j < n_my; ++j) {
@@ -380,8 +386,9 @@ __global__ void __launch_bounds__(W * 32, 12 / W) attend_rows_kernel(const __gri
       }
     }
     uint32_t pb[2][2], pb_skip[2][2];   // query groups: the weights as B operands, in two parts
-    // The first part is the next bf16 value below the weight and the second what is left, so a weight that is not zero has
-    // two positive parts: an infinite value element stays infinite (times a zero or negative part it would not).
+    // The first part is the next bf16 value below the weight and the second what is left, so a weight that is
+    // not zero has two positive parts: an infinite value element stays infinite (times a zero or negative part
+    // it would not).
     auto operands = [&](uint32_t (&b)[2][2]) {
       constexpr float kBelow = 1.f - 0x1p-24f;   // the largest float below 1
 #pragma unroll
@@ -672,8 +679,8 @@ cudaError_t with_rows_kernel(int d, bool mh, int nv, int warps, Fn fn) {
 
 }  // namespace
 
-// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone), and what
-// is resident of the one that fits least.
+// The kernels that a cache's launches can take (each of them is loaded by this, so the others are left alone),
+// and what is resident of the one that fits least.
 cudaError_t configure_rows_kernels(int d, int group, const std::vector<RowJobs>& layers, RowPlaces& places) {
   for (int& n : places.clusters) n = INT_MAX;
   for (int& n : places.per_sm) n = INT_MAX;
@@ -725,8 +732,9 @@ cudaError_t launch_attend_rows(const Params& p, const RowJobs& jobs, int n_sms, 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = p.row_cluster, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    // An SM holds eight clusters at most, clusters of one too: single CTAs beyond that are launched as what they are
-    // (1 280 rows of 19 pages 45.0 -> 31.1 us a layer, 1 760 48.0 -> 39.2; up to eight per SM clusters are the better, 1 024 26.1 against 26.4).
+    // An SM holds eight clusters at most, clusters of one too: single CTAs beyond that are launched as what
+    // they are (1 280 rows of 19 pages 45.0 -> 31.1 us a layer, 1 760 48.0 -> 39.2; up to eight per SM clusters
+    // are the better, 1 024 26.1 against 26.4).
     cfg.numAttrs = p.row_cluster > 1 || cfg.gridDim.x <= 8u * static_cast<unsigned>(n_sms) ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, p, jobs);
   });

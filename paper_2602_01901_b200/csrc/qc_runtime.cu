@@ -565,10 +565,10 @@ void grow_stream(qc_cache* c, int layer, int stream, int seq, int have, int n_ne
 
 inline int pages_for(int tokens) { return (tokens + kPage - 1) / kPage; }
 
-// The pool seen as a 2-D bf16 tensor [n_pool_pages * hkv * 16 rows][D]: a (page, head) tile is
-// 16 consecutive rows.  Box = 16 rows x 64 elements (128 bytes) with the 128-byte swizzle, so
-// a D = 128 tile is fetched as two column halves.  The driver entry point is looked up at run
-// time; nothing links against the driver library.
+// The pool as the bf16 tensors that tile copies read it through: a (page, head) tile is 16 consecutive rows of
+// [n_pool_pages * hkv * 16 rows][D].  For the decode kernels the column halves are a dimension of their own, [D / 64]
+// [rows][64], and one copy brings a tile as [D / 64][16][64]; the prompt kernel's map is two-dimensional, box 16 x 64.
+// Both with the 128-byte swizzle.  The driver entry point is looked up at run time; nothing links against the driver library.
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1323,45 +1323,8 @@ int run_group(qc_cache* c, Params& p, size_t gi, const LaunchList& launches, boo
   return QC_OK;
 }
 
-// CTAs that an output row gets in the launches of a step of the in-order schedule, and their warps, or 0: its launches
-// are cut into tile ranges.
-// As long as every row's cluster is resident at once (six-warp CTAs fit an SM twice, 296 of them; clusters of two, four and eight
-// 148, 71 and 33 times): as many CTAs per row as leave one CTA per SM (the next launch then starts in the other
-// half of each SM, and its first tiles have landed when this one ends), twice that where a warp would still have more than six
-// pages.  us per layer, tile ranges / 1, 2, 4, 8 CTAs per row (* what the rule takes): 32 rows of 43 pages 9.54 / 10.2, 7.53, 6.92*,
-// 7.74; 32 of 188 13.8 / 30.2, 17.4, 12.4, 11.6*; 34 of 500 24.2 / 68.3, 37.3, 23.8*, 31.4; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4;
-// 256 of 188 55.5 / 52.7*, 54.6, 62.2; 256 of
-// 130, GLA, 34.4 / 32.7*, 32.8, 36.9; 32 of 43, 64-wide, GLA 7.50 / 8.0, 5.9, 5.09*, 4.94; with query groups 32 of 50 11.7 / 12.3, 9.27,
-// 8.34*, 9.98; 4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1; 72 of 190 24.4 / 33.5, 21.8*, 31.0, 38.4;
-// 128 of 71 20.2 / 18.7, 17.8*, 24.4.
-// Few rows, eight CTAs each, leave SMs idle, and ranges are the better the longer the rows are; that they pay for it in merges of hundreds of
-// partials per row decides where: one query head, VLA, 4 rows of 1 000 pages 21.7 / 21.3*, of 1 880 24.7* / 35.2, 8 of 500 17.1 / 14.1*, of
-// 1 000 19.9 / 21.7*, of 1 880 26.4* / 35.7; GLA blocks of four, 8 of 1 000 24.4 / 18.0*, of 1 880 29.6 / 30.6*; query groups, VLA, 4 of 1 000
-// 45.3 / 25.1*, of 2 000 48.8 / 42.9*, of 3 760 55.8* / 74.7; 64-wide heads, 16 of 500 14.1 / 13.4*, of 606 15.2* / 16.8.  Of 64-wide heads ranges
-// are also the better for long rows where some SMs have two CTAs and most have one: 40 of 660 19.2* / 24.4, 48 of 500 20.3* / 21.0, of 250
-// 14.4 / 13.7*, 56 of 500 22.1 / 21.3*, 80 of 313 19.0* / 20.6, 96 of 198 19.5* / 21.6, 112 of 251 22.1 / 21.1*.
-// Query groups of 128-wide heads with two or three followers: their sums and tiles fit an SM once (148, 74, 33 and 15 clusters).  As many
-// CTAs per row as are resident, and ranges where a row's pages are too many for them: blocks of four, VLA_QC, 16 rows of 64 pages 13.5 / 18.6,
-// 12.7, 10.4*, 15.5; 64 of 64 16.1 / 19.1, 13.5*, 18.4; 64 of 190 22.5* / 44.6, 26.4; 128 of 21 13.6 / 11.1*, 15.1; 128 of 64 19.4* / 19.6,
-// 23.6; the same blocks in GLA, 16 of 64 10.4 / 17.6, 11.7, 8.3*, 12.3; 72 of 64 13.5 / 18.0, 12.7*, 20.9; 72 of 190 21.9* / 43.1, 24.7;
-// 80 of 64 13.8* / 18.1, 21.2; 16 of 500 24.0* / 106, 55.8, 30.1, 33.7.
-// More rows, no query groups: one CTA per row, with the most warps that leave every row resident.  Ranges / 6, 4, 3, 2, 1 warps:
-// 384 rows of 64 pages 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4; 480 of 17 18.3 / 18.5,
-// 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7; 1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*.  64-wide
-// heads, of which an SM holds more: 480 of 63 25.2 / 25.7, 20.2*, 23.1, 27.5, 43.8; 640 of 63 32.2 / 37.4, 37.0, 25.3*, 31.0, 47.6; 900 of 63
-// 40.8 / 48.7, 40.1, 46.8, 34.0*, 48.2; 640 of 19, GLA blocks of four (fewer again), 12.9 / 13.7, 11.8, 13.4, 10.2*, 14.3.
-// A launch takes as long as its longest row.  Batches whose longest row is over 1.6 times the average one stay with the
-// ranges, and so do those where it has more pages than the average one by what a launch's start and end are worth: 32 for each
-// six-warp CTA of a row (half of that for 64-wide heads), 50 for rows of fewer warps, 64 for query groups.  Ranges / rows, by pages more than the average:
-// 256 rows of 188 pages 31 45.5 / 44.8*; 240 of 251 38 68.4* / 70.3, 64 61.3* / 66.2; 480 of 251 35 86.3 / 82.6*, 58 78.1* / 78.6;
-// 384 of 188 42 61.3 / 58.8*; 64-wide, 240 of 251 46 33.2* / 34.9, 112 of 501 74 32.4* / 35.4; query groups, 240 of 251
-// 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6.
-// Followers that sweep the text alone are launches of their own in both: sequences of as many tokens, one with 3 000 of text and
-// seven with 16, 54.9* / 65.1; half of 14 with the text and the image of the others exchanged, 224 of 251 68.9* / 76.2 With query groups
-// they count for the second only: 32 of 1 500 or 16 23.9 / 22.1*, 64-wide, five of 8 800, text in two of them, 27.2* / 34.0.  Up to 1 184 rows one warp per row is for rows of one length (1 024 rows of 0.4 to 1 times
-// 38 pages 41.7 / 45.0, 40.4, 40.7*, 40.5, 43.3; beyond that, where long rows are left to ranges (1 280 of 32 42.2 / 39.3*, of 63 78.3 / 77.6*, of 80
-// 131* / 141), blocks of three run in a third wave: 1 280 of 4 to 6 pages 20.6 / 27.7, 21.3, 19.2,
-// 16.4, 15.7*, of 10 to 32 42.2 / 45.7, 40.0, 40.2, 40.4, 39.3*; 512 of up to 62 33.3 / 32.6, 33.1, 31.7*, 36.6; 256 of up to 131 31.6 / 30.8*).
+// CTAs that an output row gets in the launches of a step of the in-order schedule, and their warps, or 0: its
+// launches are cut into tile ranges.  All figures are us per layer in tile ranges / by rows; * is what the rule takes.
 struct RowSplit {
   int cluster, warps;
 };
@@ -1373,6 +1336,7 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   if (c->group == 1 && c->row_warps > 0) return RowSplit{1, c->row_warps};
   if (c->row_cluster > 0) return RowSplit{c->row_cluster, kAttendWarps};
   const int rows = n_seqs * c->items_per_chunk, n_sms = c->ctx->n_sms;
+  const bool gla = c->cfg.lazy_mode == QC_MODE_GLA;
   int64_t pages = 0, longest = 0, pages_t = 0, longest_t = 0;   // of a row in a launch; in one that sweeps the text alone
   for (int i = 0; i < n_seqs; ++i) {
     const SeqState& st = c->seqs[seq_ids[i]];
@@ -1382,7 +1346,10 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     longest = std::max(longest, n);
     longest_t = std::max(longest_t, t);
   }
-  // pages of the longest row, summed over the step's launches, and of all rows
+  // A launch takes as long as its longest row: batches whose longest row is over 1.6 times the average one stay with
+  // the ranges.  Without query groups that also goes for all of a step's launches together, those included in which
+  // followers sweep the text alone: sequences of equal totals, one with 3 000 tokens of text and seven with 16,
+  // 56.4* / 65.1 (query groups lose more to ranges: 32 of 1 500 or 16 23.9 / 22.1*).
   const int64_t text_launches = c->text_launches, launches = c->cfg.n_layers - c->no_launches - text_launches;
   const int64_t worst = launches * longest + text_launches * longest_t, all = launches * pages + text_launches * pages_t;
   if (5 * longest * n_seqs > 8 * pages || (c->group == 1 && 5 * worst * n_seqs > 8 * all)) return ranges;
@@ -1392,24 +1359,65 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   if (rows <= places(1)) {
     int n = 8;
     if (places(1) > n_sms) {
+      // Two six-warp CTAs fit an SM (296 of them; clusters of two, four and eight 148, 71 and 33 times).  As many CTAs
+      // per row as leave one CTA per SM: the next launch then starts in the other half of each SM, and its first tiles
+      // have landed when this one ends.  Twice that where a warp would still have more than six pages, if they are
+      // resident at once.  1, 2, 4, 8 CTAs per row:
+      //   32 rows of 43 pages 9.54 / 10.2, 7.53, 6.92*, 7.74; 32 of 188 13.8 / 30.2, 17.4, 12.4, 11.6*;
+      //   34 of 500 24.2 / 68.3, 37.3, 23.8*, 31.4; 128 of 43 13.0 / 11.4, 10.4*, 16.1, 27.4;
+      //   256 of 188 55.5 / 52.7*, 54.6, 62.2; 256 of 130, GLA, 34.4 / 32.7*, 32.8, 36.9;
+      //   64-wide, GLA, 32 of 43 7.50 / 8.0, 5.9, 5.09*, 4.94; query groups, 32 of 50 11.7 / 12.3, 9.27, 8.34*, 9.98;
+      //   4 of 71 12.2 / 16.3, 11.1, 8.64, 8.07*; 52 of 131 19.3 / 25.4, 17.2, 15.4*, 23.1;
+      //   72 of 190 24.4 / 33.5, 21.8*, 31.0, 38.4; 128 of 71 20.2 / 18.7, 17.8*, 24.4
       while (n > 1 && n * rows > n_sms) n /= 2;
       if (n < 8 && rows <= places(2 * n) && longest > 36 * n) n *= 2;
-      const int few = (c->D == 64 ? 600 : 1000) * ((c->cfg.lazy_mode == QC_MODE_GLA) == (c->group > 1) ? 1 : 2);
+      // Few rows, eight CTAs each, leave SMs idle, and ranges are the better the longer the rows are.  They pay for it
+      // in merges of hundreds of partials per row, most where a merge launch per layer does them (query groups, GLA):
+      //   VLA, 4 of 1 000 21.7 / 21.3*, of 1 880 24.7* / 35.2; 8 of 500 17.1 / 14.1*, of 1 000 19.9 / 21.7*,
+      //   of 1 880 26.4* / 35.7; 64-wide, 16 of 500 14.1 / 13.4*, of 606 15.2* / 16.8; GLA blocks of four, 8 of 1 000
+      //   24.4 / 18.0*, of 1 880 29.6 / 30.6*; query groups, VLA, 4 of 1 000 45.3 / 25.1*, of 2 000 48.8 / 42.9*,
+      //   of 3 760 55.8* / 74.7
+      const int few = (c->D == 64 ? 600 : 1000) * (gla == (c->group > 1) ? 1 : 2);
       if (8 * rows <= n_sms && longest > few) return ranges;
+      // Long rows of 64-wide heads where some SMs have two CTAs and most have one:
+      //   40 of 660 19.2* / 24.4; 48 of 500 20.3* / 21.0, of 250 14.4 / 13.7*; 56 of 500 22.1 / 21.3*;
+      //   80 of 313 19.0* / 20.6; 96 of 198 19.5* / 21.6; 112 of 251 22.1 / 21.1*
       if (c->D == 64 && c->group == 1 && n * rows > n_sms && 10 * n * rows < 7 * places(1) && longest > 80 * n) return ranges;
     } else {
+      // Query groups of 128-wide heads with two or three followers fit an SM once (148, 74, 33 and 15 clusters).  As
+      // many CTAs per row as are resident, and ranges where a row's pages are too many for them.  1, 2, 4, 8 CTAs per
+      // row, blocks of four:
+      //   VLA_QC, 16 of 64 13.5 / 18.6, 12.7, 10.4*, 15.5; 64 of 64 16.1 / 19.1, 13.5*, 18.4; 64 of 190 22.5* / 44.6,
+      //   26.4; 128 of 21 13.6 / 11.1*, 15.1; 128 of 64 19.4* / 19.6, 23.6;
+      //   GLA, 16 of 64 10.4 / 17.6, 11.7, 8.3*, 12.3, of 500 24.0* / 106, 55.8, 30.1, 33.7; 72 of 64 13.5 / 18.0,
+      //   12.7*, 20.9, of 190 21.9* / 43.1, 24.7; 80 of 64 13.8* / 18.1, 21.2
       while (rows > places(n)) n /= 2;
       static constexpr int kMostPages[2][4] = {{45, 135, 300, 900}, {0, 85, 270, 900}};
-      if (longest > kMostPages[c->cfg.lazy_mode == QC_MODE_GLA][n == 8 ? 3 : n / 2]) return ranges;
+      if (longest > kMostPages[gla][n == 8 ? 3 : n / 2]) return ranges;
     }
     split = RowSplit{n, kAttendWarps};
     most = c->group > 1 ? 64 : n * c->D / 4;
   } else if (c->group == 1) {
+    // More rows: one CTA per row, with the most warps that leave every row resident.  6, 4, 3, 2, 1 warps:
+    //   384 of 64 32.7 / 36.0, 29.0*, 30.3, 35.8, 52.9; 512 of 43 30.8 / 30.9, 32.0, 26.9*, 29.4, 38.4;
+    //   480 of 17 18.3 / 18.5, 17.2, 14.4*, 16.4, 20.5; 768 of 43 43.4 / 45.3, 42.8, 49.0, 38.5*, 43.7;
+    //   1 024 of 32 44.9 / 49.3, 45.4, 43.3, 46.1, 40.5*;
+    //   64-wide, of which an SM holds more, 480 of 63 25.2 / 25.7, 20.2*, 23.1, 27.5, 43.8; 640 of 63 32.2 / 37.4,
+    //   37.0, 25.3*, 31.0, 47.6; 900 of 63 40.8 / 48.7, 40.1, 46.8, 34.0*, 48.2
     for (int warps : {1, 2, 3, 4})
       if (rows <= n_sms * (warps == 1 ? kWorkersPerSm : c->row_places.per_sm[warps])) split = RowSplit{1, warps};
+    // Beyond the eight clusters that an SM holds, long rows: 1 280 of 32 42.2 / 39.3*, of 63 78.3 / 77.6*, of 80 131* / 141.
     if (rows > 8 * n_sms && longest > 64) return ranges;
+    // Up to there one warp per row is for rows of one length: 1 024 of 0.4 to 1 times 38 41.7 / 45.0, 40.4, 40.7*, 40.5,
+    // 43.3 (beyond it blocks of three run in a third wave: 1 280 of 4 to 6 20.6 / 27.7, 21.3, 19.2, 16.4, 15.7*).
     if (split.warps == 1 && rows <= 8 * n_sms && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
   }
+  // Rows that are longer than the average one by more pages than a launch's start and end are worth: 32 for each
+  // six-warp CTA of a row (half of that for 64-wide heads), 50 for rows of fewer warps, 64 for query groups.  By how many:
+  //   256 of 188 31 45.5 / 44.8*; 240 of 251 38 68.4* / 70.3, 64 61.3* / 66.2; 480 of 251 35 86.3 / 82.6*, 58 78.1* / 78.6;
+  //   384 of 188 42 61.3 / 58.8*; 64-wide, 240 of 251 46 33.2* / 34.9, 112 of 501 74 32.4* / 35.4; query groups, 240 of
+  //   251 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6; followers' text, 224 of 251 60 68.9* / 76.2, 64-wide
+  //   query groups, 40 of 552 164 27.2* / 34.0
   if (worst * n_seqs - all > most * n_seqs * (launches + text_launches)) return ranges;
   return split;
 }
@@ -1466,17 +1474,19 @@ int decode_step_core(qc_cache* c, int32_t n_seqs, const int32_t* seq_ids, const 
   }
   const int n_patches = static_cast<int>(patches.size());
   if (c->auto_split) {
-    // Larger chunks mean fewer partial results to write and merge; smaller chunks mean more
-    // work items to balance over the workers.  Take the largest chunk whose heaviest item is small against
-    // a worker's share of the launch: a third of it, half where no stream is cut.  us per layer of a step in one launch, with five items per worker
-    // asked for as before -> now: 16 sequences of 677 tokens, 8 layers 30.1 -> 26.3; 24 of them 42.0 -> 37.8; 30 of 260, 16 heads 14.0 -> 12.6;
-    // long steps are unchanged.  With query groups five items per worker (longer chunks were 4 to 17 % faster where a step has less,
-    // 13 sequences of 2 100 tokens 11.0 -> 9.5, but have fewer weights that bf16 holds exactly: the error against 64 bits grows).
-    // One and a half items per worker when it is one launch per layer (a short launch's partial rows and their
-    // merge weigh more than the balance of its tail; 1, 2 and 3 were measured too).  With several launches per
-    // step, a long stream cut small also means many partial rows per output row for every one of
-    // those launches' merges: beyond 24 rows the chunk is doubled as long as one and a half items
-    // per worker remain.
+    // Larger chunks mean fewer partial results to write and merge; smaller chunks mean more work items to balance
+    // over the workers.  Take the largest chunk whose heaviest item is small against a worker's share of the launch: a
+    // third of it, half where no stream is cut.  us per layer, with five items per worker asked for as before -> now:
+    //   a step in one launch: 16 sequences of 677 tokens, 8 layers 30.1 -> 26.3; 24 of them 42.0 -> 37.8; 30 of 260,
+    //   16 heads 14.0 -> 12.6; long steps as before;
+    //   a launch per lazy block / per two / per four: 16 of 3 000 100.4 -> 98.2 / 92.1 -> 93.1 / 88.1 -> 88.3, in GLA
+    //   blocks of four 75.4 -> 75.3 / 74.7 -> 75.3 / 72.2 -> 72.3; 8 of 4 100, VLA_EQ8, 65.8 / 63.9 / 60.7, no difference.
+    // With query groups five items per worker (longer chunks were 4 to 17 % faster where a step has less, 13 sequences
+    // of 2 100 tokens 11.0 -> 9.5, but have fewer weights that bf16 holds exactly: the error against 64 bits grows).
+    // One and a half items per worker when it is one launch per layer (a short launch's partial rows and their merge
+    // weigh more than the balance of its tail; 1, 2 and 3 were measured too).  With several launches per step, a long
+    // stream cut small also means many partial rows per output row for every one of those launches' merges: beyond 24
+    // rows the chunk is doubled as long as one and a half items per worker remain.
     const int64_t workers = static_cast<int64_t>(c->ctx->n_sms) * kWorkersPerSm * static_cast<int64_t>(c->groups.size());
     auto items_at = [&](int cp, int* max_slots) {
       int64_t cv = 0, ct = 0;
