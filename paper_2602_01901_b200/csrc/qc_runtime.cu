@@ -1355,7 +1355,7 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
   if (5 * longest * n_seqs > 8 * pages || (c->group == 1 && 5 * worst * n_seqs > 8 * all)) return ranges;
   auto places = [&](int n) { return c->row_places.clusters[n == 8 ? 3 : n / 2]; };
   RowSplit split = ranges;
-  int64_t most = 50;   // pages that the longest row may have more than the average one
+  int64_t most = 0;   // pages that the longest row may have more than the average one
   if (rows <= places(1)) {
     int n = 8;
     if (places(1) > n_sms) {
@@ -1380,9 +1380,11 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
       const int few = (c->D == 64 ? 600 : 1000) * (gla == (c->group > 1) ? 1 : 2);
       if (8 * rows <= n_sms && longest > few) return ranges;
       // Long rows of 64-wide heads where some SMs have two CTAs and most have one:
-      //   40 of 660 19.2* / 24.4; 48 of 500 20.3* / 21.0, of 250 14.4 / 13.7*; 56 of 500 22.1 / 21.3*;
-      //   80 of 313 19.0* / 20.6; 96 of 198 19.5* / 21.6; 112 of 251 22.1 / 21.1*
-      if (c->D == 64 && c->group == 1 && n * rows > n_sms && 10 * n * rows < 7 * places(1) && longest > 80 * n) return ranges;
+      //   40 of 317 15.6* / 18.1, of 660 19.2* / 24.4; 48 of 500 20.3* / 21.0, of 250 14.4 / 13.7*; 56 of 500 22.1 / 21.3*;
+      //   80 of 157 13.1* / 13.3, of 313 19.0* / 20.6; 96 of 198 19.5* / 21.6; 112 of 251 22.1 / 21.1*;
+      //   query groups, GLA, 80 of 366 19.2* / 24.1
+      const bool most_have_one = 10 * n * rows < 7 * places(1), nearly_all = 10 * n * rows < 6 * places(1);
+      if (c->D == 64 && n * rows > n_sms && most_have_one && longest > (nearly_all && c->group == 1 ? 40 : 80) * n) return ranges;
     } else {
       // Query groups of 128-wide heads with two or three followers fit an SM once (148, 74, 33 and 15 clusters).  As
       // many CTAs per row as are resident, and ranges where a row's pages are too many for them.  1, 2, 4, 8 CTAs per
@@ -1411,9 +1413,15 @@ RowSplit row_split_of(const qc_cache* c, int32_t n_seqs, const int32_t* seq_ids)
     // Up to there one warp per row is for rows of one length: 1 024 of 0.4 to 1 times 38 41.7 / 45.0, 40.4, 40.7*, 40.5,
     // 43.3 (beyond it blocks of three run in a third wave: 1 280 of 4 to 6 20.6 / 27.7, 21.3, 19.2, 16.4, 15.7*).
     if (split.warps == 1 && rows <= 8 * n_sms && 20 * longest * n_seqs > 23 * pages) split.warps = 3;
+    // 64-wide again, long rows that leave much of the chip's warps without work: 320 of 134 36.7* / 43.0.
+    if (c->D == 64 && split.warps > 1 && 10 * rows < 7 * n_sms * c->row_places.per_sm[split.warps] && longest > 80) return ranges;
+    // A few warps are a long way through text that half of the batch does not have: 600 rows of 115 or 4 pages 84.2* / 104,
+    // 320 of 81 or 7, blocks of four, 36.5* / 44.2, 512 of 94 or 3, blocks of four, 60.3* / 66.9.
+    if (text_launches > 0 && longest_t * n_seqs - pages_t > 25 * n_seqs) return ranges;
+    most = c->D == 64 ? 25 : 50;
   }
   // Rows that are longer than the average one by more pages than a launch's start and end are worth: 32 for each
-  // six-warp CTA of a row (half of that for 64-wide heads), 50 for rows of fewer warps, 64 for query groups.  By how many:
+  // six-warp CTA of a row and 50 for rows of fewer warps (half of these for 64-wide heads), 64 for query groups.  By how many:
   //   256 of 188 31 45.5 / 44.8*; 240 of 251 38 68.4* / 70.3, 64 61.3* / 66.2; 480 of 251 35 86.3 / 82.6*, 58 78.1* / 78.6;
   //   384 of 188 42 61.3 / 58.8*; 64-wide, 240 of 251 46 33.2* / 34.9, 112 of 501 74 32.4* / 35.4; query groups, 240 of
   //   251 62 58.2 / 57.2*, 80 of 251 41 27.8 / 27.8*, 69 26.1* / 27.6; followers' text, 224 of 251 60 68.9* / 76.2, 64-wide

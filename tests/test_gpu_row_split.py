@@ -77,6 +77,8 @@ def test_rows_of_many_sequences_get_the_warps_that_are_resident(heads, d, lens, 
     (40, 64, 1, 10400, BLOCKS_OF_2, qc.QC_MODE_VLA_EQ8),    # clusters of four on 160 of 296 places
     (32, 64, 3, 3140, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),     # of two on 192
     (16, 64, 1, 9700, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),     # of eight on 128
+    (4, 64, 10, 5060, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),     # of four on 160
+    (32, 64, 10, 2130, [0, 0, 0, 0], qc.QC_MODE_VLA_QC),    # 320 blocks of four warps on 592 places
     (40, 128, 32, 1240, BLOCKS_OF_4, qc.QC_MODE_VLA_EQ8),   # a warp for each of 1 280 rows
 ])
 def test_long_rows_on_part_of_the_chip(heads, d, batch, tokens, block, mode):
@@ -100,6 +102,7 @@ def test_rows_that_are_longer_than_others_by_many_pages(heads, d, lens):
 @pytest.mark.parametrize("hq,hkv,d,lens", [
     (32, 32, 128, [(3000, 16)] + [(16, 3000)] * 7),
     (32, 8, 64, [(26, 8800), (8800, 26)] * 2 + [(26, 8800)]),
+    (40, 40, 128, [(56, 1839), (1839, 56)] * 7 + [(56, 1839)]),
 ])
 def test_a_follower_whose_text_is_mostly_one_sequences_is_not_slower_than_ranges(hq, hkv, d, lens):
     _not_slower_than_ranges(hq, hkv, d, BLOCKS_OF_2, qc.QC_MODE_VLA_QC, lens)
